@@ -45,8 +45,8 @@ def listed():
     return [
         # the smallest call: a few hundred typed markers of a pilot cohort, every statistic
         _scan("pilot_2bit_p40_full", "2bit", 777, 300, 40, 2, missing=0.02, full=True),
-        # a small cohort's typed chromosome against 16 traits, hits and best markers
-        _scan("cohort2k_2bit_p16", "2bit", 2000, 10_000, 16, 4, missing=0.01),
+        # a small cohort's typed chromosome against 16 traits, every statistic
+        _scan("cohort2k_2bit_p16_full", "2bit", 2000, 10_000, 16, 4, missing=0.01, full=True),
         # the single-trait association every biobank runs: summary statistics of a dosage block
         _scan("biobank_u8_p1_full", "u8", 23_000, 8192, 1, 19, full=True),
         # a small panel over a full block of imputed dosages: bound by reading the genotypes
