@@ -881,8 +881,8 @@ tg_status tg_prepare_panel(tg_ctx* c, const float* Y, int64_t ldy, int64_t N, in
   const int64_t k = 1 + n_cov;
   auto cleanup = [&](tg_status s) { tg_panel_free(p); return s; };
   cudaError_t e;
-  int* dint = nullptr;  // [0] rank, [1..k] kept flags
-  if ((e = dalloc(&p->X, (size_t)(2 * k * N))) || (e = dalloc(&p->Q, (size_t)(k * N))) ||
+  int* dint = nullptr;  // rank
+  if ((e = dalloc(&p->X, householder_doubles(N, k))) || (e = dalloc(&p->Q, (size_t)(k * N))) ||
       (e = dalloc(&p->Yres, (size_t)(std::max<int64_t>(P, 1) * N))) ||
       (e = dalloc(&p->s, (size_t)std::max<int64_t>(P, 1))) ||
       (e = dalloc(&p->col_s, (size_t)std::max<int64_t>(P, 1))) ||
@@ -893,7 +893,7 @@ tg_status tg_prepare_panel(tg_ctx* c, const float* Y, int64_t ldy, int64_t N, in
       (e = dalloc(&p->B32, (size_t)(p->Ppad * p->Npad))) ||
       (e = dalloc(&p->QB, (size_t)(QCOLS * p->Npad))) ||
       (e = dalloc(&p->QBhi, (size_t)(QCOLS * p->Npad))) ||
-      (e = dalloc(&p->QBlo, (size_t)(QCOLS * p->Npad))) || (e = dalloc(&dint, (size_t)(1 + k))))
+      (e = dalloc(&p->QBlo, (size_t)(QCOLS * p->Npad))) || (e = dalloc(&dint, 1)))
     return cleanup(cuda_fail(e, "tg_prepare_panel allocation"));
   auto run = [&]() -> cudaError_t {
     cudaError_t r;
@@ -904,7 +904,7 @@ tg_status tg_prepare_panel(tg_ctx* c, const float* Y, int64_t ldy, int64_t N, in
     if ((r = cudaMemsetAsync(p->col_rmul, 0, sizeof(float) * p->Ppad, st))) return r;
     if ((r = cudaMemsetAsync(p->col_cs, 0, sizeof(float) * p->Ppad, st))) return r;
     if ((r = launch_build_design(p->X, C, ldc, N, n_cov, c->scratch, st))) return r;
-    if ((r = launch_householder(p->X, N, k, p->Q, dint, dint + 1, st))) return r;
+    if ((r = launch_householder(p->X, N, k, p->Q, dint, st))) return r;
     return cudaSuccess;
   };
   if ((e = run())) { cudaFree(dint); return cleanup(cuda_fail(e, "tg_prepare_panel basis")); }

@@ -158,7 +158,7 @@ struct tg_panel {
   int64_t N = 0, P = 0, n_cov = 0, q = 0, df = 0, Npad = 0, Ppad = 0;
   int64_t NS = 0;               // samples the panel's phenotypes use (N unless a subset)
   uint32_t* samples = nullptr;  // [ceil(N/32)] bit mask of those samples (subset panels only)
-  double* X = nullptr;        // [(1+n_cov)][N] design, reduced in place by the QR
+  double* X = nullptr;        // [(1+n_cov)][N] design, reduced in place by the QR; its workspace
   double* Q = nullptr;        // [q][N] (column-major N x q)
   double* Yres = nullptr;     // [P][N]
   double* s = nullptr;        // [P]
@@ -294,8 +294,11 @@ bool make_tmap_packed(CUtensorMap* m, const void* ptr, int64_t rows, int64_t ld,
 // panel kernels (k_panel.cu)
 cudaError_t launch_build_design(double* X, const double* C, int64_t ldc, int64_t N, int64_t n_cov,
                                 uint32_t* flags, cudaStream_t st);
+// X [k][N] is followed by the reflectors and the factorisation's state: householder_doubles(N, k)
+// doubles in all.
+size_t householder_doubles(int64_t N, int64_t k);
 cudaError_t launch_householder(double* X, int64_t N, int64_t k, double* Q, int* rank_out,
-                               int* kept_out, cudaStream_t st);
+                               cudaStream_t st);
 cudaError_t launch_residualise(const float* Y, int64_t ldy, const double* Q, int64_t N, int64_t P,
                                int64_t q, int64_t Npad, double* Yres, double* s, float* col_s,
                                float* col_rmul, __nv_bfloat16* Bhi, __nv_bfloat16* Blo, float* B32,

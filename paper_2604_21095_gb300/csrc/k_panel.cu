@@ -1,7 +1,7 @@
 // Panel preparation, run once per phenotype panel (Section 2.1; Section 2.2, Eq. 1).
 //
 //   1. X = [1, C] (FP64, column-major), with a non-finite check of C.
-//   2. Householder QR of X in one thread block: a column whose remaining norm is at most
+//   2. Householder QR of X: a column whose remaining norm is at most
 //      1e-9 of its own norm is dropped (rank detection); Q = H_0 ... H_{q-1} [I_q; 0].
 //   3. Per phenotype: Y_res = (I - Q Q^T)(Y - Ybar), s_p = |y_res|, and the unit-norm column
 //      y_res / s_p written as FP32 and as a BF16 pair hi = bf16(y), lo = bf16(y - hi).
@@ -15,6 +15,9 @@
 // phenotype's finite-value mask, from which such subsets are formed.
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
+
+#include <algorithm>
+#include <mutex>
 
 #include "device.cuh"
 #include "internal.h"
@@ -39,76 +42,239 @@ __global__ void k_build_design(double* __restrict__ X, const double* __restrict_
   if (bad) atomicOr(flags, 1u);
 }
 
-// One block of 1024 threads. X [k][N] is reduced in place; V keeps the reflectors.
-__global__ void __launch_bounds__(1024) k_householder(double* __restrict__ X, long long N, int k,
-                                                       double* __restrict__ V,
-                                                       double* __restrict__ Q, int* rank_out,
-                                                       int* kept_out) {
-  __shared__ double red[33];
-  __shared__ double own[QMAX];
-  __shared__ int vrow[QMAX];
-  __shared__ double vbeta[QMAX];
-  const int tid = threadIdx.x, nt = blockDim.x;
-  for (int j = 0; j < k; ++j) {
-    double s = 0.0;
-    for (long long i = tid; i < N; i += nt) s += X[j * N + i] * X[j * N + i];
-    s = block_sum(s, red);
-    if (tid == 0) own[j] = sqrt(s);
+// Householder QR of X [k][N] (reduced in place) over the whole GPU, one launch per column.
+//
+// What bounds it is not the arithmetic (N k^2 FP64 operations, 9 M at N = 23,000, k = 20) but
+// the chain of k dependent reductions over N. Reducing one column at a time against every later
+// column in a single block (two block-wide reductions per pair of columns, 1 SM) took 6.79 ms at
+// N = 23,000, k = 20; here each column costs one launch over all SMs, 0.42 ms in all. A step
+// needs only the Gram row g_c = sum_{i >= row} x_j[i] x_c[i], c >= j, of the current column: the
+// reflector is v = x_j + s |x_j| e_row, so v . x_c = g_c + s |x_j| x_c[row] for every later
+// column at once, and the pass that applies the reflector also sums the next column's Gram row.
+// Launches, not a grid-wide barrier, order the steps: every block adds the previous step's
+// per-block partial sums in the same order, so all take the same decisions, and nothing spins.
+// Row `row` of the reflector of kept column number q is row q, so the basis is
+// Q = E - V T (V^T E) (the compact form of H_0 ... H_{q-1} applied to the first q unit vectors),
+// one Gram of the reflectors and one pass over the rows.
+constexpr int kQrThreads = 256;
+constexpr int kQrBlocks = 152;
+constexpr int kQrCols = 8;  // columns whose sums a thread carries at once
+
+// Device state of the factorisation, in doubles: the partial sums of two successive steps
+// [2][kQrBlocks][2 k], the pivot rows [2][k], the columns' own norms [k], the reflectors' betas
+// [k], the number of columns kept before step j [k + 1] and the reflectors' Gram [k][k].
+struct QrWork {
+  double *part, *piv, *own, *beta, *kept, *gram;
+};
+__host__ __device__ inline QrWork qr_work(double* w, int k) {
+  QrWork r;
+  r.part = w;
+  r.piv = r.part + (size_t)2 * kQrBlocks * 2 * k;
+  r.own = r.piv + 2 * k;
+  r.beta = r.own + k;
+  r.kept = r.beta + k;
+  r.gram = r.kept + k + 1;
+  return r;
+}
+
+// The warp's sums of 8 per-lane values: lane l returns the sum of column
+// 4 [l & 16] + 2 [l & 8] + [l & 4]. Halving the columns as the lanes pair up takes 9 FP64 adds
+// per lane instead of 40 (FP64 runs at 2 lanes per cycle and SM).
+__device__ __forceinline__ double warp_sum8(const double (&a)[kQrCols], int lane) {
+  double b[4], c[2];
+  const bool h16 = lane & 16, h8 = lane & 8, h4 = lane & 4;
+#pragma unroll
+  for (int u = 0; u < 4; ++u)
+    b[u] = (h16 ? a[u + 4] : a[u]) + __shfl_xor_sync(0xffffffffu, h16 ? a[u] : a[u + 4], 16);
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+    c[u] = (h8 ? b[u + 2] : b[u]) + __shfl_xor_sync(0xffffffffu, h8 ? b[u] : b[u + 2], 8);
+  double d = (h4 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h4 ? c[0] : c[1], 4);
+  d += __shfl_xor_sync(0xffffffffu, d, 2);
+  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+
+// Block sums of 8 columns into out[0 .. n), n <= 8.
+__device__ __forceinline__ void block_sum8(const double (&a)[kQrCols], int n,
+                                           double (*red)[kQrCols], double* out) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const double s = warp_sum8(a, lane);
+  if ((lane & 3) == 0) red[warp][((lane >> 4) & 1) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] = s;
+  __syncthreads();
+  if ((int)threadIdx.x < n) {
+    double t = 0.0;
+#pragma unroll
+    for (int w = 0; w < kQrThreads / 32; ++w) t += red[w][threadIdx.x];
+    out[threadIdx.x] = t;
   }
   __syncthreads();
-  int row = 0, q = 0;
-  for (int j = 0; j < k && row < N; ++j) {
-    double* x = X + (long long)j * N;
+}
+
+// The columns' own sums of squares (partials [k, 2k)) and the first column's Gram row ([0, k)).
+__global__ void __launch_bounds__(kQrThreads) k_qr_first(const double* __restrict__ X, long long N,
+                                                         int k, double* work) {
+  __shared__ double red[kQrThreads / 32][kQrCols];
+  const QrWork w = qr_work(work, k);
+  const long long step = (long long)gridDim.x * kQrThreads;
+  const long long t0 = blockIdx.x * (long long)kQrThreads + threadIdx.x;
+  double* out = w.part + (size_t)blockIdx.x * 2 * k;
+  for (int c0 = 0; c0 < k; c0 += kQrCols) {
+    double g[kQrCols] = {}, o[kQrCols] = {};
+    for (long long i = t0; i < N; i += step) {
+      const double x0 = X[i];
+#pragma unroll
+      for (int u = 0; u < kQrCols; ++u)
+        if (c0 + u < k) {
+          const double v = X[(long long)(c0 + u) * N + i];
+          g[u] = fma(x0, v, g[u]);
+          o[u] = fma(v, v, o[u]);
+        }
+    }
+    const int n = k - c0 < kQrCols ? k - c0 : kQrCols;
+    block_sum8(g, n, red, out + c0);
+    block_sum8(o, n, red, out + k + c0);
+  }
+  if (t0 == 0) {
+    for (int c = 0; c < k; ++c) w.piv[c] = X[(long long)c * N];
+    w.kept[0] = 0.0;
+  }
+}
+
+// Step j: the reflector of column j (none if the column is dropped: what is left of it is at most
+// kRankTol of its own norm), its application to the later columns, and the Gram row of column
+// j + 1 below the next row.
+__global__ void __launch_bounds__(kQrThreads) k_qr_step(double* __restrict__ X,
+                                                        double* __restrict__ V, long long N, int k,
+                                                        int j, double* work, int* rank_out) {
+  __shared__ double red[kQrThreads / 32][kQrCols];
+  __shared__ double sums[2 * QMAX];
+  __shared__ double coef[QMAX];
+  const QrWork w = qr_work(work, k);
+  const int tid = threadIdx.x, nb = gridDim.x;
+  const double* in = w.part + (size_t)(j & 1) * kQrBlocks * 2 * k;
+  double* out = w.part + (size_t)((j + 1) & 1) * kQrBlocks * 2 * k + (size_t)blockIdx.x * 2 * k;
+  const double* piv = w.piv + (j & 1) * k;
+  // the previous launch's partial sums, four threads to a column, in the same order in every block
+  const int ncol = j == 0 ? 2 * k : k;
+  for (int c0 = j; c0 < ncol; c0 += kQrThreads / 4) {
+    const int c = c0 + tid / 4;
     double s = 0.0;
-    for (long long i = row + tid; i < N; i += nt) s += x[i] * x[i];
-    s = block_sum(s, red);
-    const double nrm = sqrt(s);
-    if (own[j] == 0.0 || nrm <= kRankTol * own[j]) {
-      if (tid == 0) kept_out[j] = 0;
-      continue;
-    }
-    const double x0 = x[row];
-    const double sg = (x0 >= 0.0) ? 1.0 : -1.0;
-    // v = x + sg |x| e_row (rows >= row); |v|^2 = 2 |x|^2 + 2 |x0| |x|
-    double* v = V + (long long)q * N;
-    for (long long i = row + tid; i < N; i += nt) v[i] = (i == row) ? x0 + sg * nrm : x[i];
-    const double beta = 2.0 / (2.0 * s + 2.0 * fabs(x0) * nrm);
-    __syncthreads();
-    for (int c = j + 1; c < k; ++c) {
-      double* xc = X + (long long)c * N;
-      double d = 0.0;
-      for (long long i = row + tid; i < N; i += nt) d += v[i] * xc[i];
-      d = block_sum(d, red) * beta;
-      for (long long i = row + tid; i < N; i += nt) xc[i] -= d * v[i];
-      __syncthreads();
-    }
+    if (c < ncol)
+      for (int b = tid & 3; b < nb; b += 4) s += in[(size_t)b * 2 * k + c];
+    s += __shfl_xor_sync(0xffffffffu, s, 1);
+    s += __shfl_xor_sync(0xffffffffu, s, 2);
+    if (c < ncol && (tid & 3) == 0) sums[c] = s;
+  }
+  __syncthreads();
+  const int q = (int)w.kept[j];  // columns kept so far = this reflector's row
+  const double s = sums[j], nrm = sqrt(s);
+  const double own = j == 0 ? sqrt(sums[k]) : w.own[j];
+  const bool keep = q < N && !(own == 0.0 || nrm <= kRankTol * own);
+  const double x0 = piv[j], shift = (x0 >= 0.0 ? 1.0 : -1.0) * nrm;
+  // v = x + sign(x0) |x| e_row, |v|^2 = 2 |x|^2 + 2 |x0| |x|
+  const double beta = keep ? 2.0 / (2.0 * s + 2.0 * fabs(x0) * nrm) : 0.0;
+  if (tid > j && tid < k) coef[tid] = beta * (sums[tid] + shift * piv[tid]);
+  const int row = keep ? q + 1 : q;  // the next step's row
+  if (blockIdx.x == 0) {
+    if (j == 0 && tid < k) w.own[tid] = sqrt(sums[k + tid]);
     if (tid == 0) {
-      kept_out[j] = 1;
-      vrow[q] = row;
-      vbeta[q] = beta;
+      if (keep) w.beta[q] = beta;
+      w.kept[j + 1] = (double)row;
+      if (j == k - 1) *rank_out = row;
+    }
+  }
+  __syncthreads();
+  double* pnext = w.piv + ((j + 1) & 1) * k;
+  const double* xj = X + (long long)j * N;
+  double* v = V + (long long)q * N;
+  const long long step = (long long)nb * kQrThreads;
+  const long long t0 = blockIdx.x * (long long)kQrThreads + tid;
+  if (j == k - 1) {
+    if (keep)
+      for (long long i = t0; i < N; i += step)
+        v[i] = i < q ? 0.0 : i == q ? x0 + shift : xj[i];
+    return;
+  }
+  for (int c0 = j + 1; c0 < k; c0 += kQrCols) {
+    const int n = k - c0 < kQrCols ? k - c0 : kQrCols;
+    double g[kQrCols] = {};
+    for (long long i = t0; i < N; i += step) {
+      const double vi = i < q ? 0.0 : i == q ? x0 + shift : xj[i];
+      if (keep && c0 == j + 1) v[i] = vi;
+      if (i < q) continue;
+      double xn = 0.0;  // column j + 1 after this reflector (updated in the first group)
+      if (c0 > j + 1) xn = X[(long long)(j + 1) * N + i];
+#pragma unroll
+      for (int u = 0; u < kQrCols; ++u)
+        if (u < n) {
+          double* xc = X + (long long)(c0 + u) * N + i;
+          double x = *xc;
+          if (keep) {
+            x = fma(-coef[c0 + u], vi, x);
+            *xc = x;
+          }
+          if (u == 0 && c0 == j + 1) xn = x;
+          if (i == row) pnext[c0 + u] = x;
+          if (i >= row) g[u] = fma(xn, x, g[u]);
+        }
+    }
+    block_sum8(g, n, red, out + c0);
+  }
+}
+
+// gram[a][b] = v_a . v_b of the reflectors, a < b, one block per pair.
+__global__ void __launch_bounds__(256) k_qr_gram(const double* __restrict__ V, long long N, int k,
+                                                 double* work) {
+  __shared__ double red[33];
+  const QrWork w = qr_work(work, k);
+  const int a = blockIdx.x, b = blockIdx.y, q = (int)w.kept[k];
+  if (a >= b || b >= q) return;
+  double s = 0.0;
+  for (long long i = b + threadIdx.x; i < N; i += blockDim.x)  // v_b is zero above row b
+    s = fma(V[(long long)a * N + i], V[(long long)b * N + i], s);
+  s = block_sum(s, red);
+  if (threadIdx.x == 0) w.gram[a * k + b] = s;
+}
+
+// Q = E - V W with W = T V_top^T: T the upper triangular factor of the compact form
+// (T_jj = beta_j, T_ij = -beta_j sum_{i <= m < j} T_im gram_mj), V_top the first q rows of V.
+// Every block forms T and W for itself (q^3 / 3 operations), then its rows.
+__global__ void __launch_bounds__(256) k_qr_basis(const double* __restrict__ V, long long N, int k,
+                                                  double* work, double* __restrict__ Q) {
+  extern __shared__ double tw[];  // T [k][k], W [k][k]
+  const QrWork w = qr_work(work, k);
+  const int q = (int)w.kept[k], tid = threadIdx.x;
+  double *T = tw, *W = tw + k * k;
+  for (int j = 0; j < q; ++j) {
+    if (tid == j) T[j * k + j] = w.beta[j];
+    if (tid < j) {
+      double s = 0.0;
+      for (int m = tid; m < j; ++m) s = fma(T[tid * k + m], w.gram[m * k + j], s);
+      T[tid * k + j] = -w.beta[j] * s;
     }
     __syncthreads();
-    ++row;
-    ++q;
   }
-  // Q[:, c] = H_0 ... H_{q-1} e_c, applying the reflectors in reverse order.
-  for (int c = 0; c < q; ++c)
-    for (long long i = tid; i < N; i += nt) Q[(long long)c * N + i] = (i == c) ? 1.0 : 0.0;
+  for (int e = tid; e < q * q; e += blockDim.x) {
+    const int a = e / q, c = e - a * q;
+    double s = 0.0;
+    for (int b = a; b <= c; ++b) s = fma(T[a * k + b], V[(long long)b * N + c], s);
+    W[a * k + c] = s;
+  }
   __syncthreads();
-  for (int r = q - 1; r >= 0; --r) {
-    const double* v = V + (long long)r * N;
-    const long long r0 = vrow[r];
-    const double beta = vbeta[r];
-    for (int c = r; c < q; ++c) {
-      double* qc = Q + (long long)c * N;
-      double d = 0.0;
-      for (long long i = r0 + tid; i < N; i += nt) d += v[i] * qc[i];
-      d = block_sum(d, red) * beta;
-      for (long long i = r0 + tid; i < N; i += nt) qc[i] -= d * v[i];
-      __syncthreads();
+  for (long long i = blockIdx.x * (long long)blockDim.x + tid; i < N;
+       i += (long long)gridDim.x * blockDim.x)
+    for (int c0 = 0; c0 < q; c0 += kQrCols) {
+      double s[kQrCols] = {};
+      for (int a = 0; a < q; ++a) {
+        const double va = V[(long long)a * N + i];
+#pragma unroll
+        for (int u = 0; u < kQrCols; ++u)
+          if (c0 + u < q) s[u] = fma(va, W[a * k + c0 + u], s[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < kQrCols; ++u)
+        if (c0 + u < q) Q[(long long)(c0 + u) * N + i] = (i == c0 + u ? 1.0 : 0.0) - s[u];
     }
-  }
-  if (tid == 0) *rank_out = q;
 }
 
 // One block per phenotype column.
@@ -347,10 +513,30 @@ cudaError_t launch_build_design(double* X, const double* C, int64_t ldc, int64_t
   return cudaGetLastError();
 }
 
+size_t householder_doubles(int64_t N, int64_t k) {
+  // X, the reflectors V, the state of the factorisation
+  return (size_t)(2 * k * N) + (size_t)2 * kQrBlocks * 2 * k + 2 * k + k + k + (k + 1) + k * k;
+}
+
 cudaError_t launch_householder(double* X, int64_t N, int64_t k, double* Q, int* rank_out,
-                               int* kept_out, cudaStream_t st) {
-  // The reflectors are stored after the k columns of X (the caller allocates 2k columns).
-  k_householder<<<1, 1024, 0, st>>>(X, N, (int)k, X + k * N, Q, rank_out, kept_out);
+                               cudaStream_t st) {
+  double* V = X + k * N;
+  double* work = V + k * N;
+  const size_t smem = sizeof(double) * 2 * (size_t)(k * k);  // 64 KB at the largest k
+  static std::once_flag once;
+  static cudaError_t attr = cudaSuccess;
+  std::call_once(once, [] {
+    attr = cudaFuncSetAttribute(k_qr_basis, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)(sizeof(double) * 2 * QMAX * QMAX));
+  });
+  if (attr != cudaSuccess) return attr;
+  // blocks of a row or so per thread, at most one per SM
+  const unsigned nb = (unsigned)std::min<int64_t>(kQrBlocks, (N + kQrThreads - 1) / kQrThreads);
+  k_qr_first<<<nb, kQrThreads, 0, st>>>(X, N, (int)k, work);
+  for (int64_t j = 0; j < k; ++j)
+    k_qr_step<<<nb, kQrThreads, 0, st>>>(X, V, N, (int)k, (int)j, work, rank_out);
+  k_qr_gram<<<dim3((unsigned)k, (unsigned)k), 256, 0, st>>>(V, N, (int)k, work);
+  k_qr_basis<<<nb, 256, smem, st>>>(V, N, (int)k, work, Q);
   return cudaGetLastError();
 }
 

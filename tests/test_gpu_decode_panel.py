@@ -162,6 +162,33 @@ def test_panel_matches_oracle(tgctx, N, P, n_cov):
         tg.tg_panel_free(panel)
 
 
+@pytest.mark.parametrize("N,n_cov,dup", [(130, 63, False), (256, 8, True), (257, 7, False),
+                                         (38912, 15, True), (38913, 3, False)])
+def test_basis_at_the_edges_of_its_launches(tgctx, N, n_cov, dup):
+    """The covariate basis with the most columns, with sample counts either side of one block's
+    rows and of one row per thread of the whole grid, and with dropped columns: the FP64 QR's own
+    basis, to k eps cond(X) (at most 1e-13 for these normal covariates) within 1e-12, and
+    orthonormal columns."""
+    cov = synth.covariates(N + n_cov, N, n_cov)
+    if dup:  # dropped columns in the middle and at the end
+        cov[n_cov // 2] = cov[0] - 3.0 * cov[1]
+        cov[-1] = 2.0 * cov[0]
+    Yt = synth.phenotypes(N, cov, 3)
+    panel = tg.tg_prepare_panel(tgctx, Yt.cuda(), N, 3, cov.cuda())
+    try:
+        ref = oracle.prepare_panel(Yt.numpy().T.astype(np.float64), cov.numpy().T)
+        assert tg.tg_panel_info(panel)[2] == ref["q"] == 1 + n_cov - (2 if dup else 0)
+        Q = tg.tg_panel_Q(panel).cpu().numpy().T[:, :ref["q"]]
+        assert np.allclose(Q, ref["Q"], atol=1e-12, rtol=0)
+        assert np.allclose(Q.T @ Q, np.eye(ref["q"]), atol=1e-12, rtol=0)
+        Yres, s = tg.tg_panel_Yres(panel)
+        scale = np.linalg.norm(ref["Y"] - ref["Y"].mean(0), axis=0).max()
+        assert np.allclose(Yres.cpu().numpy().T, ref["Yres"], atol=1e-11 * scale, rtol=0)
+        assert np.allclose(s.cpu().numpy(), ref["s"], rtol=1e-12)
+    finally:
+        tg.tg_panel_free(panel)
+
+
 def test_panel_rank_detection(tgctx):
     N, P = 500, 4
     cov = synth.covariates(3, N, 4)
