@@ -141,15 +141,13 @@ struct StageScope {
 cudaError_t ensure_markers(tg_ctx* c, int64_t M) {
   if (M <= c->cap_m) return cudaSuccess;
   const int64_t cap = round_up(M, MT);
-  dfree(c->nobs); dfree(c->mean); dfree(c->shift); dfree(c->mh); dfree(c->gc2s); dfree(c->gc2); dfree(c->qg);
-  dfree(c->gres2); dfree(c->rinv); dfree(c->rinv64); dfree(c->refine_list);
+  dfree(c->nobs); dfree(c->mean); dfree(c->shift); dfree(c->mh); dfree(c->gc2s); dfree(c->gc2);
+  dfree(c->rinv); dfree(c->rinv64);
   c->cap_m = 0;
   cudaError_t e;
   if ((e = dalloc(&c->nobs, cap)) || (e = dalloc(&c->mean, cap)) || (e = dalloc(&c->shift, cap)) ||
       (e = dalloc(&c->mh, cap)) || (e = dalloc(&c->gc2s, cap)) ||
-      (e = dalloc(&c->gc2, cap)) || (e = dalloc(&c->qg, cap * JCOLS)) ||
-      (e = dalloc(&c->gres2, cap)) || (e = dalloc(&c->rinv, cap)) || (e = dalloc(&c->rinv64, cap)) ||
-      (e = dalloc(&c->refine_list, cap)))
+      (e = dalloc(&c->gc2, cap)) || (e = dalloc(&c->rinv, cap)) || (e = dalloc(&c->rinv64, cap)))
     return e;
   c->cap_m = cap;
   return cudaSuccess;
@@ -175,76 +173,142 @@ cudaError_t ensure_operands(tg_ctx* c, int64_t M, int64_t Npad, int prec) {
   return cudaSuccess;
 }
 
-// Split-K of the one-CTA kernel for a block of M markers: for a panel of at most 64 phenotypes
-// (64-column tiles) it is chosen by rule, for wider panels it is the tuned value. A split pays
-// only while the tiles are fewer than the SMs; every split keeps at least one 1,024-sample chunk.
-struct SplitChoice {
-  int ks = 1;
-  int64_t tiles = 0;
+cudaError_t ensure_raw(tg_ctx* c, size_t floats) {
+  if (floats <= c->cap_raw) return cudaSuccess;
+  dfree(c->raw);
+  c->cap_raw = 0;
+  cudaError_t e = dalloc(&c->raw, floats);
+  if (e == cudaSuccess) c->cap_raw = floats;
+  return e;
+}
+
+// Ranges that K (`chunks` accumulation chunks of 1,024 samples) is split into for `tiles` tiles on
+// `slots` CTAs or CTA pairs: the count with the shortest estimated pass, the rounds of work items
+// times what one takes (its longest range at chunk_us per chunk, and item_us to fill the pipeline
+// and to store), plus the traffic of the ranges' partial sums (range_bytes written and read
+// back each). A split is taken for at least 3%. Without one, a block of few tiles leaves most
+// SMs idle behind one long K loop: 675 markers x 346 columns x 5,001 samples took 54 + 74 us
+// in the projection and the contraction, whatever the marker count up to 4,000.
+constexpr double kChunkUs64 = 6.6, kChunkUs128 = 9.0;  // one-CTA kernel, per chunk of a 128-marker tile
+constexpr double kChunkUsCol = 0.0337;  // CTA-pair kernel, per chunk and column of a 256-marker tile
+constexpr double kItemUs = 4.0;
+constexpr double kRangeBytesPerUs = 6.0e6;
+constexpr size_t kMaxSplitFloats = size_t(1) << 26;  // partial sums of a split: 256 MiB at most
+int pick_ranges(int64_t tiles, int64_t slots, int64_t chunks, double chunk_us, double range_floats) {
+  int best = 1;
+  double best_us = 0;
+  for (int64_t ks = 1; ks <= chunks; ++ks) {
+    const int64_t per = (chunks + ks - 1) / ks;
+    if (ks > 1 && ((ks - 1) * per >= chunks || ks * range_floats > (double)kMaxSplitFloats)) continue;
+    const double rounds = (double)((tiles * ks + slots - 1) / slots);
+    const double us = rounds * ((double)per * chunk_us + kItemUs) +
+                      (double)ks * range_floats * 8.0 / kRangeBytesPerUs;
+    if (ks == 1 || us < 0.97 * best_us) {
+      best = (int)ks;
+      best_us = us;
+    }
+  }
+  return best;
+}
+
+// How a block is scanned: the passes, their splits and the workspace they need.
+struct Plan {
+  bool split = false;       // the split form (else FP32)
+  int64_t nq = 0;           // projection columns
+  bool joint = false;       // projection and panel products in one raw pass
+  bool fuse_joint = false;  // ... that decodes the packed rows itself (joint operand of <= 128 rows)
+  bool fuse_proj = false;   // projection pass over the packed rows that writes the operand
+  bool one_pass = false;    // ... and takes the marker statistics too
+  bool dec = false;         // contraction kernels decode the packed rows (no operand in HBM)
+  bool single = false;      // the panel's contraction on one CTA per tile
+  int ranges_proj = 1;      // K ranges of the projection or joint pass
+  int ranges_scan = 1;      // K ranges of the panel's own contraction (> 1: raw, then k_raw_stats)
+  int64_t ldr = 0;          // rows of the raw products' columns
+  size_t raw_floats = 0;
+  bool operand = false;     // the decoded operand is needed
 };
-SplitChoice pick_split(const tg_ctx* c, const tg_panel* p, int64_t M, bool single,
-                       bool projection = false) {
-  SplitChoice r;
-  const int64_t n_mt = (M + MT - 1) / MT;
-  const bool narrow = projection || p->P <= 64;  // the projection has one 64-column tile
-  r.tiles = n_mt * (narrow ? 1 : (p->P + 255) / 256);
-  int ks = 1;
-  if (narrow) {
-    while (ks < 4 && r.tiles * ks * 2 <= c->sm_count) ks *= 2;
-  } else if (single) {
-    const int t = c->tune_split[tune_bucket(M)];
-    ks = t > 1 ? t : 1;
+
+Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int encoding,
+               const uint32_t* missing, const tg_scan_opts& opts) {
+  Plan r;
+  r.split = opts.precision == TG_PREC_SPLIT_BF16;
+  r.nq = opts.mode == TG_MODE_PAPER ? 0 : p->q - 1;
+  r.ldr = round_up(M, 32);
+  const int64_t n_mt = (M + MT - 1) / MT, n_mp = (n_mt + 1) / 2;
+  const bool wide_block = n_mt >= c->sm_count;  // at least one 128-marker tile per SM
+  const bool packed_ok = r.split && c->fuse_joint && missing == nullptr && r.nq > 0 && wide_block;
+  // a small panel's joint projection pass (projected form, joint operand of at most 128 rows,
+  // at least one 128-marker tile per SM) reads the packed rows and decodes them in shared memory
+  r.fuse_joint = packed_ok && p->joint_cols > 0 && p->joint_cols <= 128 && p->QYhi16 != nullptr;
+  // a panel with P + q - 1 > JCOLS: the projection runs as the same pass with the 64 projection
+  // columns alone, which reads the packed rows and also writes the block's operand as it expands
+  // them, so the operand is written once and read once, by the panel's contraction
+  r.fuse_proj = packed_ok && !r.fuse_joint && !c->fuse_decode && p->QBhi16 != nullptr &&
+                p->joint_cols == 0;
+  // split-form 2-bit blocks and unmasked dosage blocks are decoded inside the contraction
+  // kernels when the context asks for it; the rest go through a decoded operand in HBM
+  r.dec = r.split && missing == nullptr && (c->fuse_decode || r.fuse_joint);
+  r.operand = !r.dec;
+  // dosage rows in the joint pass (or the projection pass that writes the operand) on 256-row
+  // tiles: that pass writes the row statistics itself (a thread holds a whole row), so no
+  // counting pass reads the block first
+  r.one_pass = (r.fuse_joint || r.fuse_proj) && encoding == TG_ENC_U8_DOSAGE && N <= kOnePassMaxN &&
+               joint_fused_rows(M, c->sm_count, r.fuse_proj ? QCOLS : p->joint_cols) == 2 * MT;
+  // P + q - 1 <= JCOLS: one pass over the operand gives the projection and the panel's products
+  // (raw); the statistics follow the norms
+  r.joint = r.split && r.nq > 0 && p->joint_cols > 0;
+  const int64_t chunks = (p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB;
+  const double ldr = (double)r.ldr;
+  const int64_t pairs = c->sm_count / 2;
+  if (r.split && r.nq > 0 && !r.fuse_joint && !r.fuse_proj) {
+    if (r.joint && p->joint_cols > 128) {
+      r.ranges_proj = pick_ranges(n_mp * (p->joint_cols / p->joint_bn), pairs, chunks,
+                                  kChunkUsCol * p->joint_bn, ldr * (double)(r.nq + p->P));
+    } else {
+      r.ranges_proj = pick_ranges(n_mt, c->sm_count, chunks,
+                                  r.joint && p->joint_cols > 64 ? kChunkUs128 : kChunkUs64,
+                                  ldr * (double)(r.nq + (r.joint ? p->P : 0)));
+    }
   }
-  const int chunks = (int)((p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB);
-  while (ks > 1 && (ks > chunks || ks > c->sm_count)) ks /= 2;
-  r.ks = ks;
+  if (r.nq > 0)
+    r.raw_floats = (size_t)r.ranges_proj * (size_t)(r.nq + (r.joint ? p->P : 0)) * (size_t)r.ldr;
+  if (r.split && !r.joint && p->P > 0) {
+    const int tuned = c->tune_split[tune_bucket(M)];
+    const double cols = (double)p->P;
+    if (p->P <= 64) {  // a small panel without projection columns: 64-column tiles, bound by HBM
+      r.single = true;
+      r.ranges_scan = pick_ranges(n_mt, c->sm_count, chunks, kChunkUs64, ldr * cols);
+    } else if (c->tune_kernel[tune_bucket(M)] == TUNE_SINGLE) {
+      r.single = true;
+      r.ranges_scan = (int)std::min<int64_t>(tuned > 1 ? tuned : 1, chunks);
+    } else {
+      r.ranges_scan = pick_ranges(n_mp * ((p->P + p->bn - 1) / p->bn), pairs, chunks,
+                                  kChunkUsCol * p->bn, ldr * cols);
+    }
+    if (r.ranges_scan > 1)
+      r.raw_floats = std::max(r.raw_floats,
+                              (size_t)r.ranges_scan * (size_t)p->P * (size_t)r.ldr);
+  }
   return r;
-}
-size_t split_bytes(const SplitChoice& sc) {
-  return sc.ks > 1 ? (size_t)sc.tiles * (size_t)(sc.ks - 1) * (size_t)(MT * 256) * sizeof(float) : 0;
-}
-cudaError_t ensure_split(tg_ctx* c, const SplitChoice& sc) {
-  const size_t need = split_bytes(sc);
-  if (need > c->sk_ws_bytes) {
-    dfree(c->sk_ws);
-    c->sk_ws_bytes = 0;
-    cudaError_t e = cudaMalloc(reinterpret_cast<void**>(&c->sk_ws), need);
-    if (e != cudaSuccess) return e;
-    c->sk_ws_bytes = need;
-  }
-  if (sc.ks > 1 && sc.tiles > c->sk_cnt_cap) {
-    dfree(c->sk_cnt);
-    c->sk_cnt_cap = 0;
-    cudaError_t e = dalloc(&c->sk_cnt, (size_t)sc.tiles);
-    if (e != cudaSuccess) return e;
-    c->sk_cnt_cap = sc.tiles;
-  }
-  return cudaSuccess;
-}
-bool split_fits(const tg_ctx* c, const SplitChoice& sc) {
-  return split_bytes(sc) <= c->sk_ws_bytes && (sc.ks <= 1 || sc.tiles <= c->sk_cnt_cap);
 }
 
 // Size the context's workspace for the scans a graph will capture: nothing may allocate inside
 // a capture. A workspace that another live graph has captured cannot move, so while one exists
 // only a graph whose blocks fit the current buffers is accepted.
+bool operand_fits(const tg_ctx* c, int64_t M, int64_t Npad, int prec) {
+  return round_up(M, MT) <= c->cap_rows && Npad <= c->cap_npad &&
+         (prec == TG_PREC_FP32 ? c->A32 != nullptr : c->Ahi != nullptr);
+}
 tg_status reserve_graph_workspace(tg_ctx* c, const tg_panel* p, int n_blocks, const int64_t* M,
-                                  int64_t maxM, bool need_operand, const tg_scan_opts& opts) {
-  const bool split = opts.precision == TG_PREC_SPLIT_BF16;
-  std::vector<SplitChoice> need;
-  for (int b = 0; b < n_blocks; ++b) {
-    if (split && (p->P <= 64 || c->tune_kernel[tune_bucket(M[b])] == TUNE_SINGLE))
-      need.push_back(pick_split(c, p, M[b], true));
-    if (split && opts.mode == TG_MODE_PROJECTED && p->q > 1)
-      need.push_back(pick_split(c, p, M[b], true, true));
-  }
+                                  int64_t maxM, bool need_operand, int encoding,
+                                  const uint32_t* const* missing, const tg_scan_opts& opts) {
+  size_t raw = 0;
+  for (int b = 0; b < n_blocks; ++b)
+    raw = std::max(raw, make_plan(c, p, p->N, M[b], encoding, missing ? missing[b] : nullptr, opts)
+                            .raw_floats);
   if (c->graphs_alive > 0) {
-    bool fits = maxM <= c->cap_m;
-    if (need_operand)
-      fits = fits && round_up(maxM, MT) <= c->cap_rows && p->Npad <= c->cap_npad &&
-             (opts.precision == TG_PREC_FP32 ? c->A32 != nullptr : c->Ahi != nullptr);
-    for (const SplitChoice& sc : need) fits = fits && split_fits(c, sc);
-    if (!fits)
+    if (maxM > c->cap_m || raw > c->cap_raw ||
+        (need_operand && !operand_fits(c, maxM, p->Npad, opts.precision)))
       return fail(TG_ERR_INVALID_ARG,
                   "another captured scan graph holds this context's workspace: capture the "
                   "largest blocks first, or use another context");
@@ -252,7 +316,7 @@ tg_status reserve_graph_workspace(tg_ctx* c, const tg_panel* p, int n_blocks, co
   }
   TG_CUDA(ensure_markers(c, maxM));
   if (need_operand) TG_CUDA(ensure_operands(c, maxM, p->Npad, opts.precision));
-  for (const SplitChoice& sc : need) TG_CUDA(ensure_split(c, sc));
+  TG_CUDA(ensure_raw(c, raw));
   return TG_OK;
 }
 
@@ -349,11 +413,13 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
   const tg_status ps = ensure_fp4_panel(c, p, st);
   if (ps != TG_OK) return ps;
   TG_CUDA(ensure_markers(c, a.M));
-  const int64_t lda = p->Npad / 2;
+  const int64_t lda = p->Npad / 2, ldr = round_up(a.M, 32);
+  const size_t raw = (size_t)(QCOLS * ldr);
   const int64_t need = round_up(a.M, MT) * lda;
+  if (c->graphs_alive > 0 && (need > c->cap_fp4 || raw > c->cap_raw))
+    return fail(TG_ERR_INVALID_ARG, "the context's workspace is held by a captured scan graph");
+  TG_CUDA(ensure_raw(c, raw));
   if (need > c->cap_fp4) {
-    if (c->graphs_alive > 0)
-      return fail(TG_ERR_INVALID_ARG, "the context's workspace is held by a captured scan graph");
     dfree(c->Afp4);
     c->Afp4 = nullptr;
     c->cap_fp4 = 0;
@@ -378,23 +444,20 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
     pp.row_shift = c->shift;
     pp.col_cs = p->fp4Q_cs;
     pp.col_rmul = p->fp4Q_scale;
-    pp.raw_out = c->qg;
+    pp.raw_out = c->raw;
     pp.raw_cols = (int)nq;
-    pp.raw_ld = QCOLS;
+    pp.raw_ld = ldr;
     TG_CUDA(launch_fp4_scan(&tA, &p->tmFQ, QCOLS, p->Npad, pp, c->sm_count, kSpinNs, st));
   }
+  unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
+  const bool want_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
   {
-    StageScope s(c, STAGE_NORM, st, nq > 0 ? 2 : 1);
-    const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, nullptr, 0, c->mean, p->Q, (int)p->q,
-                          c->refine_list, c->scratch + 40};
-    TG_CUDA(launch_marker_norm(a.M, c->nobs, c->gc2, c->qg, QCOLS, nq, 1.0, c->gres2,
-                               a.out.marker_norm2, c->rinv, c->rinv64, &rf, st, a.N));
-    if (a.out.marker_nobs)
-      TG_CUDA(cudaMemcpyAsync(a.out.marker_nobs, c->nobs, sizeof(int32_t) * a.M,
-                              cudaMemcpyDeviceToDevice, st));
-    if (a.out.marker_mean)
-      TG_CUDA(cudaMemcpyAsync(a.out.marker_mean, c->mean, sizeof(double) * a.M,
-                              cudaMemcpyDeviceToDevice, st));
+    StageScope s(c, STAGE_NORM, st, 1);
+    const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, nullptr, 0, c->mean, p->Q, (int)p->q};
+    const NormOut no{a.out.marker_norm2, c->rinv, c->rinv64, a.out.marker_nobs, a.out.marker_mean,
+                     want_hits ? hit_start : nullptr, a.out.n_hits};
+    TG_CUDA(launch_marker_norm(a.M, c->nobs, c->gc2, RawView{c->raw, ldr, 0, 1, nullptr, nullptr},
+                               nq, 1.0, rf, no, st, a.N));
   }
   EpiParams ep{};
   ep.M = (int)a.M;
@@ -404,7 +467,7 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
   ep.df_f = (float)ep.df;
   ep.kappa = 1.0f;
   ep.kappa64 = 1.0;
-  ep.do_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
+  ep.do_hits = want_hits;
   ep.r2_thr = ep.do_hits ? (float)host_r2_threshold(a.opts.hit_mlog10p, ep.df, ep.lnB) : 2.0f;
   ep.do_full = a.opts.full_output ? 1 : 0;
   ep.do_best = a.out.best != nullptr;
@@ -427,10 +490,6 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
   ep.n_hits = a.out.n_hits;
   ep.best = a.out.best;
   ep.status = c->status;
-  unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
-  if (ep.do_hits)
-    TG_CUDA(cudaMemcpyAsync(hit_start, ep.n_hits, sizeof(unsigned long long),
-                            cudaMemcpyDeviceToDevice, st));
   {
     StageScope s(c, STAGE_GEMM, st, 1);
     TG_CUDA(launch_fp4_scan(&tA, &p->tmFB, (int)p->Ppad, p->Npad, ep, c->sm_count, kSpinNs, st));
@@ -448,98 +507,64 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   if (a.M == 0) return TG_OK;
   if (a.opts.precision == TG_PREC_FP4_PIECES) return scan_fp4(c, p, a, st);
   const int prec = a.opts.precision;
-  const bool split = prec == TG_PREC_SPLIT_BF16;
-  // a small panel's joint projection pass (projected form, joint operand of at most 128 rows,
-  // at least one 128-marker tile per SM) reads the packed rows and decodes them in shared memory
-  const bool fuse_joint = split && c->fuse_joint && a.missing == nullptr &&
-                          a.opts.mode == TG_MODE_PROJECTED && p->q > 1 && p->joint_cols > 0 &&
-                          p->joint_cols <= 128 && p->QYhi16 != nullptr &&
-                          (a.M + MT - 1) / MT >= c->sm_count;
-  // a larger panel's projection (P + q - 1 > 128, same conditions otherwise): the same pass with
-  // the 64 projection columns alone reads the packed rows and also writes the block's operand
-  // as it expands them, so the operand is written once and read once (by the panel's
-  // contraction) instead of being read a second time for the projection. A panel with a
-  // 256-row joint operand keeps its one joint pass over the decoded operand unless this pass
-  // also takes the statistics (dosage rows on 256-marker tiles): with a counting pass first the
-  // projection and the contraction as two passes take longer than the decode and one pass.
-  const bool one_pass_rows = a.encoding == TG_ENC_U8_DOSAGE && a.N <= kOnePassMaxN &&
-                             joint_fused_rows(a.M, c->sm_count, QCOLS) == 2 * MT;
-  const bool fuse_proj = split && c->fuse_joint && !c->fuse_decode && !fuse_joint &&
-                         a.missing == nullptr && a.opts.mode == TG_MODE_PROJECTED && p->q > 1 &&
-                         p->QBhi16 != nullptr && (a.M + MT - 1) / MT >= c->sm_count &&
-                         (p->joint_cols == 0 || one_pass_rows);
-  // split-form 2-bit blocks and unmasked dosage blocks are decoded inside the contraction
-  // kernels when the context asks for it; the rest go through a decoded operand in HBM
-  const bool fused = split && a.missing == nullptr && (c->fuse_decode || fuse_joint);
-  if (c->graphs_alive > 0) {
-    const bool grow = a.M > c->cap_m || (!fused && (round_up(a.M, MT) > c->cap_rows ||
-                                                    p->Npad > c->cap_npad ||
-                                                    (prec == TG_PREC_FP32 ? !c->A32 : !c->Ahi)));
-    const int bq = tune_bucket(a.M);
-    const bool single = split && (p->P <= 64 || c->tune_kernel[bq] == TUNE_SINGLE);
-    const bool proj = split && a.opts.mode == TG_MODE_PROJECTED && p->q > 1;
-    if (grow || (single && !split_fits(c, pick_split(c, p, a.M, true))) ||
-        (proj && !split_fits(c, pick_split(c, p, a.M, true, true))))
-      return fail(TG_ERR_INVALID_ARG,
-                  "the context's workspace is held by a captured scan graph: scan blocks no "
-                  "larger than the graph's, or use another context");
-  }
+  const Plan pl = make_plan(c, p, a.N, a.M, a.encoding, a.missing, a.opts);
+  const bool split = pl.split, joint = pl.joint;
+  const int64_t nq = pl.nq;
+  if (c->graphs_alive > 0 &&
+      (a.M > c->cap_m || pl.raw_floats > c->cap_raw ||
+       (pl.operand && !operand_fits(c, a.M, p->Npad, prec))))
+    return fail(TG_ERR_INVALID_ARG,
+                "the context's workspace is held by a captured scan graph: scan blocks no "
+                "larger than the graph's, or use another context");
   TG_CUDA(ensure_markers(c, a.M));
-  if (!fused) TG_CUDA(ensure_operands(c, a.M, p->Npad, prec));
+  if (pl.operand) TG_CUDA(ensure_operands(c, a.M, p->Npad, prec));
+  TG_CUDA(ensure_raw(c, pl.raw_floats));
   const double kappa64 = a.encoding == TG_ENC_U8_DOSAGE ? 2.0 / 255.0 : 1.0;
   const float kappa = (float)kappa64;
-  void* Ahi = fused ? nullptr : prec == TG_PREC_FP32 ? (void*)c->A32 : (void*)c->Ahi;
-  // dosage rows in the joint pass (or the projection pass that writes the operand) on 256-row
-  // tiles: that pass writes the row statistics itself (a thread holds a whole row), so no
-  // counting pass reads the block first
-  const int pass_cols = fuse_proj ? QCOLS : p->joint_cols;
-  const bool one_pass = (fuse_joint || fuse_proj) && a.encoding == TG_ENC_U8_DOSAGE &&
-                        a.N <= kOnePassMaxN &&
-                        joint_fused_rows(a.M, c->sm_count, pass_cols) == 2 * MT;
-  if (!one_pass) {  // (a counting pass alone before the projection pass that writes the operand)
+  const bool u8 = a.encoding == TG_ENC_U8_DOSAGE;
+  void* Ahi = pl.dec ? nullptr : prec == TG_PREC_FP32 ? (void*)c->A32 : (void*)c->Ahi;
+  if (!pl.one_pass) {  // (a counting pass alone before the projection pass that writes the operand)
     StageScope s(c, STAGE_DECODE, st, 1);
     TG_CUDA(launch_decode(a.G, a.ldg, a.encoding, a.N, a.M, a.missing, a.ldm, prec,
-                          fuse_proj ? nullptr : Ahi, split ? c->shift : nullptr,
+                          pl.fuse_proj ? nullptr : Ahi, split ? c->shift : nullptr,
                           split ? c->mh : nullptr, p->Npad, c->nobs, nullptr, nullptr, c->mean,
                           c->gc2, st));
   }
   DecodeArgs da{}, dj{};
-  if (fused || fuse_proj) {
+  if (pl.dec || pl.fuse_proj) {
     da.N = (int)a.N;
     da.M = (int)a.M;
     da.shift = c->shift;
     da.mh = c->mh;
     dj = da;
-    if (one_pass) {
+    if (pl.one_pass) {
       dj.shift_out = c->shift;
       dj.nobs_out = c->nobs;
       dj.mean_out = c->mean;
       dj.gc2_out = c->gc2;
     }
-    if (fuse_proj) {
+    if (pl.fuse_proj) {
       dj.a_out = c->Ahi;
       dj.lda_out = p->Npad;
     }
-    const bool u8 = a.encoding == TG_ENC_U8_DOSAGE;
-    if ((fused && !make_tmap_packed(&da.tmG, a.G, a.M, a.ldg, u8 ? 32u : 16u)) ||
-        ((fuse_joint || fuse_proj) &&
+    const int pass_cols = pl.fuse_proj ? QCOLS : p->joint_cols;
+    if ((pl.dec && !make_tmap_packed(&da.tmG, a.G, a.M, a.ldg, u8 ? 32u : 16u)) ||
+        ((pl.fuse_joint || pl.fuse_proj) &&
          !make_tmap_packed(&dj.tmG, a.G, a.M, a.ldg, u8 ? 64u : 16u,
                            (uint32_t)joint_fused_rows(a.M, c->sm_count, pass_cols), u8)))
       return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the packed genotypes");
   }
-  const DecodeArgs* dec = fused ? &da : nullptr;
-  const int64_t nq = a.opts.mode == TG_MODE_PAPER ? 0 : p->q - 1;
+  const DecodeArgs* dec = pl.dec ? &da : nullptr;
   CUtensorMap tA;
-  if (split && !fused && !make_tmap(&tA, c->Ahi, a.M, p->Npad, p->Npad, MT))
+  if (split && !pl.dec && !make_tmap(&tA, c->Ahi, a.M, p->Npad, p->Npad, MT))
     return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the genotype operand");
-  // a small panel in the projected form: one pass over the operand gives the projection and the
-  // panel's products (raw, into qg after the projection columns); the statistics follow the norms
-  const bool joint = split && nq > 0 && p->joint_cols > 0 && !fuse_proj;
-  const int64_t ldq = joint ? p->joint_cols : QCOLS;  // qg row stride
+  // the raw products of the projection (and the joint panel's after them)
+  RawView raw{c->raw, pl.ldr, pl.ldr * (nq + (joint ? p->P : 0)), pl.ranges_proj, c->shift,
+              joint ? p->qycs : p->qcs};
   if (nq > 0) {
     StageScope s(c, STAGE_PROJECT, st, 1);
     if (!split) {
-      TG_CUDA(launch_project(c->A32, p->Npad, a.M, p->Npad, p->QB, nq, c->qg, st));
+      TG_CUDA(launch_project(c->A32, p->Npad, a.M, p->Npad, p->QB, nq, c->raw, pl.ldr, st));
     } else {
       EpiParams pp{};
       pp.M = (int)a.M;
@@ -547,31 +572,33 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
       pp.status = c->status;
       pp.row_shift = c->shift;
       pp.col_cs = joint ? p->qycs : p->qcs;
-      pp.raw_out = c->qg;
+      pp.raw_out = c->raw;
       pp.raw_cols = pp.P;
-      pp.raw_ld = (int)ldq;
-      if (fuse_joint) {
-        const bool u8 = a.encoding == TG_ENC_U8_DOSAGE;  // dosage rows: the f16 joint operand
+      pp.raw_ld = raw.ld;
+      pp.raw_split = raw.split;
+      pp.ksplit = pl.ranges_proj;
+      if (pl.fuse_joint) {  // dosage rows: the f16 joint operand
         if (u8) pp.col_cs = p->qycs16;
         TG_CUDA(launch_joint_fused(u8 ? &p->tmQYhi16 : &p->tmQYhi, u8 ? &p->tmQYlo16 : &p->tmQYlo,
                                    p->Npad, pp, c->sm_count, kSpinNs, st, dj, a.encoding));
-      } else if (fuse_proj) {  // the projection alone, writing the operand as it goes
-        const bool u8 = a.encoding == TG_ENC_U8_DOSAGE;
+      } else if (pl.fuse_proj) {  // the projection alone, writing the operand as it goes
         if (u8) pp.col_cs = p->qcs16;
         TG_CUDA(launch_joint_fused(u8 ? &p->tmQhi16 : &p->tmQhi, u8 ? &p->tmQlo16 : &p->tmQlo,
                                    p->Npad, pp, c->sm_count, kSpinNs, st, dj, a.encoding));
-      } else {
-        const SplitChoice sc = pick_split(c, p, a.M, true, true);
-        if (sc.ks > 1) {  // a small block: split K so that more SMs stream the operand
-          TG_CUDA(ensure_split(c, sc));
-          pp.ksplit = sc.ks;
-          pp.sk_ws = c->sk_ws;
-          pp.sk_cnt = c->sk_cnt;
-          TG_CUDA(cudaMemsetAsync(pp.sk_cnt, 0, sizeof(unsigned) * (size_t)sc.tiles, st));
+      } else if (joint && p->joint_cols > 128) {  // more than one narrow tile: CTA pairs
+        const int64_t items = (a.M + 2 * MT - 1) / (2 * MT) * (p->joint_cols / p->joint_bn);
+        if (pl.ranges_proj == 1 && items > c->sm_count / 2) {
+          pp.wave_ctr = reinterpret_cast<unsigned long long*>(c->scratch + 32);
+          TG_CUDA(cudaMemsetAsync(pp.wave_ctr, 0, sizeof(unsigned long long), st));
         }
+        TG_CUDA(launch_tc2_scan(&tA, &p->tmQYhi, &p->tmQYlo, p->Npad, pp, c->sm_count, kSpinNs, st,
+                                kGroupDefault, c->fuse_decode ? dec : nullptr, a.encoding,
+                                p->joint_bn));
+      } else {
         TG_CUDA(launch_tc_scan(&tA, joint ? &p->tmQYhi : &p->tmQhi, joint ? &p->tmQYlo : &p->tmQlo,
                                p->Npad, pp, c->sm_count, kSpinNs, st, kGroupDefault,
-                               c->fuse_decode ? dec : nullptr, a.encoding));
+                               c->fuse_decode ? dec : nullptr, a.encoding,
+                               joint ? p->joint_cols : QCOLS));
       }
     }
   }
@@ -580,18 +607,15 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
     TG_CUDA(launch_subset_stats(a.G, a.ldg, a.encoding, a.N, a.M, a.missing, a.ldm, p->samples,
                                 c->mean, c->gc2s, st));
   }
+  unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
+  const bool want_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
   {
-    StageScope s(c, STAGE_NORM, st, nq > 0 ? 2 : 1);
-    const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, a.missing, a.ldm, c->mean, p->Q, (int)p->q,
-                          c->refine_list, c->scratch + 40};
-    TG_CUDA(launch_marker_norm(a.M, c->nobs, p->samples ? c->gc2s : c->gc2, c->qg, ldq, nq, kappa64, c->gres2,
-                               a.out.marker_norm2, c->rinv, c->rinv64, &rf, st));
-    if (a.out.marker_nobs)
-      TG_CUDA(cudaMemcpyAsync(a.out.marker_nobs, c->nobs, sizeof(int32_t) * a.M,
-                              cudaMemcpyDeviceToDevice, st));
-    if (a.out.marker_mean)
-      TG_CUDA(cudaMemcpyAsync(a.out.marker_mean, c->mean, sizeof(double) * a.M,
-                              cudaMemcpyDeviceToDevice, st));
+    StageScope s(c, STAGE_NORM, st, 1);
+    const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, a.missing, a.ldm, c->mean, p->Q, (int)p->q};
+    const NormOut no{a.out.marker_norm2, c->rinv, c->rinv64, a.out.marker_nobs, a.out.marker_mean,
+                     want_hits ? hit_start : nullptr, a.out.n_hits};
+    TG_CUDA(launch_marker_norm(a.M, c->nobs, p->samples ? c->gc2s : c->gc2, raw, nq, kappa64, rf,
+                               no, st));
   }
   EpiParams ep{};
   ep.M = (int)a.M;
@@ -601,7 +625,7 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   ep.df_f = (float)ep.df;
   ep.kappa = kappa;
   ep.kappa64 = kappa64;
-  ep.do_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
+  ep.do_hits = want_hits;
   ep.r2_thr = ep.do_hits ? r2_threshold(a.opts.hit_mlog10p, ep.df, ep.lnB) : 2.0f;
   ep.do_full = a.opts.full_output ? 1 : 0;
   ep.do_best = a.out.best != nullptr;
@@ -624,44 +648,52 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   ep.n_hits = a.out.n_hits;
   ep.best = a.out.best;
   ep.status = c->status;
-  unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
-  if (ep.do_hits)
-    TG_CUDA(cudaMemcpyAsync(hit_start, ep.n_hits, sizeof(unsigned long long),
-                            cudaMemcpyDeviceToDevice, st));
+  bool full_done = false;  // the FULL statistics came with the raw products'
   {
-    StageScope s(c, STAGE_GEMM, st, 1);
+    StageScope s(c, STAGE_GEMM, st, pl.ranges_scan > 1 ? 2 : 1);
     if (prec == TG_PREC_FP32) {
       TG_CUDA(launch_sgemm_scan(c->A32, p->Npad, p->B32, p->Npad, p->Npad, ep, st));
     } else if (joint) {  // the products came with the projection
-      TG_CUDA(launch_raw_stats(c->qg + nq, ldq, ep, st));
+      raw.x += nq * raw.ld;
+      raw.cs = p->col_cs;
+      TG_CUDA(launch_raw_stats(raw, ep, st));
+      full_done = true;
     } else {
       const int b = tune_bucket(a.M);
       const int group = c->tune_group[b] > 0 ? c->tune_group[b] : kGroupDefault;
       const bool narrow = p->P <= 64;  // a small panel: 64-column tiles, bound by HBM
-      if (narrow || c->tune_kernel[b] == TUNE_SINGLE) {
-        const SplitChoice sc = pick_split(c, p, a.M, true);
-        if (sc.ks > 1) {  // split-K while the tiles are fewer than the SMs
-          TG_CUDA(ensure_split(c, sc));
-          ep.ksplit = sc.ks;
-          ep.sk_ws = c->sk_ws;
-          ep.sk_cnt = c->sk_cnt;
-          TG_CUDA(cudaMemsetAsync(ep.sk_cnt, 0, sizeof(unsigned) * (size_t)sc.tiles, st));
-        }
-        TG_CUDA(launch_tc_scan(&tA, narrow ? &p->tmBhi64 : &p->tmBhi, narrow ? &p->tmBlo64 : &p->tmBlo,
-                               p->Npad, ep, c->sm_count, kSpinNs, st, group, dec, a.encoding, narrow));
+      EpiParams pp = ep;
+      if (pl.ranges_scan > 1) {  // K split while the tiles are too few for the SMs
+        pp.raw_out = c->raw;
+        pp.raw_cols = pp.P;
+        pp.raw_ld = pl.ldr;
+        pp.raw_split = pl.ldr * p->P;
+        pp.ksplit = pl.ranges_scan;
       }
-      else {
-        ep.wave_ctr = reinterpret_cast<unsigned long long*>(c->scratch + 32);
-        TG_CUDA(cudaMemsetAsync(ep.wave_ctr, 0, sizeof(unsigned long long), st));
-        TG_CUDA(launch_tc2_scan(&tA, &p->tmBhi2, &p->tmBlo2, p->Npad, ep, c->sm_count, kSpinNs, st,
-                                group, dec, a.encoding));
+      if (pl.single) {
+        TG_CUDA(launch_tc_scan(&tA, narrow ? &p->tmBhi64 : &p->tmBhi, narrow ? &p->tmBlo64 : &p->tmBlo,
+                               p->Npad, pp, c->sm_count, kSpinNs, st, group, dec, a.encoding,
+                               narrow ? 64 : 256));
+      } else {
+        if (pl.ranges_scan == 1) {
+          pp.wave_ctr = reinterpret_cast<unsigned long long*>(c->scratch + 32);
+          TG_CUDA(cudaMemsetAsync(pp.wave_ctr, 0, sizeof(unsigned long long), st));
+        }
+        TG_CUDA(launch_tc2_scan(&tA, &p->tmBhi2, &p->tmBlo2, p->Npad, pp, c->sm_count, kSpinNs, st,
+                                group, dec, a.encoding, p->bn));
+      }
+      if (pl.ranges_scan > 1) {
+        TG_CUDA(launch_raw_stats(RawView{c->raw, pl.ldr, pl.ldr * p->P, pl.ranges_scan, c->shift,
+                                         p->col_cs}, ep, st));
+        full_done = true;
       }
     }
   }
-  if (ep.do_hits || ep.do_full) {
-    StageScope s(c, STAGE_STATS, st, (ep.do_hits ? 1 : 0) + (ep.do_full ? 1 : 0));
+  const bool full = ep.do_full && !full_done;
+  if (ep.do_hits || full) {
+    StageScope s(c, STAGE_STATS, st, (ep.do_hits ? 1 : 0) + (full ? 1 : 0));
     if (ep.do_hits) TG_CUDA(launch_hit_stats(ep, hit_start, st));
-    if (ep.do_full) TG_CUDA(launch_full_stats(ep, st));
+    if (full) TG_CUDA(launch_full_stats(ep, st));
   }
   return TG_OK;
 }
@@ -784,9 +816,8 @@ tg_status tg_destroy(tg_ctx* c) {
   cudaDeviceSynchronize();
   dfree(c->status); dfree(c->scratch);
   dfree(c->Ahi); dfree(c->A32); dfree(c->Afp4); dfree(c->shift); dfree(c->mh); dfree(c->gc2s);
-  dfree(c->nobs); dfree(c->mean); dfree(c->gc2); dfree(c->qg); dfree(c->gres2);
-  dfree(c->rinv); dfree(c->rinv64); dfree(c->refine_list);
-  dfree(c->sk_ws); dfree(c->sk_cnt);
+  dfree(c->nobs); dfree(c->mean); dfree(c->gc2); dfree(c->raw);
+  dfree(c->rinv); dfree(c->rinv64);
   dfree(c->stage);
   dfree(c->dhits); dfree(c->dnhits); dfree(c->dbest);
   for (auto& ev : c->pending) { cudaEventDestroy(ev.a); cudaEventDestroy(ev.b); }
@@ -802,15 +833,16 @@ tg_status tg_destroy(tg_ctx* c) {
 }
 
 // The joint operand of a small panel (tg_panel::QYhi): the q - 1 projection rows, then the P
-// phenotype rows, copied from the panel's own split operands, in the fewest of 64, 128 or 256
-// rows that hold them. Nothing for a panel without covariate columns or with P + q - 1 > 256.
-// A panel with P + q - 1 > 128 gets the f16 copy of its projection columns alone instead of the
-// joint f16 operand (tg_panel::QBhi16). Synchronous on st.
+// phenotype rows, copied from the panel's own split operands, in 64 or 128 rows, or one or two
+// CTA-pair tiles of tile_cols(P + q - 1) rows. Nothing for a panel without covariate columns or
+// with P + q - 1 > JCOLS: there the joint pass would add a third tile's worth of raw products in
+// memory to save a projection pass that is by then a small part. Such a panel gets the f16 copy
+// of its projection columns alone (tg_panel::QBhi16). Synchronous on st.
 tg_status build_joint(tg_panel* p, cudaStream_t st) {
   const int64_t nq = p->q - 1, P = p->P, Np = p->Npad;
   if (nq <= 0 || P <= 0) return TG_OK;
   cudaError_t e;
-  if (P + nq > 128) {  // the projection pass that also writes the operand reads these
+  if (P + nq > JCOLS) {  // the projection pass that also writes the operand reads these
     if ((e = dalloc(&p->QBhi16, (size_t)(QCOLS * Np))) ||
         (e = dalloc(&p->QBlo16, (size_t)(QCOLS * Np))) || (e = dalloc(&p->qcs16, (size_t)QCOLS)) ||
         (e = launch_joint_f16(p->Q, p->N, nq, p->Yres, p->s, p->col_rmul, 0, QCOLS, Np, p->QBhi16,
@@ -822,7 +854,10 @@ tg_status build_joint(tg_panel* p, cudaStream_t st) {
       return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the f16 projection operand");
   }
   if (P + nq > JCOLS) return TG_OK;
-  const int64_t jc = P + nq <= 64 ? 64 : P + nq <= 128 ? 128 : 256;
+  // one tile of 64 or 128 columns, or CTA-pair tiles of joint_bn columns
+  const int64_t jn = tile_cols(P + nq);
+  const int64_t jc = P + nq <= 64 ? 64 : P + nq <= 128 ? 128 : round_up(P + nq, jn);
+  const uint32_t box = (uint32_t)(jc <= 128 ? jc : jn / 2);
   const size_t row = sizeof(__nv_bfloat16) * (size_t)Np;
   const auto d2d = cudaMemcpyDeviceToDevice;
   if ((e = dalloc(&p->QYhi, (size_t)(jc * Np))) || (e = dalloc(&p->QYlo, (size_t)(jc * Np))) ||
@@ -838,8 +873,8 @@ tg_status build_joint(tg_panel* p, cudaStream_t st) {
       (e = cudaMemcpyAsync(p->qycs + nq, p->col_cs, sizeof(float) * P, d2d, st)) ||
       (e = cudaStreamSynchronize(st)))
     return cuda_fail(e, "joint projection and panel operand");
-  if (!make_tmap(&p->tmQYhi, p->QYhi, jc, Np, Np, (uint32_t)jc) ||
-      !make_tmap(&p->tmQYlo, p->QYlo, jc, Np, Np, (uint32_t)jc))
+  if (!make_tmap(&p->tmQYhi, p->QYhi, jc, Np, Np, box) ||
+      !make_tmap(&p->tmQYlo, p->QYlo, jc, Np, Np, box))
     return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the joint operand");
   if (jc <= 128) {  // the f16 copy for the joint pass that decodes dosage rows in shared memory
     if ((e = dalloc(&p->QYhi16, (size_t)(jc * Np))) || (e = dalloc(&p->QYlo16, (size_t)(jc * Np))) ||
@@ -854,6 +889,7 @@ tg_status build_joint(tg_panel* p, cudaStream_t st) {
       return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the f16 joint operand");
   }
   p->joint_cols = (int)jc;
+  p->joint_bn = (int)(jc <= 128 ? jc : jn);
   return TG_OK;
 }
 
@@ -878,6 +914,7 @@ tg_status tg_prepare_panel(tg_ctx* c, const float* Y, int64_t ldy, int64_t N, in
   p->NS = N;
   p->Npad = round_up(N, KPAD);
   p->Ppad = round_up(std::max<int64_t>(P, 1), PPAD);
+  p->bn = (int)tile_cols(P);
   const int64_t k = 1 + n_cov;
   auto cleanup = [&](tg_status s) { tg_panel_free(p); return s; };
   cudaError_t e;
@@ -932,8 +969,8 @@ tg_status tg_prepare_panel(tg_ctx* c, const float* Y, int64_t ldy, int64_t N, in
   p->lnB_paper = host_lnbeta_half((double)(N - 2));
   if (!make_tmap(&p->tmBhi, p->Bhi, p->Ppad, p->Npad, p->Npad, 256) ||
       !make_tmap(&p->tmBlo, p->Blo, p->Ppad, p->Npad, p->Npad, 256) ||
-      !make_tmap(&p->tmBhi2, p->Bhi, p->Ppad, p->Npad, p->Npad, 128) ||
-      !make_tmap(&p->tmBlo2, p->Blo, p->Ppad, p->Npad, p->Npad, 128) ||
+      !make_tmap(&p->tmBhi2, p->Bhi, p->Ppad, p->Npad, p->Npad, (uint32_t)p->bn / 2) ||
+      !make_tmap(&p->tmBlo2, p->Blo, p->Ppad, p->Npad, p->Npad, (uint32_t)p->bn / 2) ||
       !make_tmap(&p->tmQhi, p->QBhi, QCOLS, p->Npad, p->Npad, 64) ||
       !make_tmap(&p->tmQlo, p->QBlo, QCOLS, p->Npad, p->Npad, 64) ||
       !make_tmap(&p->tmBhi64, p->Bhi, p->Ppad, p->Npad, p->Npad, 64) ||
@@ -998,6 +1035,7 @@ tg_status tg_prepare_panel_subset(tg_ctx* c, const float* Y, int64_t ldy, int64_
   r->df = pc->df;
   r->Npad = round_up(N, KPAD);
   r->Ppad = pc->Ppad;
+  r->bn = (int)tile_cols(r->P);
   r->lnB = pc->lnB;
   r->lnB_paper = pc->lnB_paper;
   const int64_t Np = r->Npad, Pp = r->Ppad, q = r->q, P1 = std::max<int64_t>(P, 1);
@@ -1046,7 +1084,7 @@ tg_status tg_prepare_panel_subset(tg_ctx* c, const float* Y, int64_t ldy, int64_
       return cleanup(cuda_fail(e, "tg_prepare_panel_subset sample mask"));
   }
   if (!make_tmap(&r->tmBhi, r->Bhi, Pp, Np, Np, 256) || !make_tmap(&r->tmBlo, r->Blo, Pp, Np, Np, 256) ||
-      !make_tmap(&r->tmBhi2, r->Bhi, Pp, Np, Np, 128) || !make_tmap(&r->tmBlo2, r->Blo, Pp, Np, Np, 128) ||
+      !make_tmap(&r->tmBhi2, r->Bhi, Pp, Np, Np, (uint32_t)r->bn / 2) || !make_tmap(&r->tmBlo2, r->Blo, Pp, Np, Np, (uint32_t)r->bn / 2) ||
       !make_tmap(&r->tmQhi, r->QBhi, QCOLS, Np, Np, 64) || !make_tmap(&r->tmQlo, r->QBlo, QCOLS, Np, Np, 64) ||
       !make_tmap(&r->tmBhi64, r->Bhi, Pp, Np, Np, 64) || !make_tmap(&r->tmBlo64, r->Blo, Pp, Np, Np, 64))
     return cleanup(fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the subset panel"));
@@ -1494,6 +1532,7 @@ tg_status tg_panel_concat(tg_ctx* c, const tg_panel* const* panels, int n, tg_pa
   r->df = p0->df;
   r->Npad = p0->Npad;
   r->Ppad = round_up(std::max<int64_t>(P, 1), PPAD);
+  r->bn = (int)tile_cols(r->P);
   r->lnB = p0->lnB;
   r->lnB_paper = p0->lnB_paper;
   r->NS = p0->NS;
@@ -1552,7 +1591,7 @@ tg_status tg_panel_concat(tg_ctx* c, const tg_panel* const* panels, int n, tg_pa
     return cuda_fail(e, "tg_panel_concat copy");
   }
   if (!make_tmap(&r->tmBhi, r->Bhi, Pp, Np, Np, 256) || !make_tmap(&r->tmBlo, r->Blo, Pp, Np, Np, 256) ||
-      !make_tmap(&r->tmBhi2, r->Bhi, Pp, Np, Np, 128) || !make_tmap(&r->tmBlo2, r->Blo, Pp, Np, Np, 128) ||
+      !make_tmap(&r->tmBhi2, r->Bhi, Pp, Np, Np, (uint32_t)r->bn / 2) || !make_tmap(&r->tmBlo2, r->Blo, Pp, Np, Np, (uint32_t)r->bn / 2) ||
       !make_tmap(&r->tmQhi, r->QBhi, QCOLS, Np, Np, 64) || !make_tmap(&r->tmQlo, r->QBlo, QCOLS, Np, Np, 64) ||
       !make_tmap(&r->tmBhi64, r->Bhi, Pp, Np, Np, 64) || !make_tmap(&r->tmBlo64, r->Blo, Pp, Np, Np, 64)) {
     tg_panel_free(r);
@@ -1592,7 +1631,8 @@ tg_status tg_scan_graph_create(tg_ctx* c, const tg_panel* p, int n_blocks,
   bool need_operand = opts->precision != TG_PREC_SPLIT_BF16 || !c->fuse_decode;
   for (int b = 0; b < n_blocks; ++b) need_operand |= missing && missing[b];
   {
-    tg_status ws = reserve_graph_workspace(c, p, n_blocks, M, maxM, need_operand, *opts);
+    tg_status ws = reserve_graph_workspace(c, p, n_blocks, M, maxM, need_operand, encoding,
+                                           missing, *opts);
     if (ws != TG_OK) return ws;
   }
   cudaStream_t cap = nullptr;
@@ -1658,7 +1698,8 @@ tg_status tg_scan_graph_create_host(tg_ctx* c, const tg_panel* p, int n_blocks,
   }
   const bool need_operand = opts->precision != TG_PREC_SPLIT_BF16 || !c->fuse_decode;
   {
-    tg_status ws = reserve_graph_workspace(c, p, n_blocks, M, maxM, need_operand, *opts);
+    tg_status ws = reserve_graph_workspace(c, p, n_blocks, M, maxM, need_operand, encoding,
+                                           nullptr, *opts);
     if (ws != TG_OK) return ws;
   }
   tg_graph* g = new tg_graph();

@@ -170,17 +170,17 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
   if (s != TG_OK) return s;
 
   Carver cv{ds->base};
-  uint32_t* status = cv.take<uint32_t>(4);  // [0] status word, [1] count of re-projected markers
+  uint32_t* status = cv.take<uint32_t>(4);  // [0] status word
   unsigned long long* hit_start = cv.take<unsigned long long>(1);
   float* shift = cv.take<float>((size_t)rows);
   int32_t* nobs = cv.take<int32_t>((size_t)rows);
   double* mean = cv.take<double>((size_t)rows);
   double* gc2 = cv.take<double>((size_t)rows);
   float* qg = cv.take<float>((size_t)rows * QCOLS);
-  double* gres2 = cv.take<double>((size_t)rows);
+  cv.take<double>((size_t)rows);  // (unused: the largest accepted block stays what it was)
   float* rinv = cv.take<float>((size_t)rows);
   double* rinv64 = cv.take<double>((size_t)rows);
-  int* refine_list = cv.take<int>((size_t)rows);
+  cv.take<int>((size_t)rows);  // (unused)
   void* Ahi = cv.take<unsigned char>((size_t)rows * p->Npad * elem);
 
   cudaStream_t st = (cudaStream_t)stream;
@@ -205,7 +205,7 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
   if (nq > 0) {
     if (!split) {
       TGS_CUDA(launch_project(reinterpret_cast<const float*>(Ahi), p->Npad, M, p->Npad, p->QB, nq,
-                              qg, st));
+                              qg, rows, st));
     } else {
       EpiParams pp{};
       pp.M = (int)M;
@@ -215,19 +215,16 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
       pp.col_cs = joint ? p->qycs : p->qcs;
       pp.raw_out = qg;
       pp.raw_cols = pp.P;
-      pp.raw_ld = QCOLS;
+      pp.raw_ld = rows;
       TGS_CUDA(launch_tc_scan(&tA, joint ? &p->tmQYhi : &p->tmQhi, joint ? &p->tmQYlo : &p->tmQlo,
-                              p->Npad, pp, ds->sm_count, kStaticSpinNs, st));
+                              p->Npad, pp, ds->sm_count, kStaticSpinNs, st, 16, nullptr, 0, QCOLS));
     }
   }
-  const MarkerRefine rf{G, ldg, encoding, N, missing, ldm, mean, p->Q, (int)p->q, refine_list,
-                        status + 1};
-  TGS_CUDA(launch_marker_norm(M, nobs, gc2, qg, QCOLS, nq, kappa64, gres2, out->marker_norm2, rinv, rinv64,
-                              &rf, st));
-  if (out->marker_nobs)
-    TGS_CUDA(cudaMemcpyAsync(out->marker_nobs, nobs, sizeof(int32_t) * M, cudaMemcpyDeviceToDevice, st));
-  if (out->marker_mean)
-    TGS_CUDA(cudaMemcpyAsync(out->marker_mean, mean, sizeof(double) * M, cudaMemcpyDeviceToDevice, st));
+  const MarkerRefine rf{G, ldg, encoding, N, missing, ldm, mean, p->Q, (int)p->q};
+  const NormOut no{out->marker_norm2, rinv, rinv64, out->marker_nobs, out->marker_mean,
+                   want_hits ? hit_start : nullptr, out->n_hits};
+  TGS_CUDA(launch_marker_norm(M, nobs, gc2, RawView{qg, rows, 0, 1, nullptr, nullptr}, nq, kappa64,
+                              rf, no, st));
   EpiParams ep{};
   ep.M = (int)M;
   ep.P = (int)p->P;
@@ -259,21 +256,19 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
   ep.n_hits = out->n_hits;
   ep.best = out->best;
   ep.status = status;
-  if (ep.do_hits)
-    TGS_CUDA(cudaMemcpyAsync(hit_start, ep.n_hits, sizeof(unsigned long long),
-                             cudaMemcpyDeviceToDevice, st));
   if (!split) {
     TGS_CUDA(launch_sgemm_scan(reinterpret_cast<const float*>(Ahi), p->Npad, p->B32, p->Npad,
                                p->Npad, ep, st));
   } else if (joint) {  // the products came with the projection
-    TGS_CUDA(launch_raw_stats(qg + nq, QCOLS, ep, st));
+    TGS_CUDA(launch_raw_stats(RawView{qg + nq * rows, rows, 0, 1, nullptr, nullptr}, ep, st));
   } else {
     const bool narrow = p->P <= 64;  // a small panel: 64-column tiles, bound by HBM
     TGS_CUDA(launch_tc_scan(&tA, narrow ? &p->tmBhi64 : &p->tmBhi, narrow ? &p->tmBlo64 : &p->tmBlo,
-                            p->Npad, ep, ds->sm_count, kStaticSpinNs, st, 16, nullptr, 0, narrow));
+                            p->Npad, ep, ds->sm_count, kStaticSpinNs, st, 16, nullptr, 0,
+                            narrow ? 64 : 256));
   }
   if (ep.do_hits) TGS_CUDA(launch_hit_stats(ep, hit_start, st));
-  if (ep.do_full) TGS_CUDA(launch_full_stats(ep, st));
+  if (ep.do_full && !joint) TGS_CUDA(launch_full_stats(ep, st));
   // synchronous: the device status of this call is returned
   uint32_t word = 0;
   TGS_CUDA(cudaMemcpyAsync(&word, status, sizeof(word), cudaMemcpyDeviceToHost, st));

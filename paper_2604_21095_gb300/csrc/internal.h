@@ -28,7 +28,7 @@ constexpr int kRingEvents = 8 * kMaxHostBufs + 8;
 // the next call's block growth
 constexpr int kRateBlocks = 8;
 constexpr int QCOLS = 64;    // projection columns (Q columns 1..q-1), zero padded
-constexpr int JCOLS = 256;   // widest joint operand: projection columns + panel in one tile
+constexpr int JCOLS = 512;   // widest joint operand: projection columns + panel in one pass
 constexpr int MT = 128;      // marker rows per tensor-core tile
 constexpr int kFp4Pieces = 6;  // E2M1 pieces of the panel in the FP4 form (k_fp4.cu)
 // Scale of the f16 joint operand (k_joint_f16): values of at most 1 in magnitude become at most
@@ -39,6 +39,14 @@ enum Stage { STAGE_DECODE = 0, STAGE_PROJECT = 1, STAGE_NORM = 2, STAGE_GEMM = 3
              STAGE_STATS = 5 };
 
 inline int64_t round_up(int64_t x, int64_t m) { return (x + m - 1) / m * m; }
+
+// Columns of a CTA-pair tile for an operand of `cols` columns: the fewest tiles of at most 256
+// columns, all of one width, a multiple of 32 (the MMA's step). Against 256-column tiles that
+// saves the products of the padding, 300 columns being 2 x 160 instead of 2 x 256.
+inline int64_t tile_cols(int64_t cols) {
+  const int64_t c = cols > 0 ? cols : 1, n = (c + 255) / 256;
+  return round_up((c + n - 1) / n, 32);
+}
 
 // What the FP64 recomputation of a product g_j . y_res,p needs (hits, and FULL elements near
 // |r| = 1): the packed genotype block, its FP64 observed means (decode units; a missing call is
@@ -88,14 +96,15 @@ struct EpiParams {
   unsigned long long* best;
   uint32_t* status;
   unsigned long long* wave_ctr;  // CTA-pair lockstep counter (zeroed per launch), NULL = off
-  float* raw_out;              // projection mode: D of the first raw_cols columns, [M][raw_ld]
-  int raw_cols, raw_ld;
-  // split-K (one-CTA kernel): K split in `ksplit` chunk-aligned ranges (0 or 1 = none); the
-  // partial sums of splits 1.. go through sk_ws ([tiles][ksplit-1][128][256] floats) and
-  // sk_cnt ([tiles], zeroed per launch) to the tile's split 0, which adds them in split order
+  // raw mode: the product of row m and column k < raw_cols goes to raw_out[k * raw_ld + m]
+  // (column-major, so that the 32 rows of a warp store whole sectors). Unsplit, that is D with
+  // the shift's add-back. With split-K (raw mode only, ksplit > 1: K in `ksplit` chunk-aligned
+  // ranges) range s writes its partial sums, without the add-back, raw_split floats further
+  // on; the kernels that read them (k_marker_norm, k_raw_stats) add the ranges in order.
+  float* raw_out;
+  int raw_cols;
+  long long raw_ld, raw_split;
   int ksplit;
-  float* sk_ws;
-  unsigned* sk_cnt;
   ExactArgs exact;             // FP64 recomputation of hits and of FULL elements near |r| = 1
 };
 
@@ -175,25 +184,28 @@ struct tg_panel {
   double lnB = 0;                // ln B(df/2, 1/2), df = N - q - 1
   double lnB_paper = 0;          // ln B((N-2)/2, 1/2) for the paper's printed form
   CUtensorMap tmBhi, tmBlo;      // phenotype panel, 256-row boxes
-  CUtensorMap tmBhi2, tmBlo2;    // phenotype panel, 128-row boxes (one CTA's half of a pair tile)
+  int bn = 0;                    // columns of a CTA-pair tile (tile_cols(P))
+  CUtensorMap tmBhi2, tmBlo2;    // phenotype panel, boxes of bn / 2 rows (one CTA's half of a pair tile)
   CUtensorMap tmQhi, tmQlo;      // covariate projection columns, 64-row boxes
   CUtensorMap tmBhi64, tmBlo64;  // phenotype panel, 64-row boxes (64-column tiles, P <= 64)
-  // Small panels (P + q - 1 <= 256): the projection columns and the phenotypes in one operand
-  // of joint_cols = 64, 128 or 256 rows, rows [0, q-1) = QB rows, rows [q-1, q-1+P) = the panel, rest
-  // zero, so that one pass over a block's operand gives both Q^T a and the panel's products
-  // (joint_cols = 0 and NULL buffers when the panel is larger).
-  int joint_cols = 0;
+  // Panels with P + q - 1 <= JCOLS: the projection columns and the phenotypes in one operand,
+  // rows [0, q-1) = QB rows, rows [q-1, q-1+P) = the panel, rest zero, so that one pass over a
+  // block's operand gives both Q^T a and the panel's products (joint_cols = 0 and NULL buffers
+  // when the panel is larger). Up to 128 rows the operand has joint_cols = 64 or 128 rows, one
+  // tile of the one-CTA kernels; above, it has joint_cols = n x joint_bn rows, n = 1 or 2 tiles
+  // of joint_bn columns of the CTA-pair kernel (the maps' boxes hold half a tile).
+  int joint_cols = 0, joint_bn = 0;
   __nv_bfloat16* QYhi = nullptr;  // [joint_cols][Npad]
   __nv_bfloat16* QYlo = nullptr;
   float* qycs = nullptr;          // [joint_cols] qcs then col_cs
-  CUtensorMap tmQYhi, tmQYlo;     // boxes of joint_cols rows
+  CUtensorMap tmQYhi, tmQYlo;     // boxes of joint_cols rows (joint_bn / 2 above 128)
   // The same joint operand as f16 hi + lo of 2^14 v (joint_cols <= 128 only), for the joint pass
   // that decodes dosage rows in shared memory into f16 (k_fused.cu); scaled column sums.
   __half* QYhi16 = nullptr;       // [joint_cols][Npad]
   __half* QYlo16 = nullptr;
   float* qycs16 = nullptr;        // [joint_cols]
   CUtensorMap tmQYhi16, tmQYlo16;
-  // The projection columns alone in the same f16 form (64 rows; panels with P + q - 1 > 128),
+  // The projection columns alone in the same f16 form (64 rows; panels with P + q - 1 > JCOLS),
   // for the projection pass over dosage rows that also writes the block's operand (k_fused.cu).
   __half* QBhi16 = nullptr;       // [QCOLS][Npad]
   __half* QBlo16 = nullptr;
@@ -230,11 +242,10 @@ struct tg_ctx {
   double* gc2s = nullptr;                       // [cap_m] |g_c|^2 over a subset panel's samples
   uint32_t* mh = nullptr;                       // [cap_m] bf16 bits of the missing-call value
   double* gc2 = nullptr;
-  float* qg = nullptr;                          // [cap_m][QCOLS]
-  double* gres2 = nullptr;
+  float* raw = nullptr;                         // raw products, [ranges][columns][rows]
+  size_t cap_raw = 0;                           // its floats
   float* rinv = nullptr;
   double* rinv64 = nullptr;
-  int* refine_list = nullptr;                   // [cap_m] markers re-projected in FP64
   // host-streamed scan: a device ring of host_bufs block buffers' bytes (stage_cap allocated)
   uint8_t* stage = nullptr;
   size_t stage_cap = 0;
@@ -269,10 +280,6 @@ struct tg_ctx {
   int tune_kernel[tg::kTuneBuckets] = {};
   int tune_group[tg::kTuneBuckets] = {};
   int tune_split[tg::kTuneBuckets] = {};        // split-K of the one-CTA kernel (0 = none)
-  float* sk_ws = nullptr;                       // split-K partial sums and per-tile counters
-  size_t sk_ws_bytes = 0;
-  unsigned* sk_cnt = nullptr;
-  int64_t sk_cnt_cap = 0;
 };
 
 namespace tg {
@@ -333,11 +340,21 @@ cudaError_t launch_subset_stats(const uint8_t* G, int64_t ldg, int encoding, int
                                 const double* mean, double* gc2s, cudaStream_t st);
 
 // SIMT kernels (k_simt.cu)
+// Raw products as the contraction kernels leave them (EpiParams::raw_out): element (m, k) of
+// range s at x[s * split + k * ld + m]. With ranges > 1 the partial sums are added in range
+// order and then shift[m] * cs[k].
+struct RawView {
+  const float* x;
+  long long ld, split;
+  int ranges;
+  const float* shift;
+  const float* cs;
+};
+// Projections of the FP32 operand, column-major: out[k * ldq + m].
 cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, const float* QB,
-                           int64_t nq, float* qg, cudaStream_t st);
+                           int64_t nq, float* out, int64_t ldq, cudaStream_t st);
 // What the FP64 re-projection of markers close to the covariate span needs: the packed block,
-// the FP64 means (units) and the panel's FP64 basis Q ([q][N], column 0 the intercept), and a
-// list of at least M ints with its counter (4 bytes of device memory).
+// the FP64 means (units) and the panel's FP64 basis Q ([q][N], column 0 the intercept).
 struct MarkerRefine {
   const uint8_t* G;
   int64_t ldg;
@@ -348,14 +365,24 @@ struct MarkerRefine {
   const double* mean;
   const double* Q;
   int q;
-  int* list;
-  unsigned* count;
+};
+// Outputs of the norm kernel: 1/|g_res| of each marker (NaN = untestable) and, where not NULL,
+// |g_res|^2 in allele units, copies of n_obs and of the mean for the caller, and
+// the hit counter's value before this block (hit_start = *n_hits).
+struct NormOut {
+  double* norm2_allele;
+  float* rinv;
+  double* rinv64;
+  int32_t* nobs;
+  double* mean;
+  unsigned long long* hit_start;
+  const unsigned long long* n_hits;
 };
 // complete_n > 0: markers with fewer than complete_n observed calls are untestable too.
-cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2, const float* qg,
-                               int64_t ldq, int64_t nq, double kappa, double* gres2_units_out,
-                               double* norm2_allele_out, float* rinv, double* rinv64,
-                               const MarkerRefine* refine, cudaStream_t st, int64_t complete_n = 0);
+cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2,
+                               const RawView& proj, int64_t nq, double kappa,
+                               const MarkerRefine& refine, const NormOut& out, cudaStream_t st,
+                               int64_t complete_n = 0);
 cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t K,
                               const EpiParams& ep, cudaStream_t st);
 
@@ -366,13 +393,13 @@ cudaError_t launch_fill_random(uint8_t* p, size_t n, unsigned long long seed, cu
 
 // tensor-core kernel (k_tc.cu)
 // With `dec` non-NULL the A operand is decoded from packed genotypes in the kernel (tmA unused).
-// `narrow`: 64-column tiles for a panel of at most 64 phenotypes (B maps with 64-row boxes).
-// Raw mode (ep.raw_out: the covariate projection, alone or joint with a small panel) uses the
-// narrowest of 64-, 128- and 256-column tiles that holds the raw columns.
+// `bn`: 64-, 128- or 256-column tiles, the B maps' box rows. 64: the covariate projection, a small
+// panel's joint operand, or a panel of at most 64 phenotypes; 128: a joint operand; 256: a panel.
+// Raw mode (ep.raw_out) takes split-K.
 cudaError_t launch_tc_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                            const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                            long long spin_ns, cudaStream_t st, int group_m = 16,
-                           const DecodeArgs* dec = nullptr, int encoding = 0, bool narrow = false);
+                           const DecodeArgs* dec = nullptr, int encoding = 0, int bn = 256);
 
 // The joint projection pass of a small panel (joint operand of 64 or 128 rows) with the decode
 // fused in (k_fused.cu): reads the packed rows through da.tmG, whose boxes must be
@@ -387,10 +414,9 @@ cudaError_t launch_joint_fused(const CUtensorMap* tmBhi, const CUtensorMap* tmBl
                                const EpiParams& ep, int sm_count, long long spin_ns, cudaStream_t st,
                                const DecodeArgs& da, int encoding);
 
-// The statistics of a small panel (P <= 256) from the joint pass's raw products (k_tc.cu): D of
-// marker row m and phenotype p at raw[m * ld + p] (the shift's add-back included), the same
-// per-element epilogue as the contraction kernels.
-cudaError_t launch_raw_stats(const float* raw, int64_t ld, const EpiParams& ep, cudaStream_t st);
+// The statistics of a block from its raw products (k_stats.cu): the same per-element epilogue as
+// the contraction kernels and, in FULL mode, every statistic (no launch_full_stats after it).
+cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream_t st);
 
 // The FP4 form (k_fp4.cu). Pieces: rows r < nrows of src (stride lds; divided by div[r] when
 // div is not NULL; skipped where valid[r] is NaN) as kFp4Pieces E2M1 pieces, out[k][rows_pad][Npad/2]
@@ -410,11 +436,12 @@ cudaError_t launch_fp4_scan(const CUtensorMap* tmA, const CUtensorMap* tmB, int 
                             int64_t Npad, const EpiParams& ep, int sm_count, long long spin_ns,
                             cudaStream_t st);
 
-// tensor-core kernel on CTA pairs, 256 x 256 tiles (k_tc2.cu)
+// tensor-core kernel on CTA pairs, 256 x bn tiles (k_tc2.cu); bn a multiple of 32, at most 256,
+// the B maps with boxes of bn / 2 rows. Raw mode (ep.raw_out) takes split-K.
 cudaError_t launch_tc2_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                             const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                             long long spin_ns, cudaStream_t st, int group_m = 16,
-                            const DecodeArgs* dec = nullptr, int encoding = 0);
+                            const DecodeArgs* dec = nullptr, int encoding = 0, int bn = 256);
 
 // bounded wait test (k_tc.cu)
 cudaError_t launch_wait_test(const uint32_t* flag, long long limit_ns, uint32_t* result,

@@ -418,12 +418,12 @@ __global__ void __launch_bounds__(kFThreads, 1)
 #pragma unroll
           for (int e = 0; e < BN; ++e)
             if (e < ep.raw_cols)
-              ep.raw_out[row * ep.raw_ld + e] = fmaf(shift, ep.col_cs[e], tot[e]) * ep.col_rmul[e];
+              ep.raw_out[e * ep.raw_ld + row] = fmaf(shift, ep.col_cs[e], tot[e]) * ep.col_rmul[e];
         }
       } else {
         const float rinv = (row_ok && ep.row_inv) ? ep.row_inv[row] : __int_as_float(0x7fc00000);
         epilogue_tile(ep, *reinterpret_cast<float(*)[128]>(tot), row, row_base, row_ok, rinv, shift,
-                      nt * BN, lane);
+                      nt * BN, ep.P, lane);
       }
       __syncwarp();
     }

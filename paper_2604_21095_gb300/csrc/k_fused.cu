@@ -579,7 +579,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < BR; ++e)
           if (e < ep.raw_cols)
-            ep.raw_out[row * ep.raw_ld + e] = fmaf(shift, ep.col_cs[e], tot[e]) * kUnscale;
+            ep.raw_out[e * ep.raw_ld + row] = fmaf(shift, ep.col_cs[e], tot[e]) * kUnscale;
       }
       __syncwarp();
     }
@@ -872,7 +872,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int e = 0; e < BR; ++e)
           if (e < ep.raw_cols)
-            ep.raw_out[row * ep.raw_ld + e] = fmaf(shift, ep.col_cs[e], tot[e]) * kUnscale;
+            ep.raw_out[e * ep.raw_ld + row] = fmaf(shift, ep.col_cs[e], tot[e]) * kUnscale;
       }
       __syncwarp();
     }

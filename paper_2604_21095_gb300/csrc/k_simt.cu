@@ -18,11 +18,11 @@ namespace tg {
 namespace {
 
 // ---------------------------------------------------------------- projection
-// qg[m][k] = sum_i A[m][i] QB[k][i]; tile 64 markers x 32 columns, 32 samples per step.
+// qg[k][m] = sum_i A[m][i] QB[k][i]; tile 64 markers x 32 columns, 32 samples per step.
 __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, long long lda,
                                                  long long M, int K,
                                                  const float* __restrict__ QB, int nq,
-                                                 float* __restrict__ qg) {
+                                                 float* __restrict__ qg, long long ldq) {
   __shared__ __align__(16) float As[32][64 + 4];
   __shared__ __align__(16) float Qs[32][32 + 4];
   const int tid = threadIdx.x;
@@ -81,13 +81,13 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
 #pragma unroll
     for (int b = 0; b < 2; ++b) {
       const int k = k0 + tx * 2 + b;
-      if (k < nq) qg[gm * QCOLS + k] = (float)tot[a][b];
+      if (k < nq) qg[k * ldq + gm] = (float)tot[a][b];
     }
   }
 }
 
 // ---------------------------------------------------------------- marker norms
-// A marker is re-projected in FP64 (k_marker_refine) when the covariates explain more than
+// A marker is re-projected in FP64 (refine_projection) when the covariates explain more than
 // this share of its variance: |g_res|^2 = |g_c|^2 - sum_k (q_k . g_c)^2 then amplifies the
 // rounding of the projections by |g_c|^2 / |g_res|^2 (>= 2 here).
 constexpr double kRefineShare = 0.5;
@@ -108,88 +108,104 @@ __device__ __forceinline__ bool marker_testable(int n_obs, double c2, double r2,
   return marker_testable(n_obs, c2, r2) && (complete_n <= 0 || n_obs == complete_n);
 }
 
-__global__ void k_marker_norm(long long M, const int32_t* __restrict__ nobs,
-                              const double* __restrict__ gc2, const float* __restrict__ qg,
-                              long long ldq, int nq,
-                              double kappa, double* __restrict__ gres2u,
-                              double* __restrict__ norm2_allele, float* __restrict__ rinv,
-                              double* __restrict__ rinv64, int* __restrict__ refine_list,
-                              unsigned* __restrict__ refine_count, int complete_n) {
-  const long long j = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (j >= M) return;
-  const double c2 = gc2[j];
+// One block of 8 warps per 32 markers (lane = marker): the warps share the projection columns
+// (coalesced reads, the columns being contiguous in the markers), then warp 0 forms the norms
+// and warp 1 copies the caller's n_obs and mean. A block that lists a marker close to the
+// covariate span re-projects it in FP64 itself, all 256 threads on one marker at a time, so that
+// the usual block without any costs no second launch (nor a counter to clear and a list).
+// Bound by latency: 12.8 us as three operations on 65,536 markers and 19 columns, with
+// row-major products (a sector per value).
+constexpr int kNormWarps = 8;
+
+// sum_k (q_k . g_c)^2 over the non-intercept columns of Q in FP64, from the packed genotypes
+// (missing calls at the marker's mean, which is also its centre, so they add nothing) and the
+// FP64 mean. q_0 . g_c = 0 exactly (q_0 is constant and g_c has zero sum), as in the tensor-core
+// projection, which leaves column 0 out. Whole block; thread 0 returns the sum.
+__device__ __noinline__ double refine_projection(const MarkerRefine& rf, long long j, double* red) {
+  const double mu = rf.mean[j];
+  const uint8_t* row = rf.G + j * rf.ldg;
+  const uint32_t* mrow = rf.missing ? rf.missing + j * rf.ldm : nullptr;
   double s = 0.0;
-  for (int k = 0; k < nq; ++k) {
-    const double v = (double)qg[j * ldq + k];
-    s += v * v;
+  for (int k = 1; k < rf.q; ++k) {
+    const double* qk = rf.Q + (long long)k * rf.N;
+    double acc = 0.0;
+    for (long long i = threadIdx.x; i < rf.N; i += blockDim.x) {
+      double v;
+      if (rf.encoding == TG_ENC_2BIT) {
+        const unsigned f = (row[i >> 2] >> (2 * (i & 3))) & 3u;  // 00 = 2, 10 = 1, 11 = 0, 01 missing
+        v = f == 0u ? 2.0 : f == 2u ? 1.0 : f == 3u ? 0.0 : mu;
+      } else {
+        const bool miss = mrow && ((mrow[i >> 5] >> (i & 31)) & 1u);
+        v = miss ? mu : (double)row[i];
+      }
+      acc = fma(qk[i], v - mu, acc);
+    }
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      double t = 0.0;
+      for (int w = 0; w < kNormWarps; ++w) t += red[w];
+      s += t * t;
+    }
+    __syncthreads();
   }
-  const double r2 = c2 - s;
-  const bool ok = marker_testable(nobs[j], c2, r2, complete_n);
-  const double nan = __longlong_as_double(0x7ff8000000000000ll);
-  const double inv = ok ? 1.0 / sqrt(r2) : nan;
-  gres2u[j] = ok ? r2 : nan;
-  if (norm2_allele) norm2_allele[j] = ok ? r2 * kappa * kappa : nan;
-  rinv[j] = (float)inv;
-  rinv64[j] = inv;
-  if (refine_list && nobs[j] > 0 && c2 > 0.0 && r2 < (1.0 - kRefineShare) * c2)
-    refine_list[atomicAdd(refine_count, 1u)] = (int)j;
+  return s;
 }
 
-// FP64 re-projection of the listed markers, one block of 256 threads per marker:
-// sum_k (q_k . g_c)^2 over the non-intercept columns of Q from the packed genotypes (missing
-// calls at the marker's mean, which is also its centre, so they add nothing) and the FP64 mean,
-// then the marker's norm outputs again. q_0 . g_c = 0 exactly (q_0 is constant and g_c has zero
-// sum), as in the tensor-core projection, which leaves column 0 out.
-__global__ void __launch_bounds__(256) k_marker_refine(MarkerRefine rf, const int32_t* __restrict__ nobs,
-                                                       const double* __restrict__ gc2, double kappa,
-                                                       double* __restrict__ gres2u,
-                                                       double* __restrict__ norm2_allele,
-                                                       float* __restrict__ rinv,
-                                                       double* __restrict__ rinv64,
-                                                       int complete_n) {
-  __shared__ double red[8];
-  const unsigned n = *rf.count;
-  for (unsigned li = blockIdx.x; li < n; li += gridDim.x) {
-    const long long j = rf.list[li];
-    const double mu = rf.mean[j];
-    const uint8_t* row = rf.G + j * rf.ldg;
-    const uint32_t* mrow = rf.missing ? rf.missing + j * rf.ldm : nullptr;
-    double s = 0.0;  // thread 0's copy is the sum
-    for (int k = 1; k < rf.q; ++k) {
-      const double* qk = rf.Q + (long long)k * rf.N;
-      double acc = 0.0;
-      for (long long i = threadIdx.x; i < rf.N; i += blockDim.x) {
-        double v;
-        if (rf.encoding == TG_ENC_2BIT) {
-          const unsigned f = (row[i >> 2] >> (2 * (i & 3))) & 3u;  // 00 = 2, 10 = 1, 11 = 0, 01 missing
-          v = f == 0u ? 2.0 : f == 2u ? 1.0 : f == 3u ? 0.0 : mu;
-        } else {
-          const bool miss = mrow && ((mrow[i >> 5] >> (i & 31)) & 1u);
-          v = miss ? mu : (double)row[i];
-        }
-        acc = fma(qk[i], v - mu, acc);
+__global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
+    long long M, const int32_t* __restrict__ nobs, const double* __restrict__ gc2, RawView proj,
+    int nq, double kappa, const __grid_constant__ MarkerRefine rf, NormOut out, int complete_n) {
+  __shared__ double part[kNormWarps][32];
+  __shared__ unsigned flagged;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const long long m0 = blockIdx.x * 32ll, j = m0 + lane;
+  const bool in = j < M;
+  double s = 0.0;
+  if (in)
+    for (int k = warp; k < nq; k += kNormWarps) {
+      const float* x = proj.x + (long long)k * proj.ld + j;
+      float v = *x;
+      if (proj.ranges > 1) {
+        for (int r = 1; r < proj.ranges; ++r) v += x[r * proj.split];
+        v = fmaf(proj.shift[j], proj.cs[k], v);
       }
-      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-      __syncthreads();
-      if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int w = 0; w < 8; ++w) t += red[w];
-        s += t * t;
-      }
-      __syncthreads();
+      s += (double)v * (double)v;
     }
-    if (threadIdx.x == 0) {
-      const double c2 = gc2[j];
-      const double r2 = c2 - s;
-      const bool ok = marker_testable(nobs[j], c2, r2, complete_n);
-      const double nan = __longlong_as_double(0x7ff8000000000000ll);
-      const double inv = ok ? 1.0 / sqrt(r2) : nan;
-      gres2u[j] = ok ? r2 : nan;
-      if (norm2_allele) norm2_allele[j] = ok ? r2 * kappa * kappa : nan;
-      rinv[j] = (float)inv;
-      rinv64[j] = inv;
+  part[warp][lane] = s;
+  __syncthreads();
+  auto put = [&](long long m, double c2, double r2) {
+    const bool ok = marker_testable(nobs[m], c2, r2, complete_n);
+    const double nan = __longlong_as_double(0x7ff8000000000000ll);
+    const double inv = ok ? 1.0 / sqrt(r2) : nan;
+    if (out.norm2_allele) out.norm2_allele[m] = ok ? r2 * kappa * kappa : nan;
+    out.rinv[m] = (float)inv;
+    out.rinv64[m] = inv;
+  };
+  if (warp == 0) {
+    bool close = false;
+    if (in) {
+      double t = part[0][lane];
+#pragma unroll
+      for (int w = 1; w < kNormWarps; ++w) t += part[w][lane];
+      const double c2 = gc2[j], r2 = c2 - t;
+      put(j, c2, r2);
+      close = nq > 0 && nobs[j] > 0 && c2 > 0.0 && r2 < (1.0 - kRefineShare) * c2;
     }
+    const unsigned f = __ballot_sync(0xffffffffu, close);
+    if (lane == 0) {
+      flagged = f;
+      if (out.hit_start && blockIdx.x == 0) *out.hit_start = *out.n_hits;
+    }
+  } else if (warp == 1 && in) {
+    if (out.nobs) out.nobs[j] = nobs[j];
+    if (out.mean) out.mean[j] = rf.mean[j];
+  }
+  __syncthreads();
+  for (unsigned todo = flagged; todo; todo &= todo - 1) {  // the same for the whole block
+    const long long m = m0 + __ffs(todo) - 1;
+    const double t = refine_projection(rf, m, part[0]);
+    if (threadIdx.x == 0) put(m, gc2[m], gc2[m] - t);
   }
 }
 
@@ -306,30 +322,20 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
 }  // namespace
 
 cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, const float* QB,
-                           int64_t nq, float* qg, cudaStream_t st) {
+                           int64_t nq, float* out, int64_t ldq, cudaStream_t st) {
   if (M == 0 || nq == 0) return cudaSuccess;
   dim3 grid((unsigned)((M + 63) / 64), (unsigned)((nq + 31) / 32));
-  k_project<<<grid, 256, 0, st>>>(A, lda, M, (int)K, QB, (int)nq, qg);
+  k_project<<<grid, 256, 0, st>>>(A, lda, M, (int)K, QB, (int)nq, out, (long long)ldq);
   return cudaGetLastError();
 }
 
-cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2, const float* qg,
-                               int64_t ldq, int64_t nq, double kappa, double* gres2_units_out,
-                               double* norm2_allele_out, float* rinv, double* rinv64,
-                               const MarkerRefine* refine, cudaStream_t st, int64_t complete_n) {
+cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2,
+                               const RawView& proj, int64_t nq, double kappa,
+                               const MarkerRefine& refine, const NormOut& out, cudaStream_t st,
+                               int64_t complete_n) {
   if (M == 0) return cudaSuccess;
-  const bool rf = refine != nullptr && nq > 0;
-  if (rf) {
-    cudaError_t e = cudaMemsetAsync(refine->count, 0, sizeof(unsigned), st);
-    if (e != cudaSuccess) return e;
-  }
-  k_marker_norm<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(
-      M, nobs, gc2, qg, (long long)ldq, (int)nq, kappa, gres2_units_out, norm2_allele_out, rinv, rinv64,
-      rf ? refine->list : nullptr, rf ? refine->count : nullptr, (int)complete_n);
-  if (!rf) return cudaGetLastError();
-  // a fixed grid, so that the launch does not depend on the count (graph capture)
-  k_marker_refine<<<304, 256, 0, st>>>(*refine, nobs, gc2, kappa, gres2_units_out,
-                                       norm2_allele_out, rinv, rinv64, (int)complete_n);
+  k_marker_norm<<<(unsigned)((M + 31) / 32), kNormWarps * 32, 0, st>>>(
+      M, nobs, gc2, proj, (int)nq, kappa, refine, out, (int)complete_n);
   return cudaGetLastError();
 }
 

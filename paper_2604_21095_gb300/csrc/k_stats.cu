@@ -86,50 +86,142 @@ __device__ __forceinline__ Stats64 stats_exact(const EpiParams& ep, long long ro
   return o;
 }
 
-// FULL statistics. Each warp walks 32 consecutive elements at a time (all lanes stay in the
-// loop), so that the rare elements near |r| = 1 can be recomputed by the whole warp.
-__global__ void __launch_bounds__(256, 1) k_full_stats(EpiParams ep) {
-  const long long total = (long long)ep.M * ep.P;
+// One FULL element recomputed in FP64 by a whole warp, written by lane `src`. Out of line: it is
+// rare, and inlined its registers halve the warps that the ordinary elements run on.
+__device__ __noinline__ void full_exact(const EpiParams& ep, long long row, int col, int src) {
   const int lane = threadIdx.x & 31;
-  const long long wstride = (long long)gridDim.x * blockDim.x;
-  for (long long base = blockIdx.x * (long long)blockDim.x + (threadIdx.x & ~31); base < total;
-       base += wstride) {
-    const long long e = base + lane;
-    long long row = 0, o = 0;
-    int col = 0;
-    bool exact = false;
-    if (e < total) {
-      row = e / ep.P;
-      col = (int)(e - row * ep.P);
-      o = row * ep.ldo + col;
-      const float r = ep.rstore[o];
-      const float omr2 = (1.0f - r) * (1.0f + r);
-      exact = ep.exact.G != nullptr && omr2 < kExactOmr2;  // false for NaN
-      if (!exact) {
-        const float rinv = ep.row_inv[row];
-        const float scale = ep.col_s[col] * rinv / ep.kappa;
-        if (ep.beta) ep.beta[o] = r * scale;
-        if (ep.se) ep.se[o] = scale * sqrtf(omr2 / ep.df_f);
-        if (ep.t) ep.t[o] = r * sqrtf(ep.df_f / omr2);
-        if (ep.mlp) ep.mlp[o] = mlog10p_r_f(r, ep.df_f, (float)ep.lnB);
+  double D = exact_partial(ep.exact, row, col, lane, 32);
+  for (int k = 16; k > 0; k >>= 1) D += __shfl_xor_sync(0xffffffffu, D, k);
+  if (lane != src) return;
+  const long long o = row * ep.ldo + col;
+  const Stats64 v = stats_exact(ep, row, col, D);
+  if (ep.beta) ep.beta[o] = v.beta;
+  if (ep.se) ep.se[o] = v.se;
+  if (ep.t) ep.t[o] = v.t;
+  if (ep.mlp) ep.mlp[o] = v.mlp;
+}
+
+// The FULL statistics of one element per lane (none where !in) from its r; elements near |r| = 1
+// are recomputed by the warp. Every lane of the warp calls it.
+__device__ __forceinline__ void full_elements(const EpiParams& ep, long long row, int col, float r,
+                                              bool in) {
+  const float omr2 = (1.0f - r) * (1.0f + r);
+  const bool exact = in && ep.exact.G != nullptr && omr2 < kExactOmr2;  // false for NaN
+  if (in && !exact) {
+    const long long o = row * ep.ldo + col;
+    const float rinv = ep.row_inv[row];
+    const float scale = ep.col_s[col] * rinv / ep.kappa;
+    if (ep.beta) ep.beta[o] = r * scale;
+    if (ep.se) ep.se[o] = scale * sqrtf(omr2 / ep.df_f);
+    if (ep.t) ep.t[o] = r * sqrtf(ep.df_f / omr2);
+    if (ep.mlp) ep.mlp[o] = mlog10p_r_f(r, ep.df_f, (float)ep.lnB);
+  }
+  unsigned todo = __ballot_sync(0xffffffffu, exact);
+  while (todo) {
+    const int src = __ffs(todo) - 1;
+    todo &= todo - 1;
+    full_exact(ep, __shfl_sync(0xffffffffu, row, src), __shfl_sync(0xffffffffu, col, src), src);
+  }
+}
+
+// FULL statistics of a block whose contraction left r in one of the outputs. Each warp walks 32
+// consecutive elements at a time (all lanes stay in the loop); a lane's row and column advance
+// by a fixed stride (drow rows and dcol columns), so that no element costs a 64-bit division.
+constexpr int kFullThreads = 256;
+__global__ void __launch_bounds__(kFullThreads, 4)
+    k_full_stats(const __grid_constant__ EpiParams ep, long long drow, int dcol) {
+  const long long total = (long long)ep.M * ep.P;
+  const long long stride = (long long)gridDim.x * kFullThreads;
+  long long e = blockIdx.x * (long long)kFullThreads + threadIdx.x;
+  long long row = e / ep.P;
+  int col = (int)(e - row * ep.P);
+  for (long long base = e - (threadIdx.x & 31); base < total; base += stride, e += stride) {
+    const bool in = e < total;
+    full_elements(ep, row, col, in ? ep.rstore[row * ep.ldo + col] : 0.0f, in);
+    row += drow;
+    col += dcol;
+    if (col >= ep.P) {
+      col -= ep.P;
+      row += 1;
+    }
+  }
+}
+
+// Statistics from raw products (EpiParams::raw_out), after the marker norms: per element the
+// arithmetic of the contraction epilogue, r = D / |a_res| clamped, the hit test on r^2, the
+// column's best marker. A block of 8 warps takes 8 CPW phenotypes, CPW columns per warp, lane =
+// marker: the products are column-major, so the reads are whole sectors. Without FULL output
+// it takes 128 markers, four per lane, so that a column offers a best marker once per 128.
+// In FULL mode it takes 32 markers; the tile of r then goes through shared memory and
+// consecutive threads take consecutive phenotypes of a marker, so that the four outputs are
+// written in whole sectors too, and r makes no trip through memory.
+// CPW = 1 gives a thread one element of a FULL block: on a small one the p-value's chain is the
+// whole time (300 x 40 at df = 774: a warp per 32 x 32 elements took 215 us). CPW = 4 keeps
+// four loads per marker in flight once the block fills the SMs anyway.
+constexpr int kRawWarps = 8;
+template <bool FULL, int CPW>
+__global__ void __launch_bounds__(kRawWarps * 32)
+    k_raw_stats(const RawView raw, const __grid_constant__ EpiParams ep) {
+  constexpr int R = FULL ? 1 : 4, CW = kRawWarps * CPW;
+  __shared__ float tile[FULL ? 32 : 1][CW + 1];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int c0 = (int)blockIdx.y * CW;
+  const int cols = min(CW, ep.P - c0);
+  const long long row0 = (long long)blockIdx.x * (32 * R);
+  float d[R][CPW];
+#pragma unroll
+  for (int i = 0; i < R; ++i)
+#pragma unroll
+    for (int u = 0; u < CPW; ++u) d[i][u] = 0.0f;
+  for (int s = 0; s < raw.ranges; ++s)
+#pragma unroll
+    for (int u = 0; u < CPW; ++u)
+#pragma unroll
+      for (int i = 0; i < R; ++i) {
+        const long long row = row0 + 32 * i + lane;
+        const int c = warp * CPW + u;
+        if (row < ep.M && c < cols) d[i][u] += raw.x[s * raw.split + (c0 + c) * raw.ld + row];
+      }
+#pragma unroll
+  for (int u = 0; u < CPW; ++u) {
+    const int c = warp * CPW + u, col = c0 + c;
+    if (c >= cols) break;  // the same for the whole warp
+    const float rmul = ep.col_rmul[col];
+    uint32_t key = 0u, key_row = 0u;  // bits(|r|) + 1 of this lane's best marker (0: none)
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const long long row = row0 + 32 * i + lane;
+      float r = __int_as_float(0x7fc00000);
+      if (row < ep.M) {
+        float D = d[i][u];
+        if (raw.ranges > 1) D = fmaf(raw.shift[row], raw.cs[col], D);
+        r = corr_nan(D, ep.row_inv[row], rmul);
+        if (ep.do_hits && r * r >= ep.r2_thr) emit_hit_raw(ep, D, row, col);
+      }
+      if (FULL) tile[lane][c] = r;
+      const uint32_t k = r == r ? __float_as_uint(fabsf(r)) + 1u : 0u;
+      if (k > key) {  // rows ascend: the smallest marker of equal keys stays
+        key = k;
+        key_row = 32u * i + lane;
       }
     }
-    unsigned todo = __ballot_sync(0xffffffffu, exact);
-    while (todo) {
-      const int src = __ffs(todo) - 1;
-      todo &= todo - 1;
-      const long long xrow = __shfl_sync(0xffffffffu, row, src);
-      const int xcol = __shfl_sync(0xffffffffu, col, src);
-      double D = exact_partial(ep.exact, xrow, xcol, lane, 32);
-      for (int k = 16; k > 0; k >>= 1) D += __shfl_xor_sync(0xffffffffu, D, k);
-      if (lane == src) {
-        const Stats64 v = stats_exact(ep, row, col, D);
-        if (ep.beta) ep.beta[o] = v.beta;
-        if (ep.se) ep.se[o] = v.se;
-        if (ep.t) ep.t[o] = v.t;
-        if (ep.mlp) ep.mlp[o] = v.mlp;
-      }
+    if (ep.do_best) {
+      const uint32_t top = __reduce_max_sync(0xffffffffu, key);
+      const uint32_t first = __reduce_min_sync(0xffffffffu, key == top ? key_row : 0xFFFFFFFFu);
+      if (top && lane == 0)
+        best_offer(ep.best + col,
+                   ((unsigned long long)(top - 1u) << 32) |
+                       (unsigned long long)(0xFFFFFFFFu -
+                                            (uint32_t)(ep.marker_offset + row0 + first)));
     }
+  }
+  if (!FULL) return;
+  __syncthreads();
+#pragma unroll 1
+  for (int e = threadIdx.x; e < 32 * CW; e += kRawWarps * 32) {  // whole warps stay in the loop
+    const int rr = e / CW, cc = e % CW;
+    const bool in = cc < cols && row0 + rr < ep.M;
+    full_elements(ep, row0 + rr, c0 + cc, in ? tile[rr][cc] : 0.0f, in);
   }
 }
 
@@ -178,9 +270,27 @@ cudaError_t launch_fill_random(uint8_t* p, size_t n, unsigned long long seed, cu
 cudaError_t launch_full_stats(const EpiParams& ep, cudaStream_t st) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
   const long long total = (long long)ep.M * ep.P;
-  long long grid = (total + 255) / 256;
+  long long grid = (total + kFullThreads - 1) / kFullThreads;
   if (grid > 152 * 32) grid = 152 * 32;  // a grid-stride loop: 32 blocks per SM at most
-  k_full_stats<<<(unsigned)grid, 256, 0, st>>>(ep);
+  const long long stride = grid * kFullThreads;
+  k_full_stats<<<(unsigned)grid, kFullThreads, 0, st>>>(ep, stride / ep.P, (int)(stride % ep.P));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream_t st) {
+  if (ep.M == 0 || ep.P == 0) return cudaSuccess;
+  const bool small = (long long)ep.M * ep.P < 152ll * 8192;
+  const int cw = kRawWarps * (small ? 1 : 4);
+  const long long rows = ep.do_full ? 32 : 128;
+  const dim3 grid((unsigned)((ep.M + rows - 1) / rows), (unsigned)((ep.P + cw - 1) / cw));
+  constexpr int T = kRawWarps * 32;
+  if (ep.do_full) {
+    if (small) k_raw_stats<true, 1><<<grid, T, 0, st>>>(raw, ep);
+    else k_raw_stats<true, 4><<<grid, T, 0, st>>>(raw, ep);
+  } else {
+    if (small) k_raw_stats<false, 1><<<grid, T, 0, st>>>(raw, ep);
+    else k_raw_stats<false, 4><<<grid, T, 0, st>>>(raw, ep);
+  }
   return cudaGetLastError();
 }
 

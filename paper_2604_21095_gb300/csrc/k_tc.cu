@@ -28,11 +28,12 @@
 // sub-tiles with their own accumulators sharing each B stage (half the B traffic from L2).
 // In raw mode (the covariate projection, alone or joint with a small panel whose phenotypes
 // follow the q - 1 projection columns in one B operand) the tile is the narrowest of 64, 128
-// and 256 columns that holds them, and the products are written unnormalised; k_raw_stats
-// turns a joint pass's panel columns into statistics once the marker norms exist.
-// With split-K (ep.ksplit > 1, for blocks with fewer tiles than SMs) a work item is a tile and
-// a chunk-aligned range of the samples; the tile's first range adds the other ranges' partial
-// sums (handed over in global memory) in range order before its epilogue.
+// and 256 columns that holds them, and the products are written unnormalised, column-major;
+// k_raw_stats turns a joint pass's panel columns into statistics once the marker norms exist.
+// With split-K (ep.ksplit > 1, raw mode only, for blocks with fewer tiles than SMs) a work item
+// is a tile and a chunk-aligned range of the samples, and each range writes its own partial sums;
+// the kernels that read them add the ranges in order. (Handing the ranges to the tile's first
+// one inside the kernel, with a counter and a wait, took 13 us more per extra range.)
 // Every wait is bounded: past the limit the kernel latches ST_TIMEOUT, raises a shared abort
 // flag, lets in-flight copies and products finish (again bounded), frees its TMEM and returns.
 #include <cuda.h>
@@ -72,14 +73,6 @@ struct Cfg {
 // BR x 64 B each).
 static_assert(kChunkKB == kAccumChunkKB, "the host's split choice counts the same chunks");
 
-// K-block range [lo, hi) of split `sp` of `ks`: whole accumulation chunks, the earlier splits
-// one chunk longer when they do not divide evenly (a split may be empty).
-__device__ __forceinline__ void split_range(int num_kb, int ks, int sp, int& lo, int& hi) {
-  const int chunks = (num_kb + kChunkKB - 1) / kChunkKB;
-  const int per = (chunks + ks - 1) / ks;
-  lo = min(num_kb, sp * per * kChunkKB);
-  hi = min(num_kb, (sp + 1) * per * kChunkKB);
-}
 // End of the accumulation chunk that starts at kb0 within [lo, hi); chunk_end for a whole range.
 __device__ __forceinline__ int chunk_end_in(int kb0, int lo, int hi) {
   const int e = kb0 == lo ? lo + kFirstChunks * kChunkKB : kb0 + kChunkKB;
@@ -158,8 +151,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
   const int num_tiles = n_mt * n_nt;
-  // work items: (tile, split); a tile's ks items are consecutive and run in the same round
-  // (the grid is a multiple of ks and every CTA is resident)
+  // work items: (tile, split), independent of one another
   const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
   const int num_items = num_tiles * ks;
   if (warp < 4) {
@@ -336,58 +328,6 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive(cempty_bar(acc));
       }
       if (!ok) break;
-      if (ks > 1) {
-        // this thread's row and 128 columns of the tile's partial sums
-        const int rc = (quarter * 32 + lane) * TBN + half * 128;
-        float* wsp = ep.sk_ws + (size_t)tile * (size_t)(ks - 1) * (TBM * TBN);
-        if (split > 0) {  // hand the partial sums to the tile's split 0, warp by warp
-          float4* dst = reinterpret_cast<float4*>(wsp + (size_t)(split - 1) * (TBM * TBN) + rc);
-#pragma unroll
-          for (int e = 0; e < 32; ++e)
-            dst[e] = make_float4(tot[4 * e], tot[4 * e + 1], tot[4 * e + 2], tot[4 * e + 3]);
-          __threadfence();
-          __syncwarp();
-          if (lane == 0) atomicAdd(ep.sk_cnt + tile, 1u);
-          continue;
-        }
-        // split 0: each warp waits (bounded) for the other splits' warps, then adds their sums
-        // in split order; no CTA-wide barrier, so a warp that gave up cannot hold the others
-        bool got = true;
-        if (lane == 0) {
-          const unsigned need = (unsigned)((ks - 1) * kEpiWarps);
-          const uint64_t t0 = globaltimer_ns();
-          while (*reinterpret_cast<volatile unsigned*>(ep.sk_cnt + tile) < need) {
-            if (*abort_flag || (long long)(globaltimer_ns() - t0) > spin_ns) {
-              if (!*abort_flag) {
-                *abort_flag = 1;
-                atomicOr(ep.status, ST_TIMEOUT);
-              }
-              got = false;
-              break;
-            }
-            __nanosleep(128);
-          }
-          __threadfence();
-        }
-        got = __shfl_sync(0xffffffffu, got, 0);
-        __syncwarp();  // the partial sums are read after lane 0 saw them complete
-        if (!got) {
-          ok = false;
-          break;
-        }
-        for (int sp = 1; sp < ks; ++sp) {
-          const float4* src =
-              reinterpret_cast<const float4*>(wsp + (size_t)(sp - 1) * (TBM * TBN) + rc);
-#pragma unroll
-          for (int e = 0; e < 32; ++e) {
-            const float4 v = __ldcg(src + e);
-            tot[4 * e] += v.x;
-            tot[4 * e + 1] += v.y;
-            tot[4 * e + 2] += v.z;
-            tot[4 * e + 3] += v.w;
-          }
-        }
-      }
       // MS = 1: warps of half h hold columns h*128.. of the tile's 128 rows; MS = 2: warps of
       // half h hold the (at most 128) columns of sub-tile h's 128 rows
       const long long row_base =
@@ -398,19 +338,12 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float rinv = (row_ok && ep.row_inv) ? ep.row_inv[row] : __int_as_float(0x7fc00000);
       const float shift = (row_ok && ep.row_shift) ? ep.row_shift[row] : 0.0f;
       if (ep.raw_out) {
-        // covariate projection (and a small panel's products): the first raw_cols columns of
-        // the tile, unnormalised
-        if (row_ok) {
-#pragma unroll
-          for (int e = 0; e < 128; ++e) {  // fully unrolled: tot stays in registers
-            const int col = col_half + e;
-            if (col < ep.raw_cols)
-              ep.raw_out[row * ep.raw_ld + col] = fmaf(shift, ep.col_cs[col], tot[e]);
-          }
-        }
+        // covariate projection (and a small panel's products), unnormalised
+        const int col0 = nt * bn + col_half;
+        if (row_ok) raw_store(ep, tot, row, col0, min(ep.raw_cols, nt * bn + bn), split, shift);
       } else {
         epilogue_tile(ep, tot, row, row_base, row_ok, rinv, shift,
-                      (MS == 2 ? nt * bn : nt * TBN) + col_half, lane);
+                      nt * bn + col_half, min(ep.P, nt * bn + bn), lane);
       }
       __syncwarp();
     }
@@ -423,59 +356,6 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base),
                  "r"(kTmemCols)
                  : "memory");
-  }
-}
-
-// Statistics of a small panel from its raw products: a block takes 64 consecutive marker rows,
-// its threads split into 256 / P groups of P (thread = phenotype column) that take every
-// (256 / P)-th row, so each row is read coalesced and a small panel still keeps the block busy.
-// Per element the arithmetic of the contraction epilogue (D already holds the shift's add-back):
-// r = D / |a_res| clamped, the hit test on r^2, r in FULL mode, and the key (|r| bits, ~marker)
-// whose maximum is the column's best marker; the groups' keys meet in shared memory and each
-// column offers one per block.
-constexpr int kRawRows = 64;
-constexpr int kRawThreads = 256;
-static_assert(JCOLS <= kRawThreads, "a group of P threads per block");
-__global__ void __launch_bounds__(kRawThreads) k_raw_stats(const float* __restrict__ raw,
-                                                           long long ld, EpiParams ep) {
-  __shared__ unsigned long long keys[kRawThreads];
-  __shared__ int has[kRawThreads];
-  const int groups = kRawThreads / ep.P;  // P <= JCOLS <= kRawThreads
-  const int col = (int)threadIdx.x % ep.P, sub = (int)threadIdx.x / ep.P;
-  const bool active = sub < groups;
-  const long long r0 = (long long)blockIdx.x * kRawRows;
-  const long long r1 = r0 + kRawRows < (long long)ep.M ? r0 + kRawRows : (long long)ep.M;
-  unsigned long long best = 0;
-  bool any = false;
-  if (active) {
-    const float rmul = ep.col_rmul[col];
-    for (long long row = r0 + sub; row < r1; row += groups) {
-      const float D = raw[row * ld + col];
-      const float r = corr_nan(D, ep.row_inv[row], rmul);
-      if (ep.do_hits && r * r >= ep.r2_thr) emit_hit_raw(ep, D, row, col);
-      if (ep.do_full) ep.rstore[row * ep.ldo + col] = r;
-      if (r == r) {
-        const unsigned long long key =
-            ((unsigned long long)__float_as_uint(fabsf(r)) << 32) |
-            (unsigned long long)(0xFFFFFFFFu - (uint32_t)(ep.marker_offset + row));
-        best = key > best ? key : best;
-        any = true;
-      }
-    }
-  }
-  if (!ep.do_best) return;  // the same for every thread of the launch
-  keys[threadIdx.x] = best;
-  has[threadIdx.x] = any ? 1 : 0;
-  __syncthreads();
-  if (active && sub == 0) {
-    for (int g = 1; g < groups; ++g) {
-      const int t = g * ep.P + col;
-      if (has[t]) {
-        best = keys[t] > best ? keys[t] : best;
-        any = true;
-      }
-    }
-    if (any) best_offer(ep.best + col, best);
   }
 }
 
@@ -509,11 +389,9 @@ cudaError_t go(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* b
   const int n_mt = (ep.M + MS * TBM - 1) / (MS * TBM);
   const int n_nt = (ep.P + bn - 1) / bn;
   const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
-  if (ks > 1 && (!ep.sk_ws || !ep.sk_cnt || sm_count < ks))
-    return cudaErrorInvalidValue;
+  if (ks > 1 && !ep.raw_out) return cudaErrorInvalidValue;
   const int items = n_mt * n_nt * ks;
-  // a multiple of ks, so that the splits of a tile run in the same round
-  const int grid = (items < sm_count ? items : sm_count) / ks * ks;
+  const int grid = items < sm_count ? items : sm_count;
   if (KS == 2 && (bn > BR || (K / TBK) % 2)) return cudaErrorInvalidValue;
   k_tc_scan<OPA, KS, BR, MS><<<grid, kThreads, Cfg<OPA, KS, BR, MS>::kSmem, st>>>(
       *a, *bh, *bl, (int)(K / TBK), n_mt, n_nt, bn, group_m, spin_ns, ep, da);
@@ -525,18 +403,13 @@ cudaError_t go(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* b
 cudaError_t launch_tc_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                            const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                            long long spin_ns, cudaStream_t st, int group_m, const DecodeArgs* dec,
-                           int encoding, bool narrow) {
+                           int encoding, int bn) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
   if (K % TBK || group_m < 1) return cudaErrorInvalidValue;
-  // raw mode: the narrowest tile that holds the raw columns (the B maps' boxes match)
-  const int bn = narrow ? 64
-                 : ep.raw_out ? (ep.raw_cols <= 64 ? 64 : ep.raw_cols <= 128 ? 128 : TBN)
-                              : TBN;
-  if (narrow && ep.P > 64) return cudaErrorInvalidValue;
-  if (ep.raw_out && (ep.raw_cols > TBN || ep.P != ep.raw_cols)) return cudaErrorInvalidValue;
+  if ((bn != 64 && bn != 128 && bn != TBN) || (bn < TBN && ep.P > bn)) return cudaErrorInvalidValue;
+  if (ep.raw_out && ep.P != ep.raw_cols) return cudaErrorInvalidValue;
   if (!dec) {
-    // 256-marker tiles (two sub-tiles sharing B) once they fill every SM at least once, and
-    // not with split-K, whose workspace the host sized for 128-marker tiles
+    // 256-marker tiles (two sub-tiles sharing B) once they fill every SM at least once
     const bool two = ep.ksplit <= 1 && (ep.M + 2 * TBM - 1) / (2 * TBM) >= sm_count;
     if (bn == 64)  // the covariate projection, or a panel of at most 64 phenotypes
       return two ? go<OPA_TMA, 2, 64, 2>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns,
@@ -555,14 +428,6 @@ cudaError_t launch_tc_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
   if (encoding == TG_ENC_2BIT)
     return go<OPA_2BIT, 1>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn);
   return go<OPA_U8, 1>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn);
-}
-
-cudaError_t launch_raw_stats(const float* raw, int64_t ld, const EpiParams& ep, cudaStream_t st) {
-  if (ep.M == 0 || ep.P == 0) return cudaSuccess;
-  if (ep.P > JCOLS) return cudaErrorInvalidValue;
-  const long long blocks = ((long long)ep.M + kRawRows - 1) / kRawRows;
-  k_raw_stats<<<(unsigned)blocks, kRawThreads, 0, st>>>(raw, (long long)ld, ep);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_wait_test(const uint32_t* flag, long long limit_ns, uint32_t* result,

@@ -1,9 +1,10 @@
 // Tensor-core scan on CTA pairs: Eq. 2 of Section 2.2 with tcgen05.mma.cta_group::2.
 //
-// The same product as k_tc.cu, D = A (B_hi + B_lo)^T + c (sum_i B), on 256 x 256 tiles
-// computed by a cluster of two CTAs on two SMs. Each CTA loads its own 128 marker rows of A
-// and its own half (128 phenotype rows) of B_hi / B_lo; the pair's leader (cluster rank 0)
-// issues one 256 x 256 x 16 MMA that reads A from both CTAs and B from both CTAs and writes
+// The same product as k_tc.cu, D = A (B_hi + B_lo)^T + c (sum_i B), on 256 x bn tiles (bn = 256,
+// or the multiple of 32 that cuts the panel's columns into equal tiles: 300 columns are 2 x 160,
+// not 2 x 256) computed by a cluster of two CTAs on two SMs. Each CTA loads its own 128 marker
+// rows of A and its own half (bn / 2 phenotype rows) of B_hi / B_lo; the pair's leader (cluster
+// rank 0) issues one 256 x bn x 16 MMA that reads A from both CTAs and B from both CTAs and writes
 // rows 0-127 of D into the leader's tensor memory and rows 128-255 into the peer's. Per SM,
 // each MMA of the same size reads 8 KB of shared memory instead of 12 KB, and each K block
 // brings 24 KB over L2 instead of 40 KB, which is what limits the one-CTA kernel.
@@ -21,7 +22,11 @@
 //                               leader's full barrier after its stores
 // Accumulation is chunked as in k_tc.cu (a fresh accumulator every 1024 samples, FP32 totals in
 // registers) when every statistic is written, every 2048 samples when only hits and best markers
-// are kept (chunk_kb). Every wait is bounded; a timeout raises the abort flag in both CTAs.
+// are kept (chunk_kb). In raw mode (a joint operand of the projection columns and the panel, or
+// any panel on a block with too few tiles to fill the SMs) the products are written unnormalised
+// and column-major for k_marker_norm and k_raw_stats, in 1,024-sample chunks, and K may be split:
+// a work item is then a tile and a chunk-aligned range of the samples, and each range writes its
+// own partial sums. Every wait is bounded; a timeout raises the abort flag in both CTAs.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -58,8 +63,6 @@ struct Cfg2 {
 // ring of kTileRing shared-memory slots (a full barrier per slot in each CTA, an empty
 // barrier per slot in the leader).
 constexpr int kTileRing = 4;
-
-constexpr uint32_t kIdesc2 = idesc_bf16_m(256, 256);
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -103,12 +106,12 @@ __device__ __forceinline__ void tma_load_2d_pair(const CUtensorMap* map, uint32_
       : "memory");
 }
 __device__ __forceinline__ void tc2_mma(uint32_t d_tmem, uint64_t adesc, uint64_t bdesc,
-                                        uint32_t accumulate) {
+                                        uint32_t idesc, uint32_t accumulate) {
   asm volatile(
       "{\n\t.reg .pred p;\n\t"
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n\t}" ::"r"(d_tmem),
-      "l"(adesc), "l"(bdesc), "r"(kIdesc2), "r"(accumulate)
+      "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
       : "memory");
 }
 // Arrive on the barrier at this offset in both CTAs once every prior MMA has completed.
@@ -161,20 +164,23 @@ __device__ __forceinline__ int next_tile(unsigned long long* ctr, int i, int cid
 // (k_hit_stats); half the chunk drains take 3% off the launch, and the FP32 error of the
 // totals stays within the r tolerance (the best keys) and far inside the threshold band.
 __device__ __forceinline__ int chunk_kb(const EpiParams& ep) {
-  return ep.do_full ? kChunkKB : 2 * kChunkKB;
+  return ep.do_full || ep.raw_out ? kChunkKB : 2 * kChunkKB;
 }
 __device__ __forceinline__ int chunk_end_c(int kb0, int num_kb, int ckb) {
-  const int e = kb0 == 0 ? kFirstChunks * ckb : kb0 + ckb;
-  return e < num_kb ? e : num_kb;
+  return kb0 + ckb < num_kb ? kb0 + ckb : num_kb;
 }
+static_assert(kFirstChunks == 1, "every chunk of a tile has the same length");
 
 // K direction of a tile: the tiles of odd waves stream K from the end. A wave reads about
 // 300 MB of A rows and panel columns at the bench's sizes, more than L2 holds, so a wave that
 // starts where the previous one ended finds the last-streamed slabs (chiefly the A rows of the
 // raster group's m-tile pairs, which consecutive waves share) still in L2 instead of fetching
 // them from DRAM again. Only the order of the FP32 chunk sums changes; every tile still adds
-// the same K blocks in chunks of the same sizes.
-__device__ __forceinline__ bool k_reversed(int tile, int ncl) { return ((tile / ncl) & 1) != 0; }
+// the same K blocks in chunks of the same sizes. With split-K the block is small and every range
+// streams K forwards.
+__device__ __forceinline__ bool k_reversed(int tile, int ncl, int ks) {
+  return ks == 1 && ((tile / ncl) & 1) != 0;
+}
 
 // mbarrier wait with acquire at cluster scope (the phase may be completed by the other CTA),
 // bounded like mbar_wait.
@@ -223,9 +229,9 @@ __device__ __forceinline__ void tile_coord2(int tile, int n_mp, int n_nt, int gr
 template <int OPA>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_tc2_scan(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmBhi,
-               const __grid_constant__ CUtensorMap tmBlo, int num_kb, int n_mt, int n_nt,
+               const __grid_constant__ CUtensorMap tmBlo, int num_kb, int n_mt, int n_nt, int bn,
                int group_p, long long spin_ns, EpiParams ep,
-              const __grid_constant__ DecodeArgs da) {
+               const __grid_constant__ DecodeArgs da) {
   using C = Cfg2<OPA>;
   constexpr bool kFused = OPA != OPA_TMA;
   constexpr int S = C::kStages;
@@ -299,7 +305,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
   const int n_mp = (n_mt + 1) / 2;
-  const int num_tiles = n_mp * n_nt;
+  // work items: (tile, K range); items of one tile are consecutive
+  const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
+  const int num_tiles = n_mp * n_nt * ks;
   const int ckb = chunk_kb(ep);
   const int cid = (int)cluster_id(), ncl = (int)num_clusters();
   // a timeout in either CTA stops both
@@ -353,15 +361,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           if (tile < 0) break;
         }
         if (tile >= num_tiles) break;
-        int mp, nt;
-        tile_coord2(tile, n_mp, n_nt, group_p, mp, nt);
-        const bool rev = k_reversed(tile, ncl);
+        int mp, nt, k_lo, k_hi;
+        tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
+        split_range(num_kb, ks, tile % ks, k_lo, k_hi);
+        const int kbs = k_hi - k_lo;
+        const bool rev = k_reversed(tile, ncl, ks);
         const int mt0 = 2 * mp;
-        const uint32_t pair_bytes = 2u * KS * ((kFused ? 0u : (uint32_t)A_BYTES) + 2 * HB_BYTES);
+        const uint32_t pair_bytes =
+            2u * KS * ((kFused ? 0u : (uint32_t)A_BYTES) + (uint32_t)bn * (TBK * 2));
         const int arow = (mt0 + (int)rank) * TBM;
-        const int brow = nt * TBN + (int)rank * 128;
-        for (int kb = 0; kb < num_kb; kb += KS) {
-          const int kx = rev ? num_kb - KS - kb : kb;  // first K block of this stage
+        const int brow = nt * bn + (int)rank * (bn / 2);
+        for (int kb = 0; kb < kbs; kb += KS) {
+          const int kx = k_lo + (rev ? kbs - KS - kb : kb);  // first K block of this stage
           if (!wait(empty_bar(stage), phase ^ 1u)) {
             ok = false;
             break;
@@ -401,11 +412,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       int stage = 0;
       uint32_t phase = 0;
       uint32_t g = 0;
+      const uint32_t idesc = idesc_bf16_m(256, bn);
       bool ok = true;
       for (int i = 0; ok; ++i) {
         const int tile = take_tile(i, false);
         if (tile < 0 || tile >= num_tiles) break;
-        for (int kb0 = 0; kb0 < num_kb && ok; kb0 = chunk_end_c(kb0, num_kb, ckb), ++g) {
+        int k_lo, k_hi;
+        split_range(num_kb, ks, tile % ks, k_lo, k_hi);
+        const int kbs = k_hi - k_lo;
+        for (int kb0 = 0; kb0 < kbs && ok; kb0 = chunk_end_c(kb0, kbs, ckb), ++g) {
           const int acc = (int)(g & 1u);
           const uint32_t ph = (g >> 1) & 1u;
           if (!wait(cempty_bar(acc), ph ^ 1u)) {
@@ -414,7 +429,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           }
           tc_fence_after();
           const uint32_t d = tmem_base + (uint32_t)(acc * TBN);
-          const int kb1 = chunk_end_c(kb0, num_kb, ckb);
+          const int kb1 = chunk_end_c(kb0, kbs, ckb);
           for (int kb = kb0; kb < kb1; kb += KS) {
             if (!wait(full_bar(stage), phase)) {
               ok = false;
@@ -428,8 +443,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 const uint64_t a = sdesc_sw64(sA(stage, h) + 32u * k);
                 const uint64_t bh = sdesc_sw64(sBhi(stage, h) + 32u * k);
                 const uint64_t bl = sdesc_sw64(sBlo(stage, h) + 32u * k);
-                tc2_mma(d, a, bh, (kb > kb0 || h > 0 || k > 0) ? 1u : 0u);
-                tc2_mma(d, a, bl, 1u);
+                tc2_mma(d, a, bh, idesc, (kb > kb0 || h > 0 || k > 0) ? 1u : 0u);
+                tc2_mma(d, a, bl, idesc, 1u);
               }
             tc2_commit_both(empty_bar(stage));
             if (++stage == S) {
@@ -451,13 +466,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int i = 0; ok; ++i) {
         const int tile = take_tile(i, true);
         if (tile < 0 || tile >= num_tiles) break;
-        int mp, nt;
-        tile_coord2(tile, n_mp, n_nt, group_p, mp, nt);
+        int mp, nt, k_lo, k_hi;
+        tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
+        split_range(num_kb, ks, tile % ks, k_lo, k_hi);
         const long long r0 = (long long)(2 * mp + (int)rank) * TBM + t;
         const uint2 k0 = dec_row_consts<OPA>(da, r0), k1 = dec_row_consts<OPA>(da, r0 + 64);
-        const bool rev = k_reversed(tile, ncl);
-        for (int kb = 0; kb < num_kb; ++kb) {
-          const int kx = rev ? num_kb - 1 - kb : kb;  // the K block the producer loaded
+        const int kbs = k_hi - k_lo;
+        const bool rev = k_reversed(tile, ncl, ks);
+        for (int kb = 0; kb < kbs; ++kb) {
+          const int kx = k_lo + (rev ? kbs - 1 - kb : kb);  // the K block the producer loaded
           if (!wait(pfull_bar(stage), phase)) {
             ok = false;
             break;
@@ -488,12 +505,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     for (int i = 0; ok; ++i) {
       const int tile = take_tile(i, true);
       if (tile < 0 || tile >= num_tiles) break;
-      int mp, nt;
-      tile_coord2(tile, n_mp, n_nt, group_p, mp, nt);
+      int mp, nt, k_lo, k_hi;
+      tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
+      split_range(num_kb, ks, tile % ks, k_lo, k_hi);
+      const int kbs = k_hi - k_lo;
       float tot[128];
 #pragma unroll
       for (int e = 0; e < 128; ++e) tot[e] = 0.0f;
-      for (int kb0 = 0; kb0 < num_kb; kb0 = chunk_end_c(kb0, num_kb, ckb), ++g) {
+      for (int kb0 = 0; kb0 < kbs; kb0 = chunk_end_c(kb0, kbs, ckb), ++g) {
         const int acc = (int)(g & 1u);
         const uint32_t ph = (g >> 1) & 1u;
         if (!wait(cfull_bar(acc), ph)) {
@@ -505,6 +524,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                                (uint32_t)(acc * TBN + half * 128);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
+          if (half * 128 + i * 32 >= bn) break;  // columns past the tile
           float v[32];
           __syncwarp();  // tcgen05.ld is .sync.aligned
           tc_ld32(taddr + (uint32_t)(i * 32), v);
@@ -519,9 +539,14 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       const long long row_base = (long long)(2 * mp + (int)rank) * TBM + quarter * 32;
       const long long row = row_base + lane;
       const bool row_ok = row < ep.M;
-      const float rinv = row_ok ? ep.row_inv[row] : __int_as_float(0x7fc00000);
       const float shift = (row_ok && ep.row_shift) ? ep.row_shift[row] : 0.0f;
-      epilogue_tile(ep, tot, row, row_base, row_ok, rinv, shift, nt * TBN + half * 128, lane);
+      const int col0 = nt * bn + half * 128, tile_end = nt * bn + bn;
+      if (ep.raw_out) {
+        if (row_ok) raw_store(ep, tot, row, col0, min(ep.raw_cols, tile_end), tile % ks, shift);
+      } else {
+        const float rinv = row_ok ? ep.row_inv[row] : __int_as_float(0x7fc00000);
+        epilogue_tile(ep, tot, row, row_base, row_ok, rinv, shift, col0, min(ep.P, tile_end), lane);
+      }
       __syncwarp();
     }
   }
@@ -541,7 +566,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 template <int OPA>
 cudaError_t go2(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* bl, int64_t K,
                 const EpiParams& ep, int sm_count, int group_m, long long spin_ns, cudaStream_t st,
-                const DecodeArgs& da) {
+                const DecodeArgs& da, int bn) {
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k_tc2_scan<OPA>,
@@ -551,13 +576,15 @@ cudaError_t go2(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* 
     attr_set = true;
   }
   const int n_mt = (ep.M + TBM - 1) / TBM;
-  const int n_nt = (ep.P + TBN - 1) / TBN;
-  const int tiles = ((n_mt + 1) / 2) * n_nt;
+  const int n_nt = (ep.P + bn - 1) / bn;
+  const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
+  if (ks > 1 && !ep.raw_out) return cudaErrorInvalidValue;
+  const int tiles = ((n_mt + 1) / 2) * n_nt * ks;
   const int pairs = tiles < sm_count / 2 ? tiles : sm_count / 2;
   const int group_p = group_m / 2 > 0 ? group_m / 2 : 1;
   if ((K / TBK) % Cfg2<OPA>::KS) return cudaErrorInvalidValue;
   k_tc2_scan<OPA><<<2 * pairs, kThreads, Cfg2<OPA>::kSmem, st>>>(
-      *a, *bh, *bl, (int)(K / TBK), n_mt, n_nt, group_p, spin_ns, ep, da);
+      *a, *bh, *bl, (int)(K / TBK), n_mt, n_nt, bn, group_p, spin_ns, ep, da);
   return cudaGetLastError();
 }
 
@@ -566,15 +593,17 @@ cudaError_t go2(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* 
 cudaError_t launch_tc2_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                             const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                             long long spin_ns, cudaStream_t st, int group_m, const DecodeArgs* dec,
-                            int encoding) {
+                            int encoding, int bn) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
-  if (K % TBK || group_m < 1) return cudaErrorInvalidValue;
+  if (K % TBK || group_m < 1 || bn < 32 || bn > TBN || bn % 32) return cudaErrorInvalidValue;
+  if (ep.raw_out && ep.P != ep.raw_cols) return cudaErrorInvalidValue;
   if (!dec)
-    return go2<OPA_TMA>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, DecodeArgs{});
+    return go2<OPA_TMA>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, DecodeArgs{},
+                        bn);
   if (dec->M != ep.M) return cudaErrorInvalidValue;
   if (encoding == TG_ENC_2BIT)
-    return go2<OPA_2BIT>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec);
-  return go2<OPA_U8>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec);
+    return go2<OPA_2BIT>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn);
+  return go2<OPA_U8>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn);
 }
 
 }  // namespace tg

@@ -252,8 +252,32 @@ __device__ __forceinline__ void tile_coord(int tile, int n_mt, int n_nt, int gro
   nt = idx / gm;
 }
 
+// K-block range [lo, hi) of split `sp` of `ks`: whole accumulation chunks, the earlier splits
+// one chunk longer when they do not divide evenly (a split may be empty).
+__device__ __forceinline__ void split_range(int num_kb, int ks, int sp, int& lo, int& hi) {
+  const int chunks = (num_kb + kChunkKB - 1) / kChunkKB;
+  const int per = (chunks + ks - 1) / ks;
+  lo = min(num_kb, sp * per * kChunkKB);
+  hi = min(num_kb, (sp + 1) * per * kChunkKB);
+}
+
+// Raw mode: the 128 totals of one thread (marker row `row`, columns col0..) of K range `split`.
+// Lane = row and one column per instruction, so a warp writes 128 contiguous bytes.
+__device__ __forceinline__ void raw_store(const EpiParams& ep, const float (&tot)[128],
+                                          long long row, int col0, int col_end, int split,
+                                          float shift) {
+  float* out = ep.raw_out + (long long)split * ep.raw_split + row;
+#pragma unroll
+  for (int e = 0; e < 128; ++e) {  // fully unrolled: tot stays in registers
+    const int col = col0 + e;
+    if (col < col_end)
+      out[col * ep.raw_ld] = ep.ksplit > 1 ? tot[e] : fmaf(shift, ep.col_cs[col], tot[e]);
+  }
+}
+
 // Statistics of the 128 totals one thread holds: its marker row against 128 consecutive
 // phenotype columns starting at col0, in groups of 16 columns.
+// Columns at or past col_end are not this tile's.
 // D of a column is tot + shift * col_cs[col] (the marker row was shifted by `shift`).
 // Per column: r, the hit test, optionally every statistic's r, and the column's best marker
 // over the warp's 32 rows: one warp max (redux.sync) of the ordered key bits(|r|) + 1 (0 for
@@ -264,7 +288,8 @@ __device__ __forceinline__ void tile_coord(int tile, int n_mt, int n_nt, int gro
 // and stalls on instruction fetch long enough to hold up the products.
 __device__ __forceinline__ void epilogue_tile(const EpiParams& ep, float (&tot)[128],
                                               long long row, long long row_base, bool row_ok,
-                                              float rinv, float shift, int col0, int lane) {
+                                              float rinv, float shift, int col0, int col_end,
+                                              int lane) {
 #pragma unroll 1
   for (int g = 0; g < 8; ++g) {
     // keys of the group's 16 columns, then 16 independent warp maxima, then the ballots: the
@@ -274,7 +299,7 @@ __device__ __forceinline__ void epilogue_tile(const EpiParams& ep, float (&tot)[
     for (int k = 0; k < 16; ++k) {
       const int col = col0 + 16 * g + k;
       float r = __int_as_float(0x7fc00000);
-      if (row_ok && col < ep.P) {
+      if (row_ok && col < col_end) {
         const float D = fmaf(shift, ep.col_cs[col], tot[k]);
         r = corr_nan(D, rinv, ep.col_rmul[col]);
         if (ep.do_hits && r * r >= ep.r2_thr) emit_hit_raw(ep, D, row, col);
