@@ -58,8 +58,8 @@ bool make_tmap(CUtensorMap* m, const void* ptr, int64_t rows, int64_t K, int64_t
   return r == CUDA_SUCCESS;
 }
 bool make_tmap_packed(CUtensorMap* m, const void* ptr, int64_t rows, int64_t ld, uint32_t box_bytes,
-                      uint32_t box_rows, bool swizzle64) {
-  if (swizzle64 && box_bytes != 64) return false;
+                      uint32_t box_rows, bool swizzle) {
+  if (swizzle && box_bytes != 64 && box_bytes != 128) return false;
   auto fn = encode_fn();
   if (!fn) return false;
   cuuint64_t dims[2] = {(cuuint64_t)ld, (cuuint64_t)rows};
@@ -68,7 +68,8 @@ bool make_tmap_packed(CUtensorMap* m, const void* ptr, int64_t rows, int64_t ld,
   cuuint32_t estr[2] = {1u, 1u};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(ptr), dims, strides, box,
                   estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  swizzle64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                  !swizzle ? CU_TENSOR_MAP_SWIZZLE_NONE
+                  : box_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B,
                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -142,12 +143,13 @@ cudaError_t ensure_markers(tg_ctx* c, int64_t M) {
   if (M <= c->cap_m) return cudaSuccess;
   const int64_t cap = round_up(M, MT);
   dfree(c->nobs); dfree(c->mean); dfree(c->shift); dfree(c->mh); dfree(c->gc2s); dfree(c->gc2);
-  dfree(c->rinv); dfree(c->rinv64);
+  dfree(c->rinv); dfree(c->rinv64); dfree(c->S); dfree(c->S2);
   c->cap_m = 0;
   cudaError_t e;
   if ((e = dalloc(&c->nobs, cap)) || (e = dalloc(&c->mean, cap)) || (e = dalloc(&c->shift, cap)) ||
       (e = dalloc(&c->mh, cap)) || (e = dalloc(&c->gc2s, cap)) ||
-      (e = dalloc(&c->gc2, cap)) || (e = dalloc(&c->rinv, cap)) || (e = dalloc(&c->rinv64, cap)))
+      (e = dalloc(&c->gc2, cap)) || (e = dalloc(&c->S, cap)) || (e = dalloc(&c->S2, cap)) ||
+      (e = dalloc(&c->rinv, cap)) || (e = dalloc(&c->rinv64, cap)))
     return e;
   c->cap_m = cap;
   return cudaSuccess;
@@ -193,6 +195,7 @@ constexpr double kChunkUs64 = 6.6, kChunkUs128 = 9.0;  // one-CTA kernel, per ch
 constexpr double kChunkUsCol = 0.0337;  // CTA-pair kernel, per chunk and column of a 256-marker tile
 constexpr double kItemUs = 4.0;
 constexpr double kRangeBytesPerUs = 6.0e6;
+constexpr int64_t kPackedOperandBytes = 32 << 20;
 constexpr size_t kMaxSplitFloats = size_t(1) << 26;  // partial sums of a split: 256 MiB at most
 int pick_ranges(int64_t tiles, int64_t slots, int64_t chunks, double chunk_us, double range_floats) {
   int best = 1;
@@ -211,6 +214,36 @@ int pick_ranges(int64_t tiles, int64_t slots, int64_t chunks, double chunk_us, d
   return best;
 }
 
+// The FP32 form: ranges of K for its 128 x 128 tiles, so that every SM gets the same share, and
+// for the projection's 64 x 32 tiles. Unsplit up to kFp32SplitN samples, where a tile is short.
+constexpr int64_t kFp32SplitN = 2048;
+constexpr double kFp32UsPerSample = 0.07;  // a 128 x 128 tile alone on an SM
+int pick_fp32_ranges(int64_t M, int64_t P, int64_t K, int64_t sms) {
+  if (K <= kFp32SplitN) return 1;
+  const int64_t tiles = ((M + 127) / 128) * ((P + 127) / 128);
+  int best = 1;
+  double best_us = 0;
+  for (int64_t ks = 1; ks <= 8; ++ks) {
+    const int64_t range = round_up((K + ks - 1) / ks, 16);
+    const double floats = (double)ks * (double)round_up(M, 32) * (double)P;
+    if ((ks - 1) * range >= K || (ks > 1 && floats > (double)kMaxSplitFloats)) continue;
+    const double us = (double)((tiles * ks + sms - 1) / sms) *
+                          ((double)range * kFp32UsPerSample + kItemUs) +
+                      (ks > 1 ? floats * 8.0 / kRangeBytesPerUs : 0.0);
+    if (ks == 1 || us < 0.97 * best_us) {
+      best = (int)ks;
+      best_us = us;
+    }
+  }
+  return best;
+}
+int pick_fp32_proj_ranges(int64_t M, int64_t nq, int64_t K, int64_t sms) {
+  const int64_t tiles = ((M + 63) / 64) * ((nq + 31) / 32);
+  int64_t r = std::min<int64_t>((K + 255) / 256, std::max<int64_t>(1, 4 * sms / tiles));
+  const int64_t range = round_up((K + r - 1) / r, 256);
+  return (int)((K + range - 1) / range);  // no range empty
+}
+
 // How a block is scanned: the passes, their splits and the workspace they need.
 struct Plan {
   bool split = false;       // the split form (else FP32)
@@ -218,13 +251,16 @@ struct Plan {
   bool joint = false;       // projection and panel products in one raw pass
   bool fuse_joint = false;  // ... that decodes the packed rows itself (joint operand of <= 128 rows)
   bool fuse_proj = false;   // projection pass over the packed rows that writes the operand
+  bool f16 = false;         // either pass in the f16 form (dosage rows)
   bool one_pass = false;    // ... and takes the marker statistics too
   bool dec = false;         // contraction kernels decode the packed rows (no operand in HBM)
   bool single = false;      // the panel's contraction on one CTA per tile
+  FusedUnits fu{};          // the split of either pass over the packed rows
   int ranges_proj = 1;      // K ranges of the projection or joint pass
   int ranges_scan = 1;      // K ranges of the panel's own contraction (> 1: raw, then k_raw_stats)
   int64_t ldr = 0;          // rows of the raw products' columns
   size_t raw_floats = 0;
+  size_t sums_at = 0;       // the byte sums of a one-pass block, in 32-bit words of the same buffer
   bool operand = false;     // the decoded operand is needed
 };
 
@@ -235,12 +271,14 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
   r.nq = opts.mode == TG_MODE_PAPER ? 0 : p->q - 1;
   r.ldr = round_up(M, 32);
   const int64_t n_mt = (M + MT - 1) / MT, n_mp = (n_mt + 1) / 2;
-  const bool wide_block = n_mt >= c->sm_count;  // at least one 128-marker tile per SM
-  const bool packed_ok = r.split && c->fuse_joint && missing == nullptr && r.nq > 0 && wide_block;
-  // a small panel's joint projection pass (projected form, joint operand of at most 128 rows,
-  // at least one 128-marker tile per SM) reads the packed rows and decodes them in shared memory
+  // Blocks whose passes read the packed rows and decode them on the way: those with one
+  // 128-marker tile per SM, or whose operand (bf16) is at least kPackedOperandBytes. Below that
+  // the operand's round trip stays in L2 and the decode and the pass are both a launch's latency.
+  const bool packed_ok = r.split && c->fuse_joint && missing == nullptr && r.nq > 0 &&
+                         (n_mt >= c->sm_count || M * p->Npad * 2 >= kPackedOperandBytes);
+  // a small panel's joint projection pass (projected form, joint operand of at most 128 rows)
   r.fuse_joint = packed_ok && p->joint_cols > 0 && p->joint_cols <= 128 && p->QYhi16 != nullptr;
-  // a panel with P + q - 1 > JCOLS: the projection runs as the same pass with the 64 projection
+  // a panel with P + q - 1 > JCOLS: the projection runs as the same pass with the projection
   // columns alone, which reads the packed rows and also writes the block's operand as it expands
   // them, so the operand is written once and read once, by the panel's contraction
   r.fuse_proj = packed_ok && !r.fuse_joint && !c->fuse_decode && p->QBhi16 != nullptr &&
@@ -249,18 +287,24 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
   // kernels when the context asks for it; the rest go through a decoded operand in HBM
   r.dec = r.split && missing == nullptr && (c->fuse_decode || r.fuse_joint);
   r.operand = !r.dec;
-  // dosage rows in the joint pass (or the projection pass that writes the operand) on 256-row
-  // tiles: that pass writes the row statistics itself (a thread holds a whole row), so no
-  // counting pass reads the block first
-  r.one_pass = (r.fuse_joint || r.fuse_proj) && encoding == TG_ENC_U8_DOSAGE && N <= kOnePassMaxN &&
-               joint_fused_rows(M, c->sm_count, r.fuse_proj ? QCOLS : p->joint_cols) == 2 * MT;
+  if (r.fuse_joint || r.fuse_proj) {
+    r.fu = fused_units(M, p->Npad, c->sm_count);
+    // dosage rows: the f16 form (k_fused.cu) from one 128-marker tile per SM on; smaller blocks keep
+    // the bf16 form, which is closer to the exact products. From one 256-marker tile per SM on
+    // the pass takes the byte sums itself, so no counting pass reads the block, and centres
+    // the rows on their first bytes; smaller ones stay centred on their means.
+    r.f16 = encoding == TG_ENC_U8_DOSAGE && n_mt >= c->sm_count;
+    r.one_pass = r.f16 && N <= kOnePassMaxN && (M + kFusedRows - 1) / kFusedRows >= c->sm_count;
+  }
   // P + q - 1 <= JCOLS: one pass over the operand gives the projection and the panel's products
   // (raw); the statistics follow the norms
   r.joint = r.split && r.nq > 0 && p->joint_cols > 0;
   const int64_t chunks = (p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB;
   const double ldr = (double)r.ldr;
   const int64_t pairs = c->sm_count / 2;
-  if (r.split && r.nq > 0 && !r.fuse_joint && !r.fuse_proj) {
+  if (r.fuse_joint || r.fuse_proj) {
+    r.ranges_proj = r.fu.pieces;
+  } else if (r.split && r.nq > 0) {
     if (r.joint && p->joint_cols > 128) {
       r.ranges_proj = pick_ranges(n_mp * (p->joint_cols / p->joint_bn), pairs, chunks,
                                   kChunkUsCol * p->joint_bn, ldr * (double)(r.nq + p->P));
@@ -270,8 +314,19 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
                                   ldr * (double)(r.nq + (r.joint ? p->P : 0)));
     }
   }
-  if (r.nq > 0)
-    r.raw_floats = (size_t)r.ranges_proj * (size_t)(r.nq + (r.joint ? p->P : 0)) * (size_t)r.ldr;
+  if (!r.split) {
+    if (r.nq > 0) r.ranges_proj = pick_fp32_proj_ranges(M, r.nq, p->Npad, c->sm_count);
+    if (p->P > 0) r.ranges_scan = pick_fp32_ranges(M, p->P, p->Npad, c->sm_count);
+    if (r.ranges_scan > 1)
+      r.raw_floats = (size_t)r.ranges_scan * (size_t)p->P * (size_t)r.ldr;
+  }
+  if (r.nq > 0) {
+    r.raw_floats = std::max(r.raw_floats, (size_t)r.ranges_proj * (size_t)(r.nq + (r.joint ? p->P : 0)) * (size_t)r.ldr);
+    if (r.one_pass) {  // two words in each of two parts per piece, after the products
+      r.sums_at = r.raw_floats;
+      r.raw_floats += (size_t)(4 * r.fu.pieces) * (size_t)r.ldr;
+    }
+  }
   if (r.split && !r.joint && p->P > 0) {
     const int tuned = c->tune_split[tune_bucket(M)];
     const double cols = (double)p->P;
@@ -456,7 +511,7 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
     const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, nullptr, 0, c->mean, p->Q, (int)p->q};
     const NormOut no{a.out.marker_norm2, c->rinv, c->rinv64, a.out.marker_nobs, a.out.marker_mean,
                      want_hits ? hit_start : nullptr, a.out.n_hits};
-    TG_CUDA(launch_marker_norm(a.M, c->nobs, c->gc2, RawView{c->raw, ldr, 0, 1, nullptr, nullptr},
+    TG_CUDA(launch_marker_norm(a.M, c->nobs, c->gc2, RawView{c->raw, ldr, 0, 1},
                                nq, 1.0, rf, no, st, a.N));
   }
   EpiParams ep{};
@@ -527,8 +582,8 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
     StageScope s(c, STAGE_DECODE, st, 1);
     TG_CUDA(launch_decode(a.G, a.ldg, a.encoding, a.N, a.M, a.missing, a.ldm, prec,
                           pl.fuse_proj ? nullptr : Ahi, split ? c->shift : nullptr,
-                          split ? c->mh : nullptr, p->Npad, c->nobs, nullptr, nullptr, c->mean,
-                          c->gc2, st));
+                          split ? c->mh : nullptr, p->Npad, c->nobs, c->S, c->S2, nullptr,
+                          nullptr, st));
   }
   DecodeArgs da{}, dj{};
   if (pl.dec || pl.fuse_proj) {
@@ -538,20 +593,20 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
     da.mh = c->mh;
     dj = da;
     if (pl.one_pass) {
+      dj.G = a.G;
+      dj.ldg = a.ldg;
       dj.shift_out = c->shift;
-      dj.nobs_out = c->nobs;
-      dj.mean_out = c->mean;
-      dj.gc2_out = c->gc2;
+      dj.sums = reinterpret_cast<uint32_t*>(c->raw + pl.sums_at);
+      dj.sums_ld = pl.ldr;
     }
     if (pl.fuse_proj) {
       dj.a_out = c->Ahi;
       dj.lda_out = p->Npad;
     }
-    const int pass_cols = pl.fuse_proj ? QCOLS : p->joint_cols;
     if ((pl.dec && !make_tmap_packed(&da.tmG, a.G, a.M, a.ldg, u8 ? 32u : 16u)) ||
         ((pl.fuse_joint || pl.fuse_proj) &&
-         !make_tmap_packed(&dj.tmG, a.G, a.M, a.ldg, u8 ? 64u : 16u,
-                           (uint32_t)joint_fused_rows(a.M, c->sm_count, pass_cols), u8)))
+         !make_tmap_packed(&dj.tmG, a.G, a.M, a.ldg, u8 ? 128u : 32u,
+                           (uint32_t)kFusedRows, u8)))
       return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the packed genotypes");
   }
   const DecodeArgs* dec = pl.dec ? &da : nullptr;
@@ -559,32 +614,38 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   if (split && !pl.dec && !make_tmap(&tA, c->Ahi, a.M, p->Npad, p->Npad, MT))
     return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the genotype operand");
   // the raw products of the projection (and the joint panel's after them)
-  RawView raw{c->raw, pl.ldr, pl.ldr * (nq + (joint ? p->P : 0)), pl.ranges_proj, c->shift,
-              joint ? p->qycs : p->qcs};
+  const bool packed_pass = pl.fuse_joint || pl.fuse_proj;
+  const bool f16 = pl.f16;  // the scaled f16 operand and column sums
+  RawView raw{c->raw, pl.ldr, pl.ldr * (nq + (joint ? p->P : 0)), pl.ranges_proj,
+              packed_pass || (split && pl.ranges_proj > 1), c->shift,
+              joint ? (f16 ? p->qycs16 : p->qycs) : (f16 ? p->qcs16 : p->qcs),
+              f16 ? (float)(1.0 / kJointF16Scale) : 1.0f, packed_pass ? pl.fu.per : 0,
+              pl.fu.chunks, !split};
   if (nq > 0) {
     StageScope s(c, STAGE_PROJECT, st, 1);
     if (!split) {
-      TG_CUDA(launch_project(c->A32, p->Npad, a.M, p->Npad, p->QB, nq, c->raw, pl.ldr, st));
+      TG_CUDA(launch_project(c->A32, p->Npad, a.M, p->Npad, p->QB, nq, c->raw, pl.ldr, st,
+                             pl.ranges_proj, raw.split));
     } else {
       EpiParams pp{};
       pp.M = (int)a.M;
       pp.P = (int)(joint ? nq + p->P : nq);
       pp.status = c->status;
       pp.row_shift = c->shift;
-      pp.col_cs = joint ? p->qycs : p->qcs;
+      pp.col_cs = raw.cs;
       pp.raw_out = c->raw;
       pp.raw_cols = pp.P;
       pp.raw_ld = raw.ld;
       pp.raw_split = raw.split;
-      pp.ksplit = pl.ranges_proj;
-      if (pl.fuse_joint) {  // dosage rows: the f16 joint operand
-        if (u8) pp.col_cs = p->qycs16;
-        TG_CUDA(launch_joint_fused(u8 ? &p->tmQYhi16 : &p->tmQYhi, u8 ? &p->tmQYlo16 : &p->tmQYlo,
-                                   p->Npad, pp, c->sm_count, kSpinNs, st, dj, a.encoding));
+      pp.ksplit = packed_pass ? 1 : pl.ranges_proj;
+      if (pl.fuse_joint) {
+        TG_CUDA(launch_joint_fused(f16 ? &p->tmQYhi16 : &p->tmQYhi, f16 ? &p->tmQYlo16 : &p->tmQYlo,
+                                   p->Npad, pp, c->sm_count, p->joint_bn, kSpinNs, st, dj,
+                                   a.encoding, f16));
       } else if (pl.fuse_proj) {  // the projection alone, writing the operand as it goes
-        if (u8) pp.col_cs = p->qcs16;
-        TG_CUDA(launch_joint_fused(u8 ? &p->tmQhi16 : &p->tmQhi, u8 ? &p->tmQlo16 : &p->tmQlo,
-                                   p->Npad, pp, c->sm_count, kSpinNs, st, dj, a.encoding));
+        TG_CUDA(launch_joint_fused(f16 ? &p->tmQhi16 : &p->tmQhi, f16 ? &p->tmQlo16 : &p->tmQlo,
+                                   p->Npad, pp, c->sm_count, p->proj_bn(), kSpinNs, st, dj,
+                                   a.encoding, f16));
       } else if (joint && p->joint_cols > 128) {  // more than one narrow tile: CTA pairs
         const int64_t items = (a.M + 2 * MT - 1) / (2 * MT) * (p->joint_cols / p->joint_bn);
         if (pl.ranges_proj == 1 && items > c->sm_count / 2) {
@@ -598,14 +659,20 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
         TG_CUDA(launch_tc_scan(&tA, joint ? &p->tmQYhi : &p->tmQhi, joint ? &p->tmQYlo : &p->tmQlo,
                                p->Npad, pp, c->sm_count, kSpinNs, st, kGroupDefault,
                                c->fuse_decode ? dec : nullptr, a.encoding,
-                               joint ? p->joint_cols : QCOLS));
+                               joint ? p->joint_bn : p->proj_bn()));
       }
     }
   }
-  if (p->samples) {  // a subset panel: |g_c|^2 over its samples
-    StageScope s(c, STAGE_NORM, st, 1);
+  RowSums sums{pl.one_pass ? dj.sums : nullptr, pl.ldr, (int)a.N, c->S, c->S2, c->nobs, c->mean,
+               c->gc2};
+  if (p->samples) {  // a subset panel: |g_c|^2 over its samples, which takes the means
+    StageScope s(c, STAGE_NORM, st, pl.one_pass ? 2 : 1);
+    if (pl.one_pass) {
+      TG_CUDA(launch_row_statistics(a.M, sums, raw, st));
+      sums = RowSums{};
+    }
     TG_CUDA(launch_subset_stats(a.G, a.ldg, a.encoding, a.N, a.M, a.missing, a.ldm, p->samples,
-                                c->mean, c->gc2s, st));
+                                c->mean, c->nobs, pl.one_pass ? nullptr : c->S, c->gc2s, st));
   }
   unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
   const bool want_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
@@ -615,7 +682,7 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
     const NormOut no{a.out.marker_norm2, c->rinv, c->rinv64, a.out.marker_nobs, a.out.marker_mean,
                      want_hits ? hit_start : nullptr, a.out.n_hits};
     TG_CUDA(launch_marker_norm(a.M, c->nobs, p->samples ? c->gc2s : c->gc2, raw, nq, kappa64, rf,
-                               no, st));
+                               no, st, 0, sums));
   }
   EpiParams ep{};
   ep.M = (int)a.M;
@@ -652,10 +719,22 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   {
     StageScope s(c, STAGE_GEMM, st, pl.ranges_scan > 1 ? 2 : 1);
     if (prec == TG_PREC_FP32) {
-      TG_CUDA(launch_sgemm_scan(c->A32, p->Npad, p->B32, p->Npad, p->Npad, ep, st));
+      EpiParams pp = ep;
+      if (pl.ranges_scan > 1) {
+        pp.raw_out = c->raw;
+        pp.raw_cols = pp.P;
+        pp.raw_ld = pl.ldr;
+        pp.raw_split = pl.ldr * p->P;
+        pp.ksplit = pl.ranges_scan;
+      }
+      TG_CUDA(launch_sgemm_scan(c->A32, p->Npad, p->B32, p->Npad, p->Npad, pp, st));
+      if (pl.ranges_scan > 1) {  // partial sums of the uncentred operand: no shift to add back
+        TG_CUDA(launch_raw_stats(RawView{c->raw, pl.ldr, pl.ldr * p->P, pl.ranges_scan}, ep, st));
+        full_done = true;
+      }
     } else if (joint) {  // the products came with the projection
       raw.x += nq * raw.ld;
-      raw.cs = p->col_cs;
+      raw.cs += nq;
       TG_CUDA(launch_raw_stats(raw, ep, st));
       full_done = true;
     } else {
@@ -683,8 +762,8 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
                                 group, dec, a.encoding, p->bn));
       }
       if (pl.ranges_scan > 1) {
-        TG_CUDA(launch_raw_stats(RawView{c->raw, pl.ldr, pl.ldr * p->P, pl.ranges_scan, c->shift,
-                                         p->col_cs}, ep, st));
+        TG_CUDA(launch_raw_stats(RawView{c->raw, pl.ldr, pl.ldr * p->P, pl.ranges_scan, true,
+                                         c->shift, p->col_cs, 1.0f}, ep, st));
         full_done = true;
       }
     }
@@ -817,7 +896,7 @@ tg_status tg_destroy(tg_ctx* c) {
   dfree(c->status); dfree(c->scratch);
   dfree(c->Ahi); dfree(c->A32); dfree(c->Afp4); dfree(c->shift); dfree(c->mh); dfree(c->gc2s);
   dfree(c->nobs); dfree(c->mean); dfree(c->gc2); dfree(c->raw);
-  dfree(c->rinv); dfree(c->rinv64);
+  dfree(c->rinv); dfree(c->rinv64); dfree(c->S); dfree(c->S2);
   dfree(c->stage);
   dfree(c->dhits); dfree(c->dnhits); dfree(c->dbest);
   for (auto& ev : c->pending) { cudaEventDestroy(ev.a); cudaEventDestroy(ev.b); }
@@ -849,15 +928,16 @@ tg_status build_joint(tg_panel* p, cudaStream_t st) {
                               p->QBlo16, p->qcs16, st)) ||
         (e = cudaStreamSynchronize(st)))
       return cuda_fail(e, "f16 projection operand");
-    if (!make_tmap(&p->tmQhi16, p->QBhi16, QCOLS, Np, Np, QCOLS) ||
-        !make_tmap(&p->tmQlo16, p->QBlo16, QCOLS, Np, Np, QCOLS))
+    if (!make_tmap(&p->tmQhi16, p->QBhi16, QCOLS, Np, Np, (uint32_t)p->proj_bn()) ||
+        !make_tmap(&p->tmQlo16, p->QBlo16, QCOLS, Np, Np, (uint32_t)p->proj_bn()))
       return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the f16 projection operand");
   }
   if (P + nq > JCOLS) return TG_OK;
   // one tile of 64 or 128 columns, or CTA-pair tiles of joint_bn columns
-  const int64_t jn = tile_cols(P + nq);
+  const bool pairs = P + nq > 128;
+  const int64_t jn = pairs ? tile_cols(P + nq) : round_up(P + nq, 16);
   const int64_t jc = P + nq <= 64 ? 64 : P + nq <= 128 ? 128 : round_up(P + nq, jn);
-  const uint32_t box = (uint32_t)(jc <= 128 ? jc : jn / 2);
+  const uint32_t box = (uint32_t)(pairs ? jn / 2 : jn);
   const size_t row = sizeof(__nv_bfloat16) * (size_t)Np;
   const auto d2d = cudaMemcpyDeviceToDevice;
   if ((e = dalloc(&p->QYhi, (size_t)(jc * Np))) || (e = dalloc(&p->QYlo, (size_t)(jc * Np))) ||
@@ -884,12 +964,12 @@ tg_status build_joint(tg_panel* p, cudaStream_t st) {
         (e = cudaStreamSynchronize(st)))
       return cuda_fail(e, "f16 joint projection and panel operand");
     // 2-byte elements: the bf16 map layout serves (TMA copies bytes, it converts nothing)
-    if (!make_tmap(&p->tmQYhi16, p->QYhi16, jc, Np, Np, (uint32_t)jc) ||
-        !make_tmap(&p->tmQYlo16, p->QYlo16, jc, Np, Np, (uint32_t)jc))
+    if (!make_tmap(&p->tmQYhi16, p->QYhi16, jc, Np, Np, box) ||
+        !make_tmap(&p->tmQYlo16, p->QYlo16, jc, Np, Np, box))
       return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the f16 joint operand");
   }
   p->joint_cols = (int)jc;
-  p->joint_bn = (int)(jc <= 128 ? jc : jn);
+  p->joint_bn = (int)jn;
   return TG_OK;
 }
 
@@ -971,8 +1051,8 @@ tg_status tg_prepare_panel(tg_ctx* c, const float* Y, int64_t ldy, int64_t N, in
       !make_tmap(&p->tmBlo, p->Blo, p->Ppad, p->Npad, p->Npad, 256) ||
       !make_tmap(&p->tmBhi2, p->Bhi, p->Ppad, p->Npad, p->Npad, (uint32_t)p->bn / 2) ||
       !make_tmap(&p->tmBlo2, p->Blo, p->Ppad, p->Npad, p->Npad, (uint32_t)p->bn / 2) ||
-      !make_tmap(&p->tmQhi, p->QBhi, QCOLS, p->Npad, p->Npad, 64) ||
-      !make_tmap(&p->tmQlo, p->QBlo, QCOLS, p->Npad, p->Npad, 64) ||
+      !make_tmap(&p->tmQhi, p->QBhi, QCOLS, p->Npad, p->Npad, (uint32_t)p->proj_bn()) ||
+      !make_tmap(&p->tmQlo, p->QBlo, QCOLS, p->Npad, p->Npad, (uint32_t)p->proj_bn()) ||
       !make_tmap(&p->tmBhi64, p->Bhi, p->Ppad, p->Npad, p->Npad, 64) ||
       !make_tmap(&p->tmBlo64, p->Blo, p->Ppad, p->Npad, p->Npad, 64))
     return cleanup(fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the panel"));
@@ -1085,7 +1165,7 @@ tg_status tg_prepare_panel_subset(tg_ctx* c, const float* Y, int64_t ldy, int64_
   }
   if (!make_tmap(&r->tmBhi, r->Bhi, Pp, Np, Np, 256) || !make_tmap(&r->tmBlo, r->Blo, Pp, Np, Np, 256) ||
       !make_tmap(&r->tmBhi2, r->Bhi, Pp, Np, Np, (uint32_t)r->bn / 2) || !make_tmap(&r->tmBlo2, r->Blo, Pp, Np, Np, (uint32_t)r->bn / 2) ||
-      !make_tmap(&r->tmQhi, r->QBhi, QCOLS, Np, Np, 64) || !make_tmap(&r->tmQlo, r->QBlo, QCOLS, Np, Np, 64) ||
+      !make_tmap(&r->tmQhi, r->QBhi, QCOLS, Np, Np, (uint32_t)r->proj_bn()) || !make_tmap(&r->tmQlo, r->QBlo, QCOLS, Np, Np, (uint32_t)r->proj_bn()) ||
       !make_tmap(&r->tmBhi64, r->Bhi, Pp, Np, Np, 64) || !make_tmap(&r->tmBlo64, r->Blo, Pp, Np, Np, 64))
     return cleanup(fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the subset panel"));
   const tg_status js = build_joint(r, st);
@@ -1592,7 +1672,7 @@ tg_status tg_panel_concat(tg_ctx* c, const tg_panel* const* panels, int n, tg_pa
   }
   if (!make_tmap(&r->tmBhi, r->Bhi, Pp, Np, Np, 256) || !make_tmap(&r->tmBlo, r->Blo, Pp, Np, Np, 256) ||
       !make_tmap(&r->tmBhi2, r->Bhi, Pp, Np, Np, (uint32_t)r->bn / 2) || !make_tmap(&r->tmBlo2, r->Blo, Pp, Np, Np, (uint32_t)r->bn / 2) ||
-      !make_tmap(&r->tmQhi, r->QBhi, QCOLS, Np, Np, 64) || !make_tmap(&r->tmQlo, r->QBlo, QCOLS, Np, Np, 64) ||
+      !make_tmap(&r->tmQhi, r->QBhi, QCOLS, Np, Np, (uint32_t)r->proj_bn()) || !make_tmap(&r->tmQlo, r->QBlo, QCOLS, Np, Np, (uint32_t)r->proj_bn()) ||
       !make_tmap(&r->tmBhi64, r->Bhi, Pp, Np, Np, 64) || !make_tmap(&r->tmBlo64, r->Blo, Pp, Np, Np, 64)) {
     tg_panel_free(r);
     return fail(TG_ERR_CUDA, "cuTensorMapEncodeTiled failed for the concatenated panel");

@@ -217,13 +217,14 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
       pp.raw_cols = pp.P;
       pp.raw_ld = rows;
       TGS_CUDA(launch_tc_scan(&tA, joint ? &p->tmQYhi : &p->tmQhi, joint ? &p->tmQYlo : &p->tmQlo,
-                              p->Npad, pp, ds->sm_count, kStaticSpinNs, st, 16, nullptr, 0, QCOLS));
+                              p->Npad, pp, ds->sm_count, kStaticSpinNs, st, 16, nullptr, 0,
+                              joint ? p->joint_bn : p->proj_bn()));
     }
   }
   const MarkerRefine rf{G, ldg, encoding, N, missing, ldm, mean, p->Q, (int)p->q};
   const NormOut no{out->marker_norm2, rinv, rinv64, out->marker_nobs, out->marker_mean,
                    want_hits ? hit_start : nullptr, out->n_hits};
-  TGS_CUDA(launch_marker_norm(M, nobs, gc2, RawView{qg, rows, 0, 1, nullptr, nullptr}, nq, kappa64,
+  TGS_CUDA(launch_marker_norm(M, nobs, gc2, RawView{qg, rows, 0, 1}, nq, kappa64,
                               rf, no, st));
   EpiParams ep{};
   ep.M = (int)M;
@@ -260,7 +261,7 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
     TGS_CUDA(launch_sgemm_scan(reinterpret_cast<const float*>(Ahi), p->Npad, p->B32, p->Npad,
                                p->Npad, ep, st));
   } else if (joint) {  // the products came with the projection
-    TGS_CUDA(launch_raw_stats(RawView{qg + nq * rows, rows, 0, 1, nullptr, nullptr}, ep, st));
+    TGS_CUDA(launch_raw_stats(RawView{qg + nq * rows, rows, 0, 1}, ep, st));
   } else {
     const bool narrow = p->P <= 64;  // a small panel: 64-column tiles, bound by HBM
     TGS_CUDA(launch_tc_scan(&tA, narrow ? &p->tmBhi64 : &p->tmBhi, narrow ? &p->tmBlo64 : &p->tmBlo,

@@ -52,6 +52,13 @@ __device__ __forceinline__ float corr_nan(float D, float rinv, float rmul) {
   return fminf(1.0f, fmaxf(-1.0f, r));
 }
 
+// Ranges of the raw products of marker row `row` (see RawView).
+__device__ __forceinline__ int raw_ranges(const RawView& v, long long row) {
+  if (v.per == 0) return v.ranges;
+  const int u0 = (int)(row / kFusedRows) * v.chunks;
+  return (u0 + v.chunks - 1) / v.per - u0 / v.per + 1;
+}
+
 // Append a raw hit record: marker, phenotype and the product D (in the beta slot). The
 // statistics kernel that runs after the contraction turns it into beta, se, t, -log10 p.
 __device__ __forceinline__ void emit_hit_raw(const EpiParams& ep, float D, long long row, int col) {

@@ -118,14 +118,15 @@ struct DecodeArgs {
   int M;                  // rows of the block; rows >= M are zero
   const float* shift;     // [M] row shift c
   const uint32_t* mh;     // [M] bf16 bits of (mean - c), the missing-call value
-  // Dosage rows without a mask in the joint pass on 256-row tiles: when shift_out is set, the
-  // pass takes each row's shift from the row's first 64 samples instead of reading `shift`, sums
-  // the row's bytes and their squares as it expands them, and writes the row's statistics (the
-  // counting pass's outputs: n_obs = N, mean, |g_c|^2 and the shift), so no counting pass runs.
-  float* shift_out;  // (N <= kOnePassMaxN: the sum of squared bytes fits 32 bits)
-  int32_t* nobs_out;
-  double* mean_out;
-  double* gc2_out;
+  // Dosage rows without a mask in the joint pass: when sums is set, the pass takes each row's
+  // shift from the row's first 64 samples (read through G) instead of reading `shift`, writes it
+  // to shift_out, and leaves the sums of the row's bytes and of their squares, in parts that
+  // k_marker_norm adds up (RowSums), so no counting pass runs.
+  const uint8_t* G;
+  long long ldg;
+  float* shift_out;
+  uint32_t* sums;
+  long long sums_ld;
   // The projection pass of a larger panel (the 64 projection columns alone): when a_out is set,
   // the pass also stores each expanded row as the block's bf16 operand (row-major, lda_out
   // elements per row, every column of rows < M), which the panel's contraction then reads as it
@@ -184,21 +185,24 @@ struct tg_panel {
   double lnB = 0;                // ln B(df/2, 1/2), df = N - q - 1
   double lnB_paper = 0;          // ln B((N-2)/2, 1/2) for the paper's printed form
   CUtensorMap tmBhi, tmBlo;      // phenotype panel, 256-row boxes
+  // rows of the projection operand that a pass reads: q - 1 rounded up to 16
+  int proj_bn() const { return (int)tg::round_up(q > 1 ? q - 1 : 1, 16); }
   int bn = 0;                    // columns of a CTA-pair tile (tile_cols(P))
   CUtensorMap tmBhi2, tmBlo2;    // phenotype panel, boxes of bn / 2 rows (one CTA's half of a pair tile)
-  CUtensorMap tmQhi, tmQlo;      // covariate projection columns, 64-row boxes
+  CUtensorMap tmQhi, tmQlo;      // covariate projection columns, boxes of proj_bn() rows
   CUtensorMap tmBhi64, tmBlo64;  // phenotype panel, 64-row boxes (64-column tiles, P <= 64)
   // Panels with P + q - 1 <= JCOLS: the projection columns and the phenotypes in one operand,
   // rows [0, q-1) = QB rows, rows [q-1, q-1+P) = the panel, rest zero, so that one pass over a
   // block's operand gives both Q^T a and the panel's products (joint_cols = 0 and NULL buffers
   // when the panel is larger). Up to 128 rows the operand has joint_cols = 64 or 128 rows, one
-  // tile of the one-CTA kernels; above, it has joint_cols = n x joint_bn rows, n = 1 or 2 tiles
-  // of joint_bn columns of the CTA-pair kernel (the maps' boxes hold half a tile).
+  // tile of the one-CTA kernels, which read joint_bn of them (P + q - 1 rounded up to 16, the
+  // maps' boxes); above, it has joint_cols = n x joint_bn rows, n = 1 or 2 tiles of joint_bn
+  // columns of the CTA-pair kernel (the maps' boxes hold half a tile).
   int joint_cols = 0, joint_bn = 0;
   __nv_bfloat16* QYhi = nullptr;  // [joint_cols][Npad]
   __nv_bfloat16* QYlo = nullptr;
   float* qycs = nullptr;          // [joint_cols] qcs then col_cs
-  CUtensorMap tmQYhi, tmQYlo;     // boxes of joint_cols rows (joint_bn / 2 above 128)
+  CUtensorMap tmQYhi, tmQYlo;     // boxes of joint_bn rows (joint_bn / 2 above 128)
   // The same joint operand as f16 hi + lo of 2^14 v (joint_cols <= 128 only), for the joint pass
   // that decodes dosage rows in shared memory into f16 (k_fused.cu); scaled column sums.
   __half* QYhi16 = nullptr;       // [joint_cols][Npad]
@@ -242,6 +246,8 @@ struct tg_ctx {
   double* gc2s = nullptr;                       // [cap_m] |g_c|^2 over a subset panel's samples
   uint32_t* mh = nullptr;                       // [cap_m] bf16 bits of the missing-call value
   double* gc2 = nullptr;
+  int64_t* S = nullptr;                         // sum of a row's observed calls and of their
+  int64_t* S2 = nullptr;                        // squares (decode units), from the counting pass
   float* raw = nullptr;                         // raw products, [ranges][columns][rows]
   size_t cap_raw = 0;                           // its floats
   float* rinv = nullptr;
@@ -294,9 +300,9 @@ void mode_df(const tg_panel* p, int mode, double* df, double* lnB);
 bool make_tmap(CUtensorMap* m, const void* ptr, int64_t rows, int64_t K, int64_t ld,
                uint32_t box_rows);
 // uint8 map over packed genotype rows [rows][ld], boxes of box_bytes x box_rows, zero fill;
-// swizzle64: the 64-byte swizzle (box_bytes must be 64).
+// swizzle: boxes of 64 or 128 bytes get the swizzle of that size.
 bool make_tmap_packed(CUtensorMap* m, const void* ptr, int64_t rows, int64_t ld, uint32_t box_bytes,
-                      uint32_t box_rows = 128, bool swizzle64 = false);
+                      uint32_t box_rows = 128, bool swizzle = false);
 
 // panel kernels (k_panel.cu)
 cudaError_t launch_build_design(double* X, const double* C, int64_t ldc, int64_t N, int64_t n_cov,
@@ -334,25 +340,48 @@ cudaError_t launch_decode(const uint8_t* G, int64_t ldg, int encoding, int64_t N
                           float* shift, uint32_t* mh, int64_t lda, int32_t* nobs, int64_t* S,
                           int64_t* S2, double* mean, double* gc2, cudaStream_t st);
 // |g_c|^2 over the samples of a subset panel (decode units; the imputed value is the marker's
-// all-sample mean)
+// all-sample mean, S / nobs where S is given, else `mean`)
 cudaError_t launch_subset_stats(const uint8_t* G, int64_t ldg, int encoding, int64_t N, int64_t M,
                                 const uint32_t* missing, int64_t ldm, const uint32_t* samples,
-                                const double* mean, double* gc2s, cudaStream_t st);
+                                const double* mean, const int32_t* nobs, const int64_t* S,
+                                double* gc2s, cudaStream_t st);
 
 // SIMT kernels (k_simt.cu)
 // Raw products as the contraction kernels leave them (EpiParams::raw_out): element (m, k) of
-// range s at x[s * split + k * ld + m]. With ranges > 1 the partial sums are added in range
-// order and then shift[m] * cs[k].
+// range s at x[s * split + k * ld + m]. With `partial` the ranges are partial sums, which are
+// added in range order, and then shift[m] * cs[k] * cs_scale. per > 0: the ranges are the pieces of
+// k_joint_fused's tiles, as many as the CTAs that share the row's tile (see FusedUnits).
 struct RawView {
   const float* x;
   long long ld, split;
   int ranges;
+  bool partial;
   const float* shift;
   const float* cs;
+  float cs_scale;
+  int per, chunks;
+  bool sum64;  // k_marker_norm adds the ranges in FP64 (the FP32 form; no add-back)
 };
-// Projections of the FP32 operand, column-major: out[k * ldq + m].
+// A block's integer sums, from which k_marker_norm makes the row statistics (nobs, mean, gc2):
+// byte sums of dosage rows left by the joint pass in two parts per piece (x, DecodeArgs::sums;
+// n_obs = N), or the counting pass's S and S2 with its nobs. Neither: the statistics are there.
+struct RowSums {
+  const uint32_t* x;
+  long long ld;
+  int N;
+  const int64_t* S;
+  const int64_t* S2;
+  int32_t* nobs;
+  double* mean;
+  double* gc2;
+};
+// The statistics of `sums` on their own, where something reads the means before the norms.
+cudaError_t launch_row_statistics(int64_t M, const RowSums& sums, const RawView& raw,
+                                  cudaStream_t st);
+// Projections of the FP32 operand, column-major: out[k * ldq + m], range r of K `split` floats on.
 cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, const float* QB,
-                           int64_t nq, float* out, int64_t ldq, cudaStream_t st);
+                           int64_t nq, float* out, int64_t ldq, cudaStream_t st, int ranges = 1,
+                           int64_t split = 0);
 // What the FP64 re-projection of markers close to the covariate span needs: the packed block,
 // the FP64 means (units) and the panel's FP64 basis Q ([q][N], column 0 the intercept).
 struct MarkerRefine {
@@ -382,7 +411,7 @@ struct NormOut {
 cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2,
                                const RawView& proj, int64_t nq, double kappa,
                                const MarkerRefine& refine, const NormOut& out, cudaStream_t st,
-                               int64_t complete_n = 0);
+                               int64_t complete_n = 0, const RowSums& sums = RowSums{});
 cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t K,
                               const EpiParams& ep, cudaStream_t st);
 
@@ -393,26 +422,42 @@ cudaError_t launch_fill_random(uint8_t* p, size_t n, unsigned long long seed, cu
 
 // tensor-core kernel (k_tc.cu)
 // With `dec` non-NULL the A operand is decoded from packed genotypes in the kernel (tmA unused).
-// `bn`: 64-, 128- or 256-column tiles, the B maps' box rows. 64: the covariate projection, a small
-// panel's joint operand, or a panel of at most 64 phenotypes; 128: a joint operand; 256: a panel.
+// `bn`: columns of a tile, the B maps' box rows: a multiple of 16 up to 128 (the covariate
+// projection, a small panel's joint operand, or a panel of at most 64 phenotypes), or 256.
 // Raw mode (ep.raw_out) takes split-K.
 cudaError_t launch_tc_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                            const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                            long long spin_ns, cudaStream_t st, int group_m = 16,
                            const DecodeArgs* dec = nullptr, int encoding = 0, int bn = 256);
 
-// The joint projection pass of a small panel (joint operand of 64 or 128 rows) with the decode
-// fused in (k_fused.cu): reads the packed rows through da.tmG, whose boxes must be
-// joint_fused_rows(M, sm_count, joint_cols) rows of 64 bytes with the 64-byte swizzle (dosage)
-// or 16 bytes (2-bit calls); raw mode only, no split-K, K a multiple of 64. Writes the raw
-// products launch_tc_scan writes.
-int joint_fused_rows(int64_t M, int sm_count, int joint_cols);
-// Dosage rows are expanded into f16 (b - c exact) against the f16 joint operand (tmBhi / tmBlo
-// then map QYhi16 / QYlo16 and ep.col_cs is qycs16; the raw products are scaled back by 2^-14);
-// 2-bit calls into bf16 against the bf16 joint operand.
+// The joint projection pass of a small panel (joint operand of at most 128 rows) with the decode
+// fused in (k_fused.cu): reads the packed rows through da.tmG, whose boxes must be kFusedRows
+// rows of 128 bytes with the 128-byte swizzle (dosage) or 32 bytes (2-bit calls); raw mode only, K
+// a multiple of 64, bn (a multiple of 16) the operand's box rows. Writes the raw products as
+// fused_units(M, K, sm_count).pieces partial sums per tile, without the shift's add-back.
+constexpr int kFusedRows = 256;
+// Its units (one tile x one accumulation chunk) and their even split over the CTAs: CTA w takes the
+// units [w per, (w + 1) per), so tile t is shared by the CTAs t chunks / per to
+// ((t + 1) chunks - 1) / per, at most `pieces` of them.
+struct FusedUnits {
+  int chunks, units, per, grid, pieces;
+};
+inline FusedUnits fused_units(int64_t M, int64_t K, int sm_count) {
+  FusedUnits f;
+  f.chunks = (int)((K / 32 + kAccumChunkKB - 1) / kAccumChunkKB);
+  f.units = (int)((M + kFusedRows - 1) / kFusedRows) * f.chunks;
+  const int ctas = f.units < sm_count ? f.units : sm_count;
+  f.per = (f.units + ctas - 1) / ctas;
+  f.grid = (f.units + f.per - 1) / f.per;
+  f.pieces = f.per % f.chunks == 0 ? 1 : (f.chunks + f.per - 2) / f.per + 1;
+  return f;
+}
+// f16 (dosage rows): they are expanded into f16 (b - c exact) against the f16 operand (tmBhi / tmBlo
+// then map QYhi16 / QYlo16 and the products are scaled back by 2^-14); else, and for 2-bit calls,
+// into bf16 against the bf16 operand.
 cudaError_t launch_joint_fused(const CUtensorMap* tmBhi, const CUtensorMap* tmBlo, int64_t K,
-                               const EpiParams& ep, int sm_count, long long spin_ns, cudaStream_t st,
-                               const DecodeArgs& da, int encoding);
+                               const EpiParams& ep, int sm_count, int bn, long long spin_ns,
+                               cudaStream_t st, const DecodeArgs& da, int encoding, bool f16);
 
 // The statistics of a block from its raw products (k_stats.cu): the same per-element epilogue as
 // the contraction kernels and, in FULL mode, every statistic (no launch_full_stats after it).

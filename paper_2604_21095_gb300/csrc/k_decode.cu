@@ -2,8 +2,10 @@
 //
 // One warp per marker row. Pass 1 reads the packed row with 16-byte loads and counts,
 // exactly in integers, the observed calls n, their sum S and sum of squares S2 (decode
-// units: allele-1 counts for 2-bit calls, bytes for dosages); mean = S / n is one IEEE
-// division and |g_c|^2 = (n S2 - S^2) / n one more. Pass 2 re-reads the row (cache-hot)
+// units: allele-1 counts for 2-bit calls, bytes for dosages). The scan takes the sums
+// (k_marker_norm makes mean = S / n and |g_c|^2 = (n S2 - S^2) / n of 32 markers at a time: an
+// FP64 instruction costs 16 cycles of an SM whether one lane needs it or all 32); a caller that
+// asks for the mean and |g_c|^2 gets them here. Pass 2 re-reads the row (cache-hot)
 // and writes the contraction operand with 16-byte stores, zero past N:
 //   FP32 form: the code of an observed call, the mean at a missing one.
 //   split form (bf16): the row shifted by c = the mean rounded to a grid on which every
@@ -41,16 +43,34 @@ __device__ __forceinline__ void row_stats(const uint8_t* __restrict__ row, int N
                                           unsigned long long& S2) {
   n = S = S2 = 0;
   if (ENC == TG_ENC_2BIT) {
-    const int nb = (N + 3) >> 2;
-    const int nchunk = (nb + 15) >> 4;
+    const int nchunk = (N + 63) >> 6;
+    FieldCounts f;
 #pragma unroll 4
     for (int c = lane; c < nchunk; c += 32) {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + c);
-      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+      uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + c);
+      const int left = N - c * 64;
+      if (left < 64) {  // fields past N count as 11 (no copies)
+        uint32_t* w = &v.x;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)  // word q: samples from c * 64 + q * 16
-        count16_2bit(w4[q], N - (c * 64 + q * 16), n, S, S2);
+        for (int q = 0; q < 4; ++q) {
+          const int k = left - 16 * q;
+          if (k <= 0) w[q] = 0xFFFFFFFFu;
+          else if (k < 16) w[q] |= 0xFFFFFFFFu << (2 * k);
+        }
+      }
+      f.add(v);
     }
+    f.flush();
+    // 64 nchunk fields in all: 10 (one copy) = high - both, 01 (missing) = low - both, 00 (two
+    // copies) the rest
+    const uint32_t high = __reduce_add_sync(0xffffffffu, f.high);
+    const uint32_t low = __reduce_add_sync(0xffffffffu, f.low);
+    const uint32_t both = __reduce_add_sync(0xffffffffu, f.both);
+    const uint32_t one = high - both, two = 64u * (uint32_t)nchunk - high - low + both;
+    n = (uint32_t)N - (low - both);
+    S = (unsigned long long)two * 2 + one;
+    S2 = (unsigned long long)two * 4 + one;
+    return;
   } else {
     const int nchunk = (N + 15) >> 4;
 #pragma unroll 4
@@ -61,31 +81,24 @@ __device__ __forceinline__ void row_stats(const uint8_t* __restrict__ row, int N
       if (mrow) skip = (mrow[(c * 16) >> 5] >> ((c * 16) & 31)) & 0xFFFFu;
       const int left = N - c * 16;
       if (left < 16) skip |= 0xFFFFu << left;
-      if (skip == 0) {  // 16 observed bytes: sums of bytes and of their squares by dp4a
-        uint32_t s1 = 0, s2 = 0;
+      // sums of the observed bytes and of their squares by dp4a (the rest set to 0)
+      uint32_t s1 = 0, s2 = 0;
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          s1 = __dp4a(w4[q], 0x01010101u, s1);
-          s2 = __dp4a(w4[q], w4[q], s2);
-        }
-        n += 16;
-        S += s1;
-        S2 += s2;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const uint32_t u = (w4[q] >> (8 * b)) & 0xFFu;
-            if (!((skip >> (q * 4 + b)) & 1u)) {
-              n += 1;
-              S += u;
-              S2 += u * u;
-            }
-          }
-        }
+      for (int q = 0; q < 4; ++q) {
+        const uint32_t w = skip ? keep_bytes(w4[q], (~skip >> (4 * q)) & 15u) : w4[q];
+        s1 = __dp4a(w, 0x01010101u, s1);
+        s2 = __dp4a(w, w, s2);
       }
+      n += (unsigned)__popc(~skip & 0xFFFFu);
+      S += s1;
+      S2 += s2;
     }
+  }
+  if (N <= kOnePassMaxN) {  // the row's sums fit 32 bits
+    n = __reduce_add_sync(0xffffffffu, (uint32_t)n);
+    S = __reduce_add_sync(0xffffffffu, (uint32_t)S);
+    S2 = __reduce_add_sync(0xffffffffu, (uint32_t)S2);
+    return;
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) {
@@ -120,11 +133,17 @@ __device__ __forceinline__ void load8(const uint8_t* __restrict__ row, const uin
   if (i0 + 8 > N) miss &= (N > i0) ? ((1u << (N - i0)) - 1u) : 0u;
 }
 
-// Shift of a marker row for the split form (see above); 0 when no call is observed.
 template <int ENC>
-__device__ __forceinline__ double row_shift(unsigned long long n, double mean) {
-  if (!n) return 0.0;
-  return ENC == TG_ENC_2BIT ? rint(mean * 128.0) * (1.0 / 128.0) : rint(mean);
+constexpr int kGrid = ENC == TG_ENC_2BIT ? 128 : 1;  // the shift's grid (see above): 1 / kGrid
+
+// mean and |g_c|^2 of a row with n observed calls, sum S and sum of squares S2 (NaN without one).
+__device__ __forceinline__ double row_mean(unsigned long long n, unsigned long long S) {
+  return n ? (double)S / (double)n : __longlong_as_double(0x7ff8000000000000ll);
+}
+__device__ __forceinline__ double row_gc2(unsigned long long n, unsigned long long S,
+                                          unsigned long long S2) {
+  const long long num = (long long)S2 * (long long)n - (long long)S * (long long)S;
+  return n ? (double)num / (double)n : __longlong_as_double(0x7ff8000000000000ll);
 }
 
 template <int ENC, int PREC>
@@ -141,27 +160,20 @@ __global__ void __launch_bounds__(kWarps * 32) k_decode(
   const uint32_t* mrow = miss ? miss + j * ldm : nullptr;
   unsigned long long n, S, S2;
   row_stats<ENC>(row, N, mrow, lane, n, S, S2);
-  const double dn = (double)n;
-  const double mean = n ? (double)S / dn : __longlong_as_double(0x7ff8000000000000ll);
   if (lane == 0) {
     if (nobs_out) nobs_out[j] = (int32_t)n;
     if (S_out) S_out[j] = (long long)S;
     if (S2_out) S2_out[j] = (long long)S2;
-    if (mean_out) mean_out[j] = mean;
-    if (gc2_out) {
-      const long long num = (long long)S2 * (long long)n - (long long)S * (long long)S;
-      gc2_out[j] = n ? (double)num / dn : __longlong_as_double(0x7ff8000000000000ll);
-    }
+    if (mean_out) mean_out[j] = row_mean(n, S);
+    if (gc2_out) gc2_out[j] = row_gc2(n, S, S2);
   }
   // pass 2: operand row (skipped when Ahi is NULL: the statistics and the split form's
   // per-row shift and missing value only, for the contraction that decodes in its producer)
-  const double m_imp = n ? mean : 0.0;
   const long long steps = lda >> 3;
   if (PREC == TG_PREC_SPLIT_BF16) {
-    const double c = row_shift<ENC>(n, mean);
-    const float cf = (float)c;  // exact: a multiple of 2^-7 in [0, 2] or an integer in [0, 255]
-    const __nv_bfloat16 mh = __double2bfloat16(m_imp - c);
-    const uint32_t mhu = (uint32_t)__bfloat16_as_ushort(mh);
+    float cf;  // a multiple of 2^-7 in [0, 2] or an integer in [0, 255]
+    uint32_t mhu;
+    row_shift_sums<kGrid<ENC>>((uint32_t)n, S, cf, mhu);
     if (lane == 0 && shift_out) shift_out[j] = cf;
     if (lane == 0 && mh_out) mh_out[j] = mhu;
     if (!Ahi) return;
@@ -201,7 +213,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_decode(
       }
     }
   } else {
-    const float mf = (float)m_imp;
+    const float mf = n ? (float)row_mean(n, S) : 0.0f;
     float* af = reinterpret_cast<float*>(Ahi) + j * lda;
 #pragma unroll 4
     for (long long t = lane; t < steps; t += 32) {
@@ -235,9 +247,8 @@ __global__ void __launch_bounds__(THREADS, GPT * THREADS <= 1536 ? 4 : 2) k_deco
     uint32_t* __restrict__ mh_out, long long lda, int32_t* __restrict__ nobs_out,
     long long* __restrict__ S_out, long long* __restrict__ S2_out, double* __restrict__ mean_out,
     double* __restrict__ gc2_out) {
-  __shared__ unsigned long long red[3][THREADS / 32];
-  __shared__ float s_c;
-  __shared__ uint32_t s_mh;
+  static_assert(THREADS * GPT * 16 <= kOnePassMaxN, "a row's sums fit 32 bits");
+  __shared__ uint32_t red[3][THREADS / 32];
   const long long j = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const uint8_t* row = G + j * ldg;
@@ -275,72 +286,45 @@ __global__ void __launch_bounds__(THREADS, GPT * THREADS <= 1536 ? 4 : 2) k_deco
       uint32_t skip = ms[g];
       if (left < 16) skip |= 0xFFFFu << left;
       const uint32_t w4[4] = {v[g].x, v[g].y, v[g].z, v[g].w};
-      if (skip == 0) {
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          S = __dp4a(w4[q], 0x01010101u, S);
-          S2 = __dp4a(w4[q], w4[q], S2);
-        }
-        n += 16;
-      } else {
-#pragma unroll
-        for (int q = 0; q < 4; ++q)
-#pragma unroll
-          for (int b = 0; b < 4; ++b) {
-            const uint32_t u = (w4[q] >> (8 * b)) & 0xFFu;
-            if (!((skip >> (q * 4 + b)) & 1u)) {
-              n += 1;
-              S += u;
-              S2 += u * u;
-            }
-          }
+      for (int q = 0; q < 4; ++q) {  // unobserved bytes set to 0
+        const uint32_t x = skip ? keep_bytes(w4[q], (~skip >> (4 * q)) & 15u) : w4[q];
+        S = __dp4a(x, 0x01010101u, S);
+        S2 = __dp4a(x, x, S2);
       }
+      n += __popc(~skip & 0xFFFFu);
     }
   }
-  unsigned long long n64 = n, S64 = S, S264 = S2;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    n64 += __shfl_xor_sync(0xffffffffu, n64, o);
-    S64 += __shfl_xor_sync(0xffffffffu, S64, o);
-    S264 += __shfl_xor_sync(0xffffffffu, S264, o);
-  }
+  n = __reduce_add_sync(0xffffffffu, n);
+  S = __reduce_add_sync(0xffffffffu, S);
+  S2 = __reduce_add_sync(0xffffffffu, S2);
   if (lane == 0) {
-    red[0][warp] = n64;
-    red[1][warp] = S64;
-    red[2][warp] = S264;
+    red[0][warp] = n;
+    red[1][warp] = S;
+    red[2][warp] = S2;
   }
   __syncthreads();
-  if (tid == 0) {
-    unsigned long long tn = 0, tS = 0, tS2 = 0;
+  // every thread adds the warps' sums and makes the shift from them itself
+  uint32_t tn = 0, tS = 0, tS2 = 0;
 #pragma unroll
-    for (int k = 0; k < THREADS / 32; ++k) {
-      tn += red[0][k];
-      tS += red[1][k];
-      tS2 += red[2][k];
-    }
-    const double dn = (double)tn;
-    const double mean = tn ? (double)tS / dn : __longlong_as_double(0x7ff8000000000000ll);
+  for (int k = 0; k < THREADS / 32; ++k) {
+    tn += red[0][k];
+    tS += red[1][k];
+    tS2 += red[2][k];
+  }
+  float cf;
+  uint32_t mhu;
+  row_shift_sums<kGrid<ENC>>(tn, tS, cf, mhu);
+  if (tid == 0) {
     if (nobs_out) nobs_out[j] = (int32_t)tn;
     if (S_out) S_out[j] = (long long)tS;
     if (S2_out) S2_out[j] = (long long)tS2;
-    if (mean_out) mean_out[j] = mean;
-    if (gc2_out) {
-      const long long num = (long long)tS2 * (long long)tn - (long long)tS * (long long)tS;
-      gc2_out[j] = tn ? (double)num / dn : __longlong_as_double(0x7ff8000000000000ll);
-    }
-    const double c = row_shift<ENC>(tn, mean);
-    if (shift_out) shift_out[j] = (float)c;
-    s_c = (float)c;
-    s_mh = (uint32_t)__bfloat16_as_ushort(__double2bfloat16((tn ? mean : 0.0) - c));
-    if (mh_out) mh_out[j] = s_mh;
+    if (mean_out) mean_out[j] = row_mean(tn, tS);
+    if (gc2_out) gc2_out[j] = row_gc2(tn, tS, tS2);
+    if (shift_out) shift_out[j] = cf;
+    if (mh_out) mh_out[j] = mhu;
   }
-  // without an operand (the contraction decodes in its producer): the statistics, the shift
-  // and the missing value only
-  if (!A) return;
-  __syncthreads();
   // pass 2: the operand row from registers, zeros past N
-  const float cf = s_c;
-  const uint32_t mhu = s_mh;
   uint4* ah = reinterpret_cast<uint4*>(A + j * lda);
   auto bits = [](float x) { return (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(x)); };
   const uint32_t lut0 = bits(2.0f - cf) | (mhu << 16);
@@ -368,11 +352,15 @@ __global__ void __launch_bounds__(THREADS, GPT * THREADS <= 1536 ? 4 : 2) k_deco
 }
 
 // |g_c|^2 of each marker over the samples of a subset panel, in decode units, the marker's
-// missing calls imputed with its all-sample mean m (one warp per marker). With n observed
+// missing calls imputed with its all-sample mean m. With n observed
 // calls in the subset (sum T, sum of squares U, exact integers), k imputed ones and N_S = n + k,
 // the subset mean is gbar = (T + k m) / N_S and
 //   |g_c|^2 = (n U - T^2) / n + n (T / n - gbar)^2 + k (m - gbar)^2,
-// the first term exact in integers, the others small and well conditioned.
+// the first term exact in integers, the others small and well conditioned. A block's 8 warps count
+// 16 markers, then 16 lanes of one warp take the FP64 part together (one lane per row kept the FP64
+// units busy for most of 32 us on 5,003 rows x 10,007 samples, as did a branch per byte). m comes
+// from the all-sample sums where those are given (S), else from `mean`.
+constexpr int kSubsetRows = 2 * kWarps;
 __device__ __forceinline__ uint32_t spread16(uint32_t m) {  // bit b -> bit 2b
   m = (m | (m << 8)) & 0x00FF00FFu;
   m = (m | (m << 4)) & 0x0F0F0F0Fu;
@@ -385,59 +373,72 @@ template <int ENC>
 __global__ void __launch_bounds__(kWarps * 32) k_subset_stats(
     const uint8_t* __restrict__ G, long long ldg, int N, long long M,
     const uint32_t* __restrict__ miss, long long ldm, const uint32_t* __restrict__ samples,
-    const double* __restrict__ mean, double* __restrict__ gc2s) {
+    const double* __restrict__ mean, const int32_t* __restrict__ nobs,
+    const long long* __restrict__ S, double* __restrict__ gc2s) {
+  __shared__ unsigned long long sums[4][kSubsetRows];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const long long j = (long long)blockIdx.x * kWarps + warp;
-  if (j >= M) return;
-  const uint8_t* row = G + j * ldg;
-  const uint32_t* mrow = miss ? miss + j * ldm : nullptr;
-  unsigned long long n = 0, T = 0, U = 0, k = 0;
+  const long long j0 = (long long)blockIdx.x * kSubsetRows;
   const int groups = (N + 15) >> 4;  // 16 samples each
-  for (int t = lane; t < groups; t += 32) {
-    const int left = N - t * 16;
-    const uint32_t in_n = left >= 16 ? 0xFFFFu : ((1u << left) - 1u);
-    const uint32_t s16 = (samples[t >> 1] >> ((t & 1) * 16)) & in_n;
-    if (!s16) continue;
-    if (ENC == TG_ENC_2BIT) {
-      const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(row) + t);
-      const uint32_t sm = spread16(s16);
-      const uint32_t lo = w & 0x55555555u, hi = (w >> 1) & 0x55555555u;
-      const uint32_t c2 = __popc(~lo & ~hi & sm), c1 = __popc(hi & ~lo & sm);
-      n += c2 + c1 + __popc(lo & hi & sm);
-      T += 2 * c2 + c1;
-      U += 4 * c2 + c1;
-      k += __popc(lo & ~hi & sm);
-    } else {
-      const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + t);
-      const uint32_t m16 = mrow ? (mrow[t >> 1] >> ((t & 1) * 16)) & 0xFFFFu : 0u;
-      const uint32_t use = s16 & ~m16;
-      k += __popc(s16 & m16);
-      const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+  for (int i = warp; i < kSubsetRows && j0 + i < M; i += kWarps) {
+    const uint8_t* row = G + (j0 + i) * ldg;
+    const uint32_t* mrow = miss ? miss + (j0 + i) * ldm : nullptr;
+    unsigned long long n = 0, T = 0, U = 0, k = 0;
+#pragma unroll 4
+    for (int t = lane; t < groups; t += 32) {
+      const int left = N - t * 16;
+      const uint32_t in_n = left >= 16 ? 0xFFFFu : ((1u << left) - 1u);
+      const uint32_t s16 = (samples[t >> 1] >> ((t & 1) * 16)) & in_n;
+      if (ENC == TG_ENC_2BIT) {
+        const uint32_t w = __ldg(reinterpret_cast<const uint32_t*>(row) + t);
+        const uint32_t sm = spread16(s16);
+        const uint32_t lo = w & 0x55555555u, hi = (w >> 1) & 0x55555555u;
+        const uint32_t c2 = __popc(~lo & ~hi & sm), c1 = __popc(hi & ~lo & sm);
+        n += c2 + c1 + __popc(lo & hi & sm);
+        T += 2 * c2 + c1;
+        U += 4 * c2 + c1;
+        k += __popc(lo & ~hi & sm);
+      } else {
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + t);
+        const uint32_t m16 = mrow ? (mrow[t >> 1] >> ((t & 1) * 16)) & 0xFFFFu : 0u;
+        const uint32_t use = s16 & ~m16;
+        n += __popc(use);
+        k += __popc(s16 & m16);
+        const uint32_t w4[4] = {v.x, v.y, v.z, v.w};
+        uint32_t s1 = 0, s2 = 0;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
+        for (int q = 0; q < 4; ++q) {
+          const uint32_t w = keep_bytes(w4[q], (use >> (4 * q)) & 15u);
+          s1 = __dp4a(w, 0x01010101u, s1);
+          s2 = __dp4a(w, w, s2);
+        }
+        T += s1;
+        U += s2;
+      }
+    }
 #pragma unroll
-        for (int b = 0; b < 4; ++b)
-          if ((use >> (q * 4 + b)) & 1u) {
-            const uint32_t u = (w4[q] >> (8 * b)) & 0xFFu;
-            n += 1;
-            T += u;
-            U += u * u;
-          }
+    for (int o = 16; o > 0; o >>= 1) {
+      n += __shfl_xor_sync(0xffffffffu, n, o);
+      T += __shfl_xor_sync(0xffffffffu, T, o);
+      U += __shfl_xor_sync(0xffffffffu, U, o);
+      k += __shfl_xor_sync(0xffffffffu, k, o);
+    }
+    if (lane == 0) {
+      sums[0][i] = n;
+      sums[1][i] = T;
+      sums[2][i] = U;
+      sums[3][i] = k;
     }
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    n += __shfl_xor_sync(0xffffffffu, n, o);
-    T += __shfl_xor_sync(0xffffffffu, T, o);
-    U += __shfl_xor_sync(0xffffffffu, U, o);
-    k += __shfl_xor_sync(0xffffffffu, k, o);
-  }
-  if (lane) return;
+  __syncthreads();
+  const long long j = j0 + threadIdx.x;
+  if (threadIdx.x >= kSubsetRows || j >= M) return;
+  const unsigned long long n = sums[0][lane], T = sums[1][lane], U = sums[2][lane], k = sums[3][lane];
   if (n == 0) {  // every call of the subset imputed: constant there
     gc2s[j] = 0.0;
     return;
   }
-  const double m = mean[j], dn = (double)n, dk = (double)k;
+  const double m = S ? row_mean((unsigned long long)nobs[j], (unsigned long long)S[j]) : mean[j];
+  const double dn = (double)n, dk = (double)k;
   const double gbar = ((double)T + dk * m) / (dn + dk);
   const long long num = (long long)U * (long long)n - (long long)T * (long long)T;
   const double d1 = (double)T / dn - gbar, d2 = m - gbar;
@@ -450,12 +451,12 @@ cudaError_t go(const uint8_t* G, int64_t ldg, int64_t N, int64_t M, const uint32
                int64_t* S, int64_t* S2, double* mean, double* gc2, cudaStream_t st) {
   // Split form: one block per marker row with the row in registers (read from HBM once):
   // 256 threads x 6 groups of 16 samples for dosage rows, 128 x 12 for 2-bit rows; 12 and 24
-  // groups up to twice those N, with or without the operand (Ahi NULL: statistics, shift and
-  // missing value only). Short rows (N <= kWarpRowN: at most 8 groups per lane) and long ones
-  // go to the warp-per-row kernel: a block per short row would leave most of its threads idle
-  // and take several waves of blocks for a block of short rows.
+  // groups up to twice those N. Short rows (N <= kWarpRowN: at most 8 groups per lane) and long
+  // ones go to the warp-per-row kernel: a block per short row would leave most of its threads
+  // idle and take several waves of blocks for a block of short rows. So do rows without an
+  // operand (Ahi NULL: statistics, shift and missing value only), whose bytes are read once.
   if constexpr (PREC == TG_PREC_SPLIT_BF16) {
-    if (N <= kWarpRowN) {
+    if (N <= kWarpRowN || !Ahi) {
       const unsigned grid = (unsigned)((M + kWarps - 1) / kWarps);
       k_decode<ENC, PREC><<<grid, kWarps * 32, 0, st>>>(
           G, ldg, (int)N, M, missing, ldm, Ahi, shift, mh, lda, nobs,
@@ -506,15 +507,17 @@ cudaError_t launch_decode(const uint8_t* G, int64_t ldg, int encoding, int64_t N
 
 cudaError_t launch_subset_stats(const uint8_t* G, int64_t ldg, int encoding, int64_t N, int64_t M,
                                 const uint32_t* missing, int64_t ldm, const uint32_t* samples,
-                                const double* mean, double* gc2s, cudaStream_t st) {
+                                const double* mean, const int32_t* nobs, const int64_t* S,
+                                double* gc2s, cudaStream_t st) {
   if (M == 0) return cudaSuccess;
-  const unsigned grid = (unsigned)((M + kWarps - 1) / kWarps);
+  const unsigned grid = (unsigned)((M + kSubsetRows - 1) / kSubsetRows);
+  const long long* S64 = reinterpret_cast<const long long*>(S);
   if (encoding == TG_ENC_2BIT)
     k_subset_stats<TG_ENC_2BIT><<<grid, kWarps * 32, 0, st>>>(G, ldg, (int)N, M, missing, ldm,
-                                                               samples, mean, gc2s);
+                                                               samples, mean, nobs, S64, gc2s);
   else
-    k_subset_stats<TG_ENC_U8_DOSAGE><<<grid, kWarps * 32, 0, st>>>(G, ldg, (int)N, M, missing, ldm,
-                                                                    samples, mean, gc2s);
+    k_subset_stats<TG_ENC_U8_DOSAGE><<<grid, kWarps * 32, 0, st>>>(
+        G, ldg, (int)N, M, missing, ldm, samples, mean, nobs, S64, gc2s);
   return cudaGetLastError();
 }
 

@@ -18,11 +18,14 @@ namespace tg {
 namespace {
 
 // ---------------------------------------------------------------- projection
-// qg[k][m] = sum_i A[m][i] QB[k][i]; tile 64 markers x 32 columns, 32 samples per step.
+// qg[k][m] = sum_i A[m][i] QB[k][i]; tile 64 markers x 32 columns, 32 samples per step. K is cut
+// into ranges of whole 256-sample chunks over blockIdx.z, each writing its partial sum (a block
+// per tile alone left most SMs idle: 47 blocks took 182 us on 3,001 markers x 4,099 samples).
 __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, long long lda,
-                                                 long long M, int K,
+                                                 long long M, int K, int range,
                                                  const float* __restrict__ QB, int nq,
-                                                 float* __restrict__ qg, long long ldq) {
+                                                 float* __restrict__ qg, long long ldq,
+                                                 long long split) {
   __shared__ __align__(16) float As[32][64 + 4];
   __shared__ __align__(16) float Qs[32][32 + 4];
   const int tid = threadIdx.x;
@@ -32,7 +35,9 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
   // FP32 partial sums over 256 samples, flushed into FP64 totals
   float acc[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
   double tot[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
-  for (int i0 = 0; i0 < K; i0 += 32) {
+  const int k_lo = (int)blockIdx.z * range, k_hi = min(K, k_lo + range);
+  qg += blockIdx.z * split;
+  for (int i0 = k_lo; i0 < k_hi; i0 += 32) {
 #pragma unroll
     for (int u = 0; u < 2; ++u) {  // A tile: 64 rows x 32 samples as 512 float4
       const int e = tid + u * 256;
@@ -64,7 +69,7 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
       acc[3][0] += a.w * q.x; acc[3][1] += a.w * q.y;
     }
     __syncthreads();
-    if (((i0 >> 5) & 7) == 7 || i0 + 32 >= K) {
+    if (((i0 >> 5) & 7) == 7 || i0 + 32 >= k_hi) {
 #pragma unroll
       for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -153,27 +158,63 @@ __device__ __noinline__ double refine_projection(const MarkerRefine& rf, long lo
   return s;
 }
 
+// A row's statistics from its exact integer sums: mean = S / n, |g_c|^2 = (n S2 - S^2) / n (the
+// numerator exact in 64-bit integers), NaN without an observed call. Byte sums come in two parts
+// per piece: n = N (no mask), and S2 <= 255^2 N fits 32 bits for N <= kOnePassMaxN.
+__device__ __forceinline__ void row_statistics(const RowSums& sums, long long j, int pieces) {
+  long long n, S, S2;
+  if (sums.x) {
+    uint32_t a = 0, b = 0;
+    for (int r = 0; r < 2 * pieces; ++r) {
+      a += sums.x[2 * r * sums.ld + j];
+      b += sums.x[(2 * r + 1) * sums.ld + j];
+    }
+    n = sums.N;
+    S = a;
+    S2 = b;
+    sums.nobs[j] = sums.N;
+  } else {
+    n = sums.nobs[j];
+    S = sums.S[j];
+    S2 = sums.S2[j];
+  }
+  const double dn = (double)n, nan = __longlong_as_double(0x7ff8000000000000ll);
+  sums.mean[j] = n ? (double)S / dn : nan;
+  sums.gc2[j] = n ? (double)(S2 * n - S * S) / dn : nan;
+}
+__global__ void __launch_bounds__(256) k_row_statistics(long long M, RowSums sums, RawView raw) {
+  const long long j = blockIdx.x * 256ll + threadIdx.x;
+  if (j < M) row_statistics(sums, j, raw_ranges(raw, j));
+}
+
 __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
-    long long M, const int32_t* __restrict__ nobs, const double* __restrict__ gc2, RawView proj,
-    int nq, double kappa, const __grid_constant__ MarkerRefine rf, NormOut out, int complete_n) {
+    long long M, const int32_t* nobs, const double* gc2, RawView proj,
+    int nq, double kappa, const __grid_constant__ MarkerRefine rf, NormOut out, int complete_n,
+    RowSums sums) {
   __shared__ double part[kNormWarps][32];
   __shared__ unsigned flagged;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long m0 = blockIdx.x * 32ll, j = m0 + lane;
   const bool in = j < M;
+  const int ranges = raw_ranges(proj, m0);  // the block's markers are in one tile
+  if ((sums.x || sums.S) && warp == 0 && in) row_statistics(sums, j, ranges);
   double s = 0.0;
   if (in)
     for (int k = warp; k < nq; k += kNormWarps) {
       const float* x = proj.x + (long long)k * proj.ld + j;
       float v = *x;
-      if (proj.ranges > 1) {
-        for (int r = 1; r < proj.ranges; ++r) v += x[r * proj.split];
-        v = fmaf(proj.shift[j], proj.cs[k], v);
+      if (proj.sum64) {  // the FP32 form: ranges added in FP64, rounded once
+        double w = (double)v;
+        for (int r = 1; r < ranges; ++r) w += (double)x[r * proj.split];
+        s += w * w;
+        continue;
       }
+      for (int r = 1; r < ranges; ++r) v += x[r * proj.split];
+      if (proj.partial) v = fmaf(proj.shift[j], proj.cs[k] * proj.cs_scale, v);
       s += (double)v * (double)v;
     }
   part[warp][lane] = s;
-  __syncthreads();
+  __syncthreads();  // (and the block's writes of the row statistics are visible to the block)
   auto put = [&](long long m, double c2, double r2) {
     const bool ok = marker_testable(nobs[m], c2, r2, complete_n);
     const double nan = __longlong_as_double(0x7ff8000000000000ll);
@@ -210,11 +251,26 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
 }
 
 // ---------------------------------------------------------------- FP32 scan
+// Bound by the FP32 units. A thread's 8 x 8 sums are kept as pairs of columns, so that one packed
+// instruction (fma.rn.f32x2, two FMAs with the rounding of two) does the work of two.
+// Raw mode (ep.raw_out): K may be split into ranges over blockIdx.z, which write their products
+// column-major for k_raw_stats. With 192 tiles on 152 SMs the SMs that got two tiles set the pace
+// of 740 us (3,001 markers x 1,000 phenotypes x 4,099 samples).
 constexpr int BM = 128, BN = 128, BK = 16;
+
+__device__ __forceinline__ unsigned long long pack2(float a, float b) {
+  unsigned long long r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void fma2(unsigned long long& c, unsigned long long a,
+                                     unsigned long long b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(c) : "l"(a), "l"(b));
+}
 
 __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__ A, long long lda,
                                                     const float* __restrict__ B, long long ldb,
-                                                    int K, EpiParams ep) {
+                                                    int K, int range, EpiParams ep) {
   __shared__ __align__(16) float As[2][BK][BM + 4];
   __shared__ __align__(16) float Bs[2][BK][BN + 4];
   __shared__ unsigned long long colbest[BN];
@@ -224,17 +280,21 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
   const int n0 = blockIdx.x * BN;
   // global -> smem mapping: each thread moves 2 float4 of A and 2 of B per K step
   const int lr = tid >> 2, lk = (tid & 3) * 4;
+  const int k_lo = (int)blockIdx.z * range, k_hi = min(K, k_lo + range);
+  A += k_lo;
+  B += k_lo;
+  K = k_hi - k_lo;  // a multiple of BK
   const float* Ag0 = A + (m0 + lr) * lda + lk;
   const float* Ag1 = A + (m0 + lr + 64) * lda + lk;
   const float* Bg0 = B + (long long)(n0 + lr) * ldb + lk;
   const float* Bg1 = B + (long long)(n0 + lr + 64) * ldb + lk;
   if (tid < BN) colbest[tid] = 0ull;
 
-  float acc[8][8];
+  unsigned long long acc2[8][4];  // row a, columns 2b and 2b + 1
 #pragma unroll
   for (int a = 0; a < 8; ++a)
 #pragma unroll
-    for (int b = 0; b < 8; ++b) acc[a][b] = 0.0f;
+    for (int b = 0; b < 4; ++b) acc2[a][b] = 0ull;
 
   float4 ra0 = *reinterpret_cast<const float4*>(Ag0);
   float4 ra1 = *reinterpret_cast<const float4*>(Ag1);
@@ -261,20 +321,46 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
     for (int k = 0; k < BK; ++k) {
       const float4 a0 = *reinterpret_cast<const float4*>(&As[buf][k][ty * 4]);
       const float4 a1 = *reinterpret_cast<const float4*>(&As[buf][k][64 + ty * 4]);
-      const float4 b0 = *reinterpret_cast<const float4*>(&Bs[buf][k][tx * 4]);
-      const float4 b1 = *reinterpret_cast<const float4*>(&Bs[buf][k][64 + tx * 4]);
+      const ulonglong2 b0 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][k][tx * 4]);
+      const ulonglong2 b1 = *reinterpret_cast<const ulonglong2*>(&Bs[buf][k][64 + tx * 4]);
       const float av[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
-      const float bv[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-      for (int a = 0; a < 8; ++a)
-#pragma unroll
-        for (int b = 0; b < 8; ++b) acc[a][b] = fmaf(av[a], bv[b], acc[a][b]);
+      for (int a = 0; a < 8; ++a) {
+        const unsigned long long aa = pack2(av[a], av[a]);
+        fma2(acc2[a][0], aa, b0.x);
+        fma2(acc2[a][1], aa, b0.y);
+        fma2(acc2[a][2], aa, b1.x);
+        fma2(acc2[a][3], aa, b1.y);
+      }
     }
     if (more) {
       stash(buf ^ 1);
       __syncthreads();
       buf ^= 1;
     }
+  }
+
+  float acc[8][8];
+#pragma unroll
+  for (int a = 0; a < 8; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b)
+      asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[a][2 * b]), "=f"(acc[a][2 * b + 1]) : "l"(acc2[a][b]));
+  if (ep.raw_out) {  // four rows of a column at a time (columns start 128-byte aligned)
+    float* out = ep.raw_out + (long long)blockIdx.z * ep.raw_split;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const long long row = m0 + 64 * h + ty * 4;
+      if (row >= ep.M) continue;  // raw_ld >= M rounded up to 32 holds the whole quad
+#pragma unroll
+      for (int b = 0; b < 8; ++b) {
+        const int col = n0 + (b < 4 ? tx * 4 + b : 64 + tx * 4 + (b - 4));
+        if (col < ep.raw_cols)
+          *reinterpret_cast<float4*>(out + (long long)col * ep.raw_ld + row) =
+              make_float4(acc[4 * h][b], acc[4 * h + 1][b], acc[4 * h + 2][b], acc[4 * h + 3][b]);
+      }
+    }
+    return;
   }
 
   // epilogue: rows m0 + {ty*4 + a, 64 + ty*4 + a}, columns n0 + {tx*4 + b, 64 + tx*4 + b}
@@ -322,28 +408,43 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
 }  // namespace
 
 cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, const float* QB,
-                           int64_t nq, float* out, int64_t ldq, cudaStream_t st) {
+                           int64_t nq, float* out, int64_t ldq, cudaStream_t st, int ranges,
+                           int64_t split) {
   if (M == 0 || nq == 0) return cudaSuccess;
-  dim3 grid((unsigned)((M + 63) / 64), (unsigned)((nq + 31) / 32));
-  k_project<<<grid, 256, 0, st>>>(A, lda, M, (int)K, QB, (int)nq, out, (long long)ldq);
+  const int64_t range = round_up((K + ranges - 1) / ranges, 256);
+  dim3 grid((unsigned)((M + 63) / 64), (unsigned)((nq + 31) / 32), (unsigned)ranges);
+  k_project<<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out, (long long)ldq,
+                                  (long long)split);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_row_statistics(int64_t M, const RowSums& sums, const RawView& raw,
+                                  cudaStream_t st) {
+  if (M == 0) return cudaSuccess;
+  k_row_statistics<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(M, sums, raw);
   return cudaGetLastError();
 }
 
 cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2,
                                const RawView& proj, int64_t nq, double kappa,
                                const MarkerRefine& refine, const NormOut& out, cudaStream_t st,
-                               int64_t complete_n) {
+                               int64_t complete_n, const RowSums& sums) {
   if (M == 0) return cudaSuccess;
   k_marker_norm<<<(unsigned)((M + 31) / 32), kNormWarps * 32, 0, st>>>(
-      M, nobs, gc2, proj, (int)nq, kappa, refine, out, (int)complete_n);
+      M, nobs, gc2, proj, (int)nq, kappa, refine, out, (int)complete_n, sums);
   return cudaGetLastError();
 }
 
 cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t K,
                               const EpiParams& ep, cudaStream_t st) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
-  dim3 grid((unsigned)((ep.P + BN - 1) / BN), (unsigned)((ep.M + BM - 1) / BM));
-  k_sgemm_scan<<<grid, 256, 0, st>>>(A, lda, B, ldb, (int)K, ep);
+  const int ks = ep.raw_out && ep.ksplit > 1 ? ep.ksplit : 1;
+  if (ep.raw_out && (ep.raw_cols != ep.P || ep.raw_ld % 32 || ep.raw_ld < ep.M || ep.raw_split % 4))
+    return cudaErrorInvalidValue;
+  const int64_t range = round_up((K + ks - 1) / ks, BK);
+  if ((ks - 1) * range >= K) return cudaErrorInvalidValue;
+  dim3 grid((unsigned)((ep.P + BN - 1) / BN), (unsigned)((ep.M + BM - 1) / BM), (unsigned)ks);
+  k_sgemm_scan<<<grid, 256, 0, st>>>(A, lda, B, ldb, (int)K, (int)range, ep);
   return cudaGetLastError();
 }
 

@@ -173,7 +173,8 @@ __global__ void __launch_bounds__(kRawWarps * 32)
   for (int i = 0; i < R; ++i)
 #pragma unroll
     for (int u = 0; u < CPW; ++u) d[i][u] = 0.0f;
-  for (int s = 0; s < raw.ranges; ++s)
+  const int ranges = raw_ranges(raw, row0);  // the block's rows are in one tile
+  for (int s = 0; s < ranges; ++s)
 #pragma unroll
     for (int u = 0; u < CPW; ++u)
 #pragma unroll
@@ -194,7 +195,7 @@ __global__ void __launch_bounds__(kRawWarps * 32)
       float r = __int_as_float(0x7fc00000);
       if (row < ep.M) {
         float D = d[i][u];
-        if (raw.ranges > 1) D = fmaf(raw.shift[row], raw.cs[col], D);
+        if (raw.partial) D = fmaf(raw.shift[row], raw.cs[col] * raw.cs_scale, D);
         r = corr_nan(D, ep.row_inv[row], rmul);
         if (ep.do_hits && r * r >= ep.r2_thr) emit_hit_raw(ep, D, row, col);
       }

@@ -12,7 +12,7 @@
 //   warps 2, 3     with packed genotypes instead of a decoded operand (OPA_2BIT / OPA_U8): the
 //                  decoders, which expand each A tile from the packed rows (tc_common.cuh) and
 //                  join the stage's full barrier
-//   warp 1 lane 0  MMA issuer: per 32-wide K step, 2 x 2 tcgen05.mma 128x256x16 into an
+//   warp 1         MMA issuer (one elected lane): per 32-wide K step, 2 x 2 tcgen05.mma 128x256x16 into an
 //                  FP32 accumulator in TMEM
 //   warps 4..11    epilogue: tcgen05.ld of the accumulator (thread = marker row, each warp one
 //                  TMEM lane quarter and one half of the 256 columns), r = D / |g_res|, hits
@@ -85,7 +85,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               const __grid_constant__ CUtensorMap tmBlo, int num_kb, int n_mt, int n_nt, int bn,
               int group_m, long long spin_ns, EpiParams ep,
               const __grid_constant__ DecodeArgs da) {
-  // bn = B rows per tile: 256 for the phenotype panel, 64 or 128 (<= BR) with KS = 2
+  // bn = B rows per tile: 256 for the phenotype panel, at most BR with KS = 2
   using C = Cfg<OPA, KS, BR, MS>;
   static_assert(MS == 1 || (MS == 2 && KS == 2 && BR <= 128), "two sub-tiles: two K blocks, <= 128 B rows");
   constexpr bool kFused = OPA != OPA_TMA;
@@ -204,7 +204,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (kFused) mbar_wait(pfull_bar(s), (uint32_t)armed[s], abort_flag, spin_ns, ep.status);
         mbar_wait(full_bar(s), (uint32_t)armed[s], abort_flag, spin_ns, ep.status);
       }
-    } else if (warp == 1 && lane == 0) {
+    } else if (warp == 1) {
     // ------------------------------------------------------------ MMA issuer
     // Each chunk (chunk_end) starts a fresh accumulator (no chained accumulation
     // across chunks); the two chunk accumulators alternate.
@@ -213,6 +213,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     uint32_t g = 0;
     bool ok = true;
     const uint32_t idesc = idesc_bf16(bn);
+    const bool lead = elect_one();
     for (int item = blockIdx.x; item < num_items && ok; item += gridDim.x) {
       const int tile = item / ks;
       int kb_lo, kb_hi;
@@ -220,7 +221,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       for (int kb0 = kb_lo; kb0 < kb_hi && ok; kb0 = chunk_end_in(kb0, kb_lo, kb_hi), ++g) {
         const int acc = (int)(g & 1u);
         const uint32_t ph = (g >> 1) & 1u;
-        if (!mbar_wait(cempty_bar(acc), ph ^ 1u, abort_flag, spin_ns, ep.status)) {
+        if (!mbar_wait_warp(cempty_bar(acc), ph ^ 1u, abort_flag, spin_ns, ep.status)) {
           ok = false;
           break;
         }
@@ -228,7 +229,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         const uint32_t d = tmem_base + (uint32_t)(acc * TBN);
         const int kb1 = chunk_end_in(kb0, kb_lo, kb_hi);
         for (int kb = kb0; kb < kb1; kb += KS) {
-          if (!mbar_wait(full_bar(stage), phase, abort_flag, spin_ns, ep.status)) {
+          if (!mbar_wait_warp(full_bar(stage), phase, abort_flag, spin_ns, ep.status)) {
             ok = false;
             break;
           }
@@ -243,22 +244,25 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int sub = 0; sub < MS; ++sub) {  // sub-tile accumulators at +0 and +128
                 const uint64_t a = sdesc_sw64(sAk(stage, h, sub) + 32u * k);
                 const uint32_t ds = d + (uint32_t)(sub * 128);
-                tc_mma(ds, a, bh, idesc, (kb > kb0 || h > 0 || k > 0) ? 1u : 0u);
-                tc_mma(ds, a, bl, idesc, 1u);
+                if (lead) {
+                  tc_mma(ds, a, bh, idesc, (kb > kb0 || h > 0 || k > 0) ? 1u : 0u);
+                  tc_mma(ds, a, bl, idesc, 1u);
+                }
               }
             }
-          tc_commit(empty_bar(stage));
+          if (lead) tc_commit(empty_bar(stage));
           if (++stage == S) {
             stage = 0;
             phase ^= 1u;
           }
         }
-        if (ok) tc_commit(cfull_bar(acc));
+        if (ok && lead) tc_commit(cfull_bar(acc));
       }
     }
     // every product issued so far completes before TMEM is released (bounded)
-    tc_commit(drain_bar);
-    mbar_wait(drain_bar, 0u, abort_flag, spin_ns, ep.status);
+    if (lead) tc_commit(drain_bar);
+    __syncwarp();
+    mbar_wait_warp(drain_bar, 0u, abort_flag, spin_ns, ep.status);
     } else if (kFused && warp >= 2) {
     // ------------------------------------------------------------ decoders (warps 2, 3)
     const int t = threadIdx.x - 64;  // rows t and t + 64 of each A tile
@@ -406,17 +410,18 @@ cudaError_t launch_tc_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                            int encoding, int bn) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
   if (K % TBK || group_m < 1) return cudaErrorInvalidValue;
-  if ((bn != 64 && bn != 128 && bn != TBN) || (bn < TBN && ep.P > bn)) return cudaErrorInvalidValue;
+  if (bn < 16 || bn % 16 || (bn > 128 && bn != TBN) || (bn < TBN && ep.P > bn))
+    return cudaErrorInvalidValue;
   if (ep.raw_out && ep.P != ep.raw_cols) return cudaErrorInvalidValue;
   if (!dec) {
     // 256-marker tiles (two sub-tiles sharing B) once they fill every SM at least once
     const bool two = ep.ksplit <= 1 && (ep.M + 2 * TBM - 1) / (2 * TBM) >= sm_count;
-    if (bn == 64)  // the covariate projection, or a panel of at most 64 phenotypes
+    if (bn <= 64)  // the covariate projection, or a panel of at most 64 phenotypes
       return two ? go<OPA_TMA, 2, 64, 2>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns,
                                          st, DecodeArgs{}, bn)
                  : go<OPA_TMA, 2, 64, 1>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns,
                                          st, DecodeArgs{}, bn);
-    if (bn == 128)  // the projection joint with a panel of at most 128 - (q - 1) phenotypes
+    if (bn <= 128)  // the projection joint with a panel of at most 128 - (q - 1) phenotypes
       return two ? go<OPA_TMA, 2, 128, 2>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns,
                                           st, DecodeArgs{}, bn)
                  : go<OPA_TMA, 2, 128, 1>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns,

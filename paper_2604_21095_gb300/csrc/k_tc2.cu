@@ -14,7 +14,7 @@
 //                               the leader's full barrier (cta_group::2 completion). The
 //                               leader's producer also takes the pair's next tile (next_tile)
 //                               and publishes its index to every role of both CTAs
-//   warp 1 lane 0 (leader only) MMA issuer; commits are multicast to both CTAs' barriers
+//   warp 1 (leader only)        MMA issuer (one elected lane); commits are multicast to both CTAs' barriers
 //   warps 4..11 (both CTAs)     epilogue on the local 128 rows; the drained signal goes to
 //                               the leader's chunk-empty barrier (16 arrivals: 8 per CTA)
 //   warps 2, 3 (both CTAs)      with packed genotypes (OPA_2BIT / OPA_U8): decoders of the
@@ -176,10 +176,11 @@ static_assert(kFirstChunks == 1, "every chunk of a tile has the same length");
 // starts where the previous one ended finds the last-streamed slabs (chiefly the A rows of the
 // raster group's m-tile pairs, which consecutive waves share) still in L2 instead of fetching
 // them from DRAM again. Only the order of the FP32 chunk sums changes; every tile still adds
-// the same K blocks in chunks of the same sizes. With split-K the block is small and every range
-// streams K forwards.
-__device__ __forceinline__ bool k_reversed(int tile, int ncl, int ks) {
-  return ks == 1 && ((tile / ncl) & 1) != 0;
+// the same K blocks in chunks of the same sizes. In raw mode (blocks of at most JCOLS columns,
+// whose operand stays in L2 whole, or few tiles) every tile streams K forwards: its chunks and
+// their order are then those of the other kernels' raw products, bit for bit.
+__device__ __forceinline__ bool k_reversed(int tile, int ncl, bool raw) {
+  return !raw && ((tile / ncl) & 1) != 0;
 }
 
 // mbarrier wait with acquire at cluster scope (the phase may be completed by the other CTA),
@@ -316,13 +317,18 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     if (!ok) st_cluster_u32(peer_abort, 1u);
     return ok;
   };
+  auto wait_warp = [&](uint32_t bar, uint32_t parity) {  // one answer for a whole warp
+    return __all_sync(0xffffffffu, wait(bar, parity)) != 0;
+  };
   // Tile `i` of this pair's sequence from the ring, for every consumer role: a single thread
   // (whole_warp false) or a whole warp, whose lane 0 then arrives for it. Returns num_tiles at
   // the end of the work, and -1 on timeout or abort.
   auto take_tile = [&](int i, bool whole_warp) -> int {
     const int r = i % kTileRing;
-    if (!mbar_wait_cluster(tfull_bar(r), (uint32_t)(i / kTileRing) & 1u, abort_flag, spin_ns,
-                           ep.status)) {
+    bool got = mbar_wait_cluster(tfull_bar(r), (uint32_t)(i / kTileRing) & 1u, abort_flag, spin_ns,
+                                 ep.status);
+    if (whole_warp) got = __all_sync(0xffffffffu, got) != 0;  // one answer for all lanes
+    if (!got) {
       st_cluster_u32(peer_abort, 1u);
       return -1;
     }
@@ -365,7 +371,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
         split_range(num_kb, ks, tile % ks, k_lo, k_hi);
         const int kbs = k_hi - k_lo;
-        const bool rev = k_reversed(tile, ncl, ks);
+        const bool rev = k_reversed(tile, ncl, ep.raw_out != nullptr);
         const int mt0 = 2 * mp;
         const uint32_t pair_bytes =
             2u * KS * ((kFused ? 0u : (uint32_t)A_BYTES) + (uint32_t)bn * (TBK * 2));
@@ -407,15 +413,17 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (kFused) mbar_wait(pfull_bar(s), (uint32_t)armed[s], abort_flag, spin_ns, ep.status);
         if (leader) mbar_wait(full_bar(s), (uint32_t)armed[s], abort_flag, spin_ns, ep.status);
       }
-    } else if (warp == 1 && lane == 0 && leader) {
+    } else if (warp == 1 && leader) {
       // ---------------------------------------------------------- MMA issuer (leader)
       int stage = 0;
       uint32_t phase = 0;
       uint32_t g = 0;
       const uint32_t idesc = idesc_bf16_m(256, bn);
+      const bool lead = elect_one();
       bool ok = true;
       for (int i = 0; ok; ++i) {
-        const int tile = take_tile(i, false);
+        // the reduction's result is known to be the same in every lane
+        const int tile = __reduce_min_sync(0xffffffffu, take_tile(i, true));
         if (tile < 0 || tile >= num_tiles) break;
         int k_lo, k_hi;
         split_range(num_kb, ks, tile % ks, k_lo, k_hi);
@@ -423,7 +431,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         for (int kb0 = 0; kb0 < kbs && ok; kb0 = chunk_end_c(kb0, kbs, ckb), ++g) {
           const int acc = (int)(g & 1u);
           const uint32_t ph = (g >> 1) & 1u;
-          if (!wait(cempty_bar(acc), ph ^ 1u)) {
+          if (!wait_warp(cempty_bar(acc), ph ^ 1u)) {
             ok = false;
             break;
           }
@@ -431,7 +439,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           const uint32_t d = tmem_base + (uint32_t)(acc * TBN);
           const int kb1 = chunk_end_c(kb0, kbs, ckb);
           for (int kb = kb0; kb < kb1; kb += KS) {
-            if (!wait(full_bar(stage), phase)) {
+            if (!wait_warp(full_bar(stage), phase)) {
               ok = false;
               break;
             }
@@ -443,20 +451,23 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
                 const uint64_t a = sdesc_sw64(sA(stage, h) + 32u * k);
                 const uint64_t bh = sdesc_sw64(sBhi(stage, h) + 32u * k);
                 const uint64_t bl = sdesc_sw64(sBlo(stage, h) + 32u * k);
-                tc2_mma(d, a, bh, idesc, (kb > kb0 || h > 0 || k > 0) ? 1u : 0u);
-                tc2_mma(d, a, bl, idesc, 1u);
+                if (lead) {
+                  tc2_mma(d, a, bh, idesc, (kb > kb0 || h > 0 || k > 0) ? 1u : 0u);
+                  tc2_mma(d, a, bl, idesc, 1u);
+                }
               }
-            tc2_commit_both(empty_bar(stage));
+            if (lead) tc2_commit_both(empty_bar(stage));
             if (++stage == S) {
               stage = 0;
               phase ^= 1u;
             }
           }
-          if (ok) tc2_commit_both(cfull_bar(acc));
+          if (ok && lead) tc2_commit_both(cfull_bar(acc));
         }
       }
-      tc2_commit_local(drain_bar);
-      mbar_wait(drain_bar, 0u, abort_flag, spin_ns, ep.status);
+      if (lead) tc2_commit_local(drain_bar);
+      __syncwarp();
+      mbar_wait_warp(drain_bar, 0u, abort_flag, spin_ns, ep.status);
     } else if (kFused && warp >= 2) {
       // ---------------------------------------------------------- decoders (both CTAs)
       const int t = threadIdx.x - 64;  // rows t and t + 64 of this CTA's A tile
@@ -472,7 +483,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         const long long r0 = (long long)(2 * mp + (int)rank) * TBM + t;
         const uint2 k0 = dec_row_consts<OPA>(da, r0), k1 = dec_row_consts<OPA>(da, r0 + 64);
         const int kbs = k_hi - k_lo;
-        const bool rev = k_reversed(tile, ncl, ks);
+        const bool rev = k_reversed(tile, ncl, ep.raw_out != nullptr);
         for (int kb = 0; kb < kbs; ++kb) {
           const int kx = k_lo + (rev ? kbs - 1 - kb : kb);  // the K block the producer loaded
           if (!wait(pfull_bar(stage), phase)) {

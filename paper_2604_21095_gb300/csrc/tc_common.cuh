@@ -113,6 +113,29 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
   }
 }
 
+// The same for a whole warp (every lane calls it): one answer for all lanes, so that the control flow
+// that hangs on it stays uniform.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity,
+                                               volatile int* abort_flag, long long limit_ns,
+                                               uint32_t* status) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit_ns, status)) != 0;
+}
+
+// True in one lane of a converged warp. The MMA issuer is a whole warp in uniform control flow that
+// issues under this predicate: descriptors and addresses then live in uniform registers. From
+// a branch that a single lane takes, every tcgen05.mma moves its operands there first and costs
+// 105 cycles, whatever its size; this way 128 x 64 x 16 with A in tensor memory takes 52 (in
+// shared memory 80), and 128 x 128 x 16 73 (107).
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0u;
+}
+
 __device__ __forceinline__ void tma_load_2d(const CUtensorMap* map, uint32_t dst, uint32_t bar,
                                             int x, int y) {
   asm volatile(
