@@ -45,20 +45,30 @@ __device__ __forceinline__ void row_stats(const uint8_t* __restrict__ row, int N
   if (ENC == TG_ENC_2BIT) {
     const int nchunk = (N + 63) >> 6;
     FieldCounts f;
-#pragma unroll 4
-    for (int c = lane; c < nchunk; c += 32) {
-      uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + c);
-      const int left = N - c * 64;
-      if (left < 64) {  // fields past N count as 11 (no copies)
-        uint32_t* w = &v.x;
+    // six chunks' loads in flight per lane: a row of 23,000 samples is 12 per lane
+    constexpr int kAhead = 6;
+    for (int c0 = lane; c0 < nchunk; c0 += 32 * kAhead) {
+      uint4 buf[kAhead];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          const int k = left - 16 * q;
-          if (k <= 0) w[q] = 0xFFFFFFFFu;
-          else if (k < 16) w[q] |= 0xFFFFFFFFu << (2 * k);
+      for (int i = 0; i < kAhead; ++i)
+        if (c0 + 32 * i < nchunk) buf[i] = __ldg(reinterpret_cast<const uint4*>(row) + c0 + 32 * i);
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) {
+        const int c = c0 + 32 * i;
+        if (c >= nchunk) break;
+        uint4 v = buf[i];
+        const int left = N - c * 64;
+        if (left < 64) {  // fields past N count as 11 (no copies)
+          uint32_t* w = &v.x;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            const int k = left - 16 * q;
+            if (k <= 0) w[q] = 0xFFFFFFFFu;
+            else if (k < 16) w[q] |= 0xFFFFFFFFu << (2 * k);
+          }
         }
+        f.add(v);
       }
-      f.add(v);
     }
     f.flush();
     // 64 nchunk fields in all: 10 (one copy) = high - both, 01 (missing) = low - both, 00 (two
@@ -357,10 +367,11 @@ __global__ void __launch_bounds__(THREADS, GPT * THREADS <= 1536 ? 4 : 2) k_deco
 // the subset mean is gbar = (T + k m) / N_S and
 //   |g_c|^2 = (n U - T^2) / n + n (T / n - gbar)^2 + k (m - gbar)^2,
 // the first term exact in integers, the others small and well conditioned. A block's 8 warps count
-// 16 markers, then 16 lanes of one warp take the FP64 part together (one lane per row kept the FP64
-// units busy for most of 32 us on 5,003 rows x 10,007 samples, as did a branch per byte). m comes
+// a marker each, then 8 lanes of one warp take the FP64 part together; the bytes that count are
+// picked by a mask, without a branch (32 us on 5,003 rows x 10,007 samples with one lane per row
+// in FP64 and a branch per byte). m comes
 // from the all-sample sums where those are given (S), else from `mean`.
-constexpr int kSubsetRows = 2 * kWarps;
+constexpr int kSubsetRows = kWarps;
 __device__ __forceinline__ uint32_t spread16(uint32_t m) {  // bit b -> bit 2b
   m = (m | (m << 8)) & 0x00FF00FFu;
   m = (m | (m << 4)) & 0x0F0F0F0Fu;
@@ -383,7 +394,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_subset_stats(
     const uint8_t* row = G + (j0 + i) * ldg;
     const uint32_t* mrow = miss ? miss + (j0 + i) * ldm : nullptr;
     unsigned long long n = 0, T = 0, U = 0, k = 0;
-#pragma unroll 4
+#pragma unroll 8
     for (int t = lane; t < groups; t += 32) {
       const int left = N - t * 16;
       const uint32_t in_n = left >= 16 ? 0xFFFFu : ((1u << left) - 1u);
