@@ -238,7 +238,7 @@ int pick_fp32_ranges(int64_t M, int64_t P, int64_t K, int64_t sms) {
   return best;
 }
 int pick_fp32_proj_ranges(int64_t M, int64_t nq, int64_t K, int64_t sms) {
-  const int64_t tiles = ((M + 63) / 64) * ((nq + 31) / 32);
+  const int64_t tiles = nq <= 16 ? (M + 127) / 128 : ((M + 63) / 64) * ((nq + 31) / 32);
   int64_t r = std::min<int64_t>((K + 255) / 256, std::max<int64_t>(1, 4 * sms / tiles));
   const int64_t range = round_up((K + r - 1) / r, 256);
   return (int)((K + range - 1) / range);  // no range empty

@@ -18,20 +18,23 @@ namespace tg {
 namespace {
 
 // ---------------------------------------------------------------- projection
-// qg[k][m] = sum_i A[m][i] QB[k][i]; tile 64 markers x 32 columns, 32 samples per step. K is cut
+// qg[k][m] = sum_i A[m][i] QB[k][i]; tile 2,048 / KC markers x KC columns (KC = 16 for up to 16
+// columns, else 32), 32 samples per step. K is cut
 // into ranges of whole 256-sample chunks over blockIdx.z, each writing its partial sum (a block
 // per tile alone left most SMs idle: 47 blocks took 182 us on 3,001 markers x 4,099 samples).
+template <int KC>
 __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, long long lda,
                                                  long long M, int K, int range,
                                                  const float* __restrict__ QB, int nq,
                                                  float* __restrict__ qg, long long ldq,
                                                  long long split) {
-  __shared__ __align__(16) float As[32][64 + 4];
-  __shared__ __align__(16) float Qs[32][32 + 4];
+  constexpr int TM = 2048 / KC;
+  __shared__ __align__(16) float As[32][TM + 4];
+  __shared__ __align__(16) float Qs[32][KC + 4];
   const int tid = threadIdx.x;
-  const long long m0 = (long long)blockIdx.x * 64;
-  const int k0 = blockIdx.y * 32;
-  const int tx = tid & 15, ty = tid >> 4;  // 2 columns (k) x 4 markers per thread
+  const long long m0 = (long long)blockIdx.x * TM;
+  const int k0 = blockIdx.y * KC;
+  const int tx = tid % (KC / 2), ty = tid / (KC / 2);  // 2 columns (k) x 4 markers per thread
   // FP32 partial sums over 256 samples, flushed into FP64 totals
   float acc[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
   double tot[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
@@ -39,7 +42,7 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
   qg += blockIdx.z * split;
   for (int i0 = k_lo; i0 < k_hi; i0 += 32) {
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {  // A tile: 64 rows x 32 samples as 512 float4
+    for (int u = 0; u < TM / 32; ++u) {  // A tile: TM rows x 32 samples as 8 TM float4
       const int e = tid + u * 256;
       const int r = e >> 3, c4 = (e & 7) * 4;
       const long long gm = m0 + r;
@@ -50,7 +53,7 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
       As[c4 + 2][r] = v.z;
       As[c4 + 3][r] = v.w;
     }
-    {  // Q tile: 32 columns x 32 samples
+    if (tid < KC * 8) {  // Q tile: KC columns x 32 samples
       const int r = tid >> 3, c4 = (tid & 7) * 4;
       const float4 v = *reinterpret_cast<const float4*>(QB + (long long)(k0 + r) * K + i0 + c4);
       Qs[c4 + 0][r] = v.x;
@@ -198,7 +201,10 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
   const bool in = j < M;
   const int ranges = raw_ranges(proj, m0);  // the block's markers are in one tile
   if ((sums.x || sums.S) && warp == 0 && in) row_statistics(sums, j, ranges);
-  double s = 0.0;
+  // sum of squares in pairs of floats (48 bits; FP64 instructions take 16 cycles of an SM each, and
+  // three per column were half of this kernel's time): v^2 = p + e exactly, and two-sums
+  double s64 = 0.0;
+  float hi = 0.0f, lo = 0.0f;
   if (in)
     for (int k = warp; k < nq; k += kNormWarps) {
       const float* x = proj.x + (long long)k * proj.ld + j;
@@ -206,14 +212,17 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
       if (proj.sum64) {  // the FP32 form: ranges added in FP64, rounded once
         double w = (double)v;
         for (int r = 1; r < ranges; ++r) w += (double)x[r * proj.split];
-        s += w * w;
+        s64 += w * w;
         continue;
       }
       for (int r = 1; r < ranges; ++r) v += x[r * proj.split];
       if (proj.partial) v = fmaf(proj.shift[j], proj.cs[k] * proj.cs_scale, v);
-      s += (double)v * (double)v;
+      const float p = v * v;
+      const float t = hi + p, z = t - hi;
+      lo += fmaf(v, v, -p) + ((hi - (t - z)) + (p - z));
+      hi = t;
     }
-  part[warp][lane] = s;
+  part[warp][lane] = proj.sum64 ? s64 : __hiloint2double(__float_as_int(hi), __float_as_int(lo));
   __syncthreads();  // (and the block's writes of the row statistics are visible to the block)
   auto put = [&](long long m, double c2, double r2) {
     const bool ok = marker_testable(nobs[m], c2, r2, complete_n);
@@ -226,9 +235,21 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
   if (warp == 0) {
     bool close = false;
     if (in) {
-      double t = part[0][lane];
+      double t = 0.0;
+      if (proj.sum64) {
 #pragma unroll
-      for (int w = 1; w < kNormWarps; ++w) t += part[w][lane];
+        for (int w = 0; w < kNormWarps; ++w) t += part[w][lane];
+      } else {
+        float h = 0.0f, l = 0.0f;
+#pragma unroll
+        for (int w = 0; w < kNormWarps; ++w) {
+          const float p = __int_as_float(__double2hiint(part[w][lane]));
+          const float u = h + p, z = u - h;
+          l += __int_as_float(__double2loint(part[w][lane])) + ((h - (u - z)) + (p - z));
+          h = u;
+        }
+        t = (double)h + (double)l;
+      }
       const double c2 = gc2[j], r2 = c2 - t;
       put(j, c2, r2);
       close = nq > 0 && nobs[j] > 0 && c2 > 0.0 && r2 < (1.0 - kRefineShare) * c2;
@@ -412,9 +433,14 @@ cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, co
                            int64_t split) {
   if (M == 0 || nq == 0) return cudaSuccess;
   const int64_t range = round_up((K + ranges - 1) / ranges, 256);
-  dim3 grid((unsigned)((M + 63) / 64), (unsigned)((nq + 31) / 32), (unsigned)ranges);
-  k_project<<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out, (long long)ldq,
-                                  (long long)split);
+  const int kc = nq <= 16 ? 16 : 32, tm = 2048 / kc;
+  const dim3 grid((unsigned)((M + tm - 1) / tm), (unsigned)((nq + kc - 1) / kc), (unsigned)ranges);
+  if (kc == 16)
+    k_project<16><<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out,
+                                        (long long)ldq, (long long)split);
+  else
+    k_project<32><<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out,
+                                        (long long)ldq, (long long)split);
   return cudaGetLastError();
 }
 

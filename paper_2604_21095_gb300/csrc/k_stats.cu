@@ -30,6 +30,10 @@ __device__ __forceinline__ double exact_partial(const ExactArgs& x, long long ro
   const double* y = x.Yres + (long long)col * x.ldy;
   // 2-bit fields 00 (2 copies), 10 (1), 11 (0) minus the mean; 01 (missing) is the mean itself
   const double c00 = 2.0 - mu, c10 = 1.0 - mu, c11 = -mu;
+  // dosage bytes minus the rounded mean, exactly, as (2^52 + byte) - (2^52 + round(mean)): one FP64
+  // addition instead of a conversion and a subtraction on units that do two a cycle. What is left
+  // of the centring multiplies sum_i y_res,p,i = 0; a missing call holds mean - round(mean).
+  const double cr = rint(mu), magic = 4503599627370496.0 + cr, cm = mu - cr;
   double acc0 = 0.0, acc1 = 0.0;
   for (int i0 = 8 * t; i0 < x.N; i0 += 8 * nt) {
     const bool whole = i0 + 8 <= x.N;
@@ -55,7 +59,7 @@ __device__ __forceinline__ double exact_partial(const ExactArgs& x, long long ro
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
         const unsigned byte = ((u < 4 ? b.x : b.y) >> (8 * (u & 3))) & 0xFFu;
-        v[u] = ((mb >> u) & 1u) ? 0.0 : (double)byte - mu;
+        v[u] = ((mb >> u) & 1u) ? cm : __hiloint2double(0x43300000, (int)byte) - magic;
       }
     }
 #pragma unroll
@@ -112,8 +116,9 @@ __device__ __forceinline__ void full_elements(const EpiParams& ep, long long row
     const float rinv = ep.row_inv[row];
     const float scale = ep.col_s[col] * rinv / ep.kappa;
     if (ep.beta) ep.beta[o] = r * scale;
-    if (ep.se) ep.se[o] = scale * sqrtf(omr2 / ep.df_f);
-    if (ep.t) ep.t[o] = r * sqrtf(ep.df_f / omr2);
+    const float sq = sqrtf(omr2 / ep.df_f);  // t = r sqrt(df / (1 - r^2)) = r / sq
+    if (ep.se) ep.se[o] = scale * sq;
+    if (ep.t) ep.t[o] = r / sq;
     if (ep.mlp) ep.mlp[o] = mlog10p_r_f(r, ep.df_f, (float)ep.lnB);
   }
   unsigned todo = __ballot_sync(0xffffffffu, exact);
@@ -183,22 +188,26 @@ __global__ void __launch_bounds__(kRawWarps * 32)
         const int c = warp * CPW + u;
         if (row < ep.M && c < cols) d[i][u] += raw.x[s * raw.split + (c0 + c) * raw.ld + row];
       }
+  float rinv[R], shift[R];  // NaN past the block's rows: no test, no hit, no key
+#pragma unroll
+  for (int i = 0; i < R; ++i) {
+    const long long row = row0 + 32 * i + lane;
+    const bool in = row < ep.M;
+    rinv[i] = in ? ep.row_inv[row] : __int_as_float(0x7fc00000);
+    shift[i] = in && raw.partial && raw.cs ? raw.shift[row] : 0.0f;
+  }
 #pragma unroll
   for (int u = 0; u < CPW; ++u) {
     const int c = warp * CPW + u, col = c0 + c;
     if (c >= cols) break;  // the same for the whole warp
     const float rmul = ep.col_rmul[col];
+    const float cs = raw.partial && raw.cs ? raw.cs[col] * raw.cs_scale : 0.0f;
     uint32_t key = 0u, key_row = 0u;  // bits(|r|) + 1 of this lane's best marker (0: none)
 #pragma unroll
     for (int i = 0; i < R; ++i) {
-      const long long row = row0 + 32 * i + lane;
-      float r = __int_as_float(0x7fc00000);
-      if (row < ep.M) {
-        float D = d[i][u];
-        if (raw.partial) D = fmaf(raw.shift[row], raw.cs[col] * raw.cs_scale, D);
-        r = corr_nan(D, ep.row_inv[row], rmul);
-        if (ep.do_hits && r * r >= ep.r2_thr) emit_hit_raw(ep, D, row, col);
-      }
+      const float D = raw.partial ? fmaf(shift[i], cs, d[i][u]) : d[i][u];
+      const float r = corr_nan(D, rinv[i], rmul);
+      if (ep.do_hits && r * r >= ep.r2_thr) emit_hit_raw(ep, D, row0 + 32 * i + lane, col);
       if (FULL) tile[lane][c] = r;
       const uint32_t k = r == r ? __float_as_uint(fabsf(r)) + 1u : 0u;
       if (k > key) {  // rows ascend: the smallest marker of equal keys stays
@@ -226,27 +235,55 @@ __global__ void __launch_bounds__(kRawWarps * 32)
   }
 }
 
-// Hit records: one block per hit recomputes its product in FP64 and writes the FP64 statistics.
-constexpr int kHitThreads = 512;
-__global__ void __launch_bounds__(kHitThreads) k_hit_stats(EpiParams ep,
-                                                   const unsigned long long* __restrict__ start) {
+// Hit records: a cluster of blocks per hit recomputes its product in FP64 and its first block writes
+// the FP64 statistics. A block of 80 hits or so is bound by the FP64 units (two lanes per cycle and
+// SM): with one thread block per hit half of the SMs had none (65,536 x 16 tests on 23,000 samples:
+// 33 us, 23 with 8 blocks). On short sample axes the last FP64 chain of one thread is the time
+// (17 us at 5,001 samples, 20 with 8 blocks): one block per hit up to kHitSplitN samples.
+constexpr int kHitThreads = 256, kHitCluster = 8, kHitSplitN = 8192;
+__global__ void __launch_bounds__(kHitThreads)
+    k_hit_stats(const __grid_constant__ EpiParams ep, const unsigned long long* __restrict__ start) {
   __shared__ double red[33];
+  __shared__ double parts[2][kHitCluster];  // of the first block; two in turn
   const unsigned long long s0 = *start;
   unsigned long long s1 = *ep.n_hits;
   if (s1 > (unsigned long long)ep.hit_cap) s1 = (unsigned long long)ep.hit_cap;
-  for (unsigned long long i = s0 + blockIdx.x; i < s1; i += gridDim.x) {
-    tg_hit h = ep.hits[i];
+  unsigned nrank;  // blocks per cluster
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
+  const unsigned rank = blockIdx.x % nrank;
+  int turn = 0;
+  for (unsigned long long i = s0 + blockIdx.x / nrank; i < s1; i += gridDim.x / nrank) {
+    const tg_hit h = ep.hits[i];
     const long long row = (long long)h.marker - ep.marker_offset;
-    const double D = block_sum(exact_partial(ep.exact, row, (int)h.pheno, threadIdx.x, blockDim.x), red);
+    const double D = block_sum(exact_partial(ep.exact, row, (int)h.pheno,
+                                             (int)(rank * kHitThreads + threadIdx.x),
+                                             (int)(kHitThreads * nrank)), red);
     if (threadIdx.x == 0) {
-      const Stats64 v = stats_exact(ep, row, (int)h.pheno, D);
-      h.beta = v.beta;
-      h.se = v.se;
-      h.t = v.t;
-      h.mlog10p = v.mlp;
-      ep.hits[i] = h;
+      uint32_t dst;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
+                   : "=r"(dst)
+                   : "r"((uint32_t)__cvta_generic_to_shared(&parts[turn][rank])));
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(D) : "memory");
     }
+    // every block has read the record and delivered its part; the slot of two hits ago is free,
+    // since its reader has arrived here too
+    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
+                     : "memory");
+    if (rank == 0 && threadIdx.x == 0) {
+      double sum = 0.0;
+      for (unsigned k = 0; k < nrank; ++k) sum += parts[turn][k];
+      const Stats64 v = stats_exact(ep, row, (int)h.pheno, sum);
+      tg_hit o = h;
+      o.beta = v.beta;
+      o.se = v.se;
+      o.t = v.t;
+      o.mlog10p = v.mlp;
+      ep.hits[i] = o;
+    }
+    turn ^= 1;
   }
+  // (a block's shared memory stays while others may still write to it: the last write comes
+  // before the last barrier above)
 }
 
 // Deterministic pseudo-random bytes (SplitMix64 of the index); used for timing trial blocks.
@@ -297,8 +334,18 @@ cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream
 
 cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* start, cudaStream_t st) {
   if (ep.exact.G == nullptr) return cudaErrorInvalidValue;  // hits are always recomputed in FP64
-  k_hit_stats<<<152 * 2, kHitThreads, 0, st>>>(ep, start);
-  return cudaGetLastError();
+  const unsigned nrank = ep.exact.N > kHitSplitN ? kHitCluster : 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(nrank * (nrank > 1 ? 76 : 304));
+  cfg.blockDim = dim3(kHitThreads);
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = nrank;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, k_hit_stats, ep, start);
 }
 
 }  // namespace tg
