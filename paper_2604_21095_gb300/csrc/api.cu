@@ -197,6 +197,42 @@ constexpr double kItemUs = 4.0;
 constexpr double kRangeBytesPerUs = 6.0e6;
 constexpr int64_t kPackedOperandBytes = 32 << 20;
 constexpr size_t kMaxSplitFloats = size_t(1) << 26;  // partial sums of a split: 256 MiB at most
+// How a CTA-pair pass of M markers and `cols` columns is split, by the shortest estimate: whole tiles
+// (per = 0; they waste nothing where their last wave is nearly full, and pieces of partial sums
+// cost memory), every tile in ks equal ranges (chunks rounded up to ks x per, one item per pair
+// and more pairs than fit run in turn), or all units dealt evenly (a pair's units may cross
+// into the next tile, which is a second item). Each item costs kItemUs to fill the pipeline and
+// to store.
+PairUnits pick_units(int64_t M, int64_t cols, int64_t bn, int64_t chunks, int64_t sms) {
+  const int64_t n_nt = (cols + bn - 1) / bn, tiles = ((M + 255) / 256) * n_nt, pairs = sms / 2;
+  const double floats = (double)round_up(M, 32) * (double)cols;
+  const double piece_us = 8.0 * floats / kRangeBytesPerUs, chunk_us = kChunkUsCol * (double)bn;
+  PairUnits best{(int)n_nt, (int)chunks, 0, (int)std::min(tiles, pairs), 1};
+  double best_us = 0.97 * ((double)((tiles + pairs - 1) / pairs) * ((double)chunks * chunk_us + kItemUs) +
+                           piece_us);
+  const auto offer = [&](int64_t vchunks, int64_t per, int64_t pieces, double us) {
+    if (us >= best_us || (double)pieces * floats > 2.0 * (double)kMaxSplitFloats ||
+        tiles * vchunks > INT32_MAX / 2)
+      return;
+    best = PairUnits{(int)n_nt, (int)vchunks, (int)per, (int)((tiles * vchunks + per - 1) / per),
+                     (int)pieces};
+    best_us = us;
+  };
+  for (int64_t ks = 2; ks <= chunks; ++ks) {
+    const int64_t per = (chunks + ks - 1) / ks;
+    if ((ks - 1) * per >= chunks) continue;  // no range empty
+    offer(ks * per, per, ks,
+          (double)((tiles * ks + pairs - 1) / pairs) * ((double)per * chunk_us + kItemUs) +
+              (double)ks * piece_us);
+  }
+  const int64_t per = (tiles * chunks + pairs - 1) / pairs;
+  if (per % chunks != 0) {
+    const int64_t pieces = (chunks + per - 2) / per + 1;
+    offer(chunks, per, pieces, (double)per * chunk_us + (double)(per / chunks + 2) * kItemUs +
+                                   (double)pieces * piece_us);
+  }
+  return best;
+}
 int pick_ranges(int64_t tiles, int64_t slots, int64_t chunks, double chunk_us, double range_floats) {
   int best = 1;
   double best_us = 0;
@@ -256,7 +292,8 @@ struct Plan {
   bool dec = false;         // contraction kernels decode the packed rows (no operand in HBM)
   bool single = false;      // the panel's contraction on one CTA per tile
   FusedUnits fu{};          // the split of either pass over the packed rows
-  int ranges_proj = 1;      // K ranges of the projection or joint pass
+  PairUnits pu{};           // the split of a CTA-pair pass that leaves raw products
+  int ranges_proj = 1;      // K ranges or pieces of the projection or joint pass
   int ranges_scan = 1;      // K ranges of the panel's own contraction (> 1: raw, then k_raw_stats)
   int64_t ldr = 0;          // rows of the raw products' columns
   size_t raw_floats = 0;
@@ -301,13 +338,12 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
   r.joint = r.split && r.nq > 0 && p->joint_cols > 0;
   const int64_t chunks = (p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB;
   const double ldr = (double)r.ldr;
-  const int64_t pairs = c->sm_count / 2;
   if (r.fuse_joint || r.fuse_proj) {
     r.ranges_proj = r.fu.pieces;
   } else if (r.split && r.nq > 0) {
     if (r.joint && p->joint_cols > 128) {
-      r.ranges_proj = pick_ranges(n_mp * (p->joint_cols / p->joint_bn), pairs, chunks,
-                                  kChunkUsCol * p->joint_bn, ldr * (double)(r.nq + p->P));
+      r.pu = pick_units(M, p->joint_cols, p->joint_bn, chunks, c->sm_count);
+      r.ranges_proj = r.pu.pieces;
     } else {
       r.ranges_proj = pick_ranges(n_mt, c->sm_count, chunks,
                                   r.joint && p->joint_cols > 64 ? kChunkUs128 : kChunkUs64,
@@ -337,8 +373,10 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
       r.single = true;
       r.ranges_scan = (int)std::min<int64_t>(tuned > 1 ? tuned : 1, chunks);
     } else {
-      r.ranges_scan = pick_ranges(n_mp * ((p->P + p->bn - 1) / p->bn), pairs, chunks,
-                                  kChunkUsCol * p->bn, ldr * cols);
+      // raw only with the split: whole tiles keep the fused epilogue
+      if (n_mp * ((p->P + p->bn - 1) / p->bn) < c->sm_count / 2)
+        r.pu = pick_units(M, p->P, p->bn, chunks, c->sm_count);
+      r.ranges_scan = std::max(1, r.pu.pieces);
     }
     if (r.ranges_scan > 1)
       r.raw_floats = std::max(r.raw_floats,
@@ -619,8 +657,17 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   RawView raw{c->raw, pl.ldr, pl.ldr * (nq + (joint ? p->P : 0)), pl.ranges_proj,
               packed_pass || (split && pl.ranges_proj > 1), c->shift,
               joint ? (f16 ? p->qycs16 : p->qycs) : (f16 ? p->qcs16 : p->qcs),
-              f16 ? (float)(1.0 / kJointF16Scale) : 1.0f, packed_pass ? pl.fu.per : 0,
-              pl.fu.chunks, !split};
+              f16 ? (float)(1.0 / kJointF16Scale) : 1.0f, 0, 0, 1, 1, 0, !split};
+  if (packed_pass) {
+    raw.per = pl.fu.per;
+    raw.chunks = pl.fu.chunks;
+    raw.bn = JCOLS;  // one column tile
+  } else if (joint && pl.pu.per > 0) {
+    raw.per = pl.pu.per;
+    raw.chunks = pl.pu.chunks;
+    raw.n_nt = pl.pu.n_nt;
+    raw.bn = p->joint_bn;
+  }
   if (nq > 0) {
     StageScope s(c, STAGE_PROJECT, st, 1);
     if (!split) {
@@ -647,14 +694,14 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
                                    p->Npad, pp, c->sm_count, p->proj_bn(), kSpinNs, st, dj,
                                    a.encoding, f16));
       } else if (joint && p->joint_cols > 128) {  // more than one narrow tile: CTA pairs
-        const int64_t items = (a.M + 2 * MT - 1) / (2 * MT) * (p->joint_cols / p->joint_bn);
-        if (pl.ranges_proj == 1 && items > c->sm_count / 2) {
+        const int64_t tiles = (a.M + 2 * MT - 1) / (2 * MT) * (p->joint_cols / p->joint_bn);
+        if (pl.pu.per == 0 && tiles > c->sm_count / 2) {
           pp.wave_ctr = reinterpret_cast<unsigned long long*>(c->scratch + 32);
           TG_CUDA(cudaMemsetAsync(pp.wave_ctr, 0, sizeof(unsigned long long), st));
         }
         TG_CUDA(launch_tc2_scan(&tA, &p->tmQYhi, &p->tmQYlo, p->Npad, pp, c->sm_count, kSpinNs, st,
                                 kGroupDefault, c->fuse_decode ? dec : nullptr, a.encoding,
-                                p->joint_bn));
+                                p->joint_bn, pl.pu.per > 0 ? &pl.pu : nullptr));
       } else {
         TG_CUDA(launch_tc_scan(&tA, joint ? &p->tmQYhi : &p->tmQhi, joint ? &p->tmQYlo : &p->tmQlo,
                                p->Npad, pp, c->sm_count, kSpinNs, st, kGroupDefault,
@@ -735,6 +782,7 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
     } else if (joint) {  // the products came with the projection
       raw.x += nq * raw.ld;
       raw.cs += nq;
+      raw.col0 = (int)nq;
       TG_CUDA(launch_raw_stats(raw, ep, st));
       full_done = true;
     } else {
@@ -759,11 +807,18 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
           TG_CUDA(cudaMemsetAsync(pp.wave_ctr, 0, sizeof(unsigned long long), st));
         }
         TG_CUDA(launch_tc2_scan(&tA, &p->tmBhi2, &p->tmBlo2, p->Npad, pp, c->sm_count, kSpinNs, st,
-                                group, dec, a.encoding, p->bn));
+                                group, dec, a.encoding, p->bn,
+                                pl.ranges_scan > 1 ? &pl.pu : nullptr));
       }
       if (pl.ranges_scan > 1) {
-        TG_CUDA(launch_raw_stats(RawView{c->raw, pl.ldr, pl.ldr * p->P, pl.ranges_scan, true,
-                                         c->shift, p->col_cs, 1.0f}, ep, st));
+        RawView rv{c->raw, pl.ldr, pl.ldr * p->P, pl.ranges_scan, true, c->shift, p->col_cs, 1.0f};
+        if (!pl.single) {
+          rv.per = pl.pu.per;
+          rv.chunks = pl.pu.chunks;
+          rv.n_nt = pl.pu.n_nt;
+          rv.bn = p->bn;
+        }
+        TG_CUDA(launch_raw_stats(rv, ep, st));
         full_done = true;
       }
     }

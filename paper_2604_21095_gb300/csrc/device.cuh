@@ -3,6 +3,7 @@
 
 #include <cuda_bf16.h>
 #include <cstdint>
+#include <initializer_list>
 
 #include "internal.h"
 #include "pvalue.cuh"
@@ -13,6 +14,18 @@ __device__ __forceinline__ uint64_t globaltimer_ns() {
   uint64_t t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
   return t;
+}
+
+// Programmatic dependent launch: the kernels of a scan follow one another on the stream with their
+// launch latency hidden (launch_chained). The next kernel may start once every block of this one
+// has called chain_wait, and its own chain_wait returns when this one has completed, its writes
+// visible. Called once by every thread that goes on to touch global memory, before it does.
+// Pointers whose loads the compiler may take for loads of constants (__restrict__ parameters,
+// __ldg) go through it, so that no such load can be moved ahead of the wait.
+template <class... T>
+__device__ __forceinline__ void chain_wait(T&... p) {
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+  (void)std::initializer_list<int>{([&] { asm volatile("" : "+l"(p)::"memory"); }(), 0)...};
 }
 
 // Sum over a whole thread block (any size multiple of 32, <= 1024); every thread gets it.
@@ -52,10 +65,10 @@ __device__ __forceinline__ float corr_nan(float D, float rinv, float rmul) {
   return fminf(1.0f, fmaxf(-1.0f, r));
 }
 
-// Ranges of the raw products of marker row `row` (see RawView).
-__device__ __forceinline__ int raw_ranges(const RawView& v, long long row) {
+// Ranges of the raw product of marker row `row` and column `col` (see RawView).
+__device__ __forceinline__ int raw_ranges(const RawView& v, long long row, int col) {
   if (v.per == 0) return v.ranges;
-  const int u0 = (int)(row / kFusedRows) * v.chunks;
+  const int u0 = ((int)(row / kFusedRows) * v.n_nt + (v.col0 + col) / v.bn) * v.chunks;
   return (u0 + v.chunks - 1) / v.per - u0 / v.per + 1;
 }
 

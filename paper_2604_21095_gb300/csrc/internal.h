@@ -304,6 +304,25 @@ bool make_tmap(CUtensorMap* m, const void* ptr, int64_t rows, int64_t K, int64_t
 bool make_tmap_packed(CUtensorMap* m, const void* ptr, int64_t rows, int64_t ld, uint32_t box_bytes,
                       uint32_t box_rows = 128, bool swizzle = false);
 
+// Launch a kernel that starts with chain_wait() (device.cuh) so that it may be scheduled while the
+// kernel before it on the stream still runs: each boundary between the four or five kernels of a
+// small scan cost 1.5 to 2.5 us. Behind anything else it is an ordinary launch.
+template <class... P, class... A>
+cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, unsigned block, size_t smem,
+                           cudaStream_t st, const A&... args) {
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(block);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // panel kernels (k_panel.cu)
 cudaError_t launch_build_design(double* X, const double* C, int64_t ldc, int64_t N, int64_t n_cov,
                                 uint32_t* flags, cudaStream_t st);
@@ -347,10 +366,19 @@ cudaError_t launch_subset_stats(const uint8_t* G, int64_t ldg, int encoding, int
                                 double* gc2s, cudaStream_t st);
 
 // SIMT kernels (k_simt.cu)
+// The CTA-pair kernel's units (one 256 x bn tile x one accumulation chunk) and their even split over
+// the pairs: pair w takes the units [w per, (w + 1) per), tile (m-tile pair t / n_nt, column tile
+// t % n_nt) holding the units t chunks .., so at most `pieces` pairs share a tile. chunks may be more
+// than the tile has (a multiple of per, so that no pair crosses into another tile).
+struct PairUnits {
+  int n_nt, chunks, per, pairs, pieces;
+};
+
 // Raw products as the contraction kernels leave them (EpiParams::raw_out): element (m, k) of
 // range s at x[s * split + k * ld + m]. With `partial` the ranges are partial sums, which are
 // added in range order, and then shift[m] * cs[k] * cs_scale. per > 0: the ranges are the pieces of
-// k_joint_fused's tiles, as many as the CTAs that share the row's tile (see FusedUnits).
+// a tile of 256 rows and bn columns, as many as the CTAs or pairs that share it (FusedUnits,
+// PairUnits), tiles counted over n_nt column tiles; column k here is column col0 + k of the pass.
 struct RawView {
   const float* x;
   long long ld, split;
@@ -359,7 +387,7 @@ struct RawView {
   const float* shift;
   const float* cs;
   float cs_scale;
-  int per, chunks;
+  int per, chunks, n_nt, bn, col0;
   bool sum64;  // k_marker_norm adds the ranges in FP64 (the FP32 form; no add-back)
 };
 // A block's integer sums, from which k_marker_norm makes the row statistics (nobs, mean, gc2):
@@ -482,11 +510,12 @@ cudaError_t launch_fp4_scan(const CUtensorMap* tmA, const CUtensorMap* tmB, int 
                             cudaStream_t st);
 
 // tensor-core kernel on CTA pairs, 256 x bn tiles (k_tc2.cu); bn a multiple of 32, at most 256,
-// the B maps with boxes of bn / 2 rows. Raw mode (ep.raw_out) takes split-K.
+// the B maps with boxes of bn / 2 rows. Raw mode (ep.raw_out) takes an even split of its units.
 cudaError_t launch_tc2_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                             const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                             long long spin_ns, cudaStream_t st, int group_m = 16,
-                            const DecodeArgs* dec = nullptr, int encoding = 0, int bn = 256);
+                            const DecodeArgs* dec = nullptr, int encoding = 0, int bn = 256,
+                            const PairUnits* pu = nullptr);
 
 // bounded wait test (k_tc.cu)
 cudaError_t launch_wait_test(const uint32_t* flag, long long limit_ns, uint32_t* result,

@@ -118,13 +118,14 @@ __device__ __forceinline__ void row_stats(const uint8_t* __restrict__ row, int N
   }
 }
 
-// 8 decoded samples starting at i0 (a multiple of 8): values and missing bits.
+// 8 decoded samples starting at i0 (a multiple of 8): values and missing bits. (__ldg: the loads of
+// the groups to come need not wait for the operand stores of those before.)
 template <int ENC>
 __device__ __forceinline__ void load8(const uint8_t* __restrict__ row, const uint32_t* __restrict__ mrow,
                                       int i0, int N, float v[8], uint32_t& miss) {
   miss = 0;
   if (ENC == TG_ENC_2BIT) {
-    const uint32_t w = *reinterpret_cast<const uint16_t*>(row + (i0 >> 2));
+    const uint32_t w = __ldg(reinterpret_cast<const uint16_t*>(row + (i0 >> 2)));
 #pragma unroll
     for (int s = 0; s < 8; ++s) {
       const uint32_t f = (w >> (2 * s)) & 3u;
@@ -132,8 +133,8 @@ __device__ __forceinline__ void load8(const uint8_t* __restrict__ row, const uin
       if (f == 1u && i0 + s < N) miss |= 1u << s;
     }
   } else {
-    const uint2 w = *reinterpret_cast<const uint2*>(row + i0);
-    if (mrow) miss = (mrow[i0 >> 5] >> (i0 & 31)) & 0xFFu;
+    const uint2 w = __ldg(reinterpret_cast<const uint2*>(row + i0));
+    if (mrow) miss = (__ldg(mrow + (i0 >> 5)) >> (i0 & 31)) & 0xFFu;
 #pragma unroll
     for (int s = 0; s < 8; ++s) v[s] = (float)(((s < 4 ? w.x : w.y) >> (8 * (s & 3))) & 0xFFu);
   }
@@ -165,6 +166,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_decode(
     double* __restrict__ mean_out, double* __restrict__ gc2_out) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long j = (long long)blockIdx.x * kWarps + warp;
+  chain_wait(G, miss);
   if (j >= M) return;
   const uint8_t* row = G + j * ldg;
   const uint32_t* mrow = miss ? miss + j * ldm : nullptr;
@@ -214,7 +216,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_decode(
         const int i0 = (int)(t << 4);
         uint32_t o[8] = {0, 0, 0, 0, 0, 0, 0, 0};
         if (i0 < N) {
-          const uint32_t ms = mrow ? (mrow[i0 >> 5] >> (i0 & 31)) & 0xFFFFu : 0u;
+          const uint32_t ms = mrow ? (__ldg(mrow + (i0 >> 5)) >> (i0 & 31)) & 0xFFFFu : 0u;
           split16_u8(__ldg(vrow + t), c_plus, ms, mh2, o);
           if (i0 + 16 > N) zero_tail16(o, i0, N);
         }
@@ -261,6 +263,7 @@ __global__ void __launch_bounds__(THREADS, GPT * THREADS <= 1536 ? 4 : 2) k_deco
   __shared__ uint32_t red[3][THREADS / 32];
   const long long j = blockIdx.x;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  chain_wait(G, miss);
   const uint8_t* row = G + j * ldg;
   const uint32_t* mrow = miss ? miss + j * ldm : nullptr;
   const int nvalid = (N + 15) >> 4;  // 16-sample groups holding a sample < N
@@ -390,6 +393,7 @@ __global__ void __launch_bounds__(kWarps * 32) k_subset_stats(
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long j0 = (long long)blockIdx.x * kSubsetRows;
   const int groups = (N + 15) >> 4;  // 16 samples each
+  chain_wait(G, miss, samples, mean, nobs, S);
   for (int i = warp; i < kSubsetRows && j0 + i < M; i += kWarps) {
     const uint8_t* row = G + (j0 + i) * ldg;
     const uint32_t* mrow = miss ? miss + (j0 + i) * ldm : nullptr;
@@ -469,10 +473,9 @@ cudaError_t go(const uint8_t* G, int64_t ldg, int64_t N, int64_t M, const uint32
   if constexpr (PREC == TG_PREC_SPLIT_BF16) {
     if (N <= kWarpRowN || !Ahi) {
       const unsigned grid = (unsigned)((M + kWarps - 1) / kWarps);
-      k_decode<ENC, PREC><<<grid, kWarps * 32, 0, st>>>(
+      return launch_chained(k_decode<ENC, PREC>, dim3(grid), kWarps * 32, 0, st,
           G, ldg, (int)N, M, missing, ldm, Ahi, shift, mh, lda, nobs,
           reinterpret_cast<long long*>(S), reinterpret_cast<long long*>(S2), mean, gc2);
-      return cudaGetLastError();
     }
     constexpr int T = ENC == TG_ENC_2BIT ? 128 : 256;
     constexpr int G1 = ENC == TG_ENC_2BIT ? 12 : 6;
@@ -480,22 +483,19 @@ cudaError_t go(const uint8_t* G, int64_t ldg, int64_t N, int64_t M, const uint32
     long long* S64 = reinterpret_cast<long long*>(S);
     long long* S264 = reinterpret_cast<long long*>(S2);
     if (N <= T * G1 * 16) {
-      k_decode_rows<ENC, G1, T><<<(unsigned)M, T, 0, st>>>(G, ldg, (int)N, missing, ldm, A, shift,
+      return launch_chained(k_decode_rows<ENC, G1, T>, dim3((unsigned)M), T, 0, st, G, ldg, (int)N, missing, ldm, A, shift,
                                                           mh, lda, nobs, S64, S264, mean, gc2);
-      return cudaGetLastError();
     }
     if (N <= T * 2 * G1 * 16) {
-      k_decode_rows<ENC, 2 * G1, T><<<(unsigned)M, T, 0, st>>>(G, ldg, (int)N, missing, ldm, A,
+      return launch_chained(k_decode_rows<ENC, 2 * G1, T>, dim3((unsigned)M), T, 0, st, G, ldg, (int)N, missing, ldm, A,
                                                               shift, mh, lda, nobs, S64, S264,
                                                               mean, gc2);
-      return cudaGetLastError();
     }
   }
   const unsigned grid = (unsigned)((M + kWarps - 1) / kWarps);
-  k_decode<ENC, PREC><<<grid, kWarps * 32, 0, st>>>(
+  return launch_chained(k_decode<ENC, PREC>, dim3(grid), kWarps * 32, 0, st,
       G, ldg, (int)N, M, missing, ldm, Ahi, shift, mh, lda, nobs, reinterpret_cast<long long*>(S),
       reinterpret_cast<long long*>(S2), mean, gc2);
-  return cudaGetLastError();
 }
 
 }  // namespace
@@ -524,12 +524,10 @@ cudaError_t launch_subset_stats(const uint8_t* G, int64_t ldg, int encoding, int
   const unsigned grid = (unsigned)((M + kSubsetRows - 1) / kSubsetRows);
   const long long* S64 = reinterpret_cast<const long long*>(S);
   if (encoding == TG_ENC_2BIT)
-    k_subset_stats<TG_ENC_2BIT><<<grid, kWarps * 32, 0, st>>>(G, ldg, (int)N, M, missing, ldm,
+    return launch_chained(k_subset_stats<TG_ENC_2BIT>, dim3(grid), kWarps * 32, 0, st, G, ldg, (int)N, M, missing, ldm,
                                                                samples, mean, nobs, S64, gc2s);
-  else
-    k_subset_stats<TG_ENC_U8_DOSAGE><<<grid, kWarps * 32, 0, st>>>(
+  return launch_chained(k_subset_stats<TG_ENC_U8_DOSAGE>, dim3(grid), kWarps * 32, 0, st,
         G, ldg, (int)N, M, missing, ldm, samples, mean, nobs, S64, gc2s);
-  return cudaGetLastError();
 }
 
 }  // namespace tg

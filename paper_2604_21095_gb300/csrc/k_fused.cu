@@ -220,7 +220,7 @@ __device__ __forceinline__ uint32_t first_bytes_shift_u8(const uint8_t* row, int
   uint32_t s = 0, s2 = 0;
 #pragma unroll 1
   for (int g = 0; g < 4 && 16 * g < N; ++g)
-    sums16_u8(__ldg(reinterpret_cast<const uint4*>(row) + g), 16 * g, N, s, s2);
+    sums16_u8(reinterpret_cast<const uint4*>(row)[g], 16 * g, N, s, s2);
   const int n = N < 64 ? N : 64;
   const int c = (int)rintf((float)s / (float)n);
   return (uint32_t)(c < 0 ? 0 : c > 255 ? 255 : c);
@@ -379,6 +379,7 @@ __global__ void __launch_bounds__(kFThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+  chain_wait();
   Items it(per, units, chunks, num_kb);
 
   if (warp < 4) {
@@ -641,9 +642,8 @@ cudaError_t go_fused(const CUtensorMap* bh, const CUtensorMap* bl, int64_t K, co
     attr_set = true;
   }
   const FusedUnits fu = fused_units(ep.M, K, sm_count);
-  k_joint_fused<OPA, BR><<<fu.grid, kFThreads, C::kSmem, st>>>(
+  return launch_chained(k_joint_fused<OPA, BR>, dim3(fu.grid), kFThreads, C::kSmem, st,
       *bh, *bl, (int)(K / TBK), fu.chunks, fu.per, fu.units, bn, spin_ns, ep, da);
-  return cudaGetLastError();
 }
 
 }  // namespace

@@ -38,6 +38,7 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
   // FP32 partial sums over 256 samples, flushed into FP64 totals
   float acc[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
   double tot[4][2] = {{0, 0}, {0, 0}, {0, 0}, {0, 0}};
+  chain_wait(A, QB);
   const int k_lo = (int)blockIdx.z * range, k_hi = min(K, k_lo + range);
   qg += blockIdx.z * split;
   for (int i0 = k_lo; i0 < k_hi; i0 += 32) {
@@ -187,7 +188,8 @@ __device__ __forceinline__ void row_statistics(const RowSums& sums, long long j,
 }
 __global__ void __launch_bounds__(256) k_row_statistics(long long M, RowSums sums, RawView raw) {
   const long long j = blockIdx.x * 256ll + threadIdx.x;
-  if (j < M) row_statistics(sums, j, raw_ranges(raw, j));
+  chain_wait();
+  if (j < M) row_statistics(sums, j, raw_ranges(raw, j, 0));
 }
 
 __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
@@ -199,7 +201,8 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long m0 = blockIdx.x * 32ll, j = m0 + lane;
   const bool in = j < M;
-  const int ranges = raw_ranges(proj, m0);  // the block's markers are in one tile
+  chain_wait();
+  const int ranges = raw_ranges(proj, m0, 0);  // the block's markers and the columns are in one tile
   if ((sums.x || sums.S) && warp == 0 && in) row_statistics(sums, j, ranges);
   // sum of squares in pairs of floats (48 bits; FP64 instructions take 16 cycles of an SM each, and
   // three per column were half of this kernel's time): v^2 = p + e exactly, and two-sums
@@ -301,6 +304,7 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
   const int n0 = blockIdx.x * BN;
   // global -> smem mapping: each thread moves 2 float4 of A and 2 of B per K step
   const int lr = tid >> 2, lk = (tid & 3) * 4;
+  chain_wait(A, B);
   const int k_lo = (int)blockIdx.z * range, k_hi = min(K, k_lo + range);
   A += k_lo;
   B += k_lo;
@@ -436,19 +440,16 @@ cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, co
   const int kc = nq <= 16 ? 16 : 32, tm = 2048 / kc;
   const dim3 grid((unsigned)((M + tm - 1) / tm), (unsigned)((nq + kc - 1) / kc), (unsigned)ranges);
   if (kc == 16)
-    k_project<16><<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out,
+    return launch_chained(k_project<16>, grid, 256, 0, st, A, lda, M, (int)K, (int)range, QB, (int)nq, out,
                                         (long long)ldq, (long long)split);
-  else
-    k_project<32><<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out,
+  return launch_chained(k_project<32>, grid, 256, 0, st, A, lda, M, (int)K, (int)range, QB, (int)nq, out,
                                         (long long)ldq, (long long)split);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_row_statistics(int64_t M, const RowSums& sums, const RawView& raw,
                                   cudaStream_t st) {
   if (M == 0) return cudaSuccess;
-  k_row_statistics<<<(unsigned)((M + 255) / 256), 256, 0, st>>>(M, sums, raw);
-  return cudaGetLastError();
+  return launch_chained(k_row_statistics, dim3((unsigned)((M + 255) / 256)), 256, 0, st, M, sums, raw);
 }
 
 cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2,
@@ -456,9 +457,8 @@ cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2
                                const MarkerRefine& refine, const NormOut& out, cudaStream_t st,
                                int64_t complete_n, const RowSums& sums) {
   if (M == 0) return cudaSuccess;
-  k_marker_norm<<<(unsigned)((M + 31) / 32), kNormWarps * 32, 0, st>>>(
+  return launch_chained(k_marker_norm, dim3((unsigned)((M + 31) / 32)), kNormWarps * 32, 0, st,
       M, nobs, gc2, proj, (int)nq, kappa, refine, out, (int)complete_n, sums);
-  return cudaGetLastError();
 }
 
 cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t K,
@@ -470,8 +470,7 @@ cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64
   const int64_t range = round_up((K + ks - 1) / ks, BK);
   if ((ks - 1) * range >= K) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((ep.P + BN - 1) / BN), (unsigned)((ep.M + BM - 1) / BM), (unsigned)ks);
-  k_sgemm_scan<<<grid, 256, 0, st>>>(A, lda, B, ldb, (int)K, (int)range, ep);
-  return cudaGetLastError();
+  return launch_chained(k_sgemm_scan, grid, 256, 0, st, A, lda, B, ldb, (int)K, (int)range, ep);
 }
 
 }  // namespace tg

@@ -135,6 +135,7 @@ __device__ __forceinline__ void full_elements(const EpiParams& ep, long long row
 constexpr int kFullThreads = 256;
 __global__ void __launch_bounds__(kFullThreads, 4)
     k_full_stats(const __grid_constant__ EpiParams ep, long long drow, int dcol) {
+  chain_wait();
   const long long total = (long long)ep.M * ep.P;
   const long long stride = (long long)gridDim.x * kFullThreads;
   long long e = blockIdx.x * (long long)kFullThreads + threadIdx.x;
@@ -173,20 +174,28 @@ __global__ void __launch_bounds__(kRawWarps * 32)
   const int c0 = (int)blockIdx.y * CW;
   const int cols = min(CW, ep.P - c0);
   const long long row0 = (long long)blockIdx.x * (32 * R);
+  chain_wait();
   float d[R][CPW];
 #pragma unroll
   for (int i = 0; i < R; ++i)
 #pragma unroll
     for (int u = 0; u < CPW; ++u) d[i][u] = 0.0f;
-  const int ranges = raw_ranges(raw, row0);  // the block's rows are in one tile
-  for (int s = 0; s < ranges; ++s)
+  // the block's rows are in one tile; a warp's columns may be in two
+  int ranges[CPW], most = 0;
+#pragma unroll
+  for (int u = 0; u < CPW; ++u) {
+    const int c = warp * CPW + u;
+    ranges[u] = c < cols ? raw_ranges(raw, row0, c0 + c) : 0;
+    most = max(most, ranges[u]);
+  }
+  for (int s = 0; s < most; ++s)
 #pragma unroll
     for (int u = 0; u < CPW; ++u)
 #pragma unroll
       for (int i = 0; i < R; ++i) {
         const long long row = row0 + 32 * i + lane;
-        const int c = warp * CPW + u;
-        if (row < ep.M && c < cols) d[i][u] += raw.x[s * raw.split + (c0 + c) * raw.ld + row];
+        if (row < ep.M && s < ranges[u])
+          d[i][u] += raw.x[s * raw.split + (c0 + warp * CPW + u) * raw.ld + row];
       }
   float rinv[R], shift[R];  // NaN past the block's rows: no test, no hit, no key
 #pragma unroll
@@ -245,6 +254,7 @@ __global__ void __launch_bounds__(kHitThreads)
     k_hit_stats(const __grid_constant__ EpiParams ep, const unsigned long long* __restrict__ start) {
   __shared__ double red[33];
   __shared__ double parts[2][kHitCluster];  // of the first block; two in turn
+  chain_wait(start);
   const unsigned long long s0 = *start;
   unsigned long long s1 = *ep.n_hits;
   if (s1 > (unsigned long long)ep.hit_cap) s1 = (unsigned long long)ep.hit_cap;
@@ -311,8 +321,7 @@ cudaError_t launch_full_stats(const EpiParams& ep, cudaStream_t st) {
   long long grid = (total + kFullThreads - 1) / kFullThreads;
   if (grid > 152 * 32) grid = 152 * 32;  // a grid-stride loop: 32 blocks per SM at most
   const long long stride = grid * kFullThreads;
-  k_full_stats<<<(unsigned)grid, kFullThreads, 0, st>>>(ep, stride / ep.P, (int)(stride % ep.P));
-  return cudaGetLastError();
+  return launch_chained(k_full_stats, dim3((unsigned)grid), kFullThreads, 0, st, ep, stride / ep.P, (int)(stride % ep.P));
 }
 
 cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream_t st) {
@@ -322,14 +331,11 @@ cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream
   const long long rows = ep.do_full ? 32 : 128;
   const dim3 grid((unsigned)((ep.M + rows - 1) / rows), (unsigned)((ep.P + cw - 1) / cw));
   constexpr int T = kRawWarps * 32;
-  if (ep.do_full) {
-    if (small) k_raw_stats<true, 1><<<grid, T, 0, st>>>(raw, ep);
-    else k_raw_stats<true, 4><<<grid, T, 0, st>>>(raw, ep);
-  } else {
-    if (small) k_raw_stats<false, 1><<<grid, T, 0, st>>>(raw, ep);
-    else k_raw_stats<false, 4><<<grid, T, 0, st>>>(raw, ep);
-  }
-  return cudaGetLastError();
+  if (ep.do_full)
+    return small ? launch_chained(k_raw_stats<true, 1>, grid, T, 0, st, raw, ep)
+                 : launch_chained(k_raw_stats<true, 4>, grid, T, 0, st, raw, ep);
+  return small ? launch_chained(k_raw_stats<false, 1>, grid, T, 0, st, raw, ep)
+               : launch_chained(k_raw_stats<false, 4>, grid, T, 0, st, raw, ep);
 }
 
 cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* start, cudaStream_t st) {
@@ -339,12 +345,14 @@ cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* star
   cfg.gridDim = dim3(nrank * (nrank > 1 ? 76 : 304));
   cfg.blockDim = dim3(kHitThreads);
   cfg.stream = st;
-  cudaLaunchAttribute at[1];
+  cudaLaunchAttribute at[2];
   at[0].id = cudaLaunchAttributeClusterDimension;
   at[0].val.clusterDim.x = nrank;
   at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_chained
+  at[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = at;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = 2;
   return cudaLaunchKernelEx(&cfg, k_hit_stats, ep, start);
 }
 

@@ -150,6 +150,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+  chain_wait();
   const int num_tiles = n_mt * n_nt;
   // work items: (tile, split), independent of one another
   const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
@@ -344,7 +345,8 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (ep.raw_out) {
         // covariate projection (and a small panel's products), unnormalised
         const int col0 = nt * bn + col_half;
-        if (row_ok) raw_store(ep, tot, row, col0, min(ep.raw_cols, nt * bn + bn), split, shift);
+        if (row_ok) raw_store(ep, tot, row, col0, min(ep.raw_cols, nt * bn + bn), split,
+                              ks > 1, shift);
       } else {
         epilogue_tile(ep, tot, row, row_base, row_ok, rinv, shift,
                       nt * bn + col_half, min(ep.P, nt * bn + bn), lane);
@@ -397,9 +399,9 @@ cudaError_t go(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* b
   const int items = n_mt * n_nt * ks;
   const int grid = items < sm_count ? items : sm_count;
   if (KS == 2 && (bn > BR || (K / TBK) % 2)) return cudaErrorInvalidValue;
-  k_tc_scan<OPA, KS, BR, MS><<<grid, kThreads, Cfg<OPA, KS, BR, MS>::kSmem, st>>>(
+  return launch_chained(k_tc_scan<OPA, KS, BR, MS>, dim3((unsigned)grid), kThreads,
+                           Cfg<OPA, KS, BR, MS>::kSmem, st,
       *a, *bh, *bl, (int)(K / TBK), n_mt, n_nt, bn, group_m, spin_ns, ep, da);
-  return cudaGetLastError();
 }
 
 }  // namespace

@@ -24,9 +24,9 @@
 // registers) when every statistic is written, every 2048 samples when only hits and best markers
 // are kept (chunk_kb). In raw mode (a joint operand of the projection columns and the panel, or
 // any panel on a block with too few tiles to fill the SMs) the products are written unnormalised
-// and column-major for k_marker_norm and k_raw_stats, in 1,024-sample chunks, and K may be split:
-// a work item is then a tile and a chunk-aligned range of the samples, and each range writes its
-// own partial sums. Every wait is bounded; a timeout raises the abort flag in both CTAs.
+// and column-major for k_marker_norm and k_raw_stats, in 1,024-sample chunks, and the work may be cut
+// into units of one tile x one chunk, dealt evenly to the pairs (PairUnits): each pair writes its
+// part of a tile as one piece of partial sums. Every wait is bounded; a timeout raises the abort flag in both CTAs.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -231,7 +231,7 @@ template <int OPA>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     k_tc2_scan(const __grid_constant__ CUtensorMap tmAhi, const __grid_constant__ CUtensorMap tmBhi,
                const __grid_constant__ CUtensorMap tmBlo, int num_kb, int n_mt, int n_nt, int bn,
-               int group_p, long long spin_ns, EpiParams ep,
+               int group_p, int per, int chunks, long long spin_ns, EpiParams ep,
                const __grid_constant__ DecodeArgs da) {
   using C = Cfg2<OPA>;
   constexpr bool kFused = OPA != OPA_TMA;
@@ -305,12 +305,32 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   cluster_sync_all();  // both CTAs' barriers initialised, both TMEM allocations done
   tc_fence_after();
   const uint32_t tmem_base = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
+  chain_wait();
   const int n_mp = (n_mt + 1) / 2;
-  // work items: (tile, K range); items of one tile are consecutive
-  const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
-  const int num_tiles = n_mp * n_nt * ks;
+  // The ring carries tiles of the raster or, where the work is cut into units (per > 0), the first
+  // unit of an item: the pair's consecutive units of one tile (tile u / chunks, column tiles
+  // first). Either way an index of num_items or more ends the work.
+  const int num_items = per > 0 ? n_mp * n_nt * chunks : n_mp * n_nt;
   const int ckb = chunk_kb(ep);
   const int cid = (int)cluster_id(), ncl = (int)num_clusters();
+  const int unit_end = min(num_items, (cid + 1) * per);
+  struct Item {
+    int mp, nt, k_lo, k_hi, piece;
+  };
+  auto open_item = [&](int t) -> Item {
+    Item r{0, 0, 0, num_kb, 0};
+    if (per > 0) {
+      const int tile = t / chunks, c = t - tile * chunks, n = min(chunks - c, unit_end - t);
+      r.mp = tile / n_nt;
+      r.nt = tile - r.mp * n_nt;
+      r.k_lo = c * kChunkKB;
+      r.k_hi = min(num_kb, (c + n) * kChunkKB);
+      r.piece = cid - tile * chunks / per;
+    } else {
+      tile_coord2(t, n_mp, n_nt, group_p, r.mp, r.nt);
+    }
+    return r;
+  };
   // a timeout in either CTA stops both
   auto wait = [&](uint32_t bar, uint32_t parity) {
     const bool ok = mbar_wait(bar, parity, abort_flag, spin_ns, ep.status);
@@ -320,8 +340,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
   auto wait_warp = [&](uint32_t bar, uint32_t parity) {  // one answer for a whole warp
     return __all_sync(0xffffffffu, wait(bar, parity)) != 0;
   };
-  // Tile `i` of this pair's sequence from the ring, for every consumer role: a single thread
-  // (whole_warp false) or a whole warp, whose lane 0 then arrives for it. Returns num_tiles at
+  // Item `i` of this pair's sequence from the ring, for every consumer role: a single thread
+  // (whole_warp false) or a whole warp, whose lane 0 then arrives for it. Returns num_items at
   // the end of the work, and -1 on timeout or abort.
   auto take_tile = [&](int i, bool whole_warp) -> int {
     const int r = i % kTileRing;
@@ -348,6 +368,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 #pragma unroll
       for (int s = 0; s < S; ++s) armed[s] = -1;
       bool ok = true;
+      int next_unit = cid * per;
       for (int i = 0; ok; ++i) {
         int tile;
         if (leader) {  // take the next tile and publish it to both CTAs
@@ -357,7 +378,12 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
             st_cluster_u32(peer_abort, 1u);
             break;
           }
-          tile = next_tile(ep.wave_ctr, i, cid, ncl, num_tiles);
+          if (per > 0) {  // the units after the last item's
+            tile = next_unit < unit_end ? next_unit : num_items;
+            next_unit += min(chunks - next_unit % chunks, unit_end - next_unit);
+          } else {
+            tile = next_tile(ep.wave_ctr, i, cid, ncl, num_items);
+          }
           tile_slot[r] = tile;
           st_cluster_u32(map_to_rank(smem_u32((const void*)(tile_slot + r)), 1u), (uint32_t)tile);
           mbar_arrive(tfull_bar(r));
@@ -366,17 +392,15 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
           tile = take_tile(i, false);
           if (tile < 0) break;
         }
-        if (tile >= num_tiles) break;
-        int mp, nt, k_lo, k_hi;
-        tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
-        split_range(num_kb, ks, tile % ks, k_lo, k_hi);
-        const int kbs = k_hi - k_lo;
+        if (tile >= num_items) break;
+        const Item it = open_item(tile);
+        const int k_lo = it.k_lo, kbs = it.k_hi - it.k_lo;
         const bool rev = k_reversed(tile, ncl, ep.raw_out != nullptr);
-        const int mt0 = 2 * mp;
+        const int mt0 = 2 * it.mp;
         const uint32_t pair_bytes =
             2u * KS * ((kFused ? 0u : (uint32_t)A_BYTES) + (uint32_t)bn * (TBK * 2));
         const int arow = (mt0 + (int)rank) * TBM;
-        const int brow = nt * bn + (int)rank * (bn / 2);
+        const int brow = it.nt * bn + (int)rank * (bn / 2);
         for (int kb = 0; kb < kbs; kb += KS) {
           const int kx = k_lo + (rev ? kbs - KS - kb : kb);  // first K block of this stage
           if (!wait(empty_bar(stage), phase ^ 1u)) {
@@ -424,10 +448,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       for (int i = 0; ok; ++i) {
         // the reduction's result is known to be the same in every lane
         const int tile = __reduce_min_sync(0xffffffffu, take_tile(i, true));
-        if (tile < 0 || tile >= num_tiles) break;
-        int k_lo, k_hi;
-        split_range(num_kb, ks, tile % ks, k_lo, k_hi);
-        const int kbs = k_hi - k_lo;
+        if (tile < 0 || tile >= num_items) break;
+        const Item it = open_item(tile);
+        const int kbs = it.k_hi - it.k_lo;
         for (int kb0 = 0; kb0 < kbs && ok; kb0 = chunk_end_c(kb0, kbs, ckb), ++g) {
           const int acc = (int)(g & 1u);
           const uint32_t ph = (g >> 1) & 1u;
@@ -476,13 +499,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
       bool ok = true;
       for (int i = 0; ok; ++i) {
         const int tile = take_tile(i, true);
-        if (tile < 0 || tile >= num_tiles) break;
-        int mp, nt, k_lo, k_hi;
-        tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
-        split_range(num_kb, ks, tile % ks, k_lo, k_hi);
-        const long long r0 = (long long)(2 * mp + (int)rank) * TBM + t;
+        if (tile < 0 || tile >= num_items) break;
+        const Item it = open_item(tile);
+        const int k_lo = it.k_lo, kbs = it.k_hi - it.k_lo;
+        const long long r0 = (long long)(2 * it.mp + (int)rank) * TBM + t;
         const uint2 k0 = dec_row_consts<OPA>(da, r0), k1 = dec_row_consts<OPA>(da, r0 + 64);
-        const int kbs = k_hi - k_lo;
         const bool rev = k_reversed(tile, ncl, ep.raw_out != nullptr);
         for (int kb = 0; kb < kbs; ++kb) {
           const int kx = k_lo + (rev ? kbs - 1 - kb : kb);  // the K block the producer loaded
@@ -515,11 +536,9 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
     bool ok = true;
     for (int i = 0; ok; ++i) {
       const int tile = take_tile(i, true);
-      if (tile < 0 || tile >= num_tiles) break;
-      int mp, nt, k_lo, k_hi;
-      tile_coord2(tile / ks, n_mp, n_nt, group_p, mp, nt);
-      split_range(num_kb, ks, tile % ks, k_lo, k_hi);
-      const int kbs = k_hi - k_lo;
+      if (tile < 0 || tile >= num_items) break;
+      const Item it = open_item(tile);
+      const int kbs = it.k_hi - it.k_lo;
       float tot[128];
 #pragma unroll
       for (int e = 0; e < 128; ++e) tot[e] = 0.0f;
@@ -547,13 +566,13 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive_cluster(acc ? leader_cempty1 : leader_cempty0);
       }
       if (!ok) break;
-      const long long row_base = (long long)(2 * mp + (int)rank) * TBM + quarter * 32;
+      const long long row_base = (long long)(2 * it.mp + (int)rank) * TBM + quarter * 32;
       const long long row = row_base + lane;
       const bool row_ok = row < ep.M;
       const float shift = (row_ok && ep.row_shift) ? ep.row_shift[row] : 0.0f;
-      const int col0 = nt * bn + half * 128, tile_end = nt * bn + bn;
+      const int col0 = it.nt * bn + half * 128, tile_end = it.nt * bn + bn;
       if (ep.raw_out) {
-        if (row_ok) raw_store(ep, tot, row, col0, min(ep.raw_cols, tile_end), tile % ks, shift);
+        if (row_ok) raw_store(ep, tot, row, col0, min(ep.raw_cols, tile_end), it.piece, per > 0, shift);
       } else {
         const float rinv = row_ok ? ep.row_inv[row] : __int_as_float(0x7fc00000);
         epilogue_tile(ep, tot, row, row_base, row_ok, rinv, shift, col0, min(ep.P, tile_end), lane);
@@ -577,7 +596,7 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 template <int OPA>
 cudaError_t go2(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* bl, int64_t K,
                 const EpiParams& ep, int sm_count, int group_m, long long spin_ns, cudaStream_t st,
-                const DecodeArgs& da, int bn) {
+                const DecodeArgs& da, int bn, const PairUnits* pu) {
   static bool attr_set = false;
   if (!attr_set) {
     cudaError_t e = cudaFuncSetAttribute(k_tc2_scan<OPA>,
@@ -588,15 +607,14 @@ cudaError_t go2(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* 
   }
   const int n_mt = (ep.M + TBM - 1) / TBM;
   const int n_nt = (ep.P + bn - 1) / bn;
-  const int ks = ep.ksplit > 1 ? ep.ksplit : 1;
-  if (ks > 1 && !ep.raw_out) return cudaErrorInvalidValue;
-  const int tiles = ((n_mt + 1) / 2) * n_nt * ks;
-  const int pairs = tiles < sm_count / 2 ? tiles : sm_count / 2;
+  if (pu && !ep.raw_out) return cudaErrorInvalidValue;
+  const int tiles = ((n_mt + 1) / 2) * n_nt;
+  const int pairs = pu ? pu->pairs : tiles < sm_count / 2 ? tiles : sm_count / 2;
   const int group_p = group_m / 2 > 0 ? group_m / 2 : 1;
   if ((K / TBK) % Cfg2<OPA>::KS) return cudaErrorInvalidValue;
-  k_tc2_scan<OPA><<<2 * pairs, kThreads, Cfg2<OPA>::kSmem, st>>>(
-      *a, *bh, *bl, (int)(K / TBK), n_mt, n_nt, bn, group_p, spin_ns, ep, da);
-  return cudaGetLastError();
+  return launch_chained(k_tc2_scan<OPA>, dim3((unsigned)(2 * pairs)), kThreads, Cfg2<OPA>::kSmem, st,
+      *a, *bh, *bl, (int)(K / TBK), n_mt, n_nt, bn, group_p, pu ? pu->per : 0, pu ? pu->chunks : 1, spin_ns,
+      ep, da);
 }
 
 }  // namespace
@@ -604,17 +622,17 @@ cudaError_t go2(const CUtensorMap* a, const CUtensorMap* bh, const CUtensorMap* 
 cudaError_t launch_tc2_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
                             const CUtensorMap* tmBlo, int64_t K, const EpiParams& ep, int sm_count,
                             long long spin_ns, cudaStream_t st, int group_m, const DecodeArgs* dec,
-                            int encoding, int bn) {
+                            int encoding, int bn, const PairUnits* pu) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
   if (K % TBK || group_m < 1 || bn < 32 || bn > TBN || bn % 32) return cudaErrorInvalidValue;
   if (ep.raw_out && ep.P != ep.raw_cols) return cudaErrorInvalidValue;
   if (!dec)
     return go2<OPA_TMA>(tmA, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, DecodeArgs{},
-                        bn);
+                        bn, pu);
   if (dec->M != ep.M) return cudaErrorInvalidValue;
   if (encoding == TG_ENC_2BIT)
-    return go2<OPA_2BIT>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn);
-  return go2<OPA_U8>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn);
+    return go2<OPA_2BIT>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn, pu);
+  return go2<OPA_U8>(tmBhi, tmBhi, tmBlo, K, ep, sm_count, group_m, spin_ns, st, *dec, bn, pu);
 }
 
 }  // namespace tg

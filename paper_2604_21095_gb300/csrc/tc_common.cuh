@@ -284,17 +284,18 @@ __device__ __forceinline__ void split_range(int num_kb, int ks, int sp, int& lo,
   hi = min(num_kb, (sp + 1) * per * kChunkKB);
 }
 
-// Raw mode: the 128 totals of one thread (marker row `row`, columns col0..) of K range `split`.
+// Raw mode: the 128 totals of one thread (marker row `row`, columns col0..) as range `split`, as
+// partial sums (without the shift's add-back) where the tile has others.
 // Lane = row and one column per instruction, so a warp writes 128 contiguous bytes.
 __device__ __forceinline__ void raw_store(const EpiParams& ep, const float (&tot)[128],
                                           long long row, int col0, int col_end, int split,
-                                          float shift) {
+                                          bool partial, float shift) {
   float* out = ep.raw_out + (long long)split * ep.raw_split + row;
 #pragma unroll
   for (int e = 0; e < 128; ++e) {  // fully unrolled: tot stays in registers
     const int col = col0 + e;
     if (col < col_end)
-      out[col * ep.raw_ld] = ep.ksplit > 1 ? tot[e] : fmaf(shift, ep.col_cs[col], tot[e]);
+      out[col * ep.raw_ld] = partial ? tot[e] : fmaf(shift, ep.col_cs[col], tot[e]);
   }
 }
 
