@@ -166,6 +166,7 @@ inline int tune_bucket(int64_t M) {
 struct tg_panel {
   int device = 0;
   int64_t N = 0, P = 0, n_cov = 0, q = 0, df = 0, Npad = 0, Ppad = 0;
+  std::vector<void*> memory;    // the allocations that hold every buffer below but the FP4 form's
   int64_t NS = 0;               // samples the panel's phenotypes use (N unless a subset)
   uint32_t* samples = nullptr;  // [ceil(N/32)] bit mask of those samples (subset panels only)
   double* X = nullptr;        // [(1+n_cov)][N] design, reduced in place by the QR; its workspace
