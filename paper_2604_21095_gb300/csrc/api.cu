@@ -323,8 +323,9 @@ struct Plan {
   bool operand = false;     // the decoded operand is needed
 };
 
+// whole: no pass is split, so that the raw products take at most JCOLS columns of the block's rows.
 Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int encoding,
-               const uint32_t* missing, const tg_scan_opts& opts) {
+               const uint32_t* missing, const tg_scan_opts& opts, bool whole) {
   Plan r;
   r.split = opts.precision == TG_PREC_SPLIT_BF16;
   r.nq = opts.mode == TG_MODE_PAPER ? 0 : p->q - 1;
@@ -347,7 +348,7 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
   r.dec = r.split && missing == nullptr && (c->fuse_decode || r.fuse_joint);
   r.operand = !r.dec;
   if (r.fuse_joint || r.fuse_proj) {
-    r.fu = fused_units(M, p->Npad, c->sm_count);
+    r.fu = fused_units(M, p->Npad, c->sm_count, whole);
     // dosage rows: the f16 form (k_fused.cu) from one 128-marker tile per SM on; smaller blocks keep
     // the bf16 form, which is closer to the exact products. From one 256-marker tile per SM on
     // the pass takes the byte sums itself, so no counting pass reads the block, and centres
@@ -358,7 +359,8 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
   // P + q - 1 <= JCOLS: one pass over the operand gives the projection and the panel's products
   // (raw); the statistics follow the norms
   r.joint = r.split && r.nq > 0 && p->joint_cols > 0;
-  const int64_t chunks = (p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB;
+  // (one chunk: nothing to split)
+  const int64_t chunks = whole ? 1 : (p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB;
   const double ldr = (double)r.ldr;
   if (r.fuse_joint || r.fuse_proj) {
     r.ranges_proj = r.fu.pieces;
@@ -373,8 +375,8 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
     }
   }
   if (!r.split) {
-    if (r.nq > 0) r.ranges_proj = pick_fp32_proj_ranges(M, r.nq, p->Npad, c->sm_count);
-    if (p->P > 0) r.ranges_scan = pick_fp32_ranges(M, p->P, p->Npad, c->sm_count);
+    if (r.nq > 0 && !whole) r.ranges_proj = pick_fp32_proj_ranges(M, r.nq, p->Npad, c->sm_count);
+    if (p->P > 0 && !whole) r.ranges_scan = pick_fp32_ranges(M, p->P, p->Npad, c->sm_count);
     if (r.ranges_scan > 1)
       r.raw_floats = (size_t)r.ranges_scan * (size_t)p->P * (size_t)r.ldr;
   }
@@ -417,22 +419,31 @@ bool operand_fits(const tg_ctx* c, int64_t M, int64_t Npad, int prec) {
 tg_status reserve_graph_workspace(tg_ctx* c, const tg_panel* p, int n_blocks, const int64_t* M,
                                   int64_t maxM, bool need_operand, int encoding,
                                   const uint32_t* const* missing, const tg_scan_opts& opts) {
-  size_t raw = 0;
-  for (int b = 0; b < n_blocks; ++b)
-    raw = std::max(raw, make_plan(c, p, p->N, M[b], encoding, missing ? missing[b] : nullptr, opts)
-                            .raw_floats);
-  if (c->graphs_alive > 0) {
-    if (maxM > c->cap_m || raw > c->cap_raw ||
-        (need_operand && !operand_fits(c, maxM, p->Npad, opts.precision)))
+  if (c->graphs_alive > 0) {  // (the raw products fit: see plan_scan)
+    if (maxM > c->cap_m || (need_operand && !operand_fits(c, maxM, p->Npad, opts.precision)))
       return fail(TG_ERR_INVALID_ARG,
                   "another captured scan graph holds this context's workspace: capture the "
                   "largest blocks first, or use another context");
     return TG_OK;
   }
+  size_t raw = 0;
+  for (int b = 0; b < n_blocks; ++b)
+    raw = std::max(raw, make_plan(c, p, p->N, M[b], encoding, missing ? missing[b] : nullptr, opts,
+                                  false).raw_floats);
   TG_CUDA(ensure_markers(c, maxM));
   if (need_operand) TG_CUDA(ensure_operands(c, maxM, p->Npad, opts.precision));
-  TG_CUDA(ensure_raw(c, raw));
+  // while the graph lives nothing grows: room for any unsplit pass over as many markers
+  TG_CUDA(ensure_raw(c, std::max(raw, (size_t)c->cap_m * JCOLS)));
   return TG_OK;
+}
+
+// The plan of a scan. While a captured graph holds the workspace, a scan whose split passes need more
+// room for their partial sums than there is runs unsplit.
+Plan plan_scan(const tg_ctx* c, const tg_panel* p, const ScanArgs& a) {
+  Plan r = make_plan(c, p, a.N, a.M, a.encoding, a.missing, a.opts, false);
+  if (c->graphs_alive > 0 && r.raw_floats > c->cap_raw)
+    r = make_plan(c, p, a.N, a.M, a.encoding, a.missing, a.opts, true);
+  return r;
 }
 
 }  // namespace
@@ -622,7 +633,7 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   if (a.M == 0) return TG_OK;
   if (a.opts.precision == TG_PREC_FP4_PIECES) return scan_fp4(c, p, a, st);
   const int prec = a.opts.precision;
-  const Plan pl = make_plan(c, p, a.N, a.M, a.encoding, a.missing, a.opts);
+  const Plan pl = plan_scan(c, p, a);
   const bool split = pl.split, joint = pl.joint;
   const int64_t nq = pl.nq;
   if (c->graphs_alive > 0 &&
@@ -709,11 +720,11 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
       pp.ksplit = packed_pass ? 1 : pl.ranges_proj;
       if (pl.fuse_joint) {
         TG_CUDA(launch_joint_fused(f16 ? &p->tmQYhi16 : &p->tmQYhi, f16 ? &p->tmQYlo16 : &p->tmQYlo,
-                                   p->Npad, pp, c->sm_count, p->joint_bn, kSpinNs, st, dj,
+                                   p->Npad, pp, pl.fu, p->joint_bn, kSpinNs, st, dj,
                                    a.encoding, f16));
       } else if (pl.fuse_proj) {  // the projection alone, writing the operand as it goes
         TG_CUDA(launch_joint_fused(f16 ? &p->tmQhi16 : &p->tmQhi, f16 ? &p->tmQlo16 : &p->tmQlo,
-                                   p->Npad, pp, c->sm_count, p->proj_bn(), kSpinNs, st, dj,
+                                   p->Npad, pp, pl.fu, p->proj_bn(), kSpinNs, st, dj,
                                    a.encoding, f16));
       } else if (joint && p->joint_cols > 128) {  // more than one narrow tile: CTA pairs
         const int64_t tiles = (a.M + 2 * MT - 1) / (2 * MT) * (p->joint_cols / p->joint_bn);

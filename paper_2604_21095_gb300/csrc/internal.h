@@ -463,7 +463,7 @@ cudaError_t launch_tc_scan(const CUtensorMap* tmA, const CUtensorMap* tmBhi,
 // fused in (k_fused.cu): reads the packed rows through da.tmG, whose boxes must be kFusedRows
 // rows of 128 bytes with the 128-byte swizzle (dosage) or 32 bytes (2-bit calls); raw mode only, K
 // a multiple of 64, bn (a multiple of 16) the operand's box rows. Writes the raw products as
-// fused_units(M, K, sm_count).pieces partial sums per tile, without the shift's add-back.
+// fu.pieces partial sums per tile, without the shift's add-back.
 constexpr int kFusedRows = 256;
 // Its units (one tile x one accumulation chunk) and their even split over the CTAs: CTA w takes the
 // units [w per, (w + 1) per), so tile t is shared by the CTAs t chunks / per to
@@ -471,12 +471,14 @@ constexpr int kFusedRows = 256;
 struct FusedUnits {
   int chunks, units, per, grid, pieces;
 };
-inline FusedUnits fused_units(int64_t M, int64_t K, int sm_count) {
+// whole: whole tiles only, one piece each.
+inline FusedUnits fused_units(int64_t M, int64_t K, int sm_count, bool whole = false) {
   FusedUnits f;
   f.chunks = (int)((K / 32 + kAccumChunkKB - 1) / kAccumChunkKB);
   f.units = (int)((M + kFusedRows - 1) / kFusedRows) * f.chunks;
   const int ctas = f.units < sm_count ? f.units : sm_count;
   f.per = (f.units + ctas - 1) / ctas;
+  if (whole) f.per = (f.per + f.chunks - 1) / f.chunks * f.chunks;
   f.grid = (f.units + f.per - 1) / f.per;
   f.pieces = f.per % f.chunks == 0 ? 1 : (f.chunks + f.per - 2) / f.per + 1;
   return f;
@@ -485,7 +487,7 @@ inline FusedUnits fused_units(int64_t M, int64_t K, int sm_count) {
 // then map QYhi16 / QYlo16 and the products are scaled back by 2^-14); else, and for 2-bit calls,
 // into bf16 against the bf16 operand.
 cudaError_t launch_joint_fused(const CUtensorMap* tmBhi, const CUtensorMap* tmBlo, int64_t K,
-                               const EpiParams& ep, int sm_count, int bn, long long spin_ns,
+                               const EpiParams& ep, const FusedUnits& fu, int bn, long long spin_ns,
                                cudaStream_t st, const DecodeArgs& da, int encoding, bool f16);
 
 // The statistics of a block from its raw products (k_stats.cu): the same per-element epilogue as

@@ -632,7 +632,8 @@ __global__ void __launch_bounds__(kFThreads, 1)
 
 template <int OPA, int BR>
 cudaError_t go_fused(const CUtensorMap* bh, const CUtensorMap* bl, int64_t K, const EpiParams& ep,
-                     int sm_count, int bn, long long spin_ns, cudaStream_t st, const DecodeArgs& da) {
+                     const FusedUnits& fu, int bn, long long spin_ns, cudaStream_t st,
+                     const DecodeArgs& da) {
   using C = FCfg<OPA, BR>;
   static bool attr_set = false;  // per process and instantiation
   if (!attr_set) {
@@ -641,7 +642,6 @@ cudaError_t go_fused(const CUtensorMap* bh, const CUtensorMap* bl, int64_t K, co
     if (e != cudaSuccess) return e;
     attr_set = true;
   }
-  const FusedUnits fu = fused_units(ep.M, K, sm_count);
   return launch_chained(k_joint_fused<OPA, BR>, dim3(fu.grid), kFThreads, C::kSmem, st,
       *bh, *bl, (int)(K / TBK), fu.chunks, fu.per, fu.units, bn, spin_ns, ep, da);
 }
@@ -649,7 +649,7 @@ cudaError_t go_fused(const CUtensorMap* bh, const CUtensorMap* bl, int64_t K, co
 }  // namespace
 
 cudaError_t launch_joint_fused(const CUtensorMap* tmBhi, const CUtensorMap* tmBlo, int64_t K,
-                               const EpiParams& ep, int sm_count, int bn, long long spin_ns,
+                               const EpiParams& ep, const FusedUnits& fu, int bn, long long spin_ns,
                                cudaStream_t st, const DecodeArgs& da, int encoding, bool f16) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
   // raw mode only (the projection, alone or joint with a small panel), an even number of K
@@ -664,8 +664,8 @@ cudaError_t launch_joint_fused(const CUtensorMap* tmBhi, const CUtensorMap* tmBl
     return cudaErrorInvalidValue;
   const auto go = [&](auto form) {
     constexpr int F = decltype(form)::value;
-    return bn <= 64 ? go_fused<F, 64>(tmBhi, tmBlo, K, ep, sm_count, bn, spin_ns, st, da)
-                    : go_fused<F, 128>(tmBhi, tmBlo, K, ep, sm_count, bn, spin_ns, st, da);
+    return bn <= 64 ? go_fused<F, 64>(tmBhi, tmBlo, K, ep, fu, bn, spin_ns, st, da)
+                    : go_fused<F, 128>(tmBhi, tmBlo, K, ep, fu, bn, spin_ns, st, da);
   };
   if (encoding == TG_ENC_2BIT) return f16 ? cudaErrorInvalidValue : go(std::integral_constant<int, F_2BIT>());
   return f16 ? go(std::integral_constant<int, F_U8_F16>()) : go(std::integral_constant<int, F_U8_BF16>());
