@@ -162,8 +162,8 @@ __global__ void __launch_bounds__(kFullThreads, 4)
 // consecutive threads take consecutive phenotypes of a marker, so that the four outputs are
 // written in whole sectors too, and r makes no trip through memory.
 // CPW = 1 gives a thread one element of a FULL block: on a small one the p-value's chain is the
-// whole time (300 x 40 at df = 774: a warp per 32 x 32 elements took 215 us). CPW = 4 keeps
-// four loads per marker in flight once the block fills the SMs anyway.
+// whole time (300 x 40 at df = 774: a warp per 32 x 32 elements took 215 us). CPW = 4 (2 with four
+// markers per lane) keeps more loads in flight once the block fills the SMs anyway.
 constexpr int kRawWarps = 8;
 template <bool FULL, int CPW>
 __global__ void __launch_bounds__(kRawWarps * 32)
@@ -188,15 +188,6 @@ __global__ void __launch_bounds__(kRawWarps * 32)
     ranges[u] = c < cols ? raw_ranges(raw, row0, c0 + c) : 0;
     most = max(most, ranges[u]);
   }
-  for (int s = 0; s < most; ++s)
-#pragma unroll
-    for (int u = 0; u < CPW; ++u)
-#pragma unroll
-      for (int i = 0; i < R; ++i) {
-        const long long row = row0 + 32 * i + lane;
-        if (row < ep.M && s < ranges[u])
-          d[i][u] += raw.x[s * raw.split + (c0 + warp * CPW + u) * raw.ld + row];
-      }
   float rinv[R], shift[R];  // NaN past the block's rows: no test, no hit, no key
 #pragma unroll
   for (int i = 0; i < R; ++i) {
@@ -204,6 +195,28 @@ __global__ void __launch_bounds__(kRawWarps * 32)
     const bool in = row < ep.M;
     rinv[i] = in ? ep.row_inv[row] : __int_as_float(0x7fc00000);
     shift[i] = in && raw.partial && raw.cs ? raw.shift[row] : 0.0f;
+  }
+  // two ranges' loads in flight together (added in range order)
+  for (int s = 0; s < most; s += 2) {
+    float v[2][R][CPW];
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int u = 0; u < CPW; ++u)
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          const long long row = row0 + 32 * i + lane;
+          v[k][i][u] = row < ep.M && s + k < ranges[u]
+                           ? raw.x[(s + k) * raw.split + (c0 + warp * CPW + u) * raw.ld + row]
+                           : 0.0f;
+        }
+#pragma unroll
+    for (int k = 0; k < 2; ++k)
+#pragma unroll
+      for (int u = 0; u < CPW; ++u)
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+          if (s + k < ranges[u]) d[i][u] += v[k][i][u];
   }
 #pragma unroll
   for (int u = 0; u < CPW; ++u) {
@@ -327,7 +340,7 @@ cudaError_t launch_full_stats(const EpiParams& ep, cudaStream_t st) {
 cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream_t st) {
   if (ep.M == 0 || ep.P == 0) return cudaSuccess;
   const bool small = (long long)ep.M * ep.P < 152ll * 8192;
-  const int cw = kRawWarps * (small ? 1 : 4);
+  const int cw = kRawWarps * (small ? 1 : ep.do_full ? 4 : 2);
   const long long rows = ep.do_full ? 32 : 128;
   const dim3 grid((unsigned)((ep.M + rows - 1) / rows), (unsigned)((ep.P + cw - 1) / cw));
   constexpr int T = kRawWarps * 32;
@@ -335,7 +348,7 @@ cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream
     return small ? launch_chained(k_raw_stats<true, 1>, grid, T, 0, st, raw, ep)
                  : launch_chained(k_raw_stats<true, 4>, grid, T, 0, st, raw, ep);
   return small ? launch_chained(k_raw_stats<false, 1>, grid, T, 0, st, raw, ep)
-               : launch_chained(k_raw_stats<false, 4>, grid, T, 0, st, raw, ep);
+               : launch_chained(k_raw_stats<false, 2>, grid, T, 0, st, raw, ep);
 }
 
 cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* start, cudaStream_t st) {
