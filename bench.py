@@ -715,14 +715,16 @@ def _kernel_profile():
 
 def fused_joint(M: int, P: int, q: int, sm_count: int) -> bool:
     """Whether the library scans a block with the decode fused into the small panel's joint
-    projection pass (its documented default: projected form, no mask, P + q - 1 <= 128 and at
-    least one 128-marker tile per SM)."""
+    projection pass (projected form, no mask, P + q - 1 <= 128 and at least one 128-marker tile
+    per SM; smaller blocks whose operand would take 32 MB or more go that way too, and are counted
+    here as the decoded path, which moves more)."""
     return q > 1 and P + q - 1 <= 128 and (M + 127) // 128 >= sm_count
 
 
 def fused_projection(N: int, M: int, encoding: str, P: int, q: int, sm_count: int) -> bool:
-    """Whether the library runs a larger panel's projection as the pass over the packed rows
-    that also writes the block's operand (its default for P + q - 1 > 128 in the projected form,
+    """Whether a larger panel's projection can run as the pass over the packed rows that also
+    writes the block's operand (panels of 128 < P + q - 1 <= 512 take one joint pass over the
+    decoded operand instead, which the caller looks at first; P + q - 1 > 128, projected form,
     no mask, at least one 128-marker tile per SM; a panel with a 256-row joint operand,
     P + q - 1 <= 256, only where that pass also writes the marker statistics)."""
     return (q > 1 and P + q - 1 > 128 and (M + 127) // 128 >= sm_count and
@@ -845,9 +847,13 @@ def _scan_points(w, Ps, dev, reps_for, flush_bytes=0, prec="split"):
             continue
         sms = torch.cuda.get_device_properties(dev).multi_processor_count
         fz = fused_joint(M, P, q, sms)
-        fp = fused_projection(w.N, M, w.encoding, P, q, sms)
+        # 128 < P + q - 1 <= 512: one pass over the decoded operand gives projection and products
+        wide = q > 1 and 128 < P + q - 1 <= 512
+        fp = fused_projection(w.N, M, w.encoding, P, q, sms) and not wide
         op = (fz or fp) and one_pass_joint(w.N, M, w.encoding, sms)
         byts = _hbm_bytes_per_block(w.N, M, w.encoding, P, q, fz, op, fp)
+        if wide and P + q - 1 > 256:
+            byts -= 2 * M * ((w.N + 63) // 64 * 64)  # the operand is read once, not twice
         hbm_frac = byts / (ms / 1000.0) / 1e9 / float(peaks["hbm_gbs"])
         tflops = flops / (ms / 1000.0) / 1e12
         tens_frac = tflops / float(peaks["bf16_tflops"])
