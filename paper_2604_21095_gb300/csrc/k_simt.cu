@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
       const int r = e >> 3, c4 = (e & 7) * 4;
       const long long gm = m0 + r;
       float4 v = make_float4(0, 0, 0, 0);
-      if (gm < M) v = *reinterpret_cast<const float4*>(A + gm * lda + i0 + c4);
+      if (gm < M) v = __ldg(reinterpret_cast<const float4*>(A + gm * lda + i0 + c4));
       As[c4 + 0][r] = v.x;
       As[c4 + 1][r] = v.y;
       As[c4 + 2][r] = v.z;
@@ -56,7 +56,7 @@ __global__ void __launch_bounds__(256) k_project(const float* __restrict__ A, lo
     }
     if (tid < KC * 8) {  // Q tile: KC columns x 32 samples
       const int r = tid >> 3, c4 = (tid & 7) * 4;
-      const float4 v = *reinterpret_cast<const float4*>(QB + (long long)(k0 + r) * K + i0 + c4);
+      const float4 v = __ldg(reinterpret_cast<const float4*>(QB + (long long)(k0 + r) * K + i0 + c4));
       Qs[c4 + 0][r] = v.x;
       Qs[c4 + 1][r] = v.y;
       Qs[c4 + 2][r] = v.z;
@@ -321,10 +321,10 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
 #pragma unroll
     for (int b = 0; b < 4; ++b) acc2[a][b] = 0ull;
 
-  float4 ra0 = *reinterpret_cast<const float4*>(Ag0);
-  float4 ra1 = *reinterpret_cast<const float4*>(Ag1);
-  float4 rb0 = *reinterpret_cast<const float4*>(Bg0);
-  float4 rb1 = *reinterpret_cast<const float4*>(Bg1);
+  float4 ra0 = __ldg(reinterpret_cast<const float4*>(Ag0));
+  float4 ra1 = __ldg(reinterpret_cast<const float4*>(Ag1));
+  float4 rb0 = __ldg(reinterpret_cast<const float4*>(Bg0));
+  float4 rb1 = __ldg(reinterpret_cast<const float4*>(Bg1));
   int buf = 0;
   auto stash = [&](int bf) {
     As[bf][lk + 0][lr] = ra0.x; As[bf][lk + 1][lr] = ra0.y; As[bf][lk + 2][lr] = ra0.z; As[bf][lk + 3][lr] = ra0.w;
@@ -337,10 +337,10 @@ __global__ void __launch_bounds__(256, 2) k_sgemm_scan(const float* __restrict__
   for (int k0 = 0; k0 < K; k0 += BK) {
     const bool more = k0 + BK < K;
     if (more) {
-      ra0 = *reinterpret_cast<const float4*>(Ag0 + k0 + BK);
-      ra1 = *reinterpret_cast<const float4*>(Ag1 + k0 + BK);
-      rb0 = *reinterpret_cast<const float4*>(Bg0 + k0 + BK);
-      rb1 = *reinterpret_cast<const float4*>(Bg1 + k0 + BK);
+      ra0 = __ldg(reinterpret_cast<const float4*>(Ag0 + k0 + BK));
+      ra1 = __ldg(reinterpret_cast<const float4*>(Ag1 + k0 + BK));
+      rb0 = __ldg(reinterpret_cast<const float4*>(Bg0 + k0 + BK));
+      rb1 = __ldg(reinterpret_cast<const float4*>(Bg1 + k0 + BK));
     }
 #pragma unroll
     for (int k = 0; k < BK; ++k) {
@@ -439,11 +439,16 @@ cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, co
   const int64_t range = round_up((K + ranges - 1) / ranges, 256);
   const int kc = nq <= 16 ? 16 : 32, tm = 2048 / kc;
   const dim3 grid((unsigned)((M + tm - 1) / tm), (unsigned)((nq + kc - 1) / kc), (unsigned)ranges);
+  // ordinary launches, here and of k_sgemm_scan: several blocks fit an SM, and blocks placed while
+  // the kernel before still holds other SMs pile up on the free ones (120 blocks of k_sgemm_scan:
+  // 94 us chained, 43 not)
   if (kc == 16)
-    return launch_chained(k_project<16>, grid, 256, 0, st, A, lda, M, (int)K, (int)range, QB, (int)nq, out,
+    k_project<16><<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out,
                                         (long long)ldq, (long long)split);
-  return launch_chained(k_project<32>, grid, 256, 0, st, A, lda, M, (int)K, (int)range, QB, (int)nq, out,
+  else
+    k_project<32><<<grid, 256, 0, st>>>(A, lda, M, (int)K, (int)range, QB, (int)nq, out,
                                         (long long)ldq, (long long)split);
+  return cudaGetLastError();
 }
 
 cudaError_t launch_row_statistics(int64_t M, const RowSums& sums, const RawView& raw,
@@ -470,7 +475,8 @@ cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64
   const int64_t range = round_up((K + ks - 1) / ks, BK);
   if ((ks - 1) * range >= K) return cudaErrorInvalidValue;
   dim3 grid((unsigned)((ep.P + BN - 1) / BN), (unsigned)((ep.M + BM - 1) / BM), (unsigned)ks);
-  return launch_chained(k_sgemm_scan, grid, 256, 0, st, A, lda, B, ldb, (int)K, (int)range, ep);
+  k_sgemm_scan<<<grid, 256, 0, st>>>(A, lda, B, ldb, (int)K, (int)range, ep);
+  return cudaGetLastError();
 }
 
 }  // namespace tg
