@@ -167,13 +167,14 @@ __global__ void __launch_bounds__(kFullThreads, 4)
 constexpr int kRawWarps = 8;
 template <bool FULL, int CPW>
 __global__ void __launch_bounds__(kRawWarps * 32)
-    k_raw_stats(const RawView raw, const __grid_constant__ EpiParams ep) {
+    k_raw_stats(const RawView raw, const __grid_constant__ EpiParams ep, int cgroups) {
   constexpr int R = FULL ? 1 : 4, CW = kRawWarps * CPW;
   __shared__ float tile[FULL ? 32 : 1][CW + 1];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int c0 = (int)blockIdx.y * CW;
+  // one grid dimension (the second holds 65,535 blocks), the column groups of a row block in a row
+  const int c0 = (int)(blockIdx.x % (unsigned)cgroups) * CW;
   const int cols = min(CW, ep.P - c0);
-  const long long row0 = (long long)blockIdx.x * (32 * R);
+  const long long row0 = (long long)(blockIdx.x / (unsigned)cgroups) * (32 * R);
   chain_wait();
   float d[R][CPW];
 #pragma unroll
@@ -342,13 +343,16 @@ cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream
   const bool small = (long long)ep.M * ep.P < 152ll * 8192;
   const int cw = kRawWarps * (small ? 1 : ep.do_full ? 4 : 2);
   const long long rows = ep.do_full ? 32 : 128;
-  const dim3 grid((unsigned)((ep.M + rows - 1) / rows), (unsigned)((ep.P + cw - 1) / cw));
+  const int cgroups = (ep.P + cw - 1) / cw;
+  const long long blocks = ((long long)ep.M + rows - 1) / rows * cgroups;
+  if (blocks > INT32_MAX) return cudaErrorInvalidConfiguration;
+  const dim3 grid((unsigned)blocks);
   constexpr int T = kRawWarps * 32;
   if (ep.do_full)
-    return small ? launch_chained(k_raw_stats<true, 1>, grid, T, 0, st, raw, ep)
-                 : launch_chained(k_raw_stats<true, 4>, grid, T, 0, st, raw, ep);
-  return small ? launch_chained(k_raw_stats<false, 1>, grid, T, 0, st, raw, ep)
-               : launch_chained(k_raw_stats<false, 2>, grid, T, 0, st, raw, ep);
+    return small ? launch_chained(k_raw_stats<true, 1>, grid, T, 0, st, raw, ep, cgroups)
+                 : launch_chained(k_raw_stats<true, 4>, grid, T, 0, st, raw, ep, cgroups);
+  return small ? launch_chained(k_raw_stats<false, 1>, grid, T, 0, st, raw, ep, cgroups)
+               : launch_chained(k_raw_stats<false, 2>, grid, T, 0, st, raw, ep, cgroups);
 }
 
 cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* start, cudaStream_t st) {

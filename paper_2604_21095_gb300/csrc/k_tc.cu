@@ -27,9 +27,9 @@
 // tiles of blocks with at least one 256-marker tile per SM take 256 markers, as two 128-row
 // sub-tiles with their own accumulators sharing each B stage (half the B traffic from L2).
 // In raw mode (the covariate projection, alone or joint with a small panel whose phenotypes
-// follow the q - 1 projection columns in one B operand) the tile is the narrowest of 64, 128
-// and 256 columns that holds them, and the products are written unnormalised, column-major;
-// k_raw_stats turns a joint pass's panel columns into statistics once the marker norms exist.
+// follow the q - 1 projection columns in one B operand) the tile takes the operand's columns
+// rounded up to 16, and the products are written unnormalised, column-major; k_raw_stats turns a
+// joint pass's panel columns into statistics once the marker norms exist.
 // With split-K (ep.ksplit > 1, raw mode only, for blocks with fewer tiles than SMs) a work item
 // is a tile and a chunk-aligned range of the samples, and each range writes its own partial sums;
 // the kernels that read them add the ranges in order. (Handing the ranges to the tile's first
