@@ -28,6 +28,16 @@ __device__ __forceinline__ void chain_wait(T&... p) {
   (void)std::initializer_list<int>{([&] { asm volatile("" : "+l"(p)::"memory"); }(), 0)...};
 }
 
+// The cluster's barrier in two halves, by every thread of a converged warp. Shared memory of another
+// block of the cluster may be touched only once that block is known to have started, so a kernel
+// that does passes one of these first.
+__device__ __forceinline__ void cluster_arrive() {
+  asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void cluster_wait() {
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+
 // Sum over a whole thread block (any size multiple of 32, <= 1024); every thread gets it.
 __device__ __forceinline__ double block_sum(double v, double* red /* >= 33 doubles of smem */) {
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

@@ -268,7 +268,9 @@ __global__ void __launch_bounds__(kHitThreads)
     k_hit_stats(const __grid_constant__ EpiParams ep, const unsigned long long* __restrict__ start) {
   __shared__ double red[33];
   __shared__ double parts[2][kHitCluster];  // of the first block; two in turn
-  chain_wait(start);
+  cluster_arrive();  // the cluster's blocks have all started before any writes to the first one's
+  chain_wait(start);  // shared memory; the wait for the kernel before hides it
+  cluster_wait();
   const unsigned long long s0 = *start;
   unsigned long long s1 = *ep.n_hits;
   if (s1 > (unsigned long long)ep.hit_cap) s1 = (unsigned long long)ep.hit_cap;
@@ -291,8 +293,9 @@ __global__ void __launch_bounds__(kHitThreads)
     }
     // every block has read the record and delivered its part; the slot of two hits ago is free,
     // since its reader has arrived here too
-    asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::
-                     : "memory");
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
     if (rank == 0 && threadIdx.x == 0) {
       double sum = 0.0;
       for (unsigned k = 0; k < nrank; ++k) sum += parts[turn][k];
