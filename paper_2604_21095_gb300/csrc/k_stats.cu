@@ -258,16 +258,21 @@ __global__ void __launch_bounds__(kRawWarps * 32)
   }
 }
 
-// Hit records: a cluster of blocks per hit recomputes its product in FP64 and its first block writes
-// the FP64 statistics. A block of 80 hits or so is bound by the FP64 units (two lanes per cycle and
-// SM): with one thread block per hit half of the SMs had none (65,536 x 16 tests on 23,000 samples:
-// 33 us, 23 with 8 blocks). On short sample axes the last FP64 chain of one thread is the time
-// (17 us at 5,001 samples, 20 with 8 blocks): one block per hit up to kHitSplitN samples.
+// Hit records: the product of each is recomputed in FP64 and one thread writes its FP64 statistics.
+// Bound by the FP64 units (two lanes per cycle and SM), with few hits by one hit's chain: its
+// sum, then the 17 us of the statistics' own FP64 chain. Few hits leave most SMs idle, so on long
+// sample axes the kernel runs in clusters, and while there are at most as many hits as clusters a
+// whole cluster shares a hit, each block a part of the samples, added up by the first one (80
+// hits on 23,000 samples: 33 us with one block per hit, 23 with 8). With more hits every block
+// takes its own: a cluster's blocks would wait for each hit's chain in turn (65,536 x 100 tests on
+// 23,000 samples with 6,501 hits: 3,480 us for the scan, 1,730 when each block had its own). On
+// short sample axes the chain is the time (17 us at 5,001 samples, 20 with 8 blocks): one block
+// per hit up to kHitSplitN samples.
 constexpr int kHitThreads = 256, kHitCluster = 8, kHitSplitN = 8192;
 __global__ void __launch_bounds__(kHitThreads)
     k_hit_stats(const __grid_constant__ EpiParams ep, const unsigned long long* __restrict__ start) {
   __shared__ double red[33];
-  __shared__ double parts[2][kHitCluster];  // of the first block; two in turn
+  __shared__ double parts[kHitCluster];  // of the first block of a cluster that shares a hit
   cluster_arrive();  // the cluster's blocks have all started before any writes to the first one's
   chain_wait(start);  // shared memory; the wait for the kernel before hides it
   cluster_wait();
@@ -276,30 +281,33 @@ __global__ void __launch_bounds__(kHitThreads)
   if (s1 > (unsigned long long)ep.hit_cap) s1 = (unsigned long long)ep.hit_cap;
   unsigned nrank;  // blocks per cluster
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
-  const unsigned rank = blockIdx.x % nrank;
-  int turn = 0;
-  for (unsigned long long i = s0 + blockIdx.x / nrank; i < s1; i += gridDim.x / nrank) {
+  const bool share = nrank > 1 && s1 <= s0 + gridDim.x / nrank;  // the same for the whole grid
+  const unsigned team = share ? nrank : 1, rank = blockIdx.x % team;
+  for (unsigned long long i = s0 + blockIdx.x / team; i < s1; i += gridDim.x / team) {
     const tg_hit h = ep.hits[i];
     const long long row = (long long)h.marker - ep.marker_offset;
-    const double D = block_sum(exact_partial(ep.exact, row, (int)h.pheno,
-                                             (int)(rank * kHitThreads + threadIdx.x),
-                                             (int)(kHitThreads * nrank)), red);
-    if (threadIdx.x == 0) {
-      uint32_t dst;
-      asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
-                   : "=r"(dst)
-                   : "r"((uint32_t)__cvta_generic_to_shared(&parts[turn][rank])));
-      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(D) : "memory");
+    double D = block_sum(exact_partial(ep.exact, row, (int)h.pheno,
+                                       (int)(rank * kHitThreads + threadIdx.x),
+                                       (int)(kHitThreads * team)), red);
+    if (share) {  // at most one hit per cluster
+      if (threadIdx.x == 0) {
+        uint32_t dst;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
+                     : "=r"(dst)
+                     : "r"((uint32_t)__cvta_generic_to_shared(&parts[rank])));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(D) : "memory");
+      }
+      // every block has read the record and delivered its part
+      __syncwarp();
+      cluster_arrive();
+      cluster_wait();
+      if (rank == 0 && threadIdx.x == 0) {
+        D = 0.0;
+        for (unsigned k = 0; k < nrank; ++k) D += parts[k];
+      }
     }
-    // every block has read the record and delivered its part; the slot of two hits ago is free,
-    // since its reader has arrived here too
-    __syncwarp();
-    cluster_arrive();
-    cluster_wait();
     if (rank == 0 && threadIdx.x == 0) {
-      double sum = 0.0;
-      for (unsigned k = 0; k < nrank; ++k) sum += parts[turn][k];
-      const Stats64 v = stats_exact(ep, row, (int)h.pheno, sum);
+      const Stats64 v = stats_exact(ep, row, (int)h.pheno, D);
       tg_hit o = h;
       o.beta = v.beta;
       o.se = v.se;
@@ -307,7 +315,6 @@ __global__ void __launch_bounds__(kHitThreads)
       o.mlog10p = v.mlp;
       ep.hits[i] = o;
     }
-    turn ^= 1;
   }
   // (a block's shared memory stays while others may still write to it: the last write comes
   // before the last barrier above)

@@ -37,3 +37,30 @@ def test_hit_statistics_either_side_of_the_cluster_form(tgctx, encoding, N, M, t
     j, p = res["hits"]["marker"].astype(int) - 9, res["hits"]["pheno"].astype(int)
     np.testing.assert_allclose(res["hits"]["se"], ref["se"][j, p], rtol=1e-6)
     np.testing.assert_allclose(res["hits"]["t"], ref["t"][j, p], rtol=1e-6)
+
+
+def test_many_hits_do_not_take_turns(tgctx):
+    """Long sample axes share each of a few hits over a cluster of 8 blocks; with many hits every
+    block takes its own. Clusters that took 4,800 hits in turn would need more than 60 times as
+    long as for one hit each (76 clusters); blocks of their own need about a third of that."""
+    N, M, P = 16_001, 1200, 40
+    w = synth.Workload("hits_many", N=N, M=M, P=P, n_cov=3, encoding="2bit", missing=0.01, seed=71,
+                       block=M, causal_per_pheno=1)
+    pan = synth.make_panel(w)
+    G = synth.make_block(w, 0)["G"].cuda()
+    panel = tg.tg_prepare_panel(tgctx, pan["Yt"].cuda(), N, P, pan["cov_t"].cuda())
+    ms, hits = {}, {}
+    try:
+        tg.tg_set_profiling(tgctx, True)
+        for thr in (4.0, 1.0):
+            ms[thr] = 1e9
+            for _ in range(6):
+                tg.tg_stage_times(tgctx, reset=True)
+                hits[thr] = run_scan(tgctx, panel, G, N, P, "2bit", "split", full=False,
+                                     hit_mlog10p=thr)["n_hits"]
+                ms[thr] = min(ms[thr], tg.tg_stage_times(tgctx, reset=True)["stats"][0])
+    finally:
+        tg.tg_set_profiling(tgctx, False)
+        tg.tg_panel_free(panel)
+    assert 0 < hits[4.0] <= 76 and hits[1.0] > 3000, hits
+    assert ms[1.0] < 0.7 * (hits[1.0] / 76.0) * ms[4.0], (ms, hits)
