@@ -142,7 +142,7 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
   const size_t elem = prec == TG_PREC_FP32 ? 4 : 2;
   Carver probe{nullptr};
   probe.take<uint32_t>(4);
-  probe.take<unsigned long long>(1);
+  probe.take<unsigned long long>(2);
   probe.take<float>((size_t)rows);
   probe.take<int32_t>((size_t)rows);
   probe.take<double>((size_t)rows);
@@ -171,7 +171,7 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
 
   Carver cv{ds->base};
   uint32_t* status = cv.take<uint32_t>(4);  // [0] status word
-  unsigned long long* hit_start = cv.take<unsigned long long>(1);
+  unsigned long long* hit_start = cv.take<unsigned long long>(2);
   float* shift = cv.take<float>((size_t)rows);
   int32_t* nobs = cv.take<int32_t>((size_t)rows);
   double* mean = cv.take<double>((size_t)rows);

@@ -426,7 +426,7 @@ struct MarkerRefine {
 };
 // Outputs of the norm kernel: 1/|g_res| of each marker (NaN = untestable) and, where not NULL,
 // |g_res|^2 in allele units, copies of n_obs and of the mean for the caller, and
-// the hit counter's value before this block (hit_start = *n_hits).
+// the hit counter's value before this block (hit_start[0] = *n_hits, hit_start[1] = 0).
 struct NormOut {
   double* norm2_allele;
   float* rinv;
@@ -446,7 +446,8 @@ cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64
 
 // statistics after the contraction (k_stats.cu)
 cudaError_t launch_full_stats(const EpiParams& ep, cudaStream_t st);
-cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* start, cudaStream_t st);
+// start: [0] the hit count before the block, [1] a counter, as k_marker_norm leaves them (NormOut).
+cudaError_t launch_hit_stats(const EpiParams& ep, unsigned long long* start, cudaStream_t st);
 cudaError_t launch_fill_random(uint8_t* p, size_t n, unsigned long long seed, cudaStream_t st);
 
 // tensor-core kernel (k_tc.cu)

@@ -260,7 +260,10 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
     const unsigned f = __ballot_sync(0xffffffffu, close);
     if (lane == 0) {
       flagged = f;
-      if (out.hit_start && blockIdx.x == 0) *out.hit_start = *out.n_hits;
+      if (out.hit_start && blockIdx.x == 0) {
+        out.hit_start[0] = *out.n_hits;
+        out.hit_start[1] = 0ull;
+      }
     }
   } else if (warp == 1 && in) {
     if (out.nobs) out.nobs[j] = nobs[j];

@@ -265,59 +265,74 @@ __global__ void __launch_bounds__(kRawWarps * 32)
 // whole cluster shares a hit, each block a part of the samples, added up by the first one (80
 // hits on 23,000 samples: 33 us with one block per hit, 23 with 8). With more hits every block
 // takes its own: a cluster's blocks would wait for each hit's chain in turn (65,536 x 100 tests on
-// 23,000 samples with 6,501 hits: 3,480 us for the scan, 1,730 when each block had its own). On
-// short sample axes the chain is the time (17 us at 5,001 samples, 20 with 8 blocks): one block
-// per hit up to kHitSplitN samples.
+// 23,000 samples with 6,501 hits: the scan took 3,480 us, now 1,305; with 65,319 hits 30.0 ms, now
+// 7.7). On short sample axes the chain is the time (17 us at 5,001 samples, 20 with 8 blocks): one
+// block per hit up to kHitSplitN samples.
 constexpr int kHitThreads = 256, kHitCluster = 8, kHitSplitN = 8192;
 __global__ void __launch_bounds__(kHitThreads)
-    k_hit_stats(const __grid_constant__ EpiParams ep, const unsigned long long* __restrict__ start) {
+    k_hit_stats(const __grid_constant__ EpiParams ep, unsigned long long* start) {
   __shared__ double red[33];
   __shared__ double parts[kHitCluster];  // of the first block of a cluster that shares a hit
+  __shared__ unsigned long long next[2];
   cluster_arrive();  // the cluster's blocks have all started before any writes to the first one's
-  chain_wait(start);  // shared memory; the wait for the kernel before hides it
+  chain_wait();      // shared memory; the wait for the kernel before hides it
   cluster_wait();
-  const unsigned long long s0 = *start;
+  const int tid = (int)threadIdx.x;
+  const unsigned long long s0 = start[0];
   unsigned long long s1 = *ep.n_hits;
   if (s1 > (unsigned long long)ep.hit_cap) s1 = (unsigned long long)ep.hit_cap;
+  const auto write = [&](unsigned long long i, const tg_hit& h, double D) {
+    const Stats64 v = stats_exact(ep, (long long)h.marker - ep.marker_offset, (int)h.pheno, D);
+    tg_hit o = h;
+    o.beta = v.beta;
+    o.se = v.se;
+    o.t = v.t;
+    o.mlog10p = v.mlp;
+    ep.hits[i] = o;
+  };
   unsigned nrank;  // blocks per cluster
   asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(nrank));
-  const bool share = nrank > 1 && s1 <= s0 + gridDim.x / nrank;  // the same for the whole grid
-  const unsigned team = share ? nrank : 1, rank = blockIdx.x % team;
-  for (unsigned long long i = s0 + blockIdx.x / team; i < s1; i += gridDim.x / team) {
+  if (nrank > 1 && s1 <= s0 + gridDim.x / nrank) {  // the same for the whole grid
+    const unsigned rank = blockIdx.x % nrank;
+    const unsigned long long i = s0 + blockIdx.x / nrank;
+    if (i >= s1) return;
     const tg_hit h = ep.hits[i];
-    const long long row = (long long)h.marker - ep.marker_offset;
-    double D = block_sum(exact_partial(ep.exact, row, (int)h.pheno,
-                                       (int)(rank * kHitThreads + threadIdx.x),
-                                       (int)(kHitThreads * team)), red);
-    if (share) {  // at most one hit per cluster
-      if (threadIdx.x == 0) {
-        uint32_t dst;
-        asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
-                     : "=r"(dst)
-                     : "r"((uint32_t)__cvta_generic_to_shared(&parts[rank])));
-        asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(D) : "memory");
-      }
-      // every block has read the record and delivered its part
-      __syncwarp();
-      cluster_arrive();
-      cluster_wait();
-      if (rank == 0 && threadIdx.x == 0) {
-        D = 0.0;
-        for (unsigned k = 0; k < nrank; ++k) D += parts[k];
-      }
+    double D = block_sum(exact_partial(ep.exact, (long long)h.marker - ep.marker_offset,
+                                       (int)h.pheno, (int)(rank * kHitThreads) + tid,
+                                       (int)(kHitThreads * nrank)), red);
+    if (tid == 0) {
+      uint32_t dst;
+      asm volatile("mapa.shared::cluster.u32 %0, %1, 0;"
+                   : "=r"(dst)
+                   : "r"((uint32_t)__cvta_generic_to_shared(&parts[rank])));
+      asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(dst), "d"(D) : "memory");
     }
-    if (rank == 0 && threadIdx.x == 0) {
-      const Stats64 v = stats_exact(ep, row, (int)h.pheno, D);
-      tg_hit o = h;
-      o.beta = v.beta;
-      o.se = v.se;
-      o.t = v.t;
-      o.mlog10p = v.mlp;
-      ep.hits[i] = o;
+    // every block has read the record and delivered its part; the first one stays to read them
+    __syncwarp();
+    cluster_arrive();
+    cluster_wait();
+    if (rank == 0 && tid == 0) {
+      D = 0.0;
+      for (unsigned k = 0; k < nrank; ++k) D += parts[k];
+      write(i, h, D);
     }
+    return;
   }
-  // (a block's shared memory stays while others may still write to it: the last write comes
-  // before the last barrier above)
+  // Each block starts with a hit of its own; further ones come from a counter (cleared before), one
+  // ahead: a block that starts late, the grid being more than fits at once, finds less left instead
+  // of a fixed share (65,319 hits: 7.7 ms against 10.7).
+  const bool more = s1 > s0 + gridDim.x;  // the same for the whole grid
+  unsigned long long i = s0 + blockIdx.x;
+  for (int turn = 0; i < s1; turn ^= 1) {
+    const tg_hit h = ep.hits[i];
+    if (more && tid == 0) next[turn] = s0 + gridDim.x + atomicAdd(start + 1, 1ull);
+    const double D = block_sum(exact_partial(ep.exact, (long long)h.marker - ep.marker_offset,
+                                             (int)h.pheno, tid, kHitThreads), red);
+    // (the slot is written again only past another block_sum)
+    const unsigned long long after = more ? next[turn] : s1;
+    if (tid == 0) write(i, h, D);
+    i = after;
+  }
 }
 
 // Deterministic pseudo-random bytes (SplitMix64 of the index); used for timing trial blocks.
@@ -365,7 +380,7 @@ cudaError_t launch_raw_stats(const RawView& raw, const EpiParams& ep, cudaStream
                : launch_chained(k_raw_stats<false, 2>, grid, T, 0, st, raw, ep, cgroups);
 }
 
-cudaError_t launch_hit_stats(const EpiParams& ep, const unsigned long long* start, cudaStream_t st) {
+cudaError_t launch_hit_stats(const EpiParams& ep, unsigned long long* start, cudaStream_t st) {
   if (ep.exact.G == nullptr) return cudaErrorInvalidValue;  // hits are always recomputed in FP64
   const unsigned nrank = ep.exact.N > kHitSplitN ? kHitCluster : 1;
   cudaLaunchConfig_t cfg{};
