@@ -165,13 +165,14 @@ cudaError_t ensure_markers(tg_ctx* c, int64_t M) {
   if (M <= c->cap_m) return cudaSuccess;
   const int64_t cap = round_up(M, MT);
   dfree(c->nobs); dfree(c->mean); dfree(c->shift); dfree(c->mh); dfree(c->gc2s); dfree(c->gc2);
-  dfree(c->rinv); dfree(c->rinv64); dfree(c->S); dfree(c->S2);
+  dfree(c->rinv); dfree(c->rinv64); dfree(c->S); dfree(c->S2); dfree(c->close);
   c->cap_m = 0;
   cudaError_t e;
   if ((e = dalloc(&c->nobs, cap)) || (e = dalloc(&c->mean, cap)) || (e = dalloc(&c->shift, cap)) ||
       (e = dalloc(&c->mh, cap)) || (e = dalloc(&c->gc2s, cap)) ||
       (e = dalloc(&c->gc2, cap)) || (e = dalloc(&c->S, cap)) || (e = dalloc(&c->S2, cap)) ||
-      (e = dalloc(&c->rinv, cap)) || (e = dalloc(&c->rinv64, cap)))
+      (e = dalloc(&c->rinv, cap)) || (e = dalloc(&c->rinv64, cap)) ||
+      (e = dalloc(&c->close, cap / 32)))
     return e;
   c->cap_m = cap;
   return cudaSuccess;
@@ -578,10 +579,10 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
   unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
   const bool want_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
   {
-    StageScope s(c, STAGE_NORM, st, 1);
+    StageScope s(c, STAGE_NORM, st, nq > 0 ? 2 : 1);
     const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, nullptr, 0, c->mean, p->Q, (int)p->q};
     const NormOut no{a.out.marker_norm2, c->rinv, c->rinv64, a.out.marker_nobs, a.out.marker_mean,
-                     want_hits ? hit_start : nullptr, a.out.n_hits};
+                     want_hits ? hit_start : nullptr, a.out.n_hits, c->close};
     TG_CUDA(launch_marker_norm(a.M, c->nobs, c->gc2, RawView{c->raw, ldr, 0, 1},
                                nq, 1.0, rf, no, st, a.N));
   }
@@ -757,10 +758,10 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   unsigned long long* hit_start = reinterpret_cast<unsigned long long*>(c->scratch + 16);
   const bool want_hits = a.opts.hit_mlog10p > 0.0 && a.out.n_hits != nullptr;
   {
-    StageScope s(c, STAGE_NORM, st, 1);
+    StageScope s(c, STAGE_NORM, st, nq > 0 ? 2 : 1);
     const MarkerRefine rf{a.G, a.ldg, a.encoding, a.N, a.missing, a.ldm, c->mean, p->Q, (int)p->q};
     const NormOut no{a.out.marker_norm2, c->rinv, c->rinv64, a.out.marker_nobs, a.out.marker_mean,
-                     want_hits ? hit_start : nullptr, a.out.n_hits};
+                     want_hits ? hit_start : nullptr, a.out.n_hits, c->close};
     TG_CUDA(launch_marker_norm(a.M, c->nobs, p->samples ? c->gc2s : c->gc2, raw, nq, kappa64, rf,
                                no, st, 0, sums));
   }
@@ -984,7 +985,7 @@ tg_status tg_destroy(tg_ctx* c) {
   dfree(c->status); dfree(c->scratch);
   dfree(c->Ahi); dfree(c->A32); dfree(c->Afp4); dfree(c->shift); dfree(c->mh); dfree(c->gc2s);
   dfree(c->nobs); dfree(c->mean); dfree(c->gc2); dfree(c->raw);
-  dfree(c->rinv); dfree(c->rinv64); dfree(c->S); dfree(c->S2);
+  dfree(c->rinv); dfree(c->rinv64); dfree(c->S); dfree(c->S2); dfree(c->close);
   dfree(c->stage);
   dfree(c->dhits); dfree(c->dnhits); dfree(c->dbest);
   for (auto& ev : c->pending) { cudaEventDestroy(ev.a); cudaEventDestroy(ev.b); }

@@ -180,7 +180,7 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
   cv.take<double>((size_t)rows);  // (unused: the largest accepted block stays what it was)
   float* rinv = cv.take<float>((size_t)rows);
   double* rinv64 = cv.take<double>((size_t)rows);
-  cv.take<int>((size_t)rows);  // (unused)
+  uint32_t* close = cv.take<uint32_t>((size_t)rows);  // (a bit per marker; the rest unused)
   void* Ahi = cv.take<unsigned char>((size_t)rows * p->Npad * elem);
 
   cudaStream_t st = (cudaStream_t)stream;
@@ -223,7 +223,7 @@ extern "C" tg_status tg_scan_block_static(const tg_panel* p, const uint8_t* G, i
   }
   const MarkerRefine rf{G, ldg, encoding, N, missing, ldm, mean, p->Q, (int)p->q};
   const NormOut no{out->marker_norm2, rinv, rinv64, out->marker_nobs, out->marker_mean,
-                   want_hits ? hit_start : nullptr, out->n_hits};
+                   want_hits ? hit_start : nullptr, out->n_hits, close};
   TGS_CUDA(launch_marker_norm(M, nobs, gc2, RawView{qg, rows, 0, 1}, nq, kappa64,
                               rf, no, st));
   EpiParams ep{};

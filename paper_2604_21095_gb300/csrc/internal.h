@@ -253,6 +253,7 @@ struct tg_ctx {
   size_t cap_raw = 0;                           // its floats
   float* rinv = nullptr;
   double* rinv64 = nullptr;
+  uint32_t* close = nullptr;                    // bit per marker: close to the covariate span
   // host-streamed scan: a device ring of host_bufs block buffers' bytes (stage_cap allocated)
   uint8_t* stage = nullptr;
   size_t stage_cap = 0;
@@ -435,6 +436,7 @@ struct NormOut {
   double* mean;
   unsigned long long* hit_start;
   const unsigned long long* n_hits;
+  uint32_t* close;  // [ceil(M/32)] bit per marker: re-projected in FP64 (nq > 0)
 };
 // complete_n > 0: markers with fewer than complete_n observed calls are untestable too.
 cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2,

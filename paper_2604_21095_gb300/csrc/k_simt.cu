@@ -119,47 +119,97 @@ __device__ __forceinline__ bool marker_testable(int n_obs, double c2, double r2,
 
 // One block of 8 warps per 32 markers (lane = marker): the warps share the projection columns
 // (coalesced reads, the columns being contiguous in the markers), then warp 0 forms the norms
-// and warp 1 copies the caller's n_obs and mean. A block that lists a marker close to the
-// covariate span re-projects it in FP64 itself, all 256 threads on one marker at a time, so that
-// the usual block without any costs no second launch (nor a counter to clear and a list).
-// Bound by latency: 12.8 us as three operations on 65,536 markers and 19 columns, with
-// row-major products (a sector per value).
+// and warp 1 copies the caller's n_obs and mean. Bound by latency: 12.8 us as three operations on
+// 65,536 markers and 19 columns, with row-major products (a sector per value).
 constexpr int kNormWarps = 8;
+
+// Markers close to the covariate span (bits of `close`, left by k_marker_norm) are re-projected in
+// FP64 by a kernel of their own, marker m by block m % gridDim.x: such markers are neighbours in
+// practice (those in linkage with one that is among the covariates), and one costs (q - 1) N
+// multiply-adds on units that run two lanes per cycle and SM, so neighbours go to different SMs.
+// 65,536 x 16 dosage tests on 23,000 samples with 19 covariates take 424 us, with 32 such markers
+// side by side 752 (8,100 when the block of 32 that found them took them one after another). A scan
+// without any pays 1.1 to 1.8 us for this launch.
+constexpr int kRefineBlocks = 304, kRefineThreads = 256, kRefineCols = 8;
 
 // sum_k (q_k . g_c)^2 over the non-intercept columns of Q in FP64, from the packed genotypes
 // (missing calls at the marker's mean, which is also its centre, so they add nothing) and the
 // FP64 mean. q_0 . g_c = 0 exactly (q_0 is constant and g_c has zero sum), as in the tensor-core
-// projection, which leaves column 0 out. Whole block; thread 0 returns the sum.
-__device__ __noinline__ double refine_projection(const MarkerRefine& rf, long long j, double* red) {
+// projection, which leaves column 0 out. Eight columns at a time share each sample's value. Whole
+// block; thread 0 returns the sum.
+__device__ double refine_projection(const MarkerRefine& rf, long long j,
+                                    double (*red)[kRefineCols]) {
   const double mu = rf.mean[j];
   const uint8_t* row = rf.G + j * rf.ldg;
   const uint32_t* mrow = rf.missing ? rf.missing + j * rf.ldm : nullptr;
+  const double c00 = 2.0 - mu, c10 = 1.0 - mu, c11 = -mu;  // 2-bit fields 00, 10, 11; 01 is missing
   double s = 0.0;
-  for (int k = 1; k < rf.q; ++k) {
-    const double* qk = rf.Q + (long long)k * rf.N;
-    double acc = 0.0;
-    for (long long i = threadIdx.x; i < rf.N; i += blockDim.x) {
+  for (int k0 = 1; k0 < rf.q; k0 += kRefineCols) {
+    double acc[kRefineCols] = {};
+#pragma unroll 2
+    for (long long i = threadIdx.x; i < rf.N; i += kRefineThreads) {
       double v;
       if (rf.encoding == TG_ENC_2BIT) {
-        const unsigned f = (row[i >> 2] >> (2 * (i & 3))) & 3u;  // 00 = 2, 10 = 1, 11 = 0, 01 missing
-        v = f == 0u ? 2.0 : f == 2u ? 1.0 : f == 3u ? 0.0 : mu;
+        const unsigned f = (row[i >> 2] >> (2 * (i & 3))) & 3u;
+        v = f == 0u ? c00 : f == 2u ? c10 : f == 3u ? c11 : 0.0;
       } else {
         const bool miss = mrow && ((mrow[i >> 5] >> (i & 31)) & 1u);
-        v = miss ? mu : (double)row[i];
+        v = miss ? 0.0 : (double)row[i] - mu;
       }
-      acc = fma(qk[i], v - mu, acc);
+#pragma unroll
+      for (int u = 0; u < kRefineCols; ++u)
+        if (k0 + u < rf.q) acc[u] = fma(rf.Q[(long long)(k0 + u) * rf.N + i], v, acc[u]);
     }
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+#pragma unroll
+    for (int u = 0; u < kRefineCols; ++u) {
+      for (int o = 16; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+      if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5][u] = acc[u];
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < kNormWarps; ++w) t += red[w];
-      s += t * t;
-    }
+    if (threadIdx.x == 0)
+      for (int u = 0; u < kRefineCols && k0 + u < rf.q; ++u) {
+        double t = 0.0;
+        for (int w = 0; w < kRefineThreads / 32; ++w) t += red[w][u];
+        s += t * t;
+      }
     __syncthreads();
   }
   return s;
+}
+
+// The norms of a marker from |g_c|^2 and |g_res|^2 (decode units).
+__device__ __forceinline__ void put_norms(const NormOut& out, long long m, int n_obs, double c2,
+                                          double r2, int complete_n, double kappa) {
+  const bool ok = marker_testable(n_obs, c2, r2, complete_n);
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  const double inv = ok ? 1.0 / sqrt(r2) : nan;
+  if (out.norm2_allele) out.norm2_allele[m] = ok ? r2 * kappa * kappa : nan;
+  out.rinv[m] = (float)inv;
+  out.rinv64[m] = inv;
+}
+
+__global__ void __launch_bounds__(kRefineThreads) k_marker_refine(
+    long long M, const int32_t* nobs, const double* gc2, double kappa,
+    const __grid_constant__ MarkerRefine rf, const __grid_constant__ NormOut out, int complete_n) {
+  __shared__ double red[kRefineThreads / 32][kRefineCols];
+  __shared__ unsigned todo[kRefineThreads / 32];
+  const int tid = (int)threadIdx.x;
+  const long long step = gridDim.x;
+  chain_wait();
+  for (long long m0 = blockIdx.x; m0 < M; m0 += kRefineThreads * step) {
+    const long long j = m0 + tid * step;
+    const bool close = j < M && ((out.close[j >> 5] >> (j & 31)) & 1u);
+    const unsigned f = __ballot_sync(0xffffffffu, close);
+    if ((tid & 31) == 0) todo[tid >> 5] = f;
+    if (!__syncthreads_or(close)) continue;
+    for (int w = 0; w < kRefineThreads / 32; ++w)  // the same for the whole block
+      for (unsigned t = todo[w]; t; t &= t - 1) {
+        const long long m = m0 + (32 * w + __ffs(t) - 1) * step;
+        const double p = refine_projection(rf, m, red);
+        if (tid == 0) put_norms(out, m, nobs[m], gc2[m], gc2[m] - p, complete_n, kappa);
+      }
+    __syncthreads();
+  }
 }
 
 // A row's statistics from its exact integer sums: mean = S / n, |g_c|^2 = (n S2 - S^2) / n (the
@@ -197,7 +247,6 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
     int nq, double kappa, const __grid_constant__ MarkerRefine rf, NormOut out, int complete_n,
     RowSums sums) {
   __shared__ double part[kNormWarps][32];
-  __shared__ unsigned flagged;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long m0 = blockIdx.x * 32ll, j = m0 + lane;
   const bool in = j < M;
@@ -227,14 +276,6 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
     }
   part[warp][lane] = proj.sum64 ? s64 : __hiloint2double(__float_as_int(hi), __float_as_int(lo));
   __syncthreads();  // (and the block's writes of the row statistics are visible to the block)
-  auto put = [&](long long m, double c2, double r2) {
-    const bool ok = marker_testable(nobs[m], c2, r2, complete_n);
-    const double nan = __longlong_as_double(0x7ff8000000000000ll);
-    const double inv = ok ? 1.0 / sqrt(r2) : nan;
-    if (out.norm2_allele) out.norm2_allele[m] = ok ? r2 * kappa * kappa : nan;
-    out.rinv[m] = (float)inv;
-    out.rinv64[m] = inv;
-  };
   if (warp == 0) {
     bool close = false;
     if (in) {
@@ -254,12 +295,12 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
         t = (double)h + (double)l;
       }
       const double c2 = gc2[j], r2 = c2 - t;
-      put(j, c2, r2);
+      put_norms(out, j, nobs[j], c2, r2, complete_n, kappa);
       close = nq > 0 && nobs[j] > 0 && c2 > 0.0 && r2 < (1.0 - kRefineShare) * c2;
     }
     const unsigned f = __ballot_sync(0xffffffffu, close);
     if (lane == 0) {
-      flagged = f;
+      if (out.close) out.close[blockIdx.x] = f;
       if (out.hit_start && blockIdx.x == 0) {
         out.hit_start[0] = *out.n_hits;
         out.hit_start[1] = 0ull;
@@ -268,12 +309,6 @@ __global__ void __launch_bounds__(kNormWarps * 32) k_marker_norm(
   } else if (warp == 1 && in) {
     if (out.nobs) out.nobs[j] = nobs[j];
     if (out.mean) out.mean[j] = rf.mean[j];
-  }
-  __syncthreads();
-  for (unsigned todo = flagged; todo; todo &= todo - 1) {  // the same for the whole block
-    const long long m = m0 + __ffs(todo) - 1;
-    const double t = refine_projection(rf, m, part[0]);
-    if (threadIdx.x == 0) put(m, gc2[m], gc2[m] - t);
   }
 }
 
@@ -465,8 +500,15 @@ cudaError_t launch_marker_norm(int64_t M, const int32_t* nobs, const double* gc2
                                const MarkerRefine& refine, const NormOut& out, cudaStream_t st,
                                int64_t complete_n, const RowSums& sums) {
   if (M == 0) return cudaSuccess;
-  return launch_chained(k_marker_norm, dim3((unsigned)((M + 31) / 32)), kNormWarps * 32, 0, st,
-      M, nobs, gc2, proj, (int)nq, kappa, refine, out, (int)complete_n, sums);
+  NormOut no = out;
+  if (nq == 0) no.close = nullptr;  // nothing to re-project
+  cudaError_t e = launch_chained(k_marker_norm, dim3((unsigned)((M + 31) / 32)), kNormWarps * 32, 0,
+                                 st, M, nobs, gc2, proj, (int)nq, kappa, refine, no,
+                                 (int)complete_n, sums);
+  if (e != cudaSuccess || nq == 0) return e;
+  if (!out.close) return cudaErrorInvalidValue;
+  return launch_chained(k_marker_refine, dim3((unsigned)(M < kRefineBlocks ? M : kRefineBlocks)),
+                        kRefineThreads, 0, st, M, nobs, gc2, kappa, refine, no, (int)complete_n);
 }
 
 cudaError_t launch_sgemm_scan(const float* A, int64_t lda, const float* B, int64_t ldb, int64_t K,
