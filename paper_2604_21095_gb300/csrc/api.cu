@@ -539,12 +539,13 @@ tg_status ensure_fp4_panel(tg_ctx* c, tg_panel* p, cudaStream_t st) {
 tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
   const tg_status ps = ensure_fp4_panel(c, p, st);
   if (ps != TG_OK) return ps;
-  TG_CUDA(ensure_markers(c, a.M));
   const int64_t lda = p->Npad / 2, ldr = round_up(a.M, 32);
   const size_t raw = (size_t)(QCOLS * ldr);
   const int64_t need = round_up(a.M, MT) * lda;
-  if (c->graphs_alive > 0 && (need > c->cap_fp4 || raw > c->cap_raw))
+  // (before anything grows: a captured graph holds pointers into the buffers)
+  if (c->graphs_alive > 0 && (a.M > c->cap_m || need > c->cap_fp4 || raw > c->cap_raw))
     return fail(TG_ERR_INVALID_ARG, "the context's workspace is held by a captured scan graph");
+  TG_CUDA(ensure_markers(c, a.M));
   TG_CUDA(ensure_raw(c, raw));
   if (need > c->cap_fp4) {
     dfree(c->Afp4);
