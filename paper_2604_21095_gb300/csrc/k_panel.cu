@@ -293,7 +293,7 @@ __device__ __forceinline__ float add_err(float& x, float y) {
   return e;
 }
 
-// Two phenotype columns per block, which share each load of Q.
+// Two phenotype columns per block (kResT), which share each load of Q, or one.
 //
 // FP64 arithmetic bounds it: GB300 runs 2 FP64 lanes per cycle and SM, so each FP64 instruction
 // per sample and phenotype costs about 0.08 ms at N = 23,000, P = 2,048, q = 20, where the 40
@@ -302,7 +302,13 @@ __device__ __forceinline__ float add_err(float& x, float y) {
 // eight), the centred norm comes from |y_res|^2 + |Q^T y_c|^2, and the bf16 pair and its column
 // sum are formed in FP32 from u = f + g, two floats that hold 48 bits of u (the pair is that of
 // the FP64 value, see bf16_bits_of_sum; the column sum is a compensated one): 5.86 -> 5.50 ms.
-constexpr int kResT = 2, kResCols = 10;
+//
+// Up to kResOne phenotypes a block takes one: with two, the FP64 chain of a block is twice as long
+// while SMs are idle. Preparing 1, 100, 304, 400 and 608 phenotypes at N = 23,000, q = 20 took 1,450,
+// 1,490, 1,700, 2,050 and 2,560 us with one per block against 1,800, 1,885, 1,930, 2,370 and 2,450
+// with two. A phenotype's arithmetic is the same either way.
+constexpr int kResCols = 10, kResOne = 3 * 152;
+template <int kResT>
 __global__ void __launch_bounds__(256) k_residualise(
     const float* __restrict__ Y, long long ldy, const double* __restrict__ Q, long long N, int P,
     int q, long long Npad, double* __restrict__ Yres, double* __restrict__ s_out,
@@ -607,7 +613,9 @@ cudaError_t launch_residualise(const float* Y, int64_t ldy, const double* Q, int
                                float* col_rmul, __nv_bfloat16* Bhi, __nv_bfloat16* Blo, float* B32,
                                float* col_cs, uint32_t* flags, cudaStream_t st) {
   if (P == 0) return cudaSuccess;
-  k_residualise<<<(unsigned)((P + kResT - 1) / kResT), 256, 0, st>>>(
+  const bool one = P <= kResOne;
+  const auto k = one ? k_residualise<1> : k_residualise<2>;
+  k<<<(unsigned)(one ? P : (P + 1) / 2), 256, 0, st>>>(
       Y, ldy, Q, N, (int)P, (int)q, Npad, Yres, s, col_s, col_rmul, Bhi, Blo, B32, col_cs, flags);
   return cudaGetLastError();
 }
