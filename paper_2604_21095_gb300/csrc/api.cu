@@ -198,11 +198,18 @@ cudaError_t ensure_operands(tg_ctx* c, int64_t M, int64_t Npad, int prec) {
   return cudaSuccess;
 }
 
-cudaError_t ensure_raw(tg_ctx* c, size_t floats) {
+// Room for `floats` raw products, or where the device has not that much for `least` (an unsplit
+// plan's): whoever asks looks at cap_raw.
+cudaError_t ensure_raw(tg_ctx* c, size_t floats, size_t least) {
   if (floats <= c->cap_raw) return cudaSuccess;
   dfree(c->raw);
   c->cap_raw = 0;
   cudaError_t e = dalloc(&c->raw, floats);
+  if (e == cudaErrorMemoryAllocation && least < floats) {
+    cudaGetLastError();
+    floats = least;
+    e = dalloc(&c->raw, floats);
+  }
   if (e == cudaSuccess) c->cap_raw = floats;
   return e;
 }
@@ -219,7 +226,7 @@ constexpr double kChunkUsCol = 0.0337;  // CTA-pair kernel, per chunk and column
 constexpr double kItemUs = 4.0;
 constexpr double kRangeBytesPerUs = 6.0e6;
 constexpr int64_t kPackedOperandBytes = 32 << 20;
-constexpr size_t kMaxSplitFloats = size_t(1) << 26;  // partial sums of a split: 256 MiB at most
+constexpr size_t kMaxSplitFloats = size_t(1) << 26;  // partial sums of ranges: 256 MiB at most (CTA pairs: twice)
 // How a CTA-pair pass of M markers and `cols` columns is split, by the shortest estimate: whole tiles
 // (per = 0; they waste nothing where their last wave is nearly full, and pieces of partial sums
 // cost memory), every tile in ks equal ranges (chunks rounded up to ks x per, one item per pair
@@ -427,19 +434,22 @@ tg_status reserve_graph_workspace(tg_ctx* c, const tg_panel* p, int n_blocks, co
                   "largest blocks first, or use another context");
     return TG_OK;
   }
-  size_t raw = 0;
-  for (int b = 0; b < n_blocks; ++b)
-    raw = std::max(raw, make_plan(c, p, p->N, M[b], encoding, missing ? missing[b] : nullptr, opts,
-                                  false).raw_floats);
+  size_t raw = 0, least = 0;
+  for (int b = 0; b < n_blocks; ++b) {
+    const uint32_t* ms = missing ? missing[b] : nullptr;
+    raw = std::max(raw, make_plan(c, p, p->N, M[b], encoding, ms, opts, false).raw_floats);
+    least = std::max(least, make_plan(c, p, p->N, M[b], encoding, ms, opts, true).raw_floats);
+  }
   TG_CUDA(ensure_markers(c, maxM));
   if (need_operand) TG_CUDA(ensure_operands(c, maxM, p->Npad, opts.precision));
-  // while the graph lives nothing grows: room for any unsplit pass over as many markers
-  TG_CUDA(ensure_raw(c, std::max(raw, (size_t)c->cap_m * JCOLS)));
+  // while the graph lives nothing grows: room for any unsplit pass over as many markers, or at the
+  // least for this graph's
+  TG_CUDA(ensure_raw(c, std::max(raw, (size_t)c->cap_m * JCOLS), least));
   return TG_OK;
 }
 
-// The plan of a scan. While a captured graph holds the workspace, a scan whose split passes need more
-// room for their partial sums than there is runs unsplit.
+// The plan of a scan. While a captured graph holds the workspace (or is being captured), a scan whose
+// split passes need more room for their partial sums than there is runs unsplit.
 Plan plan_scan(const tg_ctx* c, const tg_panel* p, const ScanArgs& a) {
   Plan r = make_plan(c, p, a.N, a.M, a.encoding, a.missing, a.opts, false);
   if (c->graphs_alive > 0 && r.raw_floats > c->cap_raw)
@@ -546,7 +556,7 @@ tg_status scan_fp4(tg_ctx* c, tg_panel* p, const ScanArgs& a, cudaStream_t st) {
   if (c->graphs_alive > 0 && (a.M > c->cap_m || need > c->cap_fp4 || raw > c->cap_raw))
     return fail(TG_ERR_INVALID_ARG, "the context's workspace is held by a captured scan graph");
   TG_CUDA(ensure_markers(c, a.M));
-  TG_CUDA(ensure_raw(c, raw));
+  TG_CUDA(ensure_raw(c, raw, raw));
   if (need > c->cap_fp4) {
     dfree(c->Afp4);
     c->Afp4 = nullptr;
@@ -635,9 +645,7 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
   if (a.M == 0) return TG_OK;
   if (a.opts.precision == TG_PREC_FP4_PIECES) return scan_fp4(c, p, a, st);
   const int prec = a.opts.precision;
-  const Plan pl = plan_scan(c, p, a);
-  const bool split = pl.split, joint = pl.joint;
-  const int64_t nq = pl.nq;
+  Plan pl = plan_scan(c, p, a);
   if (c->graphs_alive > 0 &&
       (a.M > c->cap_m || pl.raw_floats > c->cap_raw ||
        (pl.operand && !operand_fits(c, a.M, p->Npad, prec))))
@@ -646,7 +654,13 @@ tg_status scan_impl(tg_ctx* c, const tg_panel* pc, const ScanArgs& a, cudaStream
                 "larger than the graph's, or use another context");
   TG_CUDA(ensure_markers(c, a.M));
   if (pl.operand) TG_CUDA(ensure_operands(c, a.M, p->Npad, prec));
-  TG_CUDA(ensure_raw(c, pl.raw_floats));
+  if (pl.raw_floats > c->cap_raw) {
+    const Plan whole = make_plan(c, p, a.N, a.M, a.encoding, a.missing, a.opts, true);
+    TG_CUDA(ensure_raw(c, pl.raw_floats, whole.raw_floats));
+    if (pl.raw_floats > c->cap_raw) pl = whole;  // no room for a split's partial sums
+  }
+  const bool split = pl.split, joint = pl.joint;
+  const int64_t nq = pl.nq;
   const double kappa64 = a.encoding == TG_ENC_U8_DOSAGE ? 2.0 / 255.0 : 1.0;
   const float kappa = (float)kappa64;
   const bool u8 = a.encoding == TG_ENC_U8_DOSAGE;
@@ -1802,6 +1816,7 @@ tg_status tg_scan_graph_create(tg_ctx* c, const tg_panel* p, int n_blocks,
   const bool prof = c->prof;
   c->prof = false;
   tg_status s = TG_OK;
+  c->graphs_alive += 1;  // nothing may grow from here on
   cudaError_t e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
     for (int b = 0; b < n_blocks && s == TG_OK; ++b) {
@@ -1823,9 +1838,9 @@ tg_status tg_scan_graph_create(tg_ctx* c, const tg_panel* p, int n_blocks,
     if (g->exec) cudaGraphExecDestroy(g->exec);
     if (g->graph) cudaGraphDestroy(g->graph);
     delete g;
+    c->graphs_alive -= 1;
     return s != TG_OK ? s : cuda_fail(e, "tg_scan_graph_create capture");
   }
-  c->graphs_alive += 1;
   *graph = g;
   return TG_OK;
 }
@@ -1893,6 +1908,7 @@ tg_status tg_scan_graph_create_host(tg_ctx* c, const tg_panel* p, int n_blocks,
   const bool prof = c->prof;
   c->prof = false;
   tg_status s = TG_OK;
+  c->graphs_alive += 1;  // nothing may grow from here on
   e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
   if (e == cudaSuccess) {
     auto step = [&]() -> tg_status {
@@ -1932,8 +1948,10 @@ tg_status tg_scan_graph_create_host(tg_ctx* c, const tg_panel* p, int n_blocks,
   }
   if (s == TG_OK && (e = cudaGraphInstantiate(&g->exec, g->graph, 0)))
     s = cuda_fail(e, "tg_scan_graph_create_host instantiate");
-  if (s != TG_OK) return release(s);
-  c->graphs_alive += 1;
+  if (s != TG_OK) {
+    c->graphs_alive -= 1;
+    return release(s);
+  }
   *graph = g;
   return release(TG_OK);
 }

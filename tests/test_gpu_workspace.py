@@ -45,3 +45,52 @@ def test_fp4_scan_leaves_a_captured_graphs_buffers_alone():
         tg.tg_destroy(ctx)
     assert before.all() and np.array_equal(best.cpu().numpy(), before)
     assert np.array_equal(again["best_key"], first["best_key"])
+
+
+def test_scans_and_graphs_run_unsplit_where_memory_is_short():
+    """A block whose passes are split would need 362 MB for their partial sums, unsplit half of
+    that: with room for the half alone it is scanned, and captured, unsplit. (1,100 samples are two
+    accumulation chunks, so an even split over the SMs cuts some tiles in two.)"""
+    N, P, M, n_cov = 1100, 110, 400_000, 3
+    whole = 4 * (P + n_cov) * M
+    gen = torch.Generator(device="cuda").manual_seed(4)
+    G = torch.randint(0, 256, (M, 288), generator=gen, dtype=torch.uint8, device="cuda")
+    cov = synth.covariates(31, N, n_cov)
+    Yt = synth.phenotypes(32, cov, P)
+    best = torch.zeros(P, dtype=torch.int64, device="cuda")
+    out = tg.make_outputs(best=best)
+    opts = tg.tg_scan_opts(tg.TG_PREC_SPLIT_BF16, 0, 0.0)
+    filler, res = None, []
+    for short in (False, True):
+        ctx = tg.tg_create(0)
+        panel = tg.tg_prepare_panel(ctx, Yt.cuda(), N, P, cov.cuda())
+        graph = None
+        try:
+            tg.tg_set_fused_decode(ctx, True)  # (a graph then reserves no decoded operand)
+            tg.tg_scan_block(ctx, panel, G[:256], N, 256, tg.TG_ENC_2BIT, opts, out)
+            torch.cuda.synchronize()
+            torch.cuda.empty_cache()
+            if short:  # room for the marker arrays (under 100 bytes each) and the unsplit products
+                room = whole + 100 * M + (32 << 20)
+                assert room < 2 * whole
+                filler = torch.empty(torch.cuda.mem_get_info()[0] - room, dtype=torch.uint8,
+                                     device="cuda")
+            for captured in (False, True):
+                best.zero_()
+                if captured:
+                    graph = tg.tg_scan_graph_create(ctx, panel, [G], N, tg.TG_ENC_2BIT, opts, out, [0])
+                    tg.tg_scan_graph_launch(graph)
+                else:
+                    tg.tg_scan_block(ctx, panel, G, N, M, tg.TG_ENC_2BIT, opts, out)
+                assert tg.tg_status_poll(ctx) == tg.TG_OK
+                res.append(best.cpu().numpy().view(np.uint64).copy())
+        finally:
+            filler = None
+            torch.cuda.empty_cache()
+            if graph is not None:
+                tg.tg_scan_graph_free(graph)
+            tg.tg_panel_free(panel)
+            tg.tg_destroy(ctx)
+    for keys in res[1:]:  # |r| in the upper half; two partial sums of chunks or one, in the same order
+        absr = [(k >> 32).astype(np.uint32).view(np.float32) for k in (keys, res[0])]
+        np.testing.assert_allclose(absr[0], absr[1], atol=1e-6, rtol=0)
