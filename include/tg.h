@@ -392,7 +392,9 @@ tg_status tg_scan_graph_free(tg_graph* graph);
 /* Time the tensor-core scan of an M-marker block of this panel with each candidate kernel
  * (CTA pairs on 256 x 256 tiles, or one CTA per 128 x 256 tile) and raster group, on a
  * pseudo-random block, and keep the fastest for blocks of this size (same power of two) in the
- * context. Synchronous; allocates a temporary block. */
+ * context. Scans that do not look at the choice are not timed: a panel of at most 64 phenotypes
+ * leaves it as it is, and one whose phenotypes and covariate columns share one pass
+ * (P + q - 1 <= 512) is timed in the paper's mode. Synchronous; allocates a temporary block. */
 tg_status tg_autotune(tg_ctx* ctx, const tg_panel* panel, int32_t encoding, int64_t M,
                       void* stream);
 /* The tuned choice for M-marker blocks: kernel 2 = CTA pairs, 1 = one CTA per tile; group =

@@ -1983,6 +1983,13 @@ tg_status tg_autotune(tg_ctx* c, const tg_panel* p, int32_t encoding, int64_t M,
   TG_ARG(c && p && M > 0, "bad arguments");
   TG_ARG(encoding == TG_ENC_2BIT || encoding == TG_ENC_U8_DOSAGE, "unknown encoding");
   TG_CUDA(cudaSetDevice(c->device));
+  // Scans of at most 64 phenotypes, and projected ones whose phenotypes and covariate columns share
+  // a pass, do not look at the choice: their candidates would be ranked by noise, and the winner
+  // kept for other panels of the bucket. The first have nothing to tune, the others their scans in
+  // the paper's mode.
+  if (p->P <= 64) return TG_OK;
+  tg_scan_opts opts{TG_PREC_SPLIT_BF16, 0, 7.30103};
+  if (make_plan(c, p, p->N, M, encoding, nullptr, opts, false).joint) opts.mode = TG_MODE_PAPER;
   cudaStream_t st = (cudaStream_t)stream;
   const int64_t ldg = round_up(encoding == TG_ENC_2BIT ? (p->N + 3) / 4 : p->N, 16);
   uint8_t* G = nullptr;
@@ -2010,17 +2017,15 @@ tg_status tg_autotune(tg_ctx* c, const tg_panel* p, int32_t encoding, int64_t M,
   o.hit_capacity = kTrialHits;
   o.n_hits = cnt;
   o.best = best;
-  const tg_scan_opts opts{TG_PREC_SPLIT_BF16, 0, 7.30103};
   ScanArgs a{G, ldg, encoding, p->N, M, 0, nullptr, 0, opts, o};
   const int b = tune_bucket(M);
-  // kernel, raster group, split-K (the one-CTA kernel splits K when its tiles are fewer than
-  // the SMs; panels of at most 64 phenotypes take 64-column tiles whatever the choice)
+  // kernel, raster group, split-K (the one-CTA kernel splits K when its tiles are fewer than the SMs)
   const int kinds[] = {TUNE_PAIR, TUNE_PAIR, TUNE_PAIR, TUNE_PAIR, TUNE_SINGLE, TUNE_SINGLE,
                        TUNE_SINGLE, TUNE_SINGLE, TUNE_SINGLE};
   const int groups[] = {4, 8, 16, 32, 8, 16, 32, 16, 16};
   const int splits[] = {1, 1, 1, 1, 1, 1, 1, 2, 4};
   const int64_t single_tiles = ((M + MT - 1) / MT) * ((p->P + 255) / 256);
-  const int n_cand = p->P > 64 && single_tiles * 2 <= c->sm_count ? 9 : 7;
+  const int n_cand = single_tiles * 2 <= c->sm_count ? 9 : 7;
   const int save_k = c->tune_kernel[b], save_g = c->tune_group[b], save_s = c->tune_split[b];
   const bool prof = c->prof;
   // the trial launches do not count in the caller's stage statistics

@@ -94,3 +94,25 @@ def test_scans_and_graphs_run_unsplit_where_memory_is_short():
     for keys in res[1:]:  # |r| in the upper half; two partial sums of chunks or one, in the same order
         absr = [(k >> 32).astype(np.uint32).view(np.float32) for k in (keys, res[0])]
         np.testing.assert_allclose(absr[0], absr[1], atol=1e-6, rtol=0)
+
+
+@pytest.mark.parametrize("P,tuned", [(40, False), (300, True)])
+def test_autotune_keeps_no_choice_that_the_scans_ignore(tmp_path, P, tuned):
+    """A panel of at most 64 phenotypes has no kernel to choose, so tuning it leaves the context's
+    choice for the block size as it was; one with a joint pass is tuned for the paper's mode."""
+    N, M = 1500, 700
+    cov = synth.covariates(85, N, 3)
+    ctx = tg.tg_create(0)
+    panel = tg.tg_prepare_panel(ctx, synth.phenotypes(85, cov, P).cuda(), N, P, cov.cuda())
+    try:
+        tg.tg_autotune(ctx, panel, tg.TG_ENC_2BIT, M)
+        path = tmp_path / "tuning.json"
+        tg.tg_tuning_save(ctx, str(path))
+        assert ("min_markers" in path.read_text()) == tuned
+        if not tuned:
+            tg.tg_set_tuning(ctx, M, "single", 8)
+            tg.tg_autotune(ctx, panel, tg.TG_ENC_2BIT, M)
+            assert tg.tg_tuning(ctx, M) == {"kernel": "single", "group_m": 8}
+    finally:
+        tg.tg_panel_free(panel)
+        tg.tg_destroy(ctx)
