@@ -137,10 +137,11 @@ tg_status tg_destroy(tg_ctx* ctx);
  * Builds X = [1, C], an orthonormal basis Q of span(X) by FP64 Householder QR (a column
  * whose remaining norm is <= 1e-9 of its own norm is dropped; q = rank), the residualised
  * panel Y_res = (I - Q Q^T)(Y - Ybar) in FP64, the column norms s_p = |y_res,p| and the
- * unit-norm panel in the forms the scan consumes. A panel with P + q - 1 <= 256 also keeps a
- * joint copy of its split operand behind the q - 1 projection columns (64, 128 or 256 rows of
- * round_up(N, 64) bf16 pairs), so that split-form scans in the projected mode take the
- * projection and the panel's products from one pass over each block.
+ * unit-norm panel in the forms the scan consumes. A panel with P + q - 1 <= 512 also keeps a
+ * joint copy of its split operand behind the q - 1 projection columns (64 or 128 rows of
+ * round_up(N, 64) bf16 pairs, and as many of f16 pairs, or above 128 columns one or two tiles of
+ * equal width), so that split-form scans in the projected mode take the projection and the
+ * panel's products from one pass over each block.
  *   Y: device, float [P][ldy] storage = column-major N x P (phenotype p at Y + p*ldy), ldy >= N.
  *   C: device, double column-major N x n_cov (covariate k at C + k*ldc), ldc >= N; NULL if n_cov = 0.
  *      The intercept is added by the library and must not be passed.
@@ -228,7 +229,9 @@ tg_status tg_decode_block(tg_ctx* ctx, const uint8_t* G, int64_t ldg, int32_t en
  *   marker_offset: global index of the block's first marker (used in hits and best).
  *   opts: precision, full output and hit threshold. out: see tg_outputs.
  * Workspace is grown on demand (cudaMalloc); a call with a larger M than any before may
- * therefore synchronise the device. M = 0 is a no-op. */
+ * therefore synchronise the device. Passes with few tiles split the sample axis and leave up to
+ * 512 MiB of partial sums; where the device has not that much memory left they run unsplit.
+ * M = 0 is a no-op. */
 tg_status tg_scan_block(tg_ctx* ctx, const tg_panel* panel, const uint8_t* G, int64_t ldg,
                         int32_t encoding, int64_t N, int64_t M, int64_t marker_offset,
                         const uint32_t* missing, int64_t ldm, const tg_scan_opts* opts,
@@ -317,27 +320,30 @@ tg_status tg_host_block_sizes(int64_t M, int64_t block_markers, double factor, i
 /* Where split-form scans decode the genotypes inside the contraction kernels instead of first
  * writing the decoded operand (about 2 x round_up(N, 64) bytes per marker) to device memory.
  * The fused forms apply to 2-bit blocks and to dosage blocks without a missing mask (others always
- * use the decoded operand). They compute bit-identical results, except the small-panel pass on
- * dosage blocks (enable = 2 or 1), which expands the bytes into f16 (b - c exactly) against an
- * f16 hi + lo copy of the joint operand (about 22 significant bits against bf16's 16): its
- * results differ from the decoded operand's within the float tolerance.
+ * use the decoded operand). Their products are those of the decoded operand, added up in chunks of
+ * 1,024 samples as there; a pass that splits the sample axis adds the sums of its ranges, so r may
+ * differ in its last bits from a pass that splits it elsewhere (up to two chunks, N <= 2,048, it
+ * does not). Dosage rows differ within the float tolerance where they are expanded into f16 (b - c
+ * exactly) against an f16 hi + lo copy of the operand (about 22 significant bits against bf16's
+ * 16): in the passes of enable = 2 on blocks of at least one 128-marker tile per SM.
  *   enable = 2 (the default): only the joint projection pass of a small panel (projected mode,
- *     P + q - 1 <= 128, blocks of at least one 128-marker tile per SM), where the scan is one pass
- *     bound by the bytes it reads: the pass reads the packed rows (1 or 1/4 byte per sample)
- *     and decodes them on chip with 8 decoder warps, removing the operand's write and read
- *     (Section 2.4: the scan is bound by the reader's bandwidth). A counting pass over the rows
+ *     P + q - 1 <= 128, blocks of at least one 128-marker tile per SM or whose decoded operand would
+ *     take 32 MiB or more), where the scan is one pass bound by the bytes it reads: the pass reads
+ *     the packed rows (1 or 1/4 byte per sample) and decodes them on chip with 16 decoder warps,
+ *     removing the operand's write and read (Section 2.4: the scan is bound by the reader's
+ *     bandwidth). A counting pass over the rows
  *     (n_obs, sums, the mean each row is centred on) comes first, except for dosage rows on
- *     256-marker tiles (blocks of at least 256 markers per SM, N <= 66,051): there the pass
+ *     blocks of at least 256 markers per SM (N <= 66,051): there the pass
  *     centres each row on the rounded mean of its first 64 bytes and takes the row's exact
  *     sums as it expands it, so the block is read once. The statistics are the same integers
  *     and the same FP64 mean either way.
- *   The same setting runs a larger panel's projection (P + q - 1 > 128; same conditions
+ *   The same setting runs a larger panel's projection (P + q - 1 > 512; same conditions
  *     otherwise) as that pass with the q - 1 projection columns alone, which also writes the
  *     block's decoded operand as it expands the rows (the contraction of the panel then reads
  *     it): the operand is written once and read once instead of read a second time for the
- *     projection. Dosage rows take f16 projection columns there and, on 256-marker tiles, the
- *     one-pass statistics above; 2-bit calls give results bit-identical to enable = 0 for
- *     panels with P + q - 1 > 256.
+ *     projection. Dosage rows take the f16 projection columns and the one-pass statistics there on
+ *     the same blocks as above. (Panels of 128 < P + q - 1 <= 512 take one joint pass over the
+ *     decoded operand.)
  *   enable = 1: also the contraction kernels of larger panels, whose two decoder warps per CTA
  *     take about 3,000 cycles per 32-sample K block against 512 for the products, so on GB300
  *     they are slower there.

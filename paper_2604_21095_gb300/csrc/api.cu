@@ -365,7 +365,12 @@ Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int enc
     r.one_pass = r.f16 && N <= kOnePassMaxN && (M + kFusedRows - 1) / kFusedRows >= c->sm_count;
   }
   // P + q - 1 <= JCOLS: one pass over the operand gives the projection and the panel's products
-  // (raw); the statistics follow the norms
+  // (raw); the statistics follow the norms. Above 128 columns (two CTA-pair tiles hold JCOLS; a third
+  // would cost more raw products than the projection pass it saves) against the pass that writes
+  // the operand and the panel's own contraction, 65,536 dosage rows of 23,000 samples, 19
+  // covariates: P = 150 1,398 us against 1,598, 256 1,875 against 1,805, 300 1,900 against 2,062, 400
+  // 2,180 against 2,295, 490 2,390 against 2,480. (40,000 rows of 5,000 samples, P = 400: 478 against
+  // 444.)
   r.joint = r.split && r.nq > 0 && p->joint_cols > 0;
   // (one chunk: nothing to split)
   const int64_t chunks = whole ? 1 : (p->Npad / 32 + kAccumChunkKB - 1) / kAccumChunkKB;

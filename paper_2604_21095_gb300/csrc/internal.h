@@ -367,7 +367,6 @@ cudaError_t launch_subset_stats(const uint8_t* G, int64_t ldg, int encoding, int
                                 const double* mean, const int32_t* nobs, const int64_t* S,
                                 double* gc2s, cudaStream_t st);
 
-// SIMT kernels (k_simt.cu)
 // The CTA-pair kernel's units (one 256 x bn tile x one accumulation chunk) and their even split over
 // the pairs: pair w takes the units [w per, (w + 1) per), tile (m-tile pair t / n_nt, column tile
 // t % n_nt) holding the units t chunks .., so at most `pieces` pairs share a tile. chunks may be more
@@ -408,6 +407,7 @@ struct RowSums {
 // The statistics of `sums` on their own, where something reads the means before the norms.
 cudaError_t launch_row_statistics(int64_t M, const RowSums& sums, const RawView& raw,
                                   cudaStream_t st);
+// SIMT kernels (k_simt.cu)
 // Projections of the FP32 operand, column-major: out[k * ldq + m], range r of K `split` floats on.
 cudaError_t launch_project(const float* A, int64_t lda, int64_t M, int64_t K, const float* QB,
                            int64_t nq, float* out, int64_t ldq, cudaStream_t st, int ranges = 1,

@@ -269,15 +269,15 @@ __device__ __forceinline__ void expand32(uint32_t slot, int r, int q, uint2 k, b
   }
 }
 
-// Write a stage of the block's bf16 operand from the expanded rows of one decoder warp: lane l
-// holds 32 samples of row l of the warp's 32 (16 words, two 16-bit values each). The rows go through the warp's staging area in shared memory (`stg`, 32 rows of
-// 64 bytes; 16-byte chunk c of row l at chunk c ^ ((l >> 1) & 3), which keeps each quarter warp on
-// distinct banks both ways), then each store instruction writes 8 rows of 64 bytes, whole
-// segments, instead of 32 scattered 16-byte pieces. Row l
-// goes to dst0 + l * ld (16-byte aligned); rows at or past `rows` are skipped.
-// 2-bit values are bf16 already. Dosage values are f16 of b - c, integers of magnitude at most
-// 255 (or 0 past N), which bf16 holds exactly, so the conversion through f32 is exact and gives
-// the decoded operand's bits.
+// Write one K block of a stage to the block's bf16 operand from the expanded rows of one decoder
+// warp: lane l holds 32 samples of row l of the warp's 32 (16 words, two 16-bit values each). The
+// rows go through the warp's staging area in shared memory (`stg`, 32 rows of 64 bytes; 16-byte
+// chunk c of row l at chunk c ^ ((l >> 1) & 3), which keeps each quarter warp on distinct banks
+// both ways), then each store instruction writes 8 rows of 64 bytes, whole segments, instead of
+// 32 scattered 16-byte pieces. Row l goes to dst0 + l * ld (16-byte aligned); rows at or past
+// `rows` are skipped. The bf16 forms' values go out as they are; the f16 form's are b - c,
+// integers of magnitude at most 255 (or 0 past N), which bf16 holds exactly, so the conversion
+// through f32 is exact and gives the decoded operand's values.
 template <int OPA>
 __device__ __forceinline__ void store_operand_warp(uint32_t stg, const uint32_t (&o)[16], int lane,
                                                    __nv_bfloat16* dst0, long long ld, int rows) {
