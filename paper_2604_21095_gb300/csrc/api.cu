@@ -331,6 +331,7 @@ struct Plan {
   bool operand = false;     // the decoded operand is needed
 };
 
+// The plan of a block of M >= 1 markers.
 // whole: no pass is split, so that the raw products take at most JCOLS columns of the block's rows.
 Plan make_plan(const tg_ctx* c, const tg_panel* p, int64_t N, int64_t M, int encoding,
                const uint32_t* missing, const tg_scan_opts& opts, bool whole) {
@@ -441,6 +442,7 @@ tg_status reserve_graph_workspace(tg_ctx* c, const tg_panel* p, int n_blocks, co
   }
   size_t raw = 0, least = 0;
   for (int b = 0; b < n_blocks; ++b) {
+    if (M[b] == 0) continue;  // an empty block is no scan and has no plan
     const uint32_t* ms = missing ? missing[b] : nullptr;
     raw = std::max(raw, make_plan(c, p, p->N, M[b], encoding, ms, opts, false).raw_floats);
     least = std::max(least, make_plan(c, p, p->N, M[b], encoding, ms, opts, true).raw_floats);

@@ -116,3 +116,32 @@ def test_autotune_keeps_no_choice_that_the_scans_ignore(tmp_path, P, tuned):
     finally:
         tg.tg_panel_free(panel)
         tg.tg_destroy(ctx)
+
+
+@pytest.mark.parametrize("precision", [tg.TG_PREC_FP32, tg.TG_PREC_SPLIT_BF16])
+def test_graph_with_empty_blocks(precision):
+    """Empty blocks are accepted and add nothing. (Their plan divided by their number of tiles in the
+    FP32 form, which ends the process on hosts whose integer division traps.)"""
+    N, P, M = 900, 5, 300
+    gen = torch.Generator(device="cuda").manual_seed(6)
+    G = torch.randint(0, 256, (M, 240), generator=gen, dtype=torch.uint8, device="cuda")
+    cov = synth.covariates(41, N, 2)
+    ctx = tg.tg_create(0)
+    panel = tg.tg_prepare_panel(ctx, synth.phenotypes(42, cov, P).cuda(), N, P, cov.cuda())
+    got = []
+    try:
+        for blocks, offsets in (([G], [0]), ([G[:0], G[:100], G[100:100], G[100:]], [0, 0, 100, 100])):
+            best = torch.zeros(P, dtype=torch.int64, device="cuda")
+            graph = tg.tg_scan_graph_create(ctx, panel, blocks, N, tg.TG_ENC_2BIT,
+                                            tg.tg_scan_opts(precision, 0, 0.0),
+                                            tg.make_outputs(best=best), offsets)
+            try:
+                tg.tg_scan_graph_launch(graph)
+                torch.cuda.synchronize()
+            finally:
+                tg.tg_scan_graph_free(graph)
+            got.append(best.cpu().numpy())
+    finally:
+        tg.tg_panel_free(panel)
+        tg.tg_destroy(ctx)
+    assert got[0].all() and np.array_equal(got[0], got[1])
